@@ -8,7 +8,7 @@ HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 OUT_DIR = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libttn.so")
-SOURCES = ["ttn.cu", "gemm_f64.cu", "gemm_split.cu", "kernels.cu", "qr.cu", "noalloc.cu", "svd.cu", "sample.cu"]
+SOURCES = ["ttn.cu", "gemm_f64.cu", "gemm_split.cu", "gemm_digits.cu", "kernels.cu", "qr.cu", "noalloc.cu", "svd.cu", "sample.cu"]
 NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 FLAGS = ["-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-lineinfo", "-std=c++17",
          "-Xcompiler", "-fPIC", "--expt-relaxed-constexpr", "-I" + os.path.join(HERE, "..", "include")]
@@ -17,7 +17,8 @@ FLAGS = ["-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-lineinfo", "-std
 def _compile(src):
     obj = os.path.join(OUT_DIR, src.replace(".cu", ".o"))
     srcp = os.path.join(CSRC, src)
-    deps = [srcp, os.path.join(CSRC, "common.cuh"), os.path.join(HERE, "..", "include", "ttn.h")]
+    deps = [srcp, os.path.join(CSRC, "common.cuh"), os.path.join(CSRC, "tcgen05.cuh"),
+            os.path.join(HERE, "..", "include", "ttn.h")]
     if os.path.exists(obj) and all(os.path.getmtime(obj) >= os.path.getmtime(d) for d in deps):
         return obj
     cmd = [NVCC] + FLAGS + ["-c", srcp, "-o", obj]

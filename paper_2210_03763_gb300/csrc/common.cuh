@@ -25,6 +25,15 @@ struct GemmArgs {
 // tiles cannot fill the GPU split K into ranges summed in fixed order.
 int launch_zgemm_f64(const GemmArgs& g, cudaStream_t stream, void* workspace = nullptr, size_t workspace_bytes = 0);
 size_t f64_workspace_bytes(const GemmArgs& g);
+// C = alpha sum_ks W[ks] + beta C, W[((ks * Bo + bo) * Bi + bi) * M * N + m + n M].
+int launch_splitk_f64(const GemmArgs& g, int nsplit, const cplx* W, cudaStream_t stream);
+// The same contraction by exact digit products on the tensor cores
+// (gemm_digits.cu): whether it pays for this shape, its workspace (first int:
+// the error flag a timed-out wait sets), and the launch (kernels launched; -1
+// when it is not handled there, -2 when the workspace is too small).
+bool digits_wanted(const GemmArgs& g);
+size_t digits_workspace_bytes(const GemmArgs& g);
+int launch_zgemm_digits(const GemmArgs& g, cudaStream_t stream, void* workspace, size_t workspace_bytes);
 
 // ---- split-precision building blocks (gemm_split.cu) -------------------------
 // Packing of one side of a split contraction into TF32 hi/lo planes: complex

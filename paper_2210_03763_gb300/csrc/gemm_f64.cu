@@ -348,9 +348,12 @@ int launch_zgemm_f64(const GemmArgs& g, cudaStream_t stream, void* workspace, si
     if (bm == 16) launch_n<16>(g, stream, bn, ns, ks_len, W);
     else if (bm == 32) launch_n<32>(g, stream, bn, ns, ks_len, W);
     else launch_n<64>(g, stream, bn, ns, ks_len, W);
-    if (ns == 1) return 1;
+    return ns == 1 ? 1 : 1 + launch_splitk_f64(g, ns, W, stream);
+}
+
+int launch_splitk_f64(const GemmArgs& g, int nsplit, const cplx* W, cudaStream_t stream) {
     const long long total = (long long)g.M * g.N * g.Bi * g.Bo;
     const unsigned grid = (unsigned)std::min<long long>((total + 255) / 256, 152 * 8);
-    splitk_f64_kernel<<<grid, 256, 0, stream>>>(g, ns, W);
-    return 2;
+    splitk_f64_kernel<<<grid, 256, 0, stream>>>(g, nsplit, W);
+    return 1;
 }

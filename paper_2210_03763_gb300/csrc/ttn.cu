@@ -159,8 +159,9 @@ struct ttn_ctx {
     std::vector<ProfRec> prof;
     std::vector<cudaEvent_t> ev_pool;
     size_t ev_next = 0;
-    void* split_ws = nullptr;   // packed operands of the split GEMM (+ error flag)
+    void* split_ws = nullptr;   // packed operands of the tensor-core GEMMs (+ error flag)
     size_t split_cap = 0;
+    bool digits_run = false;    // an FP64 contraction ran on the tensor cores since the flag was last read
     void* f64_ws = nullptr;     // split-K partial sums of FP64 contractions
     size_t f64_cap = 0;
     // split-precision H_eff of one node visit (see SplitHeff): per leg the
@@ -229,8 +230,8 @@ long long ipow3_capped(int k, long long cap) {
 int leg_dim(const ttn_ctx* c, int k, int leg) { return c->nodes[k].d[leg]; }
 
 // ------------------------------------------------------------------ GEMMs
-void grow_split_ws(ttn_ctx* c, size_t bytes) {
-    if (bytes <= c->split_cap) return;
+bool try_grow_split_ws(ttn_ctx* c, size_t bytes) {
+    if (bytes <= c->split_cap) return true;
     CUDA_OK(cudaStreamSynchronize(c->stream));
     int flag = 0;
     if (c->split_ws) {
@@ -240,10 +241,18 @@ void grow_split_ws(ttn_ctx* c, size_t bytes) {
         c->split_cap = 0;
     }
     size_t cap = bytes + bytes / 4;
-    if (test_take_alloc_fail() || cudaMalloc(&c->split_ws, cap) != cudaSuccess)
-        throw TtnError(TTN_ERR_ALLOC, "split workspace");
+    if (test_take_alloc_fail() || cudaMalloc(&c->split_ws, cap) != cudaSuccess) {
+        c->split_ws = nullptr;
+        cudaGetLastError();   // reported by the caller, not by a later check
+        return false;
+    }
     CUDA_OK(cudaMemcpy(c->split_ws, &flag, sizeof(int), cudaMemcpyHostToDevice));
     c->split_cap = cap;
+    return true;
+}
+
+void grow_split_ws(ttn_ctx* c, size_t bytes) {
+    if (!try_grow_split_ws(c, bytes)) throw TtnError(TTN_ERR_ALLOC, "split workspace");
 }
 
 // Profile kinds: 0 tensor-core GEMM, 1 split packing, 2 FP64 GEMM, 3 QR,
@@ -327,6 +336,14 @@ void gemm(ttn_ctx* c, const GemmArgs& g) {
             }
         }
     }
+    if (n < 0 && digits_wanted(g)) {   // large FP64 contractions: exact digit products on the tensor cores
+        const size_t need = digits_workspace_bytes(g);
+        if (try_grow_split_ws(c, need)) {   // no room: the FP64 kernels below need none
+            ProfScope ps(c, PK_F64, fl, 0.0, &g);
+            n = launch_zgemm_digits(g, c->stream, c->split_ws, c->split_cap);
+            if (n >= 0) c->digits_run = true;
+        }
+    }
     if (n < 0) {
         const size_t wb = f64_workspace_bytes(g);
         if (wb > c->f64_cap) {   // split-K partials of small-output FP64 contractions
@@ -358,6 +375,13 @@ void check_split_flag(ttn_ctx* c) {
         CUDA_OK(cudaMemcpy(c->split_ws, &zero, sizeof(int), cudaMemcpyHostToDevice));
         throw TtnError(TTN_ERR_TIMEOUT, "tensor-core GEMM pipeline wait timed out");
     }
+    c->digits_run = false;
+}
+
+// The same at the end of a call that contracts in FP64 only: nothing to read
+// unless one of its contractions ran on the tensor cores.
+void check_digits(ttn_ctx* c) {
+    if (c->digits_run) check_split_flag(c);
 }
 
 GemmArgs base_args() {
@@ -1716,6 +1740,7 @@ void root_expect(ttn_ctx* c, const cplx* st0, int n0, const cplx* st1, int n1, s
     std::vector<cplx> h(n0 + n1);
     CUDA_OK(cudaMemcpyAsync(h.data(), res, sizeof(cplx) * (n0 + n1), cudaMemcpyDeviceToHost, c->stream));
     CUDA_OK(cudaStreamSynchronize(c->stream));
+    check_digits(c);
     for (int i = 0; i < n0 + n1; ++i) out[i] = zc(h[i].x, h[i].y);
 }
 
@@ -1726,6 +1751,7 @@ double root_norm(ttn_ctx* c) {
     cplx h;
     CUDA_OK(cudaMemcpyAsync(&h, c->Gbuf[2], sizeof(cplx), cudaMemcpyDeviceToHost, c->stream));
     CUDA_OK(cudaStreamSynchronize(c->stream));
+    check_digits(c);
     return h.x;
 }
 
@@ -1825,6 +1851,7 @@ zc overlap(ttn_ctx* psi, const ttn_ctx* tgt) {
     CUDA_OK(cudaMemcpyAsync(&h, M[c->root], sizeof(cplx), cudaMemcpyDeviceToHost, c->stream));
     CUDA_OK(cudaStreamSynchronize(c->stream));
     for (void* p : temp) cudaFree(p);
+    check_digits(c);
     return zc(h.x, h.y);
 }
 
@@ -1848,6 +1875,7 @@ double energy(ttn_ctx* c) {
     cplx h;
     CUDA_OK(cudaMemcpyAsync(&h, c->Gbuf[2], sizeof(cplx), cudaMemcpyDeviceToHost, c->stream));
     CUDA_OK(cudaStreamSynchronize(c->stream));
+    check_digits(c);
     return h.x;
 }
 
@@ -3008,6 +3036,7 @@ void transition_rdms(ttn_ctx* ket, ttn_ctx* bra, std::vector<zc>& out, std::vect
     for (int l = 0; l < c->n_leaves; ++l)
         CUDA_OK(cudaMemcpyAsync(h.data() + 9 * l, dn[nn + l], 9 * sizeof(cplx), cudaMemcpyDeviceToHost, c->stream));
     CUDA_OK(cudaStreamSynchronize(c->stream));
+    check_digits(c);
     out.assign(9 * (size_t)c->N, zc(0.0));
     for (int l = 0; l < c->n_leaves; ++l) {
         const int a = c->leaf_atom[l];
