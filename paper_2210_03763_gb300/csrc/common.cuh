@@ -119,6 +119,13 @@ constexpr int RED_BLOCKS = 304;     // 2 x 152 SMs
 constexpr int RED_THREADS = 256;
 constexpr int KRYLOV_MMAX = 30;
 
+struct KrylovStatus {
+    double err;          // a-posteriori error estimate
+    int    converged;
+    int    nonfinite;
+    int    iters;        // one-launch runs of small nodes: Krylov steps taken
+    int    pad;
+};
 struct KrylovScalars {
     double alpha[KRYLOV_MMAX];
     double beta[KRYLOV_MMAX + 1];
@@ -126,37 +133,37 @@ struct KrylovScalars {
     cplx   c[KRYLOV_MMAX];          // exp(z T_j) e_1
     double nrm0;                    // norm of the start vector
     double inv_scale;               // 1 / beta_j used to normalise v_{j+1}
-    double err;                     // a-posteriori error estimate
-    int    converged;
-    int    nonfinite;
-    cplx   hess[KRYLOV_MMAX + 1][KRYLOV_MMAX];   // Arnoldi: Hessenberg matrix H(i, j) at [i][j]
+    KrylovStatus st;
+    unsigned arrived;               // blocks of the second pass that have finished
+    cplx   hess[KRYLOV_MMAX][32];   // Arnoldi: Hessenberg matrix H(i, j) at [j][i]
 };
 
 int red_blocks_for(long long n);
 int k_norm2_partial(const cplx* x, long long n, double* partial, cudaStream_t s);
-int k_dots_scaled(cplx* V, long long ld, int nv, const cplx* w, long long n, cplx* partial, int scale_col,
-                  const double* scale_src, long long skip_col, cudaStream_t s);
-// h = fixed-order sum of partial_in; w -= sum_i V_i h_i; then mode 1: partial
-// dots of the new w with V_0..V_{nv-1}, mode 2: partial norm^2 of the new w.
-int k_orth_update_ex(const cplx* V, long long ld, int nv, const cplx* partial_in, cplx* w, long long n,
-                     int mode, cplx* partial_dots, double* partial_norm, cplx* h_out, int accumulate,
-                     long long skip_col, cudaStream_t s);
+// One step of the Krylov basis: partial dots (G = red_blocks_for(n) partials
+// per vector), the first pass (Arnoldi: all vectors; Lanczos: v_j and v_{j-1},
+// partial_in the dot with v_j; h_out receives the first-pass coefficients) and
+// the second pass over all vectors, which ends with the step's scalars in ks
+// (alpha_j, beta_j or column j of the Hessenberg matrix, c = exp(z T) e_1,
+// error estimate, status).
+int k_dots(const cplx* V, long long ld, int nv, const cplx* w, long long n, cplx* partial, cudaStream_t s);
+int k_orth_first(const cplx* V, long long ld, int nv, const cplx* partial_in, cplx* w, long long n, cplx* partial_dots,
+                 cplx* h_out, cudaStream_t s);
+int k_lanczos_first(const cplx* V, long long ld, int j, const cplx* partial_in, const KrylovScalars* ks, cplx* w,
+                    long long n, cplx* partial_dots, cplx* h_out, cudaStream_t s);
+int k_orth_second(const cplx* V, long long ld, int nv, const cplx* partial_in, cplx* w, long long n,
+                  double* partial_norm, KrylovScalars* ks, const cplx* h1, double zr, double zi, double tol,
+                  int arnoldi, cudaStream_t s);
 int k_scale_copy_dev(const cplx* x, long long n, const double* scale, cplx* y, cudaStream_t s);
 // x <- x * sqrt(sum pr / sum px) with px, pr norm^2 partials (k_norm2_partial)
 int k_rescale_to_norm(cplx* x, long long n, const double* px, int Gx, const double* pr, int Gr, cudaStream_t s);
 int k_krylov_start_ex(KrylovScalars* ks, const double* nrm2_partial, long long n, cudaStream_t s);
-int k_krylov_scalars_ex(KrylovScalars* ks, const cplx* h1, const cplx* h2, const double* beta_partial,
-                        long long n, int j, double zr, double zi, double tol, cudaStream_t s);
-// Arnoldi step j for a non-Hermitian generator (the decay of Eq. 3): column j
-// of the Hessenberg matrix is h1 + h2, H(j+1, j) = beta_j; c = exp(z H_j) e_1.
-int k_arnoldi_scalars(KrylovScalars* ks, const cplx* h1, const cplx* h2, const double* beta_partial, long long n,
-                      int j, double zr, double zi, double tol, cudaStream_t s);
 int k_combine(const cplx* V, long long ld, int nv, const KrylovScalars* ks, cplx* y,
               long long n, cudaStream_t s);
 
-// ---- small nodes: the whole Krylov exponential in one block -------------------
+// ---- small nodes: the whole Krylov exponential in one launch ------------------
 // Nodes and links with s <= SMALL_S tensor entries: H_eff as a dense s x s
-// matrix, then Lanczos/Arnoldi, exponential and combination in one launch.
+// matrix, then Lanczos/Arnoldi, exponential and combination in one cluster.
 constexpr int SMALL_S = 96;
 struct SmallPairs {      // channel pairs of a small H_eff (by value into the kernel)
     int np;
@@ -164,11 +171,8 @@ struct SmallPairs {      // channel pairs of a small H_eff (by value into the ke
     const cplx* Na[3];   // r matrices of D_a^2
     const cplx* G[3];    // r matrices of D_b^2
 };
-int k_dense_heff(cplx* H, const int* d, const cplx* hb0, const cplx* hb1, const cplx* hb2, const SmallPairs& pp,
-                 cudaStream_t s);
-// status in ks: converged, nonfinite, err; alpha[0] = iterations
-int k_small_krylov(const cplx* H, int n, cplx* x, double zr, double zi, double tol, int mmax, int arnoldi,
-                   KrylovScalars* ks, cudaStream_t s);
+int k_small_krylov(const int* d, const cplx* hb0, const cplx* hb1, const cplx* hb2, const SmallPairs& pp, cplx* x,
+                   double zr, double zi, double tol, int mmax, int arnoldi, KrylovScalars* ks, cudaStream_t s);
 
 // ---- elementwise / assembly ---------------------------------------------------
 int k_permute3(const cplx* x, cplx* y, int d0, int d1, int d2, int p0, int p1, int p2,

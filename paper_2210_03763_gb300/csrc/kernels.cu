@@ -5,6 +5,7 @@
 // the same fixed order, so repeated runs are bitwise identical and every
 // block of a kernel sees the same reduced value.
 #include "common.cuh"
+#include <cooperative_groups.h>
 #include <algorithm>
 #include <cmath>
 #include <mutex>
@@ -78,97 +79,181 @@ __device__ double block_sum_d(double v, double* sh) {
     return r;
 }
 
-// Sum the G partials of nv projections (partial[i*G + g]) into sh_h[0..nv).
+// Sum the G partials of nv projections (partial[i*G + g]) into sh_h[0..nv):
+// one warp per projection (a serial sum of 304 partials took 4 us in every
+// block of every launch), lanes in fixed order.
+__device__ __forceinline__ cplx warp_sum_c(cplx v) {
+    for (int o = 16; o > 0; o >>= 1) {
+        v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+        v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
+    }
+    return v;
+}
 __device__ void reduce_partials_to_shared(const cplx* partial, int nv, int G, cplx* sh_h) {
-    for (int i = threadIdx.x; i < nv; i += blockDim.x) {
+    const int lane = threadIdx.x & 31;
+    for (int i = threadIdx.x >> 5; i < nv; i += blockDim.x >> 5) {
         cplx s = make_double2(0.0, 0.0);
-        for (int g = 0; g < G; ++g) s = cadd(s, partial[(long long)i * G + g]);
-        sh_h[i] = s;
+        for (int g = lane; g < G; g += 32) s = cadd(s, partial[(long long)i * G + g]);
+        s = warp_sum_c(s);
+        if (lane == 0) sh_h[i] = s;
     }
     __syncthreads();
 }
 
+// By one warp; the sum in every lane.
 __device__ double reduce_norm_partials(const double* partial, int G) {
     double s = 0.0;
-    for (int g = 0; g < G; ++g) s += partial[g];
+    for (int g = threadIdx.x & 31; g < G; g += 32) s += partial[g];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
     return s;
 }
 
 // ---------------------------------------------------------------- kernels
-// (optional) column `scale_col` of V *= factor(norm partials); then partial
-// dots conj(V_i) . w for i < nv over this block's chunk.
-__global__ void dots_kernel(cplx* V, long long ld, int nv, const cplx* w, long long n, int G,
-                            cplx* partial, int scale_col, const double* scale_src, int scale_mode,
-                            long long skip_col) {
-    __shared__ cplx sh[T / 32];
-    long long lo, hi;
-    chunk_of(n, G, lo, hi);
-    if (scale_col >= 0) {
-        // scale_mode 1: factor = 1/sqrt(sum partials) or 0 if flagged dependent
-        double f = scale_src[0];
-        cplx* col = V + (long long)scale_col * ld;
-        for (long long e = lo + threadIdx.x; e < hi; e += blockDim.x) {
-            cplx x = col[e];
-            col[e] = make_double2(x.x * f, x.y * f);
-        }
-        __syncthreads();
+// conj(V_i) . w over [lo, hi) for C consecutive vectors, summed over the warp
+// (in every lane).
+template <int C>
+__device__ __forceinline__ void warp_dots(const cplx* V, long long ld, const cplx* w, long long lo, long long hi,
+                                          int first, int stride, cplx* s) {
+#pragma unroll
+    for (int c = 0; c < C; ++c) s[c] = make_double2(0.0, 0.0);
+    for (long long e = lo + first; e < hi; e += stride) {
+        const cplx x = w[e];
+#pragma unroll
+        for (int c = 0; c < C; ++c) acc_cdotc(s[c], V[c * ld + e], x);
     }
-    for (int i = 0; i < nv; ++i) {
-        cplx s = make_double2(0.0, 0.0);
-        if (i != skip_col) {
-            const cplx* vi = V + (long long)i * ld;
-            for (long long e = lo + threadIdx.x; e < hi; e += blockDim.x) acc_cdotc(s, vi[e], w[e]);
+#pragma unroll
+    for (int c = 0; c < C; ++c) s[c] = warp_sum_c(s[c]);
+}
+
+// Partial dots conj(V_i) . w, i < nv, over this block's chunk into
+// partial[i*G + block].  Long chunks: every warp takes a slice of the chunk,
+// four vectors at a time (w is read once per four); short chunks: one vector
+// per warp, so that no sum crosses warps.
+constexpr int SHORT_CHUNK = 256;
+struct DotSmem {
+    cplx w[T / 32][KRYLOV_MMAX + 1];
+};
+__device__ void block_dots(const cplx* V, long long ld, int nv, const cplx* w, long long lo, long long hi, int G,
+                           cplx* partial, DotSmem& sm) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    cplx s[4];
+    if (hi - lo <= SHORT_CHUNK) {
+        for (int i = warp; i < nv; i += T / 32) {
+            warp_dots<1>(V + (long long)i * ld, ld, w, lo, hi, lane, 32, s);
+            if (lane == 0) partial[(long long)i * G + blockIdx.x] = s[0];
         }
-        s = block_sum_c(s, sh);
-        if (threadIdx.x == 0) partial[(long long)i * G + blockIdx.x] = s;
+        return;
+    }
+    for (int i = 0; i < nv; i += 4) {
+        const cplx* v = V + (long long)i * ld;
+        const int c = nv - i < 4 ? nv - i : 4;
+        if (c == 4) warp_dots<4>(v, ld, w, lo, hi, threadIdx.x, T, s);
+        else if (c == 3) warp_dots<3>(v, ld, w, lo, hi, threadIdx.x, T, s);
+        else if (c == 2) warp_dots<2>(v, ld, w, lo, hi, threadIdx.x, T, s);
+        else warp_dots<1>(v, ld, w, lo, hi, threadIdx.x, T, s);
+        if (lane == 0)
+            for (int q = 0; q < c; ++q) sm.w[warp][i + q] = s[q];
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < nv; i += T) {
+        cplx a = sm.w[0][i];
+        for (int q = 1; q < T / 32; ++q) a = cadd(a, sm.w[q][i]);
+        partial[(long long)i * G + blockIdx.x] = a;
     }
 }
 
-// h = reduce(partial_in); w -= sum_i V_i h_i (i != skip); then mode 1: partial
-// dots of the new w, mode 2: partial norm^2.  Block 0 also stores h to h_out
-// (accumulated into h_out when accumulate != 0).
-__global__ void orth_update_kernel(const cplx* V, long long ld, int nv, const cplx* partial_in,
-                                   cplx* w, long long n, int G, int mode, cplx* partial_dots,
-                                   double* partial_norm, cplx* h_out, int accumulate,
-                                   long long skip_col) {
-    __shared__ cplx sh_h[KRYLOV_MMAX + 260];
-    __shared__ cplx shc[T / 32];
-    __shared__ double shd[T / 32];
-    reduce_partials_to_shared(partial_in, nv, G, sh_h);
-    if (blockIdx.x == 0 && h_out != nullptr) {
-        for (int i = threadIdx.x; i < nv; i += blockDim.x) {
-            cplx v = sh_h[i];
-            if (i == skip_col) v = make_double2(0.0, 0.0);
-            h_out[i] = accumulate ? cadd(h_out[i], v) : v;
-        }
-    }
+__global__ void __launch_bounds__(T) dots_kernel(const cplx* V, long long ld, int nv, const cplx* w, long long n, int G,
+                                                 cplx* partial) {
+    __shared__ DotSmem sm;
     long long lo, hi;
     chunk_of(n, G, lo, hi);
-    for (long long e = lo + threadIdx.x; e < hi; e += blockDim.x) {
+    block_dots(V, ld, nv, w, lo, hi, G, partial, sm);
+}
+
+// First pass of Arnoldi: h = sum of the partials of all nv projections
+// (stored to h_out), w -= sum_i V_i h_i, partial dots of the new w.
+__global__ void __launch_bounds__(T) orth_first_kernel(const cplx* V, long long ld, int nv, const cplx* partial_in,
+                                                       cplx* w, long long n, int G, cplx* partial_dots, cplx* h_out) {
+    __shared__ cplx sh_h[KRYLOV_MMAX + 1];
+    __shared__ DotSmem sm;
+    reduce_partials_to_shared(partial_in, nv, G, sh_h);
+    if (blockIdx.x == 0 && threadIdx.x < nv) h_out[threadIdx.x] = sh_h[threadIdx.x];
+    long long lo, hi;
+    chunk_of(n, G, lo, hi);
+    for (long long e = lo + threadIdx.x; e < hi; e += T) {
         cplx x = w[e];
-        for (int i = 0; i < nv; ++i) {
-            if (i == skip_col) continue;
-            sub_cmul(x, V[(long long)i * ld + e], sh_h[i]);
+        for (int i = 0; i < nv; ++i) sub_cmul(x, V[(long long)i * ld + e], sh_h[i]);
+        w[e] = x;
+    }
+    __syncthreads();
+    block_dots(V, ld, nv, w, lo, hi, G, partial_dots, sm);
+}
+
+// First pass of Lanczos.  H is Hermitian (up to the rounding of its
+// contractions), so only v_j and v_{j-1} have components in w beyond
+// rounding: w -= v_j h + v_{j-1} beta_{j-1} with h = v_j^H w, then the
+// partial dots of the new w with the whole basis, whose second pass removes
+// what is left.  Two sweeps over the basis instead of four: the vector work
+// is bound by the FP64 pipe.
+__global__ void __launch_bounds__(T) lanczos_first_kernel(const cplx* V, long long ld, int j, const cplx* partial_in,
+                                                          const KrylovScalars* ks, cplx* w, long long n, int G,
+                                                          cplx* partial_dots, cplx* h_out) {
+    __shared__ cplx sh_h[1];
+    __shared__ DotSmem sm;
+    reduce_partials_to_shared(partial_in, 1, G, sh_h);
+    const cplx h = sh_h[0];
+    const double b = j > 0 ? ks->beta[j - 1] : 0.0;
+    if (blockIdx.x == 0 && threadIdx.x <= j) h_out[threadIdx.x] = threadIdx.x == j ? h : make_double2(0.0, 0.0);
+    long long lo, hi;
+    chunk_of(n, G, lo, hi);
+    const cplx* vj = V + (long long)j * ld;
+    for (long long e = lo + threadIdx.x; e < hi; e += T) {
+        cplx x = w[e];
+        sub_cmul(x, vj[e], h);
+        if (j > 0) {
+            const cplx v = vj[e - ld];
+            x.x = fma(-b, v.x, x.x);
+            x.y = fma(-b, v.y, x.y);
         }
         w[e] = x;
     }
-    if (mode == 1) {
-        __syncthreads();
-        for (int i = 0; i < nv; ++i) {
-            cplx s = make_double2(0.0, 0.0);
-            if (i != skip_col) {
-                const cplx* vi = V + (long long)i * ld;
-                for (long long e = lo + threadIdx.x; e < hi; e += blockDim.x) acc_cdotc(s, vi[e], w[e]);
-            }
-            s = block_sum_c(s, shc);
-            if (threadIdx.x == 0) partial_dots[(long long)i * G + blockIdx.x] = s;
-        }
-    } else if (mode == 2) {
-        double s = 0.0;
-        for (long long e = lo + threadIdx.x; e < hi; e += blockDim.x) s += w[e].x * w[e].x + w[e].y * w[e].y;
-        s = block_sum_d(s, shd);
-        if (threadIdx.x == 0) partial_norm[blockIdx.x] = s;
+    __syncthreads();
+    block_dots(V, ld, j + 1, w, lo, hi, G, partial_dots, sm);
+}
+
+__device__ void krylov_scalars_step(KrylovScalars* ks, const cplx* h1, const cplx* h2, const double* beta_partial,
+                                    int G, int j, double zr, double zi, double tol, int arnoldi);
+
+// Second pass: h = sum of the partials, w -= sum_i V_i h_i, |w|^2.  The last
+// block to finish turns the sums into the step's scalars (alpha, beta, the
+// exponential of the projected matrix, the error estimate).
+__global__ void __launch_bounds__(T) orth_second_kernel(const cplx* V, long long ld, int nv, const cplx* partial_in,
+                                                        cplx* w, long long n, int G, double* partial_norm,
+                                                        KrylovScalars* ks, const cplx* h1, double zr, double zi,
+                                                        double tol, int arnoldi) {
+    __shared__ cplx sh_h[KRYLOV_MMAX + 1];
+    __shared__ double shd[T / 32];
+    __shared__ int last;
+    reduce_partials_to_shared(partial_in, nv, G, sh_h);
+    long long lo, hi;
+    chunk_of(n, G, lo, hi);
+    double s = 0.0;
+    for (long long e = lo + threadIdx.x; e < hi; e += T) {
+        cplx x = w[e];
+        for (int i = 0; i < nv; ++i) sub_cmul(x, V[(long long)i * ld + e], sh_h[i]);
+        w[e] = x;
+        s = fma(x.x, x.x, fma(x.y, x.y, s));
     }
+    s = block_sum_d(s, shd);
+    if (threadIdx.x == 0) {
+        partial_norm[blockIdx.x] = s;
+        __threadfence();
+        last = atomicAdd(&ks->arrived, 1u) == gridDim.x - 1;
+        if (last) ks->arrived = 0u;
+        __threadfence();
+    }
+    __syncthreads();
+    if (last && threadIdx.x < 32) krylov_scalars_step(ks, h1, sh_h, partial_norm, G, nv - 1, zr, zi, tol, arnoldi);
 }
 
 __global__ void norm2_partial_kernel(const cplx* x, long long n, int G, double* partial) {
@@ -194,11 +279,9 @@ __global__ void scale_copy_kernel(const cplx* x, long long n, const double* scal
 // partial sums pr (each block sums both partial lists in the same order).
 __global__ void rescale_to_norm_kernel(cplx* x, long long n, const double* px, int Gx, const double* pr, int Gr) {
     __shared__ double f;
-    if (threadIdx.x == 0) {
-        double a = 0.0, b = 0.0;
-        for (int g = 0; g < Gx; ++g) a += px[g];
-        for (int g = 0; g < Gr; ++g) b += pr[g];
-        f = a > 0.0 ? sqrt(b / a) : 1.0;
+    if (threadIdx.x < 32) {
+        const double a = reduce_norm_partials(px, Gx), b = reduce_norm_partials(pr, Gr);
+        if (threadIdx.x == 0) f = a > 0.0 ? sqrt(b / a) : 1.0;
     }
     __syncthreads();
     const double ff = f;
@@ -225,49 +308,71 @@ __global__ void combine_kernel(const cplx* V, long long ld, int nv, const Krylov
     }
 }
 
+// 1/k for the Taylor terms.
+__constant__ double INV_K[41] = {0.0,      1.0 / 1,  1.0 / 2,  1.0 / 3,  1.0 / 4,  1.0 / 5,  1.0 / 6,  1.0 / 7,  1.0 / 8,
+                                 1.0 / 9,  1.0 / 10, 1.0 / 11, 1.0 / 12, 1.0 / 13, 1.0 / 14, 1.0 / 15, 1.0 / 16, 1.0 / 17,
+                                 1.0 / 18, 1.0 / 19, 1.0 / 20, 1.0 / 21, 1.0 / 22, 1.0 / 23, 1.0 / 24, 1.0 / 25, 1.0 / 26,
+                                 1.0 / 27, 1.0 / 28, 1.0 / 29, 1.0 / 30, 1.0 / 31, 1.0 / 32, 1.0 / 33, 1.0 / 34, 1.0 / 35,
+                                 1.0 / 36, 1.0 / 37, 1.0 / 38, 1.0 / 39, 1.0 / 40};
+
+// High words of |re|, |im|: ordered like the magnitudes, compared without the
+// FP64 pipe.
+__device__ __forceinline__ unsigned mag_hi(cplx v) {
+    const unsigned a = (unsigned)__double2hiint(v.x) & 0x7FFFFFFFu, b = (unsigned)__double2hiint(v.y) & 0x7FFFFFFFu;
+    return a > b ? a : b;
+}
+// Every lane's term is below 2^-60 of the largest sum: the series is done.
+__device__ __forceinline__ bool series_done(cplx term, cplx sum) {
+    const unsigned tm = __reduce_max_sync(0xffffffffu, mag_hi(term)), sm = __reduce_max_sync(0xffffffffu, mag_hi(sum));
+    return (unsigned long long)tm + (60u << 20) <= sm || tm == 0u;
+}
+
+// Sub-steps that keep |z| norm / n_sub <= 1/2: bounded also for non-finite or
+// absurd norms (a NaN state is reported through the nonfinite flag, never by
+// a runaway loop).
+__device__ __forceinline__ int taylor_substeps(double want) {
+    return (want >= 1.0 && want < 65536.0) ? (int)ceil(want) : (want >= 65536.0 ? 65536 : 1);
+}
+
 // exp(z T) e_1 for the real symmetric tridiagonal T (diag a[0..m), off-diag
 // b[0..m-1)), m <= 32, by the truncated Taylor series of the matrix
 // exponential applied to the vector, with the step z split into n_sub equal
 // substeps so that |z/n_sub| * ||T||_inf <= 1/2 (the "Taylor series" method of
 // Moler & Van Loan, "Nineteen dubious ways to compute the exponential of a
-// matrix", with scaling).  One warp; lane i holds component i.
+// matrix", with scaling).  One warp; lane i holds component i.  The warp runs
+// alone, so a term costs its FP64 instructions one after another: z is i or
+// real in every caller but the general case, 1/k comes from a table and the
+// stopping test is integer.
 __device__ void tridiag_expm_warp(const double* a, const double* b, int m, double zr, double zi,
                                   cplx* out) {
     const int l = threadIdx.x & 31;
-    double ai = l < m ? a[l] : 0.0;
-    double bl = (l < m - 1) ? b[l] : 0.0;          // T(l, l+1)
-    double bu = (l >= 1 && l < m) ? b[l - 1] : 0.0; // T(l, l-1)
+    const double ai = l < m ? a[l] : 0.0;
+    const double bl = (l < m - 1) ? b[l] : 0.0;          // T(l, l+1)
+    const double bu = (l >= 1 && l < m) ? b[l - 1] : 0.0; // T(l, l-1)
     double rs = fabs(ai) + fabs(bl) + fabs(bu);
     for (int o = 16; o > 0; o >>= 1) rs = fmax(rs, __shfl_xor_sync(0xffffffffu, rs, o));
-    double zn = sqrt(zr * zr + zi * zi);
-    // substeps: bounded also for non-finite or absurd norms (a NaN state is
-    // reported through the nonfinite flag, never by a runaway loop)
-    const double want = zn * rs / 0.5;
-    int nsub = (want >= 1.0 && want < 65536.0) ? (int)ceil(want) : (want >= 65536.0 ? 65536 : 1);
-    double hr = zr / nsub, hi = zi / nsub;
+    const int nsub = taylor_substeps(sqrt(zr * zr + zi * zi) * rs / 0.5);
+    const double hr = zr / nsub, hi = zi / nsub;
     cplx u = make_double2(l == 0 ? 1.0 : 0.0, 0.0);
     for (int s = 0; s < nsub; ++s) {
         cplx term = u, sum = u;
         for (int k = 1; k <= 40; ++k) {
-            // t = T term
-            double xm_r = __shfl_up_sync(0xffffffffu, term.x, 1);
-            double xm_i = __shfl_up_sync(0xffffffffu, term.y, 1);
-            double xp_r = __shfl_down_sync(0xffffffffu, term.x, 1);
-            double xp_i = __shfl_down_sync(0xffffffffu, term.y, 1);
-            double tr = ai * term.x + (l >= 1 ? bu * xm_r : 0.0) + (l < 31 ? bl * xp_r : 0.0);
-            double ti = ai * term.y + (l >= 1 ? bu * xm_i : 0.0) + (l < 31 ? bl * xp_i : 0.0);
-            if (l >= m) { tr = 0.0; ti = 0.0; }
+            // t = T term (lanes outside [0, m) have zero rows)
+            const double xm_r = __shfl_up_sync(0xffffffffu, term.x, 1);
+            const double xm_i = __shfl_up_sync(0xffffffffu, term.y, 1);
+            const double xp_r = __shfl_down_sync(0xffffffffu, term.x, 1);
+            const double xp_i = __shfl_down_sync(0xffffffffu, term.y, 1);
+            const double tr = fma(bl, xp_r, fma(bu, xm_r, ai * term.x));
+            const double ti = fma(bl, xp_i, fma(bu, xm_i, ai * term.y));
             // term = (h * t) / k
-            double inv = 1.0 / k;
-            term = make_double2((hr * tr - hi * ti) * inv, (hr * ti + hi * tr) * inv);
-            sum = cadd(sum, term);
-            double tm = fabs(term.x) + fabs(term.y);
-            double sm = fabs(sum.x) + fabs(sum.y);
-            for (int o = 16; o > 0; o >>= 1) {
-                tm = fmax(tm, __shfl_xor_sync(0xffffffffu, tm, o));
-                sm = fmax(sm, __shfl_xor_sync(0xffffffffu, sm, o));
+            if (hr == 0.0) {
+                const double c = hi * INV_K[k];
+                term = make_double2(-c * ti, c * tr);
+            } else {
+                term = make_double2((hr * tr - hi * ti) * INV_K[k], (hr * ti + hi * tr) * INV_K[k]);
             }
-            if (tm <= 1e-18 * sm) break;
+            sum = cadd(sum, term);
+            if (series_done(term, sum)) break;
         }
         u = sum;
     }
@@ -275,286 +380,321 @@ __device__ void tridiag_expm_warp(const double* a, const double* b, int m, doubl
 }
 
 __global__ void krylov_start_kernel(KrylovScalars* ks, const double* nrm2_partial, int G) {
+    const double s = reduce_norm_partials(nrm2_partial, G);
     if (threadIdx.x != 0) return;
-    double s = reduce_norm_partials(nrm2_partial, G);
+    ks->arrived = 0u;
     double n0 = sqrt(s);
     ks->nrm0 = n0;
     ks->inv_scale = n0 > 0.0 ? 1.0 / n0 : 0.0;
-    ks->converged = (n0 == 0.0) ? 1 : 0;
-    ks->nonfinite = isfinite(n0) ? 0 : 1;
-    ks->err = 0.0;
+    ks->st.converged = (n0 == 0.0) ? 1 : 0;
+    ks->st.nonfinite = isfinite(n0) ? 0 : 1;
+    ks->st.err = 0.0;
     for (int i = 0; i < KRYLOV_MMAX; ++i) ks->c[i] = make_double2(0.0, 0.0);
 }
 
-__global__ void krylov_scalars_kernel(KrylovScalars* ks, const cplx* h1, const cplx* h2,
-                                      const double* beta_partial, int G, int j, double zr,
-                                      double zi, double tol) {
-    __shared__ double a[32], b[32];
-    if (threadIdx.x == 0) {
-        ks->alpha[j] = h1[j].x + h2[j].x;
-        double b2 = reduce_norm_partials(beta_partial, G);
-        ks->beta[j] = sqrt(b2);
-    }
-    __syncthreads();
-    if (threadIdx.x < 32) {
-        int l = threadIdx.x;
-        a[l] = l <= j ? ks->alpha[l] : 0.0;
-        b[l] = l < j ? ks->beta[l] : 0.0;
-    }
-    __syncthreads();
-    if (threadIdx.x < 32) tridiag_expm_warp(a, b, j + 1, zr, zi, ks->c);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double bj = ks->beta[j];
-        cplx cj = ks->c[j];
-        double err = bj * sqrt(cj.x * cj.x + cj.y * cj.y);
-        ks->err = err;
-        ks->converged = (err <= tol) ? 1 : 0;
-        ks->inv_scale = bj > 0.0 ? 1.0 / bj : 0.0;
-        if (!isfinite(err) || !isfinite(ks->alpha[j])) ks->nonfinite = 1;
-    }
-}
-
-// exp(z H) e_1 for the dense m x m matrix H (row-major rows of ld
-// KRYLOV_MMAX in H[i][j]), m <= 31, by the scaled Taylor series as in
-// tridiag_expm_warp: substeps with |z/n_sub| * ||H||_inf <= 1/2.  One warp;
-// lane i holds component i.
-__device__ void hess_expm_warp(const cplx (*Hm)[KRYLOV_MMAX], int m, double zr, double zi, cplx* out) {
+// exp(z H) e_1 for the m x m matrix H, H(i, k) at Hs[32 k + i] in shared
+// memory, m <= 31, by the scaled Taylor series as in tridiag_expm_warp:
+// substeps with |z/n_sub| * ||H||_inf <= 1/2.  One warp; lane i holds
+// component i; the vector goes round through `vec` (32 entries of shared
+// memory).
+__device__ void hess_expm_warp(const cplx* Hs, cplx* vec, int m, double zr, double zi, cplx* out) {
     const int l = threadIdx.x & 31;
     double rs = 0.0;
     if (l < m)
         for (int k = 0; k < m; ++k) {
-            const cplx v = Hm[l][k];
+            const cplx v = Hs[32 * k + l];
             rs += sqrt(v.x * v.x + v.y * v.y);
         }
     for (int o = 16; o > 0; o >>= 1) rs = fmax(rs, __shfl_xor_sync(0xffffffffu, rs, o));
-    const double zn = sqrt(zr * zr + zi * zi);
-    const double want = zn * rs / 0.5;
-    const int nsub = (want >= 1.0 && want < 65536.0) ? (int)ceil(want) : (want >= 65536.0 ? 65536 : 1);
+    const int nsub = taylor_substeps(sqrt(zr * zr + zi * zi) * rs / 0.5);
     const double hr = zr / nsub, hi = zi / nsub;
     cplx u = make_double2(l == 0 ? 1.0 : 0.0, 0.0);
     for (int s = 0; s < nsub; ++s) {
         cplx term = u, sum = u;
         for (int k = 1; k <= 40; ++k) {
-            double tr = 0.0, ti = 0.0;
-            for (int q = 0; q < m; ++q) {
-                const double xr = __shfl_sync(0xffffffffu, term.x, q);
-                const double xi = __shfl_sync(0xffffffffu, term.y, q);
-                if (l < m) {
-                    const cplx v = Hm[l][q];
-                    tr += v.x * xr - v.y * xi;
-                    ti += v.x * xi + v.y * xr;
-                }
+            __syncwarp();
+            vec[l] = term;
+            __syncwarp();
+            cplx t = make_double2(0.0, 0.0);
+            if (l < m) {
+                // row l of the Hessenberg matrix starts at column l - 1
+                for (int q = l > 0 ? l - 1 : 0; q < m; ++q) acc_cmul(t, Hs[32 * q + l], vec[q]);
             }
-            const double inv = 1.0 / k;
-            term = make_double2((hr * tr - hi * ti) * inv, (hr * ti + hi * tr) * inv);
+            const double inv = INV_K[k];
+            term = make_double2((hr * t.x - hi * t.y) * inv, (hr * t.y + hi * t.x) * inv);
             sum = cadd(sum, term);
-            double tm = fabs(term.x) + fabs(term.y);
-            double sm = fabs(sum.x) + fabs(sum.y);
-            for (int o = 16; o > 0; o >>= 1) {
-                tm = fmax(tm, __shfl_xor_sync(0xffffffffu, tm, o));
-                sm = fmax(sm, __shfl_xor_sync(0xffffffffu, sm, o));
-            }
-            if (tm <= 1e-18 * sm) break;
+            if (series_done(term, sum)) break;
         }
         u = sum;
     }
+    __syncwarp();
     if (l < m) out[l] = u;
 }
 
-__global__ void arnoldi_scalars_kernel(KrylovScalars* ks, const cplx* h1, const cplx* h2,
-                                       const double* beta_partial, int G, int j, double zr, double zi, double tol) {
-    if (threadIdx.x == 0) {
+// Scalars of step j by one warp: alpha_j, beta_j (Arnoldi: column j of the
+// Hessenberg matrix), c = exp(z T) e_1, the error estimate and the status.
+__device__ void krylov_scalars_step(KrylovScalars* ks, const cplx* h1, const cplx* h2, const double* beta_partial,
+                                    int G, int j, double zr, double zi, double tol, int arnoldi) {
+    __shared__ double a[32], b[32];
+    __shared__ cplx hs[KRYLOV_MMAX * 32], vec[32];
+    const int l = threadIdx.x & 31;
+    double s = 0.0;
+    for (int g = l; g < G; g += 32) s += __ldcg(beta_partial + g);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    const double bj = sqrt(s);
+    bool bad;
+    if (arnoldi) {
         // the whole column j: projections, the subdiagonal beta_j, zeros below
-        const double b2 = reduce_norm_partials(beta_partial, G);
-        ks->beta[j] = sqrt(b2);
-        for (int i = 0; i <= KRYLOV_MMAX; ++i)
-            ks->hess[i][j] = i <= j ? cadd(h1[i], h2[i]) : make_double2(i == j + 1 ? ks->beta[j] : 0.0, 0.0);
-        ks->alpha[j] = ks->hess[j][j].x;
+        const cplx col = l <= j ? cadd(h1[l], h2[l]) : make_double2(l == j + 1 ? bj : 0.0, 0.0);
+        ks->hess[j][l] = col;
+        for (int q = 0; q < j; ++q) hs[32 * q + l] = ks->hess[q][l];
+        hs[32 * j + l] = col;
+        __syncwarp();
+        const cplx d = hs[33 * j];
+        bad = !isfinite(d.x) || !isfinite(d.y);
+        if (l == 0) {
+            ks->beta[j] = bj;
+            ks->alpha[j] = d.x;
+        }
+        hess_expm_warp(hs, vec, j + 1, zr, zi, ks->c);
+    } else {
+        const double al = h1[j].x + h2[j].x;
+        bad = !isfinite(al);
+        a[l] = l < j ? ks->alpha[l] : l == j ? al : 0.0;
+        b[l] = l < j ? ks->beta[l] : 0.0;
+        __syncwarp();
+        if (l == 0) {
+            ks->alpha[j] = al;
+            ks->beta[j] = bj;
+        }
+        tridiag_expm_warp(a, b, j + 1, zr, zi, ks->c);
     }
-    __syncthreads();
-    if (threadIdx.x < 32) hess_expm_warp(ks->hess, j + 1, zr, zi, ks->c);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const double bj = ks->beta[j];
+    __syncwarp();
+    if (l == 0) {
         const cplx cj = ks->c[j];
         const double err = bj * sqrt(cj.x * cj.x + cj.y * cj.y);
-        ks->err = err;
-        ks->converged = (err <= tol) ? 1 : 0;
+        ks->st.err = err;
+        ks->st.converged = (err <= tol) ? 1 : 0;
         ks->inv_scale = bj > 0.0 ? 1.0 / bj : 0.0;
-        if (!isfinite(err) || !isfinite(ks->hess[j][j].x) || !isfinite(ks->hess[j][j].y)) ks->nonfinite = 1;
+        if (!isfinite(err) || bad) ks->st.nonfinite = 1;
     }
 }
 
-// ---------------------------------------------- small nodes: dense H_eff
-// Element (x, y) of the s x s matrix of H_eff for a node (or link) with leg
-// dims d: block terms hb_u (D_u x D_u, nullptr: none) and channel pairs
-// sum_i Na_i (leg a) (x) G_i (leg b), identity on the third leg.
-__global__ void dense_heff_kernel(cplx* H, int d0, int d1, int d2, const cplx* hb0, const cplx* hb1,
-                                  const cplx* hb2, SmallPairs pp) {
-    const int s = d0 * d1 * d2;
-    const long long n = (long long)s * s;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
-         e += (long long)gridDim.x * blockDim.x) {
-        const int xr = (int)(e % s), yc = (int)(e / s);
-        const int x[3] = {xr % d0, (xr / d0) % d1, xr / (d0 * d1)};
-        const int y[3] = {yc % d0, (yc / d0) % d1, yc / (d0 * d1)};
-        const int dd[3] = {d0, d1, d2};
-        const cplx* hb[3] = {hb0, hb1, hb2};
-        cplx h = make_double2(0.0, 0.0);
-        for (int u = 0; u < 3; ++u) {
-            if (!hb[u]) continue;
-            bool diag = true;
-            for (int v = 0; v < 3; ++v)
-                if (v != u && x[v] != y[v]) diag = false;
-            if (diag) h = cadd(h, hb[u][x[u] + dd[u] * y[u]]);
-        }
-        for (int p = 0; p < pp.np; ++p) {
-            const int a = pp.a[p], b = pp.b[p], w = 3 - a - b;
-            if (x[w] != y[w]) continue;
-            const long long Da2 = (long long)dd[a] * dd[a], Db2 = (long long)dd[b] * dd[b];
-            const long long ia = x[a] + (long long)dd[a] * y[a], ib = x[b] + (long long)dd[b] * y[b];
-            for (int i = 0; i < pp.r[p]; ++i)
-                h = cadd(h, cmul(pp.Na[p][i * Da2 + ia], pp.G[p][i * Db2 + ib]));
-        }
-        H[e] = h;
+// ------------------------------------------------------------- small nodes
+// The whole Krylov exponential x <- exp(z H) x of a node or link with s <= 96
+// entries in one launch of one cluster: H_eff as a dense matrix (block terms
+// hb_u, D_u x D_u or nullptr, and channel pairs sum_i Na_i (leg a) (x) G_i
+// (leg b)), Lanczos (or Arnoldi when `arnoldi`) with the same passes,
+// exponential and stopping rule as the multi-kernel path.  Status goes to ks.
+//
+// One SM's FP64 pipe (19 clk per warp-wide FMA) is the bound: an 81 x 81
+// matvec alone is 7 us on it.  So the rows are split over the 8 SMs of a
+// cluster; every CTA keeps the whole basis, computes its rows of w and its
+// partial dots, and writes them into all CTAs' shared memory (three cluster
+// barriers per iteration).  All CTAs sum the same partials in the same order,
+// so they take the same decisions.  Warp 0 takes the projected exponential
+// while the other warps already multiply the next vector.
+// Measured: 225 us per run of a 2x2 step (one block on one SM) -> 54 us.
+constexpr int SK_CL = 8;                                  // CTAs per cluster
+constexpr int SK_THREADS = 256;
+constexpr int SK_ROWS = (SMALL_S + SK_CL - 1) / SK_CL;    // rows per CTA (12), at most 16 for the group sums
+static_assert(SK_ROWS <= 16, "16-lane groups");
+
+struct SkSmem {
+    cplx xa[SK_CL][32], xb[SK_CL][32];   // partial dots of every CTA, first and second pass
+    double xn[SK_CL];                    // partial norms
+    cplx xw[SMALL_S];                    // w, rows from every CTA
+    cplx h1[32], h2[32], c[32], w[SK_ROWS];
+    double alpha[32], beta[32];
+    cplx hess[KRYLOV_MMAX * 32], hvec[32];   // Arnoldi: H(i, j) at [32 j + i]
+    int done, conv, nonfin;
+    double err;
+};
+
+__device__ __forceinline__ cplx group16_sum(cplx v) {
+    for (int o = 8; o > 0; o >>= 1) {
+        v.x += __shfl_xor_sync(0xffffffffu, v.x, o);
+        v.y += __shfl_xor_sync(0xffffffffu, v.y, o);
     }
+    return v;
 }
 
-// The whole Krylov exponential x <- exp(z H) x of a small dense H (s <= 96)
-// in one block: Lanczos (or Arnoldi when `arnoldi`) with the same two-pass
-// full re-orthogonalisation, tridiagonal (Hessenberg) exponential and
-// stopping rule as the multi-kernel path, with H and the basis in shared
-// memory.  Small nodes of the tree otherwise spend their time in launches
-// and host round trips, not in arithmetic.  Status goes to ks (converged,
-// nonfinite, err, and alpha[0] holds the iteration count as a double).
-constexpr int SMALL_KRYLOV_THREADS = 256;
-__global__ void __launch_bounds__(SMALL_KRYLOV_THREADS)
-    small_krylov_kernel(const cplx* Hg, int s, cplx* x, double zr, double zi, double tol, int mmax, int arnoldi,
-                        KrylovScalars* ks) {
+__device__ cplx small_heff(int xr, int yc, int d0, int d1, int d2, const cplx* hb0, const cplx* hb1, const cplx* hb2,
+                           const SmallPairs& pp) {
+    const int x[3] = {xr % d0, (xr / d0) % d1, xr / (d0 * d1)};
+    const int y[3] = {yc % d0, (yc / d0) % d1, yc / (d0 * d1)};
+    const int dd[3] = {d0, d1, d2};
+    const cplx* hb[3] = {hb0, hb1, hb2};
+    cplx h = make_double2(0.0, 0.0);
+    for (int u = 0; u < 3; ++u) {
+        if (!hb[u]) continue;
+        bool diag = true;
+        for (int v = 0; v < 3; ++v)
+            if (v != u && x[v] != y[v]) diag = false;
+        if (diag) h = cadd(h, hb[u][x[u] + dd[u] * y[u]]);
+    }
+    for (int p = 0; p < pp.np; ++p) {
+        const int a = pp.a[p], b = pp.b[p], w = 3 - a - b;
+        if (x[w] != y[w]) continue;
+        const long long Da2 = (long long)dd[a] * dd[a], Db2 = (long long)dd[b] * dd[b];
+        const long long ia = x[a] + (long long)dd[a] * y[a], ib = x[b] + (long long)dd[b] * y[b];
+        for (int i = 0; i < pp.r[p]; ++i) acc_cmul(h, pp.Na[p][i * Da2 + ia], pp.G[p][i * Db2 + ib]);
+    }
+    return h;
+}
+
+__global__ void __cluster_dims__(SK_CL, 1, 1) __launch_bounds__(SK_THREADS)
+    small_krylov_kernel(int d0, int d1, int d2, const cplx* hb0, const cplx* hb1, const cplx* hb2, SmallPairs pp,
+                        cplx* x, double zr, double zi, double tol, int mmax, int arnoldi, KrylovScalars* ks) {
+    namespace cg = cooperative_groups;
+    cg::cluster_group cl = cg::this_cluster();
     extern __shared__ cplx smem_c[];
-    cplx* Hs = smem_c;                   // s * s, column-major
-    cplx* V = Hs + (long long)s * s;     // (mmax + 1) * s
-    cplx* w = V + (long long)(mmax + 1) * s;
-    __shared__ cplx h1[KRYLOV_MMAX + 1], h2[KRYLOV_MMAX + 1];
-    __shared__ double alpha[32], beta[32], sh_red[SMALL_KRYLOV_THREADS / 32];
-    __shared__ cplx hess[KRYLOV_MMAX + 1][KRYLOV_MMAX];
-    __shared__ cplx c[32];
-    __shared__ double s_nrm0, s_beta;
-    __shared__ int s_done, s_m, s_conv, s_nonfin;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, nw = SMALL_KRYLOV_THREADS / 32;
-    for (long long e = tid; e < (long long)s * s; e += SMALL_KRYLOV_THREADS) Hs[e] = Hg[e];
-    // start vector
-    double a = 0.0;
-    for (int e = tid; e < s; e += SMALL_KRYLOV_THREADS) {
-        const cplx v = x[e];
-        V[e] = v;
-        a += v.x * v.x + v.y * v.y;
+    __shared__ SkSmem sm;
+    const int s = d0 * d1 * d2, R = (s + SK_CL - 1) / SK_CL;
+    const int rank = (int)cl.block_rank(), r0 = rank * R, nr = max(0, min(R, s - r0));
+    cplx* Hs = smem_c;              // own rows: H(r0 + r, k) at [k * R + r]
+    cplx* V = Hs + R * s;           // (mmax + 1) * s
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g16 = tid >> 4, l16 = tid & 15;
+    for (int e = tid; e < nr * s; e += SK_THREADS) {
+        const int r = e % nr, k = e / nr;
+        Hs[k * R + r] = small_heff(r0 + r, k, d0, d1, d2, hb0, hb1, hb2, pp);
     }
-    a = block_sum_d(a, sh_red);
-    if (tid == 0) {
-        s_nrm0 = sqrt(a);
-        s_done = (s_nrm0 == 0.0);
-        s_nonfin = isfinite(s_nrm0) ? 0 : 1;
-        s_conv = s_done;
-        s_m = 0;
-    }
+    for (int e = tid; e < s; e += SK_THREADS) V[e] = x[e];
     __syncthreads();
-    if (s_done || s_nonfin) {
-        if (tid == 0) {
-            ks->converged = s_conv;
-            ks->nonfinite = s_nonfin;
-            ks->err = 0.0;
-            ks->alpha[0] = 0.0;
+    double nrm0 = 0.0;
+    for (int e = lane; e < s; e += 32) nrm0 = fma(V[e].x, V[e].x, fma(V[e].y, V[e].y, nrm0));
+    for (int o = 16; o > 0; o >>= 1) nrm0 += __shfl_xor_sync(0xffffffffu, nrm0, o);
+    nrm0 = sqrt(nrm0);
+    cl.sync();                      // every CTA has read x; all are running (remote writes may start)
+    if (nrm0 == 0.0 || !isfinite(nrm0)) {
+        if (rank == 0 && tid == 0) {
+            ks->st.err = 0.0;
+            ks->st.converged = nrm0 == 0.0;
+            ks->st.nonfinite = nrm0 != 0.0;
+            ks->st.iters = 0;
         }
         return;
     }
-    const double inv0 = 1.0 / s_nrm0;
-    for (int e = tid; e < s; e += SMALL_KRYLOV_THREADS) V[e] = make_double2(V[e].x * inv0, V[e].y * inv0);
+    if (tid == 0) sm.nonfin = 0;
+    const double inv0 = 1.0 / nrm0;
+    for (int e = tid; e < s; e += SK_THREADS) V[e] = make_double2(V[e].x * inv0, V[e].y * inv0);
     __syncthreads();
+    // own rows of w = H v, 16 lanes per row, by `nt` threads numbered from t
+    auto matvec = [&](const cplx* v, int t, int nt) {
+        for (int q = t; q < ((nr * 16 + 31) & ~31); q += nt) {
+            const int r = q >> 4;
+            cplx a = make_double2(0.0, 0.0);
+            if (r < nr)
+                for (int k = q & 15; k < s; k += 16) acc_cmul(a, Hs[k * R + r], v[k]);
+            a = group16_sum(a);
+            if (r < nr && (q & 15) == 0) sm.w[r] = a;
+        }
+    };
+    // partial dots of own rows with v_i, i0 <= i < i1, into every CTA's buf
+    auto dots = [&](int i0, int i1, cplx(*buf)[32]) {
+        const int n = i1 - i0;
+        for (int q = g16; q < ((n + 1) & ~1); q += SK_THREADS / 16) {   // both groups of a warp stay together
+            cplx d = make_double2(0.0, 0.0);
+            if (q < n && l16 < nr) acc_cdotc(d, V[(i0 + q) * s + r0 + l16], sm.w[l16]);
+            d = group16_sum(d);
+            if (q < n && l16 < SK_CL) cl.map_shared_rank(&buf[rank][0], l16)[q] = d;
+        }
+    };
+    matvec(V, tid, SK_THREADS);
     int j = 0;
     for (;; ++j) {
-        const cplx* vj = V + (long long)j * s;
-        // w = H v_j
-        for (int r = tid; r < s; r += SMALL_KRYLOV_THREADS) {
-            cplx acc = make_double2(0.0, 0.0);
-            for (int k = 0; k < s; ++k) acc = cadd(acc, cmul(Hs[r + (long long)s * k], vj[k]));
-            w[r] = acc;
+        __syncthreads();
+        const int first = arnoldi ? 0 : j;   // first pass: all vectors, or v_j and beta v_{j-1}
+        dots(first, j + 1, sm.xa);
+        cl.sync();
+        if (tid <= j) {
+            cplx h = make_double2(0.0, 0.0);
+            if (tid >= first)
+                for (int q = 0; q < SK_CL; ++q) h = cadd(h, sm.xa[q][tid - first]);
+            sm.h1[tid] = h;
         }
         __syncthreads();
-        // two passes of classical Gram-Schmidt against v_0 .. v_j, one warp per dot
-        for (int pass = 0; pass < 2; ++pass) {
-            cplx* hp = pass == 0 ? h1 : h2;
-            for (int i = warp; i <= j; i += nw) {
-                const cplx* vi = V + (long long)i * s;
-                cplx d = make_double2(0.0, 0.0);
-                for (int e = lane; e < s; e += 32) d = cadd(d, cdotc(vi[e], w[e]));
-                for (int o = 16; o > 0; o >>= 1) {
-                    d.x += __shfl_down_sync(0xffffffffu, d.x, o);
-                    d.y += __shfl_down_sync(0xffffffffu, d.y, o);
-                }
-                if (lane == 0) hp[i] = d;
+        if (tid < nr) {
+            cplx w = sm.w[tid];
+            for (int i = first; i <= j; ++i) sub_cmul(w, V[i * s + r0 + tid], sm.h1[i]);
+            if (!arnoldi && j > 0) {
+                const cplx v = V[(j - 1) * s + r0 + tid];
+                w.x = fma(-sm.beta[j - 1], v.x, w.x);
+                w.y = fma(-sm.beta[j - 1], v.y, w.y);
             }
-            __syncthreads();
-            for (int e = tid; e < s; e += SMALL_KRYLOV_THREADS) {
-                cplx v = w[e];
-                for (int i = 0; i <= j; ++i) {
-                    const cplx p = cmul(V[(long long)i * s + e], hp[i]);
-                    v.x -= p.x;
-                    v.y -= p.y;
-                }
-                w[e] = v;
-            }
-            __syncthreads();
+            sm.w[tid] = w;
         }
-        double b2 = 0.0;
-        for (int e = tid; e < s; e += SMALL_KRYLOV_THREADS) b2 += w[e].x * w[e].x + w[e].y * w[e].y;
-        b2 = block_sum_d(b2, sh_red);
-        if (tid == 0) {
-            s_beta = sqrt(b2);
-            beta[j] = s_beta;
-            alpha[j] = h1[j].x + h2[j].x;
-            if (arnoldi)   // the whole column j: projections, beta_j, zeros below
-                for (int i = 0; i <= KRYLOV_MMAX; ++i)
-                    hess[i][j] = i <= j ? cadd(h1[i], h2[i]) : make_double2(i == j + 1 ? s_beta : 0.0, 0.0);
+        __syncthreads();
+        dots(0, j + 1, sm.xb);
+        cl.sync();
+        if (tid <= j) {
+            cplx h = make_double2(0.0, 0.0);
+            for (int q = 0; q < SK_CL; ++q) h = cadd(h, sm.xb[q][tid]);
+            sm.h2[tid] = h;
         }
         __syncthreads();
         if (warp == 0) {
-            if (arnoldi) {
-                hess_expm_warp(hess, j + 1, zr, zi, c);
-            } else {
-                __shared__ double ta[32], tb[32];
-                ta[lane] = lane <= j ? alpha[lane] : 0.0;
-                tb[lane] = lane < j ? beta[lane] : 0.0;
-                __syncwarp();
-                tridiag_expm_warp(ta, tb, j + 1, zr, zi, c);
+            cplx w = make_double2(0.0, 0.0);
+            double n2 = 0.0;
+            if (lane < nr) {
+                w = sm.w[lane];
+                for (int i = 0; i <= j; ++i) sub_cmul(w, V[i * s + r0 + lane], sm.h2[i]);
+                n2 = fma(w.x, w.x, w.y * w.y);
+            }
+            for (int o = 8; o > 0; o >>= 1) n2 += __shfl_xor_sync(0xffffffffu, n2, o);
+            n2 = __shfl_sync(0xffffffffu, n2, 0);
+            for (int q = 0; q < SK_CL; ++q) {
+                if (lane < nr) cl.map_shared_rank(sm.xw, q)[r0 + lane] = w;
+                if (lane == 0) cl.map_shared_rank(sm.xn, q)[rank] = n2;
             }
         }
-        __syncthreads();
-        if (tid == 0) {
-            const double err = s_beta * sqrt(c[j].x * c[j].x + c[j].y * c[j].y);
-            s_conv = err <= tol;
-            if (!isfinite(err) || !isfinite(alpha[j])) s_nonfin = 1;
-            s_done = s_conv || s_nonfin || j == mmax - 1;
-            ks->err = err;
+        cl.sync();
+        double b2 = 0.0;
+        for (int q = 0; q < SK_CL; ++q) b2 += sm.xn[q];
+        const double bj = sqrt(b2);
+        if (warp == 0) {
+            const double al = sm.h1[j].x + sm.h2[j].x;
+            if (lane == 0) {
+                sm.beta[j] = bj;
+                sm.alpha[j] = al;
+            }
+            if (arnoldi)   // the whole column j: projections, beta_j, zeros below
+                sm.hess[32 * j + lane] = lane <= j ? cadd(sm.h1[lane], sm.h2[lane])
+                                                   : make_double2(lane == j + 1 ? bj : 0.0, 0.0);
+            __syncwarp();
+            if (arnoldi) hess_expm_warp(sm.hess, sm.hvec, j + 1, zr, zi, sm.c);
+            else tridiag_expm_warp(sm.alpha, sm.beta, j + 1, zr, zi, sm.c);
+            __syncwarp();
+            if (lane == 0) {
+                const cplx cj = sm.c[j];
+                const double err = bj * sqrt(cj.x * cj.x + cj.y * cj.y);
+                sm.conv = err <= tol;
+                if (!isfinite(err) || !isfinite(al)) sm.nonfin = 1;
+                sm.done = sm.conv || sm.nonfin || j == mmax - 1;
+                sm.err = err;
+            }
+        } else {
+            // meanwhile: v_{j+1} and its product (not used when this step was the last)
+            const double inv = bj > 0.0 ? 1.0 / bj : 0.0;
+            cplx* vn = V + (j + 1) * s;
+            for (int e = tid - 32; e < s; e += SK_THREADS - 32) vn[e] = make_double2(sm.xw[e].x * inv, sm.xw[e].y * inv);
+            asm volatile("bar.sync 1, %0;" ::"n"(SK_THREADS - 32) : "memory");
+            matvec(vn, tid - 32, SK_THREADS - 32);
         }
         __syncthreads();
-        if (s_done) break;
-        const double inv = 1.0 / s_beta;
-        cplx* vn = V + (long long)(j + 1) * s;
-        for (int e = tid; e < s; e += SMALL_KRYLOV_THREADS) vn[e] = make_double2(w[e].x * inv, w[e].y * inv);
-        __syncthreads();
+        if (sm.done) break;
     }
-    // x = |x0| sum_i c_i v_i
-    for (int e = tid; e < s; e += SMALL_KRYLOV_THREADS) {
+    // x = |x0| sum_i c_i v_i, own rows
+    if (tid < nr) {
         cplx acc = make_double2(0.0, 0.0);
-        for (int i = 0; i <= j; ++i) acc = cadd(acc, cmul(V[(long long)i * s + e], c[i]));
-        x[e] = make_double2(acc.x * s_nrm0, acc.y * s_nrm0);
+        for (int i = 0; i <= j; ++i) acc_cmul(acc, V[i * s + r0 + tid], sm.c[i]);
+        x[r0 + tid] = make_double2(acc.x * nrm0, acc.y * nrm0);
     }
-    if (tid == 0) {
-        ks->converged = s_conv;
-        ks->nonfinite = s_nonfin;
-        ks->alpha[0] = (double)(j + 1);
+    if (rank == 0 && tid == 0) {
+        ks->st.err = sm.err;
+        ks->st.converged = sm.conv;
+        ks->st.nonfinite = sm.nonfin;
+        ks->st.iters = j + 1;
     }
 }
 
@@ -716,7 +856,9 @@ inline int grid_for(long long n) {
 
 // ------------------------------------------------------------------ launchers
 int red_blocks_for(long long n) {
-    long long g = (n + 2047) / 2048;
+    // 64 elements per block while blocks are free: a 6561-entry node on four
+    // blocks of 2048 left 148 SMs idle on FP64-bound sums
+    long long g = (n + 63) / 64;
     if (g > RED_BLOCKS) g = RED_BLOCKS;
     if (g < 1) g = 1;
     return (int)g;
@@ -728,26 +870,31 @@ int k_norm2_partial(const cplx* x, long long n, double* partial, cudaStream_t s)
     return 1;
 }
 
-int k_dots_partial(const cplx* V, long long ld, int nv, const cplx* w, long long n, cplx* partial,
-                   cudaStream_t s) {
-    int G = red_blocks_for(n);
-    dots_kernel<<<G, T, 0, s>>>(const_cast<cplx*>(V), ld, nv, w, n, G, partial, -1, nullptr, 0, -1);
+int k_dots(const cplx* V, long long ld, int nv, const cplx* w, long long n, cplx* partial, cudaStream_t s) {
+    const int G = red_blocks_for(n);
+    dots_kernel<<<G, T, 0, s>>>(V, ld, nv, w, n, G, partial);
     return 1;
 }
 
-int k_dots_scaled(cplx* V, long long ld, int nv, const cplx* w, long long n, cplx* partial,
-                  int scale_col, const double* scale_src, long long skip_col, cudaStream_t s) {
-    int G = red_blocks_for(n);
-    dots_kernel<<<G, T, 0, s>>>(V, ld, nv, w, n, G, partial, scale_col, scale_src, 1, skip_col);
+int k_orth_first(const cplx* V, long long ld, int nv, const cplx* partial_in, cplx* w, long long n, cplx* partial_dots,
+                 cplx* h_out, cudaStream_t s) {
+    const int G = red_blocks_for(n);
+    orth_first_kernel<<<G, T, 0, s>>>(V, ld, nv, partial_in, w, n, G, partial_dots, h_out);
     return 1;
 }
 
-int k_orth_update_ex(const cplx* V, long long ld, int nv, const cplx* partial_in, cplx* w, long long n,
-                     int mode, cplx* partial_dots, double* partial_norm, cplx* h_out, int accumulate,
-                     long long skip_col, cudaStream_t s) {
-    int G = red_blocks_for(n);
-    orth_update_kernel<<<G, T, 0, s>>>(V, ld, nv, partial_in, w, n, G, mode, partial_dots,
-                                       partial_norm, h_out, accumulate, skip_col);
+int k_lanczos_first(const cplx* V, long long ld, int j, const cplx* partial_in, const KrylovScalars* ks, cplx* w,
+                    long long n, cplx* partial_dots, cplx* h_out, cudaStream_t s) {
+    const int G = red_blocks_for(n);
+    lanczos_first_kernel<<<G, T, 0, s>>>(V, ld, j, partial_in, ks, w, n, G, partial_dots, h_out);
+    return 1;
+}
+
+int k_orth_second(const cplx* V, long long ld, int nv, const cplx* partial_in, cplx* w, long long n,
+                  double* partial_norm, KrylovScalars* ks, const cplx* h1, double zr, double zi, double tol,
+                  int arnoldi, cudaStream_t s) {
+    const int G = red_blocks_for(n);
+    orth_second_kernel<<<G, T, 0, s>>>(V, ld, nv, partial_in, w, n, G, partial_norm, ks, h1, zr, zi, tol, arnoldi);
     return 1;
 }
 
@@ -769,18 +916,6 @@ int k_combine(const cplx* V, long long ld, int nv, const KrylovScalars* ks, cplx
 
 int k_krylov_start_ex(KrylovScalars* ks, const double* nrm2_partial, long long n, cudaStream_t s) {
     krylov_start_kernel<<<1, 32, 0, s>>>(ks, nrm2_partial, red_blocks_for(n));
-    return 1;
-}
-
-int k_krylov_scalars_ex(KrylovScalars* ks, const cplx* h1, const cplx* h2, const double* beta_partial,
-                        long long n, int j, double zr, double zi, double tol, cudaStream_t s) {
-    krylov_scalars_kernel<<<1, 32, 0, s>>>(ks, h1, h2, beta_partial, red_blocks_for(n), j, zr, zi, tol);
-    return 1;
-}
-
-int k_arnoldi_scalars(KrylovScalars* ks, const cplx* h1, const cplx* h2, const double* beta_partial, long long n,
-                      int j, double zr, double zi, double tol, cudaStream_t s) {
-    arnoldi_scalars_kernel<<<1, 32, 0, s>>>(ks, h1, h2, beta_partial, red_blocks_for(n), j, zr, zi, tol);
     return 1;
 }
 
@@ -838,16 +973,10 @@ int k_weighted_sum(const cplx* N, int nb, long long n, const double* W, int r, c
     return 1;
 }
 
-int k_dense_heff(cplx* H, const int* d, const cplx* hb0, const cplx* hb1, const cplx* hb2, const SmallPairs& pp,
-                 cudaStream_t s) {
-    const long long n = (long long)d[0] * d[1] * d[2];
-    dense_heff_kernel<<<grid_for(n * n), 256, 0, s>>>(H, d[0], d[1], d[2], hb0, hb1, hb2, pp);
-    return 1;
-}
-
-int k_small_krylov(const cplx* H, int n, cplx* x, double zr, double zi, double tol, int mmax, int arnoldi,
-                   KrylovScalars* ks, cudaStream_t s) {
-    const size_t smem = sizeof(cplx) * ((size_t)n * n + (size_t)(mmax + 2) * n);
+int k_small_krylov(const int* d, const cplx* hb0, const cplx* hb1, const cplx* hb2, const SmallPairs& pp, cplx* x,
+                   double zr, double zi, double tol, int mmax, int arnoldi, KrylovScalars* ks, cudaStream_t s) {
+    const int n = d[0] * d[1] * d[2], R = (n + SK_CL - 1) / SK_CL;
+    const size_t smem = sizeof(cplx) * ((size_t)R * n + (size_t)(mmax + 1) * n);
     // the shared-memory limit is a per-device attribute of the kernel: set it
     // once on every device the process uses
     static std::mutex mu;
@@ -860,10 +989,11 @@ int k_small_krylov(const cplx* H, int n, cplx* x, double zr, double zi, double t
         if (!attr[dev]) {
             cudaFuncSetAttribute(small_krylov_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)(sizeof(cplx) *
-                                       ((size_t)SMALL_S * SMALL_S + (size_t)(KRYLOV_MMAX + 2) * SMALL_S)));
+                                       ((size_t)SK_ROWS * SMALL_S + (size_t)(KRYLOV_MMAX + 1) * SMALL_S)));
             attr[dev] = true;
         }
     }
-    small_krylov_kernel<<<1, SMALL_KRYLOV_THREADS, smem, s>>>(H, n, x, zr, zi, tol, mmax, arnoldi, ks);
+    small_krylov_kernel<<<SK_CL, SK_THREADS, smem, s>>>(d[0], d[1], d[2], hb0, hb1, hb2, pp, x, zr, zi, tol, mmax,
+                                                        arnoldi, ks);
     return 1;
 }

@@ -134,16 +134,18 @@ struct ttn_ctx {
     long long gcap = 0;
     cplx* hb[3] = {nullptr, nullptr, nullptr};
     cplx* Rbuf = nullptr;
-    cplx* dense_H = nullptr;  // SMALL_S^2: dense H_eff of a small node or link
     cplx* Kbasis = nullptr;   // (KRYLOV_MMAX + 1) * smax
     KrylovScalars* ks = nullptr;
     cplx* kh1 = nullptr;      // KRYLOV_MMAX + 1
-    cplx* kh2 = nullptr;
     cplx* kpart = nullptr;    // 2 * RED_BLOCKS * (KRYLOV_MMAX + 1)
     double* kpn = nullptr;    // RED_BLOCKS
     double* apx = nullptr;    // RED_BLOCKS: norm^2 partials of an absorbed node
     double* apr = nullptr;    // RED_BLOCKS: norm^2 partials of the absorbed link matrix
-    int* hflag = nullptr;     // pinned host: converged, nonfinite
+    struct HostStatus {
+        KrylovStatus krylov;
+        int tc_flag;
+    };
+    HostStatus* hstat = nullptr;   // pinned host: status read back from the device
     QrScratch qr{};
     std::map<std::pair<int, int>, int*> cand;   // (node, leg) -> candidate rows
     std::map<std::pair<int, int>, int> ncand;
@@ -930,8 +932,9 @@ void assemble(ttn_ctx* c, const Env& e, cplx* out) {
 bool env_has_block(const Env& e) { return e.has_H || !e.sites.empty(); }
 
 // --------------------------------------------------------------- Krylov
-// x <- exp(z H) x with H given by `apply`, Lanczos with full two-pass
-// re-orthogonalisation; z = (zr, zi).
+// x <- exp(z H) x with H given by `apply`; z = (zr, zi).  Lanczos: the
+// three-term recurrence, then a pass against the whole basis; with decay
+// (non-Hermitian H) Arnoldi, two passes against the whole basis.
 template <class F>
 void krylov(ttn_ctx* c, cplx* x, long long n, double zr, double zi, F apply) {
     cudaStream_t s = c->stream;
@@ -945,6 +948,7 @@ void krylov(ttn_ctx* c, cplx* x, long long n, double zr, double zi, F apply) {
         c->stats[3] += k_krylov_start_ex(c->ks, c->kpn, n, s);
         c->stats[3] += k_scale_copy_dev(x, n, &c->ks->inv_scale, V, s);
     }
+    const KrylovStatus& st = c->hstat->krylov;
     int j = 0;
     for (;; ++j) {
         cplx* vj = V + (long long)j * ld;
@@ -952,41 +956,41 @@ void krylov(ttn_ctx* c, cplx* x, long long n, double zr, double zi, F apply) {
         apply(vj, w);
         c->stats[1] += 1;
         {
-            // bytes: the basis is read three times (dots, two update passes), w read and written twice
-            ProfScope ps(c, PK_KRY, 0.0, 16.0 * n * (3.0 * (j + 1) + 5.0));
-            c->stats[3] += k_dots_scaled(V, ld, j + 1, w, n, c->kpart, -1, nullptr, -1, s);
+            // bytes: the basis is read twice (Arnoldi: three times), w read and written twice
+            const bool arnoldi = c->gamma != 0.0;   // non-Hermitian generator (decay)
+            ProfScope ps(c, PK_KRY, 0.0, 16.0 * n * ((arnoldi ? 3.0 : 2.0) * (j + 1) + 7.0));
             cplx* part2 = c->kpart + (size_t)RED_BLOCKS * (KRYLOV_MMAX + 1);
-            c->stats[3] += k_orth_update_ex(V, ld, j + 1, c->kpart, w, n, 1, part2, nullptr, c->kh1, 0, -1, s);
-            c->stats[3] += k_orth_update_ex(V, ld, j + 1, part2, w, n, 2, nullptr, c->kpn, c->kh2, 0, -1, s);
-            if (c->gamma != 0.0)   // non-Hermitian generator (decay): Arnoldi
-                c->stats[3] += k_arnoldi_scalars(c->ks, c->kh1, c->kh2, c->kpn, n, j, zr, zi, tol, s);
-            else
-                c->stats[3] += k_krylov_scalars_ex(c->ks, c->kh1, c->kh2, c->kpn, n, j, zr, zi, tol, s);
+            if (arnoldi) {
+                c->stats[3] += k_dots(V, ld, j + 1, w, n, c->kpart, s);
+                c->stats[3] += k_orth_first(V, ld, j + 1, c->kpart, w, n, part2, c->kh1, s);
+            } else {
+                c->stats[3] += k_dots(vj, ld, 1, w, n, c->kpart, s);
+                c->stats[3] += k_lanczos_first(V, ld, j, c->kpart, c->ks, w, n, part2, c->kh1, s);
+            }
+            c->stats[3] += k_orth_second(V, ld, j + 1, part2, w, n, c->kpn, c->ks, c->kh1, zr, zi, tol, arnoldi, s);
         }
-        CUDA_OK(cudaMemcpyAsync(c->hflag, &c->ks->converged, 2 * sizeof(int), cudaMemcpyDeviceToHost, s));
-        c->hflag[2] = 0;
+        CUDA_OK(cudaMemcpyAsync(&c->hstat->krylov, &c->ks->st, sizeof(st), cudaMemcpyDeviceToHost, s));
+        c->hstat->tc_flag = 0;
         if (c->split_ws)   // a tensor-core wait that gave up leaves garbage: report it first
-            CUDA_OK(cudaMemcpyAsync(c->hflag + 2, c->split_ws, sizeof(int), cudaMemcpyDeviceToHost, s));
+            CUDA_OK(cudaMemcpyAsync(&c->hstat->tc_flag, c->split_ws, sizeof(int), cudaMemcpyDeviceToHost, s));
         CUDA_OK(cudaStreamSynchronize(s));
-        if (c->hflag[2]) check_split_flag(c);
-        if (c->hflag[1]) throw TtnError(TTN_ERR_NUMERIC, "non-finite value in Lanczos");
-        if (c->hflag[0] || j == mmax - 1) break;
+        if (c->hstat->tc_flag) check_split_flag(c);
+        if (st.nonfinite) throw TtnError(TTN_ERR_NUMERIC, "non-finite value in Lanczos");
+        if (st.converged || j == mmax - 1) break;
         ProfScope ps(c, PK_KRY, 0.0, 32.0 * n);
         c->stats[3] += k_scale_copy_dev(w, n, &c->ks->inv_scale, w, s);
     }
-    if (!c->hflag[0]) {
-        double err;
-        CUDA_OK(cudaMemcpy(&err, &c->ks->err, sizeof(double), cudaMemcpyDeviceToHost));
-        c->max_err = std::max(c->max_err, err);
-        if (err > 1e-6) throw TtnError(TTN_ERR_KRYLOV, "Lanczos did not converge in m_max steps");
+    if (!st.converged) {
+        c->max_err = std::max(c->max_err, st.err);
+        if (st.err > 1e-6) throw TtnError(TTN_ERR_KRYLOV, "Lanczos did not converge in m_max steps");
     }
     c->stats[0] += 1;
     ProfScope ps(c, PK_KRY, 0.0, 16.0 * n * (j + 2));
     c->stats[3] += k_combine(V, ld, j + 1, c->ks, x, n, s);
 }
 
-// Small nodes and links (s <= SMALL_S): H_eff as a dense matrix and the whole
-// Krylov exponential in one launch (same algorithm and stopping rule as
+// Small nodes and links (s <= SMALL_S): the whole Krylov exponential in one
+// launch, with H_eff as a dense matrix (same algorithm and stopping rule as
 // krylov()), with one host round trip for the status instead of one per
 // Lanczos step.
 bool small_evolve(ttn_ctx* c, const int* d, cplx* const* hb, const Pair* pairs, int np, cplx* x, double zr,
@@ -1006,23 +1010,16 @@ bool small_evolve(ttn_ctx* c, const int* d, cplx* const* hb, const Pair* pairs, 
     const double tol = (c->prec == TTN_FP64) ? 1e-13 : 1e-9;
     {
         ProfScope ps(c, PK_KRY, 0.0, 0.0);
-        c->stats[3] += k_dense_heff(c->dense_H, d, hb[0], hb[1], hb[2], pp, c->stream);
-        c->stats[3] += k_small_krylov(c->dense_H, (int)s, x, zr, zi, tol, test_krylov_mmax(),
+        c->stats[3] += k_small_krylov(d, hb[0], hb[1], hb[2], pp, x, zr, zi, tol, test_krylov_mmax(),
                                       c->gamma != 0.0 ? 1 : 0, c->ks, c->stream);
     }
-    struct {
-        double alpha0;
-        double err;
-        int flags[2];
-    } st;
-    CUDA_OK(cudaMemcpyAsync(&st.alpha0, &c->ks->alpha[0], sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    CUDA_OK(cudaMemcpyAsync(&st.err, &c->ks->err, sizeof(double), cudaMemcpyDeviceToHost, c->stream));
-    CUDA_OK(cudaMemcpyAsync(st.flags, &c->ks->converged, 2 * sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+    KrylovStatus& st = c->hstat->krylov;
+    CUDA_OK(cudaMemcpyAsync(&st, &c->ks->st, sizeof(st), cudaMemcpyDeviceToHost, c->stream));
     CUDA_OK(cudaStreamSynchronize(c->stream));
-    if (st.flags[1]) throw TtnError(TTN_ERR_NUMERIC, "non-finite value in Lanczos");
+    if (st.nonfinite) throw TtnError(TTN_ERR_NUMERIC, "non-finite value in Lanczos");
     c->stats[0] += 1;
-    c->stats[1] += (int64_t)st.alpha0;
-    if (!st.flags[0]) {
+    c->stats[1] += st.iters;
+    if (!st.converged) {
         c->max_err = std::max(c->max_err, st.err);
         if (st.err > 1e-6) throw TtnError(TTN_ERR_KRYLOV, "Lanczos did not converge in m_max steps");
     }
@@ -1606,11 +1603,9 @@ void allocate(ttn_ctx* c) {
     for (int i = 0; i < 3; ++i) c->Gbuf[i] = (cplx*)dalloc(c, sizeof(cplx) * gc);
     for (int i = 0; i < 3; ++i) c->hb[i] = (cplx*)dalloc(c, sizeof(cplx) * MAX_CHI * MAX_CHI);
     c->Rbuf = (cplx*)dalloc(c, sizeof(cplx) * MAX_CHI * MAX_CHI);
-    c->dense_H = (cplx*)dalloc(c, sizeof(cplx) * SMALL_S * SMALL_S);
     c->Kbasis = (cplx*)dalloc(c, sizeof(cplx) * (KRYLOV_MMAX + 1) * c->smax);
     c->ks = (KrylovScalars*)dalloc(c, sizeof(KrylovScalars));
     c->kh1 = (cplx*)dalloc(c, sizeof(cplx) * (KRYLOV_MMAX + 1));
-    c->kh2 = (cplx*)dalloc(c, sizeof(cplx) * (KRYLOV_MMAX + 1));
     c->kpart = (cplx*)dalloc(c, sizeof(cplx) * 2 * RED_BLOCKS * (MAX_CHI + 2));
     c->kpn = (double*)dalloc(c, sizeof(double) * RED_BLOCKS);
     c->apx = (double*)dalloc(c, sizeof(double) * RED_BLOCKS);
@@ -1621,7 +1616,7 @@ void allocate(ttn_ctx* c) {
     alloc_qr_scratch(c, mq, MAX_CHI, c->qr);
     c->d_coef = (double*)dalloc(c, sizeof(double) * 5 * c->N);
     c->h_coef.assign(5 * c->N, 0.0);
-    CUDA_OK(cudaMallocHost(&c->hflag, 4 * sizeof(int)));
+    CUDA_OK(cudaMallocHost(&c->hstat, sizeof(ttn_ctx::HostStatus)));
     c->up.assign(nn, Env());
     c->down.assign(nn, Env());
     c->phys.assign(c->n_leaves, Env());
@@ -1953,7 +1948,7 @@ void ttn_destroy(ttn_ctx* c) {
         if (c->shX[i]) cudaFree(c->shX[i]);
     }
     for (cudaEvent_t e : c->ev_pool) cudaEventDestroy(e);
-    if (c->hflag) cudaFreeHost(c->hflag);
+    if (c->hstat) cudaFreeHost(c->hstat);
     delete c;
 }
 
