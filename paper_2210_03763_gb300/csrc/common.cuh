@@ -190,10 +190,12 @@ double k_fp64_probe(int method, int blocks, int iters, double* out, cudaStream_t
 int k_weighted_sum(const cplx* N, int nb, long long n, const double* W, int r, cplx* G, cudaStream_t s);
 
 // ---- QR (qr.cu) ----------------------------------------------------------------
-// QR kernels use one block per QR_ROWS rows; partial sums are sized
-// G = ceil(M / QR_ROWS) per column (part: 2 * G * (D + 1) complex), and the
+// QR kernels use one block per QR_ROWS rows (the column loop of smaller
+// matrices: fewer rows, at most QR_SMALL_BLOCKS blocks); partial sums are sized
+// G = max(ceil(M / QR_ROWS), QR_SMALL_BLOCKS) per column (part: 2 * G * (D + 1) complex), and the
 // Frobenius pass uses up to QR_FROB_BLOCKS partials (pnorm >= max of both).
 constexpr int QR_ROWS = 128;
+constexpr int QR_SMALL_BLOCKS = 152;
 constexpr int QR_FROB_BLOCKS = 1024;
 struct QrScratch {
     cplx* part;         // 2 * row blocks * (2 * MAX_CHI + 4) partial sums
@@ -213,7 +215,8 @@ struct QrScratch {
     int* row_rank;      // M: step at which a row was accepted (INT_MAX: never)
     int* cand_used;     // M: candidate accepted flags
     unsigned* bar;      // 2: grid barrier of the cooperative column loop
-    int* err;           // set when a bounded device wait gave up
+    int* err;           // [0] set when a bounded device wait gave up, [1] when the panel path gave up
+    cplx* panel;        // panel path: 3 (D + QR_PANEL) QR_PANEL + 3 QR_PANEL^2
 };
 constexpr int QR_SC_MAXR = 64;   // structured completion when the kept rank r <= this
 // In-place QR of the column-major M x D matrix A (lda = M): A <- Q, R (D x D,
@@ -224,6 +227,17 @@ constexpr int QR_SC_MAXR = 64;   // structured completion when the kept rank r <
 // dependence threshold of the completion rule, 1e-10 for every QR of the
 // library).
 constexpr double QR_TOL_FP64 = 1e-10;
+constexpr int QR_PANEL = 32;
+// QR of a well-conditioned matrix by panels (qr_panel.cu): columns [first,
+// last) of A in place and of R (zeroed before), ws.scal[0] = |A|_F^2 and
+// ws.err[1] = 0 before the first call.  ws.err[1] != 0 afterwards: not
+// well-conditioned, A and R undefined.  Workspace as launch_zgemm_digits (of
+// qr_panel_workspace bytes).  Returns launches, -1 when not available.
+size_t qr_panel_workspace(int M, int D);
+int qr_panel(cplx* A, int M, int D, cplx* R, QrScratch& ws, cudaStream_t s, void* workspace, size_t workspace_bytes,
+             int first, int last);
+// |A|_F^2 into ws.scal[0].
+int qr_frobenius(const cplx* A, long long n, QrScratch& ws, cudaStream_t s);
 int qr_cgs2(cplx* A, int M, int D, cplx* R, const int* cand, int ncand,
             QrScratch& ws, cudaStream_t s, int* n_dependent_host, double tol = QR_TOL_FP64);
 

@@ -117,8 +117,10 @@ __device__ void max_exps(const DigitSide& s, const cplx* const* base, int k0, in
 }
 
 // x on the grid 2^(E - 55), E = emax - 1022: the integer t, round to nearest
-// even, as seven signed digits (d[0] the highest).
-__device__ __forceinline__ void digits_of(double x, int emax, int* d) {
+// even, plus 128 in each of its six low bytes.  Byte i of the result minus 128
+// is then the signed digit of weight 256^i, and bits 48.. the highest digit:
+// one 64-bit addition carries for all of them.
+__device__ __forceinline__ unsigned long long biased_digits(double x, int emax) {
     const unsigned long long u = (unsigned long long)__double_as_longlong(x);
     const int e = (int)((u >> 52) & 0x7FF);
     unsigned long long m = u & 0xFFFFFFFFFFFFFULL;
@@ -133,18 +135,22 @@ __device__ __forceinline__ void digits_of(double x, int emax, int* d) {
     } else {
         m = 0;
     }
-    long long t = (u >> 63) ? -(long long)m : (long long)m;
-#pragma unroll
-    for (int i = ND - 1; i > 0; --i) {
-        const int c = (int)(signed char)(t & 0xFF);
-        d[i] = c;
-        t = (t - c) >> 8;
-    }
-    d[0] = (int)t;
+    const long long t = (u >> 63) ? -(long long)m : (long long)m;
+    return (unsigned long long)t + 0x808080808080ULL;
 }
 
-__device__ __forceinline__ uint32_t bf16_pair(int lo, int hi) {   // exact for |d| <= 256
-    return __byte_perm(__float_as_uint((float)lo), __float_as_uint((float)hi), 0x7632);
+// Digit q (0 the highest) of biased digits t as a float: the byte under the
+// exponent of 2^23, minus 2^23 + 128 (the highest digit through a conversion).
+__device__ __forceinline__ float digit_float(unsigned long long t, int q) {
+    if (q == 0) return (float)(int)((long long)t >> 48);
+    const uint32_t w = q <= 2 ? (uint32_t)(t >> 32) : (uint32_t)t;
+    const int byte = q <= 2 ? 2 - q : 6 - q;   // byte of the word
+    return __uint_as_float(__byte_perm(w, 0x4B000000u, 0x7440u | (uint32_t)byte)) - 8388736.0f;
+}
+// (lo, hi) as a bf16 pair: digits are integers up to 128, so the upper half of
+// the float is exact.
+__device__ __forceinline__ uint32_t bf16_pair(float lo, float hi) {
+    return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);
 }
 
 // Row exponents over blocks of K (long K only): exps zeroed before.
@@ -220,25 +226,26 @@ __global__ void __launch_bounds__(PK_THREADS) digit_pack_kernel(DigitSide sp, Di
             const int r = warp + 8 * i;
             const long long f = f0 + r;
             if (f >= nrow || k >= s.Kc) continue;
-            const cplx v = tile[lane][r];
-            int dr[ND], di[ND];
-            const bool special = mx[r] == 0x7FF;   // the epilogue recomputes such rows
-            digits_of(special ? 0.0 : v.x, mx[r], dr);
-            digits_of(special ? 0.0 : v.y, mx[r], di);
-            if (s.conj)
-#pragma unroll
-                for (int q = 0; q < ND; ++q) di[q] = -di[q];
-            if (s.embed) {
-                uint16_t* o = s.planes + (2 * f) * 2LL * s.Kc + 2LL * k;
+            uint16_t* o = s.planes + (s.embed ? 2 * f : f) * 2LL * s.Kc + 2LL * k;
+            if (!base[r] || mx[r] == 0x7FF) {   // padding; rows that the epilogue recomputes
 #pragma unroll
                 for (int q = 0; q < ND; ++q) {
-                    *reinterpret_cast<uint32_t*>(o + q * plane) = bf16_pair(dr[q], -di[q]);
-                    *reinterpret_cast<uint32_t*>(o + q * plane + 2LL * s.Kc) = bf16_pair(di[q], dr[q]);
+                    *reinterpret_cast<uint32_t*>(o + q * plane) = 0u;
+                    if (s.embed) *reinterpret_cast<uint32_t*>(o + q * plane + 2LL * s.Kc) = 0u;
                 }
-            } else {
-                uint16_t* o = s.planes + f * 2LL * s.Kc + 2LL * k;
+                continue;
+            }
+            const cplx v = tile[lane][r];
+            const unsigned long long tr = biased_digits(v.x, mx[r]), ti = biased_digits(s.conj ? -v.y : v.y, mx[r]);
 #pragma unroll
-                for (int q = 0; q < ND; ++q) *reinterpret_cast<uint32_t*>(o + q * plane) = bf16_pair(dr[q], di[q]);
+            for (int q = 0; q < ND; ++q) {
+                const uint32_t w = bf16_pair(digit_float(tr, q), digit_float(ti, q));   // (re, im)
+                if (s.embed) {   // (re, -im) and (im, re)
+                    *reinterpret_cast<uint32_t*>(o + q * plane) = w ^ 0x80000000u;
+                    *reinterpret_cast<uint32_t*>(o + q * plane + 2LL * s.Kc) = __byte_perm(w, 0u, 0x1032);
+                } else {
+                    *reinterpret_cast<uint32_t*>(o + q * plane) = w;
+                }
             }
         }
         __syncthreads();
@@ -461,7 +468,11 @@ __global__ void __launch_bounds__(THREADS, 1)
                         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                         const uint32_t base = smem_u32(smem + s * STAGE_BYTES);
                         const uint64_t dp = sdesc64(base), dq = sdesc64(base + P_BYTES);
+                        // unrolled: the descriptors are then immediate offsets (a loop over the digits
+                        // took 110 clk per MMA to issue, the MMA 32 to 48)
+#pragma unroll
                         for (int l = 0; l < NLEV; ++l) {
+                            if (!ok) break;
                             if (st == c0 && cg > 0) {
                                 if (!mbar_wait(&lempty[l], (cg - 1) & 1, ea.err)) {
                                     ok = false;
@@ -469,7 +480,8 @@ __global__ void __launch_bounds__(THREADS, 1)
                                 }
                                 asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
                             }
-                            const int i0 = max(0, l - (ND - 1)), i1 = min(ND - 1, l);
+                            const int i0 = l > ND - 1 ? l - (ND - 1) : 0, i1 = l < ND - 1 ? l : ND - 1;
+#pragma unroll
                             for (int i = i0; i <= i1; ++i) {
                                 const uint64_t a = dp + (uint64_t)(i * P_PLANE >> 4);
                                 const uint64_t q = dq + (uint64_t)((l - i) * Q_PLANE >> 4);
@@ -625,7 +637,7 @@ DPlan plan(const GemmArgs& g) {
     d.nsplit = 1;
     d.cps = nchunk;
     long long best = (t + N_SM - 1) / N_SM * (nchunk + 1);
-    for (int n = 2; n <= std::min(nchunk, 64); ++n) {
+    for (int n = 2; n <= std::min(nchunk, N_SM); ++n) {
         const int c = (nchunk + n - 1) / n, k = (nchunk + c - 1) / c;
         const long long cost = (t * k + N_SM - 1) / N_SM * (c + 1) + 1;
         if (cost < best) {

@@ -157,8 +157,9 @@ __global__ void splitk_f64_kernel(GemmArgs g, int nsplit, const cplx* W) {
          e += (long long)gridDim.x * blockDim.x) {
         const long long b = e / MN, mn = e - b * MN;
         const int m = (int)(mn % g.M), n = (int)(mn / g.M);
-        cplx v = W[b * MN + mn];
-        for (int ks = 1; ks < nsplit; ++ks) {
+        cplx v = make_double2(0.0, 0.0);
+#pragma unroll 8
+        for (int ks = 0; ks < nsplit; ++ks) {   // several loads in flight
             const cplx w = W[((long long)ks * nbatch + b) * MN + mn];
             v.x += w.x;
             v.y += w.y;
@@ -353,7 +354,7 @@ int launch_zgemm_f64(const GemmArgs& g, cudaStream_t stream, void* workspace, si
 
 int launch_splitk_f64(const GemmArgs& g, int nsplit, const cplx* W, cudaStream_t stream) {
     const long long total = (long long)g.M * g.N * g.Bi * g.Bo;
-    const unsigned grid = (unsigned)std::min<long long>((total + 255) / 256, 152 * 8);
-    splitk_f64_kernel<<<grid, 256, 0, stream>>>(g, nsplit, W);
+    const unsigned grid = (unsigned)std::min<long long>((total + 63) / 64, 152 * 16);   // small outputs: more SMs
+    splitk_f64_kernel<<<grid, 64, 0, stream>>>(g, nsplit, W);
     return 1;
 }

@@ -110,7 +110,10 @@ __global__ void frob_partial_kernel(const cplx* A, long long n, double* partial)
 }
 
 __global__ void frob_finish_kernel(const double* partial, int G, double* scal) {
-    if (threadIdx.x == 0) scal[0] = sum_norm(partial, G);
+    double s = 0.0;
+    for (int g = threadIdx.x; g < G; g += 32) s += partial[g];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) scal[0] = s;
 }
 
 // norm^2 partials of column 0 (no projections)
@@ -270,8 +273,7 @@ __device__ __forceinline__ unsigned long long qr_global_ns() {
     asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
     return t;
 }
-constexpr int QCS = QB + 1;            // cache column stride (odd: no bank conflicts)
-constexpr int QC_MAX = 32;             // kept columns cached in shared memory
+constexpr int QC_MAX = 32;             // kept columns cached in shared memory when several blocks share an SM
 constexpr int PSTRIDE = 2 * MAXD + 4;  // partial row length
 
 struct CoopSm {
@@ -397,14 +399,23 @@ __device__ void sum_rows(const cplx* part, int G, int E, cplx* out, CoopSm& sm) 
     __syncthreads();
 }
 
+// Rows per block RB (8 to 128): small matrices are cut finer than QB rows, so
+// that their FP64 work is spread over as many SMs as they have rows for (one
+// block of 128 rows took 57 us per column of a 128 x 128 matrix, 38 of them
+// on its SM's FP64 pipe).  QB threads per block: QB / RB of them share a row
+// in the combinations Q h (slices of the columns, summed by shuffles).
+// Cache column stride: RB + 1 (odd: no bank conflicts).
+
 // Row rr of kept column j (shared-memory cache or global).
+template <int RB>
 __device__ __forceinline__ cplx qcol(const cplx* A, long long M, long long r0, const cplx* qc, int nc, int j, int rr,
                                      const CoopSm& sm) {
-    return j < nc ? qc[j * QCS + rr] : A[r0 + rr + (long long)sm.nz[j] * M];
+    return j < nc ? qc[j * (RB + 1) + rr] : A[r0 + rr + (long long)sm.nz[j] * M];
 }
 
 // This block's partials of X(k): out[j] = Q_j^H v1, out[n + j] = Q_j^H a_next
 // (j < n), out[2n] = v1^H a_next, out[2n + 1] = (|v1|^2, fro) over its rows.
+template <int RB>
 __device__ void coop_partials(const cplx* A, long long M, long long r0, int nrows, int n, const cplx* qc, int nc,
                               double fro, cplx* out, CoopSm& sm) {
     const int t = threadIdx.x;
@@ -412,7 +423,7 @@ __device__ void coop_partials(const cplx* A, long long M, long long r0, int nrow
         for (int j = t; j < n; j += QB) {
             cplx sv = make_double2(0.0, 0.0), sa = sv;
             for (int rr = 0; rr < nrows; ++rr) {
-                cplx a = qcol(A, M, r0, qc, nc, j, rr, sm), v = sm.v1[rr], b = sm.an[rr];
+                cplx a = qcol<RB>(A, M, r0, qc, nc, j, rr, sm), v = sm.v1[rr], b = sm.an[rr];
                 sv.x = fma(a.x, v.x, fma(a.y, v.y, sv.x));
                 sv.y = fma(a.x, v.y, fma(-a.y, v.x, sv.y));
                 sa.x = fma(a.x, b.x, fma(a.y, b.y, sa.x));
@@ -432,7 +443,7 @@ __device__ void coop_partials(const cplx* A, long long M, long long r0, int nrow
         if (j < n) {
 #pragma unroll 2
             for (int rr = q; rr < nrows; rr += sl) {
-                cplx a = qcol(A, M, r0, qc, nc, j, rr, sm), v = sm.v1[rr], b = sm.an[rr];
+                cplx a = qcol<RB>(A, M, r0, qc, nc, j, rr, sm), v = sm.v1[rr], b = sm.an[rr];
                 sv.x = fma(a.x, v.x, fma(a.y, v.y, sv.x));
                 sv.y = fma(a.x, v.y, fma(-a.y, v.x, sv.y));
                 sa.x = fma(a.x, b.x, fma(a.y, b.y, sa.x));
@@ -477,26 +488,38 @@ __device__ void coop_partials(const cplx* A, long long M, long long r0, int nrow
     __syncthreads();
 }
 
-// sum_j Q[r, nz_j] h[j] for this thread's row (j < n).
-__device__ __forceinline__ cplx coop_combo(const cplx* A, long long M, long long r0, int t, const cplx* qc, int nc,
-                                           int n, const cplx* h, const CoopSm& sm) {
+// sum_j Q[r, nz_j] h[j] (j < n) for row rr of the block, by the QB / RB
+// threads of the row (slice sl); the sum in all of them.  Called by whole
+// warps; rows past the matrix (own false) give zero.
+template <int RB>
+__device__ __forceinline__ cplx coop_combo(const cplx* A, long long M, long long r0, int rr, int sl, bool own,
+                                           const cplx* qc, int nc, int n, const cplx* h, const CoopSm& sm) {
+    constexpr int SL = QB / RB;
     cplx u0 = make_double2(0.0, 0.0), u1 = u0;
-    int j = 0;
+    if (own) {
+        int j = sl;
 #pragma unroll 2
-    for (; j + 1 < n; j += 2) {
-        cplx a = qcol(A, M, r0, qc, nc, j, t, sm), b = qcol(A, M, r0, qc, nc, j + 1, t, sm);
-        cplx ha = h[j], hb = h[j + 1];
-        u0.x = fma(a.x, ha.x, fma(-a.y, ha.y, u0.x));
-        u0.y = fma(a.x, ha.y, fma(a.y, ha.x, u0.y));
-        u1.x = fma(b.x, hb.x, fma(-b.y, hb.y, u1.x));
-        u1.y = fma(b.x, hb.y, fma(b.y, hb.x, u1.y));
+        for (; j + SL < n; j += 2 * SL) {
+            cplx a = qcol<RB>(A, M, r0, qc, nc, j, rr, sm), b = qcol<RB>(A, M, r0, qc, nc, j + SL, rr, sm);
+            cplx ha = h[j], hb = h[j + SL];
+            u0.x = fma(a.x, ha.x, fma(-a.y, ha.y, u0.x));
+            u0.y = fma(a.x, ha.y, fma(a.y, ha.x, u0.y));
+            u1.x = fma(b.x, hb.x, fma(-b.y, hb.y, u1.x));
+            u1.y = fma(b.x, hb.y, fma(b.y, hb.x, u1.y));
+        }
+        if (j < n) {
+            cplx a = qcol<RB>(A, M, r0, qc, nc, j, rr, sm), ha = h[j];
+            u0.x = fma(a.x, ha.x, fma(-a.y, ha.y, u0.x));
+            u0.y = fma(a.x, ha.y, fma(a.y, ha.x, u0.y));
+        }
     }
-    if (j < n) {
-        cplx a = qcol(A, M, r0, qc, nc, j, t, sm), ha = h[j];
-        u0.x = fma(a.x, ha.x, fma(-a.y, ha.y, u0.x));
-        u0.y = fma(a.x, ha.y, fma(a.y, ha.x, u0.y));
+    u0 = cadd(u0, u1);
+#pragma unroll
+    for (int o = SL / 2; o > 0; o >>= 1) {
+        u0.x += __shfl_xor_sync(0xffffffffu, u0.x, o);
+        u0.y += __shfl_xor_sync(0xffffffffu, u0.y, o);
     }
-    return cadd(u0, u1);
+    return u0;
 }
 
 // Sums of the partial rows of one synchronisation into sm.hb (E entries).
@@ -547,9 +570,10 @@ constexpr int LA_WMAX = 16;
 
 // One vector of the block's rows: 0 = kept column i, 1 = window vector i,
 // 2 = column i of A.
+template <int RB>
 __device__ __forceinline__ cplx la_vec(int kind, int i, int rr, const cplx* A, long long M, long long r0,
-                                       const cplx* qc, int nc, const cplx (*vw)[QB], const CoopSm& sm) {
-    if (kind == 0) return qcol(A, M, r0, qc, nc, i, rr, sm);
+                                       const cplx* qc, int nc, const cplx (*vw)[RB], const CoopSm& sm) {
+    if (kind == 0) return qcol<RB>(A, M, r0, qc, nc, i, rr, sm);
     if (kind == 1) return vw[i][rr];
     return A[r0 + rr + (long long)i * M];
 }
@@ -557,9 +581,9 @@ __device__ __forceinline__ cplx la_vec(int kind, int i, int rr, const cplx* A, l
 // out[p] = sum over the block's rows of conj(L_p) R_p for p < P, where
 // pair(p, lk, li, rk, ri) names the two vectors; row slices of a power-of-two
 // width are reduced by shuffles (as in coop_partials).
-template <class PairF>
+template <int RB, class PairF>
 __device__ void la_dots(int P, PairF pair, cplx* out, const cplx* A, long long M, long long r0, int nrows,
-                        const cplx* qc, int nc, const cplx (*vw)[QB], CoopSm& sm) {
+                        const cplx* qc, int nc, const cplx (*vw)[RB], CoopSm& sm) {
     const int t = threadIdx.x;
     if (P > QB) {
         for (int p = t; p < P; p += QB) {
@@ -567,7 +591,7 @@ __device__ void la_dots(int P, PairF pair, cplx* out, const cplx* A, long long M
             pair(p, lk, li, rk, ri);
             cplx s0 = make_double2(0.0, 0.0);
             for (int rr = 0; rr < nrows; ++rr) {
-                cplx a = la_vec(lk, li, rr, A, M, r0, qc, nc, vw, sm), b = la_vec(rk, ri, rr, A, M, r0, qc, nc, vw, sm);
+                cplx a = la_vec<RB>(lk, li, rr, A, M, r0, qc, nc, vw, sm), b = la_vec<RB>(rk, ri, rr, A, M, r0, qc, nc, vw, sm);
                 s0.x = fma(a.x, b.x, fma(a.y, b.y, s0.x));
                 s0.y = fma(a.x, b.y, fma(-a.y, b.x, s0.y));
             }
@@ -584,7 +608,7 @@ __device__ void la_dots(int P, PairF pair, cplx* out, const cplx* A, long long M
         int lk, li, rk, ri;
         pair(p, lk, li, rk, ri);
         for (int rr = q; rr < nrows; rr += sl) {
-            cplx a = la_vec(lk, li, rr, A, M, r0, qc, nc, vw, sm), b = la_vec(rk, ri, rr, A, M, r0, qc, nc, vw, sm);
+            cplx a = la_vec<RB>(lk, li, rr, A, M, r0, qc, nc, vw, sm), b = la_vec<RB>(rk, ri, rr, A, M, r0, qc, nc, vw, sm);
             sv.x = fma(a.x, b.x, fma(a.y, b.y, sv.x));
             sv.y = fma(a.x, b.y, fma(-a.y, b.x, sv.y));
         }
@@ -605,35 +629,40 @@ __device__ void la_dots(int P, PairF pair, cplx* out, const cplx* A, long long M
     __syncthreads();
 }
 
+template <int RB>
 __global__ void __launch_bounds__(QB) qr_coop_kernel(cplx* A, long long M, int D, cplx* R, int* flags, cplx* part,
                                                      cplx* red_out, unsigned* bar, int* err, int nc_max, double tol,
-                                                     int la_max) {
-    // dynamic shared memory: nc_max cached columns of QCS rows, then the
+                                                     int la_max, int rpb) {
+    // dynamic shared memory: nc_max cached columns of RB + 1 rows, then the
     // look-ahead window of at most la_max (<= LA_WMAX) columns (this block's
     // rows of v1_j)
     extern __shared__ cplx dyn[];
     cplx* qc = dyn;
-    cplx(*vw)[QB] = reinterpret_cast<cplx(*)[QB]>(dyn + (long long)nc_max * QCS);
+    cplx(*vw)[RB] = reinterpret_cast<cplx(*)[RB]>(dyn + (long long)nc_max * (RB + 1));
     __shared__ CoopSm sm;
     __shared__ cplx la_g[PSTRIDE];     // look-ahead: g_j = Q^H a_j (column j at j * nq)
     __shared__ double la_s2[LA_WMAX];
     const int G = gridDim.x, t = threadIdx.x;
-    const long long r0 = (long long)blockIdx.x * QB;
-    const int nrows = (int)min((long long)QB, M - r0);
-    const bool own = t < nrows;
-    const long long r = r0 + t;
+    constexpr int SL = QB / RB;
+    const int rr = t / SL, sl = t % SL;    // row of the block, slice of the row's work
+    const long long r0 = (long long)blockIdx.x * rpb;   // rpb <= RB rows per block
+    const int nrows = (int)min((long long)rpb, M - r0);
+    const bool own = rr < nrows, lead = own && sl == 0;   // lead: the thread that stores the row
+    const long long r = r0 + rr;
     const bool b0 = blockIdx.x == 0;
 
     // |A|_F^2 over this block's rows; v1_0 = a_0, a_next = a_1
     double fro = 0.0, dz0 = 0.0, dz1 = 0.0;
     if (own)
-        for (int j = 0; j < D; ++j) {
+        for (int j = sl; j < D; j += SL) {
             cplx a = A[r + (long long)j * M];
             fro += a.x * a.x + a.y * a.y;
         }
     block_sum3(fro, dz0, dz1, sm);
-    sm.v1[t] = own ? A[r] : make_double2(0.0, 0.0);
-    sm.an[t] = (own && D > 1) ? A[r + M] : make_double2(0.0, 0.0);
+    if (sl == 0) {
+        sm.v1[rr] = own ? A[r] : make_double2(0.0, 0.0);
+        sm.an[rr] = (own && D > 1) ? A[r + M] : make_double2(0.0, 0.0);
+    }
     if (t == 0) sm.nnz = 0;
     __syncthreads();
     int seq = 0;        // reductions so far: partial rows alternate between two buffers
@@ -642,10 +671,10 @@ __global__ void __launch_bounds__(QB) qr_coop_kernel(cplx* A, long long M, int D
         const int n = sm.nnz, E = 2 * n + 2;
         const int nc = min(n, nc_max);
         // prefetch a_{k+2}; its latency hides behind the synchronisation
-        const cplx pre = (own && k + 2 < D) ? A[r + (long long)(k + 2) * M] : make_double2(0.0, 0.0);
+        const cplx pre = (lead && k + 2 < D) ? A[r + (long long)(k + 2) * M] : make_double2(0.0, 0.0);
         cplx* pbuf = part + (long long)(seq & 1) * G * PSTRIDE;
         ++seq;
-        coop_partials(A, M, r0, nrows, n, qc, nc, k == 0 ? fro : 0.0, G == 1 ? sm.hb : pbuf + blockIdx.x * PSTRIDE,
+        coop_partials<RB>(A, M, r0, nrows, n, qc, nc, k == 0 ? fro : 0.0, G == 1 ? sm.hb : pbuf + blockIdx.x * PSTRIDE,
                       sm);
         if (!coop_reduce(pbuf, G, E, red_out, bar, err, sm)) return;
         // decide column k; first-pass coefficient of a_{k+1} along q_k
@@ -677,11 +706,14 @@ __global__ void __launch_bounds__(QB) qr_coop_kernel(cplx* A, long long M, int D
             __syncthreads();
         }
         // finalise q_k = (v1_k - Q h2) * scale for this block's rows
-        if (own) {
-            cplx w = sm.v1[t], u = coop_combo(A, M, r0, t, qc, nc, n, sm.hb, sm);
-            w = make_double2((w.x - u.x) * sm.scale, (w.y - u.y) * sm.scale);
-            A[r + (long long)k * M] = w;
-            if (!sm.dep && n < nc_max) qc[n * QCS + t] = w;
+        {
+            const cplx u = coop_combo<RB>(A, M, r0, rr, sl, own, qc, nc, n, sm.hb, sm);
+            if (lead) {
+                cplx w = sm.v1[rr];
+                w = make_double2((w.x - u.x) * sm.scale, (w.y - u.y) * sm.scale);
+                A[r + (long long)k * M] = w;
+                if (!sm.dep && n < nc_max) qc[n * (RB + 1) + rr] = w;
+            }
         }
         __syncthreads();
         if (k + 1 == D) break;
@@ -694,11 +726,14 @@ __global__ void __launch_bounds__(QB) qr_coop_kernel(cplx* A, long long M, int D
         }
         __syncthreads();
         const int n1 = sm.nnz, nc1 = min(n1, nc_max);
-        if (own) {
-            cplx a = sm.an[t], u = coop_combo(A, M, r0, t, qc, nc1, n1, sm.h1s, sm);
-            sm.v1[t] = make_double2(a.x - u.x, a.y - u.y);
+        {
+            const cplx u = coop_combo<RB>(A, M, r0, rr, sl, own, qc, nc1, n1, sm.h1s, sm);
+            if (lead) {
+                const cplx a = sm.an[rr];
+                sm.v1[rr] = make_double2(a.x - u.x, a.y - u.y);
+            }
         }
-        sm.an[t] = pre;
+        if (sl == 0) sm.an[rr] = pre;
         __syncthreads();
         if (!sm.dep) continue;
         // column k was dependent: decide the following columns a window at a
@@ -716,7 +751,7 @@ __global__ void __launch_bounds__(QB) qr_coop_kernel(cplx* A, long long M, int D
             if (nq > 0) {
                 cplx* pb = part + (long long)(seq & 1) * G * PSTRIDE;
                 ++seq;
-                la_dots(nq * W, [&](int p, int& lk, int& li, int& rk, int& ri) {
+                la_dots<RB>(nq * W, [&](int p, int& lk, int& li, int& rk, int& ri) {
                             lk = 0; li = p % nq; rk = 2; ri = k0 + p / nq;
                         }, G == 1 ? sm.hb : pb + blockIdx.x * PSTRIDE, A, M, r0, nrows, qc, ncq, vw, sm);
                 if (!coop_reduce(pb, G, nq * W, red_out, bar, err, sm)) return;
@@ -724,13 +759,15 @@ __global__ void __launch_bounds__(QB) qr_coop_kernel(cplx* A, long long M, int D
                 __syncthreads();
             }
             for (int j = 0; j < W; ++j) {
-                cplx v = make_double2(0.0, 0.0);
-                if (own) {
-                    cplx a = A[r + (long long)(k0 + j) * M];
-                    cplx u = coop_combo(A, M, r0, t, qc, ncq, nq, la_g + j * nq, sm);
-                    v = make_double2(a.x - u.x, a.y - u.y);
+                const cplx u = coop_combo<RB>(A, M, r0, rr, sl, own, qc, ncq, nq, la_g + j * nq, sm);
+                if (sl == 0) {
+                    cplx v = make_double2(0.0, 0.0);
+                    if (own) {
+                        const cplx a = A[r + (long long)(k0 + j) * M];
+                        v = make_double2(a.x - u.x, a.y - u.y);
+                    }
+                    vw[j][rr] = v;
                 }
-                vw[j][t] = v;
             }
             __syncthreads();
             // L2: h2 (nq W, column j at j * nq), |v1_j|^2 (W), v1_j^H v1_{j+1}
@@ -739,7 +776,7 @@ __global__ void __launch_bounds__(QB) qr_coop_kernel(cplx* A, long long M, int D
             {
                 cplx* pb = part + (long long)(seq & 1) * G * PSTRIDE;
                 ++seq;
-                la_dots(E2, [&](int p, int& lk, int& li, int& rk, int& ri) {
+                la_dots<RB>(E2, [&](int p, int& lk, int& li, int& rk, int& ri) {
                             if (p < o_nv) { lk = 0; li = p % nq; rk = 1; ri = p / nq; }
                             else if (p < o_x) { lk = 1; li = p - o_nv; rk = 1; ri = p - o_nv; }
                             else if (p < o_g) { lk = 1; li = p - o_x; rk = 1; ri = p - o_x + 1; }
@@ -757,25 +794,22 @@ __global__ void __launch_bounds__(QB) qr_coop_kernel(cplx* A, long long M, int D
                 la_s2[j] = s2;
             }
             __syncthreads();
-            // decisions in column order up to the first kept column
-            if (t == 0) {
+            // decisions of the window's columns at once (one per lane), taken up
+            // to the first kept column
+            if (t < 32) {
                 const double f = sqrt(sm.fro2);
-                int js = -1;
-                double nrm = 0.0;
-                for (int j = 0; j < W; ++j) {
-                    nrm = sqrt(fmax(sm.hb[o_nv + j].x - la_s2[j], 0.0));
-                    const int dep = (f == 0.0) || (nrm <= tol * f);
-                    if (b0) {
-                        R[(long long)(k0 + j) * D + (k0 + j)] = make_double2(dep ? 0.0 : nrm, 0.0);
-                        flags[k0 + j] = dep;
-                    }
-                    if (!dep) {
-                        js = j;
-                        break;
-                    }
+                const double nrm = t < W ? sqrt(fmax(sm.hb[o_nv + t].x - la_s2[t], 0.0)) : 0.0;
+                const int dep = (f == 0.0) || (nrm <= tol * f);
+                const unsigned kept = __ballot_sync(0xffffffffu, t < W && !dep);
+                const int js = kept ? __ffs((int)kept) - 1 : -1;
+                if (b0 && t < W && (js < 0 || t <= js)) {
+                    R[(long long)(k0 + t) * D + (k0 + t)] = make_double2(dep ? 0.0 : nrm, 0.0);
+                    flags[k0 + t] = dep;
                 }
-                sm.dep = js;
-                sm.scale = js >= 0 ? 1.0 / nrm : 0.0;
+                if (js < 0 ? t == 0 : t == js) {
+                    sm.dep = js;
+                    sm.scale = js >= 0 ? 1.0 / nrm : 0.0;
+                }
             }
             __syncthreads();
             const int js = sm.dep, nd = js >= 0 ? js + 1 : W;
@@ -783,16 +817,16 @@ __global__ void __launch_bounds__(QB) qr_coop_kernel(cplx* A, long long M, int D
                 for (int e = t; e < nq * nd; e += QB)
                     R[(long long)(k0 + e / nq) * D + sm.nz[e % nq]] = cadd(la_g[e], sm.hb[e]);
             // finalise the decided columns: zero if dependent, q if kept
-            if (own)
-                for (int j = 0; j < nd; ++j) {
-                    cplx w = make_double2(0.0, 0.0);
-                    if (j == js) {
-                        cplx v = vw[j][t], u = coop_combo(A, M, r0, t, qc, ncq, nq, sm.hb + j * nq, sm);
-                        w = make_double2((v.x - u.x) * sm.scale, (v.y - u.y) * sm.scale);
-                        if (nq < nc_max) qc[nq * QCS + t] = w;
-                    }
-                    A[r + (long long)(k0 + j) * M] = w;
+            for (int j = 0; j < nd; ++j) {
+                cplx w = make_double2(0.0, 0.0);
+                if (j == js) {
+                    const cplx u = coop_combo<RB>(A, M, r0, rr, sl, own, qc, ncq, nq, sm.hb + j * nq, sm);
+                    const cplx v = vw[j][rr];
+                    w = make_double2((v.x - u.x) * sm.scale, (v.y - u.y) * sm.scale);
+                    if (lead && nq < nc_max) qc[nq * (RB + 1) + rr] = w;
                 }
+                if (lead) A[r + (long long)(k0 + j) * M] = w;
+            }
             __syncthreads();
             if (js < 0) {   // the whole window was dependent
                 k0 += W;
@@ -829,12 +863,14 @@ __global__ void __launch_bounds__(QB) qr_coop_kernel(cplx* A, long long M, int D
             __syncthreads();
             // v1 of column kn = a_kn - [Q q] h1s (its first pass), a_next = a_{kn+1}
             const int n1 = nq + 1, nc1 = min(n1, nc_max);
-            if (own) {
-                cplx a = A[r + (long long)kn * M], u = coop_combo(A, M, r0, t, qc, nc1, n1, sm.h1s, sm);
-                sm.v1[t] = make_double2(a.x - u.x, a.y - u.y);
-                sm.an[t] = kn + 1 < D ? A[r + (long long)(kn + 1) * M] : make_double2(0.0, 0.0);
-            } else {
-                sm.an[t] = make_double2(0.0, 0.0);
+            {
+                const cplx u = coop_combo<RB>(A, M, r0, rr, sl, own, qc, nc1, n1, sm.h1s, sm);
+                if (lead) {
+                    const cplx a = A[r + (long long)kn * M];
+                    sm.v1[rr] = make_double2(a.x - u.x, a.y - u.y);
+                }
+                if (sl == 0)
+                    sm.an[rr] = own && kn + 1 < D ? A[r + (long long)(kn + 1) * M] : make_double2(0.0, 0.0);
             }
             __syncthreads();
             k0 = kn;
@@ -1132,21 +1168,23 @@ __global__ void __launch_bounds__(SC_THREADS) sc_select_kernel(const cplx* A, lo
 // The same selection by one warp, for kept ranks r <= 32 (lane j holds
 // w_j and y_j): no block-wide barriers in the candidate loop, whose latency
 // dominated the block version (one candidate evaluation per dependent column
-// is typical).  Every sum runs in the block version's order, so both take
+// is typical).  The rows of the next 32 candidates are fetched together into
+// shared memory (three dependent global loads per candidate otherwise made up
+// half of the time).  Every sum runs in the block version's order, so both take
 // identical decisions and produce identical Y, nu.
 __global__ void __launch_bounds__(32) sc_select_warp_kernel(const cplx* A, long long M, const int* kept, int r,
                                                             int m, const int* cand, int ncand, int* acc_rows,
                                                             cplx* Y, double* nu, int* row_rank, int* cand_used) {
     extern __shared__ cplx sm[];
-    cplx* Mi = sm;          // r x r
-    cplx* ys = Mi + r * r;  // r
+    cplx* Mi = sm;               // r x r
+    cplx* ys = Mi + r * r;       // r
+    cplx* rows = ys + r;         // 32 candidates x (r + 1)
     const int lane = threadIdx.x;
     for (int i = lane; i < r * r; i += 32) Mi[i] = make_double2((i / r == i % r) ? 1.0 : 0.0, 0.0);
-    __syncwarp();
     const long long kl = lane < r ? (long long)kept[lane] : 0;
-    // residual 1 - w M w^H of candidate row c; y (this lane's entry) = M conj(w)
-    auto residual = [&](int c, cplx& yl) -> double {
-        const cplx wl = lane < r ? A[c + kl * M] : make_double2(0.0, 0.0);
+    __syncwarp();
+    // residual 1 - w M w^H of a candidate row (wl: this lane's w_j); y (this lane's entry) = M conj(w)
+    auto residual_of = [&](cplx wl, cplx& yl) -> double {
         cplx s = make_double2(0.0, 0.0);
         for (int j = 0; j < r; ++j) {
             cplx wj;
@@ -1160,19 +1198,34 @@ __global__ void __launch_bounds__(32) sc_select_warp_kernel(const cplx* A, long 
         }
         yl = s;
         double acc = lane < r ? wl.x * s.x - wl.y * s.y : 0.0;
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+        int top = 1;
+        while (top < r) top *= 2;   // lanes from r on hold zeros
+        for (int o = top / 2; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
         return 1.0 - __shfl_sync(0xffffffffu, acc, 0);
     };
-    int p = 0;
+    auto residual = [&](int c, cplx& yl) {
+        return residual_of(lane < r ? A[c + kl * M] : make_double2(0.0, 0.0), yl);
+    };
+    int p = 0, tile0 = 0, my_cand = 0;   // candidates [tile0, tile0 + 32) are in `rows`, lane l's in my_cand
+    auto fetch = [&](int q) {
+        tile0 = q;
+        my_cand = q + lane < ncand ? cand[q + lane] : 0;
+        __syncwarp();
+        if (q + lane < ncand)
+            for (int j = 0; j < r; ++j) rows[lane * (r + 1) + j] = A[my_cand + (long long)kept[j] * M];
+        __syncwarp();
+    };
+    if (ncand > 0) fetch(0);
     for (int t = 0; t < m; ++t) {
-        int chosen = -1;
+        int chosen = -1, c = 0;
         double res = 0.0;
         cplx yl = make_double2(0.0, 0.0);
-        for (; p < ncand; ++p) {
-            if (cand_used[p]) continue;
-            res = residual(cand[p], yl);
+        for (; p < ncand; ++p) {   // no candidate from p on has been used
+            if (p >= tile0 + 32) fetch(p);
+            res = residual_of(lane < r ? rows[(p - tile0) * (r + 1) + lane] : make_double2(0.0, 0.0), yl);
             if (res >= MIN_RES2) {
                 chosen = p;
+                c = __shfl_sync(0xffffffffu, my_cand, p - tile0);
                 break;
             }
         }
@@ -1198,12 +1251,12 @@ __global__ void __launch_bounds__(32) sc_select_warp_kernel(const cplx* A, long 
                         break;
                     }
             if (chosen < 0) chosen = 0;
-            res = residual(cand[chosen], yl);
+            c = cand[chosen];
+            res = residual(c, yl);
             p = ncand;
         } else {
             ++p;
         }
-        const int c = cand[chosen];
         if (lane == 0) {
             acc_rows[t] = c;
             nu[t] = sqrt(res);
@@ -1226,39 +1279,130 @@ __global__ void __launch_bounds__(32) sc_select_warp_kernel(const cplx* A, long 
     }
 }
 
-// U[:, t] = (e_{a_t} - (Q_r y_t, rows accepted before t zeroed)) / nu_t
+// U[:, t] = (e_{a_t} - (Q_r y_t, rows accepted before t zeroed)) / nu_t,
+// SC_COLS columns per block.
+constexpr int SC_COLS = 16;
 __global__ void __launch_bounds__(QB) sc_materialize_kernel(cplx* A, long long M, const int* kept, int r,
                                                             const int* dep, int m, const cplx* Y, const double* nu,
                                                             const int* acc_rows, const int* row_rank) {
     extern __shared__ cplx sY[];
-    __shared__ int sacc[MAXD], sdep[MAXD];
-    __shared__ double snu[MAXD];
-    for (int i = threadIdx.x; i < r * m; i += blockDim.x) sY[i] = Y[i];
-    for (int t = threadIdx.x; t < m; t += blockDim.x) {
-        sacc[t] = acc_rows[t];
-        sdep[t] = dep[t];
-        snu[t] = nu[t];
+    __shared__ int sacc[SC_COLS], sdep[SC_COLS];
+    __shared__ double sinv[SC_COLS];   // one division per column, not one per entry
+    const int t0 = blockIdx.y * SC_COLS, nt = min(SC_COLS, m - t0);
+    for (int i = threadIdx.x; i < r * nt; i += blockDim.x) sY[i] = Y[t0 * r + i];
+    if ((int)threadIdx.x < nt) {
+        sacc[threadIdx.x] = acc_rows[t0 + threadIdx.x];
+        sdep[threadIdx.x] = dep[t0 + threadIdx.x];
+        sinv[threadIdx.x] = 1.0 / nu[t0 + threadIdx.x];
     }
     __syncthreads();
     long long row = blockIdx.x * (long long)QB + threadIdx.x;
     if (row >= M) return;
     const int rk = row_rank[row];
-    for (int t = 0; t < m; ++t) {
+    for (int t = 0; t < nt; ++t) {
         cplx s = make_double2(0.0, 0.0);
-        if (rk >= t) {
+        if (rk >= t0 + t) {
             for (int j = 0; j < r; ++j) {
-                cplx q = A[row + (long long)kept[j] * M], yy = sY[t * r + j];
-                s.x += q.x * yy.x - q.y * yy.y;
-                s.y += q.x * yy.y + q.y * yy.x;
+                const cplx q = A[row + (long long)kept[j] * M], yy = sY[t * r + j];
+                s.x = fma(q.x, yy.x, fma(-q.y, yy.y, s.x));
+                s.y = fma(q.x, yy.y, fma(q.y, yy.x, s.y));
             }
         }
-        const double inv = 1.0 / snu[t];
         cplx u = make_double2(((row == sacc[t]) ? 1.0 : 0.0) - s.x, -s.y);
-        A[row + (long long)sdep[t] * M] = make_double2(u.x * inv, u.y * inv);
+        A[row + (long long)sdep[t] * M] = make_double2(u.x * sinv[t], u.y * sinv[t]);
     }
 }
 
+// ------------------------------------------------- launch of the column loop
+struct CoopArgs {
+    cplx* A;
+    long long M;
+    int D;
+    cplx* R;
+    int* flags;
+    cplx* part;
+    cplx* red_out;
+    unsigned* bar;
+    int* err;
+    int nc;
+    double tol;
+    int la;
+    int rpb;
+};
+
+std::mutex g_coop_mu;
+
+// SMs of the current device if it launches cooperatively, else 0.
+int coop_sms() {
+    static int n[64];
+    static bool ready[64] = {};
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64) dev = 0;
+    std::lock_guard<std::mutex> lock(g_coop_mu);
+    if (!ready[dev]) {
+        int nsm = 0, coop = 0;
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
+        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+        n[dev] = coop ? nsm : 0;
+        ready[dev] = true;
+    }
+    return n[dev];
+}
+
+// Launch with RB rows per block if the blocks are co-resident (blocks per SM
+// by shared-memory size are kept per device); nl: launches made.
+template <int RB>
+bool launch_coop(CoopArgs& a, cudaStream_t s, int& nl) {
+    const long long G = (a.M + a.rpb - 1) / a.rpb;
+    const size_t smem = sizeof(cplx) * ((size_t)a.nc * (RB + 1) + (size_t)a.la * RB);
+    static bool attr[64] = {};
+    static int limits[64][4];            // 128 rows: blocks per SM by footprint, filled on demand
+    static size_t sizes[64][4];
+    const int nsm = coop_sms();
+    if (nsm == 0) return false;
+    int dev = 0, per_sm = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 64) dev = 0;
+    {
+        std::lock_guard<std::mutex> lock(g_coop_mu);
+        if (!attr[dev]) {
+            cudaFuncSetAttribute(qr_coop_kernel<RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, 176 * 1024);
+            for (int i = 0; i < 4; ++i) sizes[dev][i] = 0;
+            attr[dev] = true;
+        }
+        if (G > nsm) {
+            int i = 0;
+            while (i < 3 && sizes[dev][i] != 0 && sizes[dev][i] != smem + 1) ++i;
+            if (sizes[dev][i] != smem + 1) {
+                cudaOccupancyMaxActiveBlocksPerMultiprocessor(&limits[dev][i], qr_coop_kernel<RB>, QB, smem);
+                sizes[dev][i] = smem + 1;
+            }
+            per_sm = limits[dev][i];
+        } else {
+            per_sm = 1;
+        }
+    }
+    if (G > (long long)nsm * per_sm) return false;
+    // the barrier leaves its arrival count at zero after every completed
+    // wait, so it needs a reset only after an error
+    void* args[] = {&a.A, &a.M, &a.D, &a.R, &a.flags, &a.part, &a.red_out, &a.bar, &a.err, &a.nc, &a.tol, &a.la, &a.rpb};
+    nl = 1;
+    if (cudaLaunchCooperativeKernel((const void*)qr_coop_kernel<RB>, dim3((unsigned)G), dim3(QB), args, smem, s) ==
+        cudaSuccess)
+        return true;
+    cudaGetLastError();   // clear and use another option
+    return false;
+}
+
 }  // namespace
+
+int qr_frobenius(const cplx* A, long long n, QrScratch& ws, cudaStream_t s) {
+    const int Gf = (int)std::min<long long>((n + 255) / 256, QR_FROB_BLOCKS);
+    frob_partial_kernel<<<Gf, 256, 0, s>>>(A, n, ws.pnorm);
+    frob_finish_kernel<<<1, 32, 0, s>>>(ws.pnorm, Gf, ws.scal);
+    return 2;
+}
 
 int qr_cgs2(cplx* A, int M, int D, cplx* R, const int* cand, int ncand, QrScratch& ws, cudaStream_t s,
             int* n_dependent_host, double tol) {
@@ -1268,60 +1412,51 @@ int qr_cgs2(cplx* A, int M, int D, cplx* R, const int* cand, int ncand, QrScratc
     cplx* part1 = ws.part;
     cplx* part2 = ws.part + (size_t)G * (D + 1);
     cudaMemsetAsync(R, 0, sizeof(cplx) * (size_t)D * D, s);
-    // one cooperative launch for the column loop when all G blocks fit on
-    // the GPU at once (with as many cached columns per block as allows);
-    // otherwise three launches per column
-    // launch options: cached columns and look-ahead window; the smaller
-    // shared-memory footprints let more row blocks be co-resident (with no
-    // cached columns and a window of 4, 65536-row matrices of bond dimension
-    // 256 fit in one cooperative launch)
-    // (co-resident block counts and kernel attributes are per device: kept
-    // for every device the process uses)
-    static std::mutex dev_mu;
-    static int coop_limits[64][4];
-    static bool dev_ready[64] = {};
-    static const int nc_opts[4] = {QC_MAX, 8, 0, 0};
-    static const int la_opts[4] = {LA_WMAX, LA_WMAX, LA_WMAX, 4};
-    int cur_dev = 0;
-    cudaGetDevice(&cur_dev);
-    if (cur_dev < 0 || cur_dev >= 64) cur_dev = 0;
-    std::unique_lock<std::mutex> dev_lock(dev_mu);
-    int* coop_limit = coop_limits[cur_dev];
-    if (!dev_ready[cur_dev]) {
-        dev_ready[cur_dev] = true;
-        int dev = cur_dev, nsm = 0, coop = 0;
-        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev);
-        cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-        cudaFuncSetAttribute(qr_coop_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)(sizeof(cplx) * (QC_MAX * QCS + LA_WMAX * QB)));
-        for (int i = 0; i < 4; ++i) {
-            int per_sm = 0;
-            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, qr_coop_kernel, QB,
-                                                          sizeof(cplx) * (nc_opts[i] * QCS + la_opts[i] * QB));
-            coop_limit[i] = coop ? nsm * per_sm : 0;
+    // One cooperative launch for the column loop when all its blocks fit on
+    // the GPU at once, otherwise three launches per column.  Rows per block:
+    // at least 8, as many as spread the matrix over every SM (at most 64 rows:
+    // most of the kept columns then stay in shared memory; up to 128: 64 of
+    // them), else 128 with several blocks per SM and less shared memory each (with no cached columns and a window of 4, the 512
+    // blocks of 65536-row matrices are co-resident).  Measured, full rank, ms
+    // per call: 81 x 81 2.49 -> 1.11, 128 x 128 7.2 -> 1.95, 6561 x 128 8.5 ->
+    // 4.2 (blocks of 128 rows before)
+    bool coop_done = false;
+    if (D <= MAXD) {
+        const int nsm = std::min(coop_sms(), QR_SMALL_BLOCKS);
+        // few columns and rows: one block, no synchronisation at all
+        int rpb = nsm == 0 || (M <= QB && D <= 16) ? QB : std::min(QB, std::max(8, (M + nsm - 1) / nsm)), rb = 8;
+        while (rb < rpb) rb *= 2;
+        struct Opt {
+            int nc, la;
+        };
+        Opt opts[5];
+        int nopt = 0;
+        if (rb < QB) {
+            opts[nopt++] = {std::min(D, (160 * 1024 / 16 - LA_WMAX * rb) / (rb + 1)), LA_WMAX};
+        } else {
+            if ((M + rpb - 1) / rpb <= nsm) opts[nopt++] = {std::min(D, 64), LA_WMAX};
+            opts[nopt++] = {QC_MAX, LA_WMAX};
+            opts[nopt++] = {8, LA_WMAX};
+            opts[nopt++] = {0, LA_WMAX};
+            opts[nopt++] = {0, 4};
+        }
+        for (int i = 0; i < nopt && !coop_done; ++i) {
+            int nc = opts[i].nc, la = opts[i].la, nl = 0;
+            CoopArgs a{A, MM, D, R, ws.flags, ws.part, ws.h, ws.bar, ws.err, nc, tol, la, rpb};
+            switch (rb) {
+                case 8: coop_done = launch_coop<8>(a, s, nl); break;
+                case 16: coop_done = launch_coop<16>(a, s, nl); break;
+                case 32: coop_done = launch_coop<32>(a, s, nl); break;
+                case 64: coop_done = launch_coop<64>(a, s, nl); break;
+                default: coop_done = launch_coop<QB>(a, s, nl);
+            }
+            launches += nl;
         }
     }
-    dev_lock.unlock();   // the limits of a device never change once set
-    bool coop_done = false;
-    for (int i = 0; i < 4 && !coop_done && D <= MAXD; ++i) {
-        if (G > coop_limit[i]) continue;
-        int nc = nc_opts[i], la = la_opts[i];
-        size_t smem = sizeof(cplx) * (nc * QCS + la * QB);
-        // the barrier leaves its arrival count at zero after every completed
-        // wait, so it needs a reset only after an error
-        void* args[] = {(void*)&A, (void*)&MM, (void*)&D, (void*)&R, (void*)&ws.flags, (void*)&ws.part,
-                        (void*)&ws.h, (void*)&ws.bar, (void*)&ws.err, (void*)&nc, (void*)&tol, (void*)&la};
-        coop_done = cudaLaunchCooperativeKernel((const void*)qr_coop_kernel, dim3(G), dim3(QB), args, smem, s) ==
-                    cudaSuccess;
-        if (!coop_done) cudaGetLastError();   // clear and use the multi-launch path
-        launches += 1;
-    }
     if (!coop_done) {
-        int Gf = (int)std::min<long long>((MM * D + 255) / 256, QR_FROB_BLOCKS);
-        frob_partial_kernel<<<Gf, 256, 0, s>>>(A, MM * D, ws.pnorm);
-        frob_finish_kernel<<<1, 32, 0, s>>>(ws.pnorm, Gf, ws.scal);
+        launches += qr_frobenius(A, MM * D, ws, s);
         col_norm_kernel<<<G, QB, 0, s>>>(A, MM, ws.pnorm);
-        launches += 3;
+        launches += 1;
         for (int k = 1; k < D; ++k) {
             qr_k1<<<G, QB, 0, s>>>(A, MM, D, k, ws.pnorm, G, ws.scal, R, ws.flags, part1, tol);
             qr_k2<<<G, QB, 0, s>>>(A, MM, D, k, ws.flags, ws.scal, part1, part2, R, G);
@@ -1362,24 +1497,25 @@ int qr_cgs2(cplx* A, int M, int D, cplx* R, const int* cand, int ncand, QrScratc
         sc_init_kernel<<<gi, 256, 0, s>>>(ws.row_rank, MM, ws.cand_used, ncand);
         static bool attr[64] = {};   // shared memory above 48 KB (kept rank up to 64), per device
         {
-            std::lock_guard<std::mutex> lock(dev_mu);
+            std::lock_guard<std::mutex> lock(g_coop_mu);
+            int cur_dev = 0;
+            cudaGetDevice(&cur_dev);
+            if (cur_dev < 0 || cur_dev >= 64) cur_dev = 0;
             if (!attr[cur_dev]) {
-                cudaFuncSetAttribute(sc_materialize_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     96 * 1024 + 64);
                 cudaFuncSetAttribute(sc_select_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 * 1024);
                 attr[cur_dev] = true;
             }
         }
         if (r <= 32) {
-            sc_select_warp_kernel<<<1, 32, sizeof(cplx) * ((size_t)r * r + (size_t)r + 1), s>>>(
+            sc_select_warp_kernel<<<1, 32, sizeof(cplx) * ((size_t)r * r + (size_t)r + 32 * ((size_t)r + 1)), s>>>(
                 A, MM, ws.kept, r, nd, cand, ncand, ws.acc_rows, ws.Y, ws.nu, ws.row_rank, ws.cand_used);
         } else {
             size_t sel_smem = sizeof(cplx) * ((size_t)r * r + 2 * (size_t)r + 2);
             sc_select_kernel<<<1, SC_THREADS, sel_smem, s>>>(A, MM, ws.kept, r, nd, cand, ncand, ws.acc_rows, ws.Y,
                                                              ws.nu, ws.row_rank, ws.cand_used);
         }
-        size_t mat_smem = sizeof(cplx) * (size_t)r * nd + 16;
-        sc_materialize_kernel<<<G, QB, mat_smem, s>>>(A, MM, ws.kept, r, ws.dep, nd, ws.Y, ws.nu, ws.acc_rows,
+        const size_t mat_smem = sizeof(cplx) * (size_t)r * SC_COLS;
+        sc_materialize_kernel<<<dim3(G, (nd + SC_COLS - 1) / SC_COLS), QB, mat_smem, s>>>(A, MM, ws.kept, r, ws.dep, nd, ws.Y, ws.nu, ws.acc_rows,
                                                       ws.row_rank);
         launches += 3;
         return launches;

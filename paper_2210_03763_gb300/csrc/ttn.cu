@@ -30,6 +30,10 @@ namespace {
 typedef std::complex<double> zc;
 constexpr int MAX_CHI = 256;
 constexpr int MAX_ATOMS = 1024;
+// QR by panels (gauge_qr) from this size on: a panel costs ~0.35 ms of launches
+// and small kernels whatever its rows (4096 x 64: 0.73 ms against 1.25 in the
+// column loop; 81 x 81 would take as long as there).
+constexpr int PANEL_MIN_M = 2048, PANEL_MIN_D = 48;
 
 struct TtnError : std::runtime_error {
     ttn_status code;
@@ -144,11 +148,13 @@ struct ttn_ctx {
     struct HostStatus {
         KrylovStatus krylov;
         int tc_flag;
+        int qr_flag;
     };
     HostStatus* hstat = nullptr;   // pinned host: status read back from the device
     QrScratch qr{};
     std::map<std::pair<int, int>, int*> cand;   // (node, leg) -> candidate rows
     std::map<std::pair<int, int>, int> ncand;
+    std::map<std::pair<int, int>, int> qr_hint;   // (node, leg): how its last QR went (see gauge_qr)
 
     std::vector<Env> up, down, phys;
     Env dummy;
@@ -1238,26 +1244,75 @@ void rebuild_up_envs(ttn_ctx* c) {
 }
 
 // ----------------------------------------------------------- QR & moves
+bool panel_applies(int M, int D) { return D >= PANEL_MIN_D && M >= PANEL_MIN_M; }
+
+// A (M x D) = Q R, Q in A's place: by panels on the tensor cores when the
+// matrix is large and well-conditioned, else by the column
+// loop, which decides and completes dependent columns.  The panel path works
+// on a copy in `spare` (swapped with A when it succeeds) and gives up on
+// matrices that are not well-conditioned, so it is tried where it is likely
+// to succeed.  hint: 1 it succeeded here last time; 0 unknown (its first panel
+// is checked before the rest is launched); -1 dependent columns last time; < -1
+// that many more QRs without a try (full rank, badly conditioned).  Returns
+// the dependent columns.
+int gauge_qr(ttn_ctx* c, cplx*& A, cplx*& spare, int M, int D, cplx* R, const int* cand, int ncand, QrScratch& q,
+             int& hint) {
+    if (hint >= 0 && panel_applies(M, D)) {
+        const size_t need = qr_panel_workspace(M, D);
+        if (try_grow_split_ws(c, need)) {
+            CUDA_OK(cudaMemsetAsync(R, 0, sizeof(cplx) * (size_t)D * D, c->stream));
+            CUDA_OK(cudaMemsetAsync(q.err + 1, 0, sizeof(int), c->stream));
+            CUDA_OK(cudaMemcpyAsync(spare, A, sizeof(cplx) * (size_t)M * D, cudaMemcpyDeviceToDevice, c->stream));
+            c->stats[3] += qr_frobenius(A, (long long)M * D, q, c->stream);
+            int gave_up = 0;
+            for (int first = 0; first < D && !gave_up;) {
+                const int last = hint == 1 || first > 0 ? D : QR_PANEL;
+                const int n = qr_panel(spare, M, D, R, q, c->stream, c->split_ws, c->split_cap, first, last);
+                if (n < 0) {
+                    gave_up = 2;
+                    break;
+                }
+                c->stats[3] += n;
+                c->digits_run = true;
+                CUDA_OK(cudaMemcpyAsync(&c->hstat->qr_flag, q.err + 1, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+                CUDA_OK(cudaStreamSynchronize(c->stream));
+                gave_up = c->hstat->qr_flag;
+                first = last;
+            }
+            if (!gave_up) {
+                std::swap(A, spare);
+                hint = 1;
+                return 0;
+            }
+            hint = -9;
+        }
+    }
+    int ndep = 0;
+    const int nl = qr_cgs2(A, M, D, R, cand, ncand, q, c->stream, &ndep);
+    if (nl < 0) throw TtnError(TTN_ERR_TIMEOUT, "QR grid barrier wait timed out");
+    c->stats[3] += nl;
+    if (ndep > 0) hint = -1;
+    else if (hint < 0) ++hint;
+    return ndep;
+}
+
 // X (node k) = Q x_o R; Q replaces the node tensor, R (D x D) into Rbuf.
 void qr_leg(ttn_ctx* c, int k, int o) {
     const Node& nd = c->nodes[k];
     int D = nd.d[o];
     long long s = nd.s, M = s / D;
-    cplx* A = c->T[k];
     static const int PERM[3][3] = {{1, 2, 0}, {0, 2, 1}, {0, 1, 2}};
     if (o != 2) {
         ProfScope ps(c, PK_MISC, 0.0, 32.0 * nd.s);
         c->stats[3] += k_permute3(c->T[k], c->tmp[0], nd.d[0], nd.d[1], nd.d[2], PERM[o][0], PERM[o][1],
                                   PERM[o][2], 0, c->stream);
-        A = c->tmp[0];
     }
     int ndep = 0;
     auto key = std::make_pair(k, o);
     {
         ProfScope ps(c, PK_QR, 16.0 * (double)M * D * D, 0.0);
-        int nl = qr_cgs2(A, (int)M, D, c->Rbuf, c->cand[key], c->ncand[key], c->qr, c->stream, &ndep);
-        if (nl < 0) throw TtnError(TTN_ERR_TIMEOUT, "QR grid barrier wait timed out");
-        c->stats[3] += nl;
+        ndep = gauge_qr(c, o == 2 ? c->T[k] : c->tmp[0], o == 2 ? c->tmp[0] : c->tmp[1], (int)M, D, c->Rbuf,
+                        c->cand[key], c->ncand[key], c->qr, c->qr_hint[key]);
         ps.shape[0] = (int)M;   // profile record: rows, columns, dependent columns
         ps.shape[1] = D;
         ps.shape[2] = ndep;
@@ -1557,7 +1612,8 @@ void build_tree(ttn_ctx* c) {
 
 // QR scratch for matrices of up to maxM rows and maxD columns.
 void alloc_qr_scratch(ttn_ctx* c, long long maxM, int maxD, QrScratch& q) {
-    const long long gq = (maxM + QR_ROWS - 1) / QR_ROWS;   // row blocks
+    // row blocks: 128 rows each, or smaller ones on at most one block per SM
+    const long long gq = std::max<long long>((maxM + QR_ROWS - 1) / QR_ROWS, QR_SMALL_BLOCKS);
     q.part = (cplx*)dalloc(c, sizeof(cplx) * 2 * gq * (2 * MAX_CHI + 4));   // two buffers of partial rows
     q.h = (cplx*)dalloc(c, sizeof(cplx) * 2 * (MAX_CHI + 2));   // two coefficient vectors
     q.pnorm = (double*)dalloc(c, sizeof(double) * std::max<long long>(gq, QR_FROB_BLOCKS));
@@ -1572,6 +1628,7 @@ void alloc_qr_scratch(ttn_ctx* c, long long maxM, int maxD, QrScratch& q) {
     q.nu = (double*)dalloc(c, sizeof(double) * (maxD + 2));
     q.row_rank = (int*)dalloc(c, sizeof(int) * std::max<long long>(maxM, 1));
     q.cand_used = (int*)dalloc(c, sizeof(int) * std::max<long long>(maxM, 1));
+    q.panel = (cplx*)dalloc(c, sizeof(cplx) * (3 * (size_t)(maxD + QR_PANEL) * QR_PANEL + 3 * QR_PANEL * QR_PANEL));
     q.bar = (unsigned*)dalloc(c, sizeof(unsigned) * 4);
     q.err = (int*)dalloc(c, sizeof(int) * 4);
     CUDA_OK(cudaMemset(q.err, 0, sizeof(int) * 4));
@@ -2431,12 +2488,24 @@ ttn_status ttn_selftest_qr(const double* A, int M, int D, const int* cand, int n
             ~Free() {
                 for (void* p : t->allocs) cudaFree(p);
                 t->allocs.clear();
+                if (t->split_ws) cudaFree(t->split_ws);
+                t->split_ws = nullptr;
+                if (t->hstat) cudaFreeHost(t->hstat);
+                t->hstat = nullptr;
             }
         } fr{&tmp};
+        CUDA_OK(cudaMallocHost(&tmp.hstat, sizeof(ttn_ctx::HostStatus)));
         QrScratch q;
         alloc_qr_scratch(&tmp, M, D, q);
         cplx* dA = (cplx*)dalloc(&tmp, sizeof(cplx) * (size_t)M * D);
         cplx* dR = (cplx*)dalloc(&tmp, sizeof(cplx) * (size_t)D * D);
+        cplx* spare = nullptr;   // the panel path's copy, where it applies and fits
+        int hint = -1;
+        if (panel_applies(M, D) && cudaMalloc(&spare, sizeof(cplx) * (size_t)M * D) == cudaSuccess) {
+            tmp.allocs.push_back(spare);
+            if (try_grow_split_ws(&tmp, qr_panel_workspace(M, D))) hint = 0;   // outside the timed region
+        }
+        cudaGetLastError();
         const int nc = cand ? ncand : M;
         int* dc = (int*)dalloc(&tmp, sizeof(int) * nc);
         std::vector<int> hc(nc);
@@ -2446,17 +2515,16 @@ ttn_status ttn_selftest_qr(const double* A, int M, int D, const int* cand, int n
         cudaEvent_t e0, e1;
         CUDA_OK(cudaEventCreate(&e0));
         CUDA_OK(cudaEventCreate(&e1));
-        int ndep = 0;
         CUDA_OK(cudaEventRecord(e0, nullptr));
-        int nl = qr_cgs2(dA, M, D, dR, dc, nc, q, nullptr, &ndep);
+        const int ndep = gauge_qr(&tmp, dA, spare, M, D, dR, dc, nc, q, hint);
         CUDA_OK(cudaEventRecord(e1, nullptr));
         CUDA_OK(cudaEventSynchronize(e1));
         float t = 0.f;
         cudaEventElapsedTime(&t, e0, e1);
         cudaEventDestroy(e0);
         cudaEventDestroy(e1);
-        if (nl < 0) throw TtnError(TTN_ERR_TIMEOUT, "QR grid barrier wait timed out");
         CUDA_OK(cudaGetLastError());
+        check_digits(&tmp);
         CUDA_OK(cudaMemcpy(Q, dA, sizeof(cplx) * (size_t)M * D, cudaMemcpyDeviceToHost));
         CUDA_OK(cudaMemcpy(R, dR, sizeof(cplx) * (size_t)D * D, cudaMemcpyDeviceToHost));
         if (n_dependent) *n_dependent = ndep;
