@@ -170,6 +170,8 @@ struct ttn_ctx {
     void* split_ws = nullptr;   // packed operands of the tensor-core GEMMs (+ error flag)
     size_t split_cap = 0;
     bool digits_run = false;    // an FP64 contraction ran on the tensor cores since the flag was last read
+    cplx* obs_ws = nullptr;     // densities of ttn_measure, overlap environments
+    size_t obs_cap = 0;
     void* f64_ws = nullptr;     // split-K partial sums of FP64 contractions
     size_t f64_cap = 0;
     // split-precision H_eff of one node visit (see SplitHeff): per leg the
@@ -1768,25 +1770,27 @@ void set_V(ttn_ctx* c) {
 }
 
 // ------------------------------------------------------------- observables
-// <psi| op_i |psi> for ops renormalised to the root legs (centre at root).
+// <psi| op_i |psi> = sum_mn op_i(m, n) P(m, n) for ops renormalised to the root
+// legs (centre at root), P(m, n) = sum conj(T(m, .)) T(n, .) the density of the
+// leg.
 void root_expect(ttn_ctx* c, const cplx* st0, int n0, const cplx* st1, int n1, std::vector<zc>& out) {
     ForceFp64 f64;
     const Node& nd = c->nodes[c->root];
-    long long s = nd.s;
     out.assign(n0 + n1, zc(0.0));
     cplx* res = c->Gbuf[2];
     const cplx* st[2] = {st0, st1};
-    int ns[2] = {n0, n1};
+    const int ns[2] = {n0, n1};
     int off = 0;
     for (int u = 0; u < 2; ++u) {
         if (ns[u] == 0) continue;
-        long long DD = (long long)nd.d[u] * nd.d[u];
-        int chunk = (int)std::max<long long>(1, c->zcap / s);
-        for (int i0 = 0; i0 < ns[u]; i0 += chunk) {
-            int nb = std::min(chunk, ns[u] - i0);
-            leg_apply(c, st[u] + i0 * DD, nd.d[u], c->T[c->root], nd.d, u, c->Z, 0.0, nb, DD, s);
-            project(c, c->T[c->root], nd.d, c->Z, nd.d, 2, res + off + i0, nb, s, 1);
-        }
+        const int DD = nd.d[u] * nd.d[u];
+        project(c, c->T[c->root], nd.d, c->T[c->root], nd.d, u, c->tmp[0], 1, 0, 0);
+        GemmArgs g = base_args();
+        g.M = ns[u]; g.N = 1; g.Ki = DD;
+        g.A = st[u]; g.a_m = DD; g.a_ki = 1;
+        g.B = c->tmp[0]; g.b_ki = 1; g.b_n = DD;
+        g.C = res + off; g.c_m = 1; g.c_n = ns[u];
+        gemm(c, g);
         off += ns[u];
     }
     std::vector<cplx> h(n0 + n1);
@@ -1807,67 +1811,61 @@ double root_norm(ttn_ctx* c) {
     return h.x;
 }
 
-// Renormalise one diagonal one-site operator (per atom) up to the root legs.
+// Observable workspace, kept by the context: at least n complex.
+cplx* obs_buffer(ttn_ctx* c, size_t n) {
+    if (n > c->obs_cap) {
+        CUDA_OK(cudaStreamSynchronize(c->stream));
+        if (c->obs_ws) cudaFree(c->obs_ws);
+        c->obs_ws = nullptr;
+        c->obs_cap = 0;
+        if (test_take_alloc_fail() || cudaMalloc(&c->obs_ws, sizeof(cplx) * n) != cudaSuccess) {
+            c->obs_ws = nullptr;
+            cudaGetLastError();
+            throw TtnError(TTN_ERR_ALLOC, "observable workspace");
+        }
+        c->obs_cap = n;
+    }
+    return c->obs_ws;
+}
+
+// <|level><level|> of every atom (centre at the root): the density matrix of
+// every bond from the root down -- the other child's leg contracted with
+// itself, the parent leg through the density above -- and the diagonal of each
+// leaf's.  Three contractions per node; carrying one operator per atom up the
+// tree takes as many per atom below a bond (8x8, chi = 128, in FP64: 45 ms
+// against 4).
 void measure_projector(ttn_ctx* c, int level_index, std::vector<double>& out) {
     ForceFp64 f64;
-    // bare operator: |level><level|
-    cplx bare[9];
-    for (int i = 0; i < 9; ++i) bare[i] = C(0.0);
-    bare[level_index * 4] = C(1.0);
-    int nn = (int)c->nodes.size();
-    std::vector<cplx*> stack(nn, nullptr);
-    std::vector<std::vector<int>> sites(nn);
-    cplx* dbare = c->Gbuf[1];
-    CUDA_OK(cudaMemcpyAsync(dbare, bare, sizeof(bare), cudaMemcpyHostToDevice, c->stream));
-    std::vector<void*> temp;
-    for (auto& lev : c->level_nodes)
-        for (int k : lev) {
-            if (k == c->root) continue;
-            const Node& nd = c->nodes[k];
-            long long DDo = (long long)nd.d[2] * nd.d[2];
-            cplx* st = nullptr;
-            CUDA_OK(cudaMalloc(&st, sizeof(cplx) * DDo * std::max<size_t>(1, nd.sites.size())));
-            temp.push_back(st);
-            long long off = 0;
-            for (int u = 0; u < 2; ++u) {
-                int ch = nd.child[u];
-                if (ch < 0) {
-                    if (c->leaf_atom[-ch - 1] < 0) continue;
-                    renorm_stack(c, c->T[k], nd.d, u, 2, dbare, 1, st + off * DDo);
-                    sites[k].push_back(c->leaf_atom[-ch - 1]);
-                    off += 1;
-                } else {
-                    int n = (int)sites[ch].size();
-                    renorm_stack(c, c->T[k], nd.d, u, 2, stack[ch], n, st + off * DDo);
-                    sites[k].insert(sites[k].end(), sites[ch].begin(), sites[ch].end());
-                    off += n;
-                }
-            }
-            stack[k] = st;
-        }
-    const Node& rn = c->nodes[c->root];
-    const cplx* st[2];
-    int ns[2];
-    std::vector<int> order;
-    std::vector<cplx*> extra;
-    for (int u = 0; u < 2; ++u) {
-        int ch = rn.child[u];
-        if (ch >= 0) {
-            st[u] = stack[ch];
-            ns[u] = (int)sites[ch].size();
-            order.insert(order.end(), sites[ch].begin(), sites[ch].end());
-        } else {
-            int a = c->leaf_atom[-ch - 1];
-            st[u] = dbare;
-            ns[u] = a >= 0 ? 1 : 0;
-            if (a >= 0) order.push_back(a);
-        }
+    const int nn = (int)c->nodes.size(), nl = c->n_leaves;
+    std::vector<size_t> off(nn);
+    size_t n = 9 * (size_t)nl;   // leaves first
+    for (int k = 0; k < nn; ++k) {
+        off[k] = n;
+        n += (size_t)c->nodes[k].d[2] * c->nodes[k].d[2];
     }
-    std::vector<zc> vals;
-    root_expect(c, st[0], ns[0], st[1], ns[1], vals);
+    cplx* ws = obs_buffer(c, n);
+    c->stats[3] += k_fill(ws + off[c->root], 1, C(1.0), c->stream);
+    for (int li = (int)c->level_nodes.size() - 1; li >= 0; --li)
+        for (int k : c->level_nodes[li]) {
+            const Node& nd = c->nodes[k];
+            const cplx* Y = c->T[k];   // rho x_2 X (the root's density is [[1]])
+            if (k != c->root) {
+                leg_apply(c, ws + off[k], nd.d[2], c->T[k], nd.d, 2, c->tmp[0], 0.0);
+                Y = c->tmp[0];
+            }
+            for (int u = 0; u < 2; ++u) {
+                const int ch = nd.child[u];
+                if (ch < 0 && c->leaf_atom[-ch - 1] < 0) continue;
+                project(c, c->T[k], nd.d, Y, nd.d, u, ch >= 0 ? ws + off[ch] : ws + 9 * (size_t)(-ch - 1), 1, 0, 0);
+            }
+        }
+    std::vector<cplx> h(9 * (size_t)nl);
+    CUDA_OK(cudaMemcpyAsync(h.data(), ws, sizeof(cplx) * h.size(), cudaMemcpyDeviceToHost, c->stream));
+    CUDA_OK(cudaStreamSynchronize(c->stream));
+    check_digits(c);
     out.assign(c->N, 0.0);
-    for (size_t i = 0; i < order.size(); ++i) out[order[i]] = vals[i].real();
-    for (void* p : temp) cudaFree(p);
+    for (int l = 0; l < nl; ++l)
+        if (c->leaf_atom[l] >= 0) out[c->leaf_atom[l]] = h[9 * (size_t)l + 4 * level_index].x;
 }
 
 zc overlap(ttn_ctx* psi, const ttn_ctx* tgt) {
@@ -1875,7 +1873,9 @@ zc overlap(ttn_ctx* psi, const ttn_ctx* tgt) {
     ttn_ctx* c = psi;
     int nn = (int)c->nodes.size();
     std::vector<cplx*> M(nn, nullptr);
-    std::vector<void*> temp;
+    size_t need = 0;
+    for (int k = 0; k < nn; ++k) need += (size_t)tgt->nodes[k].d[2] * c->nodes[k].d[2];
+    cplx* ws = obs_buffer(c, need);
     for (auto& lev : c->level_nodes)
         for (int k : lev) {
             const Node& nd = c->nodes[k];
@@ -1893,16 +1893,13 @@ zc overlap(ttn_ctx* psi, const ttn_ctx* tgt) {
                 cur = bufs[bi];
                 bi ^= 1;
             }
-            cplx* out = nullptr;
-            CUDA_OK(cudaMalloc(&out, sizeof(cplx) * (size_t)nt.d[2] * nd.d[2]));
-            temp.push_back(out);
-            project(c, tgt->T[k], nt.d, cur, d, 2, out, 1, 0, 0);
-            M[k] = out;
+            M[k] = ws;
+            ws += (size_t)nt.d[2] * nd.d[2];
+            project(c, tgt->T[k], nt.d, cur, d, 2, M[k], 1, 0, 0);
         }
     cplx h;
     CUDA_OK(cudaMemcpyAsync(&h, M[c->root], sizeof(cplx), cudaMemcpyDeviceToHost, c->stream));
     CUDA_OK(cudaStreamSynchronize(c->stream));
-    for (void* p : temp) cudaFree(p);
     check_digits(c);
     return zc(h.x, h.y);
 }
@@ -1998,6 +1995,7 @@ void ttn_destroy(ttn_ctx* c) {
     for (void* p : c->allocs) cudaFree(p);
     if (c->split_ws) cudaFree(c->split_ws);
     if (c->f64_ws) cudaFree(c->f64_ws);
+    if (c->obs_ws) cudaFree(c->obs_ws);
     for (int i = 0; i < 3; ++i) {
         if (c->shP[i]) cudaFree(c->shP[i]);
         if (c->shQ[i]) cudaFree(c->shQ[i]);
