@@ -211,7 +211,7 @@ struct QrScratch {
     int* dep;           // D: dependent column positions
     int* acc_rows;      // D: accepted candidate row per completed column
     cplx* Y;            // QR_SC_MAXR * D: coefficients y_t
-    double* nu;         // D: residual norms
+    double* nu;         // D: squared residual norms
     int* row_rank;      // M: step at which a row was accepted (INT_MAX: never)
     int* cand_used;     // M: candidate accepted flags
     unsigned* bar;      // 2: grid barrier of the cooperative column loop

@@ -747,26 +747,46 @@ __global__ void __launch_bounds__(QB) qr_coop_kernel(cplx* A, long long M, int D
             const int W = min(min(min(la_w, la_max), D - k0), cap);   // >= 1
             const bool after = k0 + W < D;
             const int ka = k0 + W;                // the column after the window
+            // the window's columns into vw: all loads in flight at once (three
+            // passes of dependent loads from L2 were half of a window's time)
+            if (own) {
+                cplx* vr = &vw[0][rr];
+                const cplx* ar = A + r + (long long)k0 * M;
+#pragma unroll 4
+                for (int j = sl; j < W; j += SL) vr[j * RB] = ar[j * M];
+            } else {
+                for (int j = sl; j < W; j += SL) vw[j][rr] = make_double2(0.0, 0.0);
+            }
+            __syncthreads();
             // L1: g_j = Q^H a_j, kept in la_g; v1_j = a_j - Q g_j into vw
             if (nq > 0) {
                 cplx* pb = part + (long long)(seq & 1) * G * PSTRIDE;
                 ++seq;
                 la_dots<RB>(nq * W, [&](int p, int& lk, int& li, int& rk, int& ri) {
-                            lk = 0; li = p % nq; rk = 2; ri = k0 + p / nq;
+                            lk = 0; li = p % nq; rk = 1; ri = p / nq;
                         }, G == 1 ? sm.hb : pb + blockIdx.x * PSTRIDE, A, M, r0, nrows, qc, ncq, vw, sm);
                 if (!coop_reduce(pb, G, nq * W, red_out, bar, err, sm)) return;
                 for (int e = t; e < nq * W; e += QB) la_g[e] = sm.hb[e];
                 __syncthreads();
             }
-            for (int j = 0; j < W; ++j) {
-                const cplx u = coop_combo<RB>(A, M, r0, rr, sl, own, qc, ncq, nq, la_g + j * nq, sm);
-                if (sl == 0) {
-                    cplx v = make_double2(0.0, 0.0);
-                    if (own) {
-                        const cplx a = A[r + (long long)(k0 + j) * M];
-                        v = make_double2(a.x - u.x, a.y - u.y);
+            if (nq <= 32 || W >= SL) {   // one column per slice: no sums across threads
+                if (own)
+                    for (int j = sl; j < W; j += SL) {
+                        cplx v = vw[j][rr];
+                        for (int i = 0; i < nq; ++i) {
+                            const cplx a = qcol<RB>(A, M, r0, qc, ncq, i, rr, sm), h = la_g[j * nq + i];
+                            v.x = fma(-a.x, h.x, fma(a.y, h.y, v.x));
+                            v.y = fma(-a.x, h.y, fma(-a.y, h.x, v.y));
+                        }
+                        vw[j][rr] = v;
                     }
-                    vw[j][rr] = v;
+            } else {
+                for (int j = 0; j < W; ++j) {
+                    const cplx u = coop_combo<RB>(A, M, r0, rr, sl, own, qc, ncq, nq, la_g + j * nq, sm);
+                    if (lead) {
+                        const cplx a = vw[j][rr];
+                        vw[j][rr] = make_double2(a.x - u.x, a.y - u.y);
+                    }
                 }
             }
             __syncthreads();
@@ -1145,10 +1165,9 @@ __global__ void __launch_bounds__(SC_THREADS) sc_select_kernel(const cplx* A, lo
             ++p;
         }
         const int c = cand[chosen];
-        const double n = sqrt(res);
         if (threadIdx.x == 0) {
             acc_rows[t] = c;
-            nu[t] = n;
+            nu[t] = res;
             row_rank[c] = t;
             cand_used[chosen] = 1;
         }
@@ -1259,7 +1278,7 @@ __global__ void __launch_bounds__(32) sc_select_warp_kernel(const cplx* A, long 
         }
         if (lane == 0) {
             acc_rows[t] = c;
-            nu[t] = sqrt(res);
+            nu[t] = res;
             row_rank[c] = t;
             cand_used[chosen] = 1;
         }
@@ -1287,13 +1306,13 @@ __global__ void __launch_bounds__(QB) sc_materialize_kernel(cplx* A, long long M
                                                             const int* acc_rows, const int* row_rank) {
     extern __shared__ cplx sY[];
     __shared__ int sacc[SC_COLS], sdep[SC_COLS];
-    __shared__ double sinv[SC_COLS];   // one division per column, not one per entry
+    __shared__ double sinv[SC_COLS];   // 1 / nu_t: one division per column, not one per entry
     const int t0 = blockIdx.y * SC_COLS, nt = min(SC_COLS, m - t0);
     for (int i = threadIdx.x; i < r * nt; i += blockDim.x) sY[i] = Y[t0 * r + i];
     if ((int)threadIdx.x < nt) {
         sacc[threadIdx.x] = acc_rows[t0 + threadIdx.x];
         sdep[threadIdx.x] = dep[t0 + threadIdx.x];
-        sinv[threadIdx.x] = 1.0 / nu[t0 + threadIdx.x];
+        sinv[threadIdx.x] = 1.0 / sqrt(nu[t0 + threadIdx.x]);
     }
     __syncthreads();
     long long row = blockIdx.x * (long long)QB + threadIdx.x;
