@@ -126,14 +126,34 @@ struct KrylovStatus {
     int    iters;        // one-launch runs of small nodes: Krylov steps taken
     int    pad;
 };
+// Status that kernels write into pinned host memory: the fields, then the
+// sequence number of the launch.  The host polls the number instead of
+// copying and synchronising (8 to 10 us per round trip: a 2x2 step of 18 round
+// trips takes 1.83 ms instead of 2.0).
+struct HostStatus {
+    KrylovStatus krylov[KRYLOV_MMAX];   // per Krylov step (one-launch runs: [0])
+    int tc_flag;                        // a tensor-core wait gave up
+    int qr_flag;                        // panel QR: not well-conditioned
+    int qr_dep[256];                    // column loop: dependent columns
+    unsigned seq;
+};
+struct Publish {                        // where and as which launch a kernel reports; hs null: not at all
+    HostStatus* hs;
+    unsigned seq;
+    const int* tc_flag;                 // may be null
+};
+// Wait until launch `seq` on stream s has reported.  False: the stream ran dry
+// (or failed) without it.
+bool wait_status(const HostStatus* hs, unsigned seq, cudaStream_t s);
+
 struct KrylovScalars {
     double alpha[KRYLOV_MMAX];
     double beta[KRYLOV_MMAX + 1];
     cplx   h[KRYLOV_MMAX + 1];      // projections of the current pass
-    cplx   c[KRYLOV_MMAX];          // exp(z T_j) e_1
+    cplx   c[KRYLOV_MMAX][KRYLOV_MMAX];   // [j]: exp(z T_j) e_1 of step j
     double nrm0;                    // norm of the start vector
     double inv_scale;               // 1 / beta_j used to normalise v_{j+1}
-    KrylovStatus st;
+    int nonfinite;
     unsigned arrived;               // blocks of the second pass that have finished
     cplx   hess[KRYLOV_MMAX][32];   // Arnoldi: Hessenberg matrix H(i, j) at [j][i]
 };
@@ -153,11 +173,13 @@ int k_lanczos_first(const cplx* V, long long ld, int j, const cplx* partial_in, 
                     long long n, cplx* partial_dots, cplx* h_out, cudaStream_t s);
 int k_orth_second(const cplx* V, long long ld, int nv, const cplx* partial_in, cplx* w, long long n,
                   double* partial_norm, KrylovScalars* ks, const cplx* h1, double zr, double zi, double tol,
-                  int arnoldi, cudaStream_t s);
+                  int arnoldi, const Publish& pub, cudaStream_t s);
 int k_scale_copy_dev(const cplx* x, long long n, const double* scale, cplx* y, cudaStream_t s);
 // x <- x * sqrt(sum pr / sum px) with px, pr norm^2 partials (k_norm2_partial)
 int k_rescale_to_norm(cplx* x, long long n, const double* px, int Gx, const double* pr, int Gr, cudaStream_t s);
-int k_krylov_start_ex(KrylovScalars* ks, const double* nrm2_partial, long long n, cudaStream_t s);
+// |x|^2 and the start scalars (nrm0, inv_scale), the flags cleared.
+int k_krylov_start(KrylovScalars* ks, const cplx* x, long long n, double* partial, cudaStream_t s);
+// y = nrm0 sum_i c[nv - 1][i] V_i
 int k_combine(const cplx* V, long long ld, int nv, const KrylovScalars* ks, cplx* y,
               long long n, cudaStream_t s);
 
@@ -172,7 +194,7 @@ struct SmallPairs {      // channel pairs of a small H_eff (by value into the ke
     const cplx* G[3];    // r matrices of D_b^2
 };
 int k_small_krylov(const int* d, const cplx* hb0, const cplx* hb1, const cplx* hb2, const SmallPairs& pp, cplx* x,
-                   double zr, double zi, double tol, int mmax, int arnoldi, KrylovScalars* ks, cudaStream_t s);
+                   double zr, double zi, double tol, int mmax, int arnoldi, const Publish& pub, cudaStream_t s);
 
 // ---- elementwise / assembly ---------------------------------------------------
 int k_permute3(const cplx* x, cplx* y, int d0, int d1, int d2, int p0, int p1, int p2,
@@ -217,6 +239,8 @@ struct QrScratch {
     unsigned* bar;      // 2: grid barrier of the cooperative column loop
     int* err;           // [0] set when a bounded device wait gave up, [1] when the panel path gave up
     cplx* panel;        // panel path: 3 (D + QR_PANEL) QR_PANEL + 3 QR_PANEL^2
+    HostStatus* hs;     // status in host memory (null: read back by copies)
+    unsigned* seq;      // last sequence number used with it
 };
 constexpr int QR_SC_MAXR = 64;   // structured completion when the kept rank r <= this
 // In-place QR of the column-major M x D matrix A (lda = M): A <- Q, R (D x D,
@@ -230,12 +254,12 @@ constexpr double QR_TOL_FP64 = 1e-10;
 constexpr int QR_PANEL = 32;
 // QR of a well-conditioned matrix by panels (qr_panel.cu): columns [first,
 // last) of A in place and of R (zeroed before), ws.scal[0] = |A|_F^2 and
-// ws.err[1] = 0 before the first call.  ws.err[1] != 0 afterwards: not
-// well-conditioned, A and R undefined.  Workspace as launch_zgemm_digits (of
+// ws.err[1] = 0 before the first call.  Reports qr_flag with the last launch;
+// not 0: not well-conditioned, A and R undefined.  Workspace as launch_zgemm_digits (of
 // qr_panel_workspace bytes).  Returns launches, -1 when not available.
 size_t qr_panel_workspace(int M, int D);
 int qr_panel(cplx* A, int M, int D, cplx* R, QrScratch& ws, cudaStream_t s, void* workspace, size_t workspace_bytes,
-             int first, int last);
+             int first, int last, const Publish& pub);
 // |A|_F^2 into ws.scal[0].
 int qr_frobenius(const cplx* A, long long n, QrScratch& ws, cudaStream_t s);
 int qr_cgs2(cplx* A, int M, int D, cplx* R, const int* cand, int ncand,

@@ -7,6 +7,7 @@
 #include "common.cuh"
 #include <cooperative_groups.h>
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <mutex>
 
@@ -222,7 +223,14 @@ __global__ void __launch_bounds__(T) lanczos_first_kernel(const cplx* V, long lo
 }
 
 __device__ void krylov_scalars_step(KrylovScalars* ks, const cplx* h1, const cplx* h2, const double* beta_partial,
-                                    int G, int j, double zr, double zi, double tol, int arnoldi);
+                                    int G, int j, double zr, double zi, double tol, int arnoldi, const Publish& pub);
+
+// The fields are written; make them visible to the host, then the number.
+__device__ __forceinline__ void publish(const Publish& pub) {
+    if (pub.tc_flag && *(volatile const int*)pub.tc_flag) pub.hs->tc_flag = 1;
+    __threadfence_system();
+    *(volatile unsigned*)&pub.hs->seq = pub.seq;
+}
 
 // Second pass: h = sum of the partials, w -= sum_i V_i h_i, |w|^2.  The last
 // block to finish turns the sums into the step's scalars (alpha, beta, the
@@ -230,7 +238,7 @@ __device__ void krylov_scalars_step(KrylovScalars* ks, const cplx* h1, const cpl
 __global__ void __launch_bounds__(T) orth_second_kernel(const cplx* V, long long ld, int nv, const cplx* partial_in,
                                                         cplx* w, long long n, int G, double* partial_norm,
                                                         KrylovScalars* ks, const cplx* h1, double zr, double zi,
-                                                        double tol, int arnoldi) {
+                                                        double tol, int arnoldi, Publish pub) {
     __shared__ cplx sh_h[KRYLOV_MMAX + 1];
     __shared__ double shd[T / 32];
     __shared__ int last;
@@ -253,7 +261,7 @@ __global__ void __launch_bounds__(T) orth_second_kernel(const cplx* V, long long
         __threadfence();
     }
     __syncthreads();
-    if (last && threadIdx.x < 32) krylov_scalars_step(ks, h1, sh_h, partial_norm, G, nv - 1, zr, zi, tol, arnoldi);
+    if (last && threadIdx.x < 32) krylov_scalars_step(ks, h1, sh_h, partial_norm, G, nv - 1, zr, zi, tol, arnoldi, pub);
 }
 
 __global__ void norm2_partial_kernel(const cplx* x, long long n, int G, double* partial) {
@@ -296,7 +304,7 @@ __global__ void combine_kernel(const cplx* V, long long ld, int nv, const Krylov
                                long long n) {
     __shared__ cplx c[KRYLOV_MMAX];
     if (threadIdx.x < nv) {
-        cplx ci = ks->c[threadIdx.x];
+        cplx ci = ks->c[nv - 1][threadIdx.x];
         c[threadIdx.x] = make_double2(ci.x * ks->nrm0, ci.y * ks->nrm0);
     }
     __syncthreads();
@@ -379,17 +387,34 @@ __device__ void tridiag_expm_warp(const double* a, const double* b, int m, doubl
     if (l < m) out[l] = u;
 }
 
-__global__ void krylov_start_kernel(KrylovScalars* ks, const double* nrm2_partial, int G) {
-    const double s = reduce_norm_partials(nrm2_partial, G);
-    if (threadIdx.x != 0) return;
-    ks->arrived = 0u;
-    double n0 = sqrt(s);
-    ks->nrm0 = n0;
-    ks->inv_scale = n0 > 0.0 ? 1.0 / n0 : 0.0;
-    ks->st.converged = (n0 == 0.0) ? 1 : 0;
-    ks->st.nonfinite = isfinite(n0) ? 0 : 1;
-    ks->st.err = 0.0;
-    for (int i = 0; i < KRYLOV_MMAX; ++i) ks->c[i] = make_double2(0.0, 0.0);
+// |x|^2; the last block to finish sets the start scalars.
+__global__ void __launch_bounds__(T) krylov_start_kernel(KrylovScalars* ks, const cplx* x, long long n, int G,
+                                                         double* partial, unsigned* arrived) {
+    __shared__ double shd[T / 32];
+    __shared__ int last;
+    long long lo, hi;
+    chunk_of(n, G, lo, hi);
+    double s = 0.0;
+    for (long long e = lo + threadIdx.x; e < hi; e += T) s = fma(x[e].x, x[e].x, fma(x[e].y, x[e].y, s));
+    s = block_sum_d(s, shd);
+    if (threadIdx.x == 0) {
+        partial[blockIdx.x] = s;
+        __threadfence();
+        last = atomicAdd(arrived, 1u) == gridDim.x - 1;
+        if (last) *arrived = 0u;
+        __threadfence();
+    }
+    __syncthreads();
+    if (!last || threadIdx.x >= 32) return;
+    double t = 0.0;
+    for (int g = threadIdx.x; g < G; g += 32) t += __ldcg(partial + g);
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (threadIdx.x == 0) {
+        const double n0 = sqrt(t);
+        ks->nrm0 = n0;
+        ks->inv_scale = n0 > 0.0 ? 1.0 / n0 : 0.0;
+        ks->nonfinite = isfinite(n0) ? 0 : 1;
+    }
 }
 
 // exp(z H) e_1 for the m x m matrix H, H(i, k) at Hs[32 k + i] in shared
@@ -434,7 +459,7 @@ __device__ void hess_expm_warp(const cplx* Hs, cplx* vec, int m, double zr, doub
 // Scalars of step j by one warp: alpha_j, beta_j (Arnoldi: column j of the
 // Hessenberg matrix), c = exp(z T) e_1, the error estimate and the status.
 __device__ void krylov_scalars_step(KrylovScalars* ks, const cplx* h1, const cplx* h2, const double* beta_partial,
-                                    int G, int j, double zr, double zi, double tol, int arnoldi) {
+                                    int G, int j, double zr, double zi, double tol, int arnoldi, const Publish& pub) {
     __shared__ double a[32], b[32];
     __shared__ cplx hs[KRYLOV_MMAX * 32], vec[32];
     const int l = threadIdx.x & 31;
@@ -456,7 +481,7 @@ __device__ void krylov_scalars_step(KrylovScalars* ks, const cplx* h1, const cpl
             ks->beta[j] = bj;
             ks->alpha[j] = d.x;
         }
-        hess_expm_warp(hs, vec, j + 1, zr, zi, ks->c);
+        hess_expm_warp(hs, vec, j + 1, zr, zi, ks->c[j]);
     } else {
         const double al = h1[j].x + h2[j].x;
         bad = !isfinite(al);
@@ -467,16 +492,19 @@ __device__ void krylov_scalars_step(KrylovScalars* ks, const cplx* h1, const cpl
             ks->alpha[j] = al;
             ks->beta[j] = bj;
         }
-        tridiag_expm_warp(a, b, j + 1, zr, zi, ks->c);
+        tridiag_expm_warp(a, b, j + 1, zr, zi, ks->c[j]);
     }
     __syncwarp();
     if (l == 0) {
-        const cplx cj = ks->c[j];
+        const cplx cj = ks->c[j][j];
         const double err = bj * sqrt(cj.x * cj.x + cj.y * cj.y);
-        ks->st.err = err;
-        ks->st.converged = (err <= tol) ? 1 : 0;
         ks->inv_scale = bj > 0.0 ? 1.0 / bj : 0.0;
-        if (!isfinite(err) || bad) ks->st.nonfinite = 1;
+        if (!isfinite(err) || bad) ks->nonfinite = 1;
+        KrylovStatus& st = pub.hs->krylov[j];
+        st.err = err;
+        st.converged = (err <= tol) ? 1 : 0;
+        st.nonfinite = ks->nonfinite;
+        publish(pub);
     }
 }
 
@@ -545,7 +573,7 @@ __device__ cplx small_heff(int xr, int yc, int d0, int d1, int d2, const cplx* h
 
 __global__ void __cluster_dims__(SK_CL, 1, 1) __launch_bounds__(SK_THREADS)
     small_krylov_kernel(int d0, int d1, int d2, const cplx* hb0, const cplx* hb1, const cplx* hb2, SmallPairs pp,
-                        cplx* x, double zr, double zi, double tol, int mmax, int arnoldi, KrylovScalars* ks) {
+                        cplx* x, double zr, double zi, double tol, int mmax, int arnoldi, Publish pub) {
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     extern __shared__ cplx smem_c[];
@@ -568,10 +596,12 @@ __global__ void __cluster_dims__(SK_CL, 1, 1) __launch_bounds__(SK_THREADS)
     cl.sync();                      // every CTA has read x; all are running (remote writes may start)
     if (nrm0 == 0.0 || !isfinite(nrm0)) {
         if (rank == 0 && tid == 0) {
-            ks->st.err = 0.0;
-            ks->st.converged = nrm0 == 0.0;
-            ks->st.nonfinite = nrm0 != 0.0;
-            ks->st.iters = 0;
+            KrylovStatus& st = pub.hs->krylov[0];
+            st.err = 0.0;
+            st.converged = nrm0 == 0.0;
+            st.nonfinite = nrm0 != 0.0;
+            st.iters = 0;
+            publish(pub);
         }
         return;
     }
@@ -691,10 +721,12 @@ __global__ void __cluster_dims__(SK_CL, 1, 1) __launch_bounds__(SK_THREADS)
         x[r0 + tid] = make_double2(acc.x * nrm0, acc.y * nrm0);
     }
     if (rank == 0 && tid == 0) {
-        ks->st.err = sm.err;
-        ks->st.converged = sm.conv;
-        ks->st.nonfinite = sm.nonfin;
-        ks->st.iters = j + 1;
+        KrylovStatus& st = pub.hs->krylov[0];
+        st.err = sm.err;
+        st.converged = sm.conv;
+        st.nonfinite = sm.nonfin;
+        st.iters = j + 1;
+        publish(pub);
     }
 }
 
@@ -973,9 +1005,10 @@ int k_lanczos_first(const cplx* V, long long ld, int j, const cplx* partial_in, 
 
 int k_orth_second(const cplx* V, long long ld, int nv, const cplx* partial_in, cplx* w, long long n,
                   double* partial_norm, KrylovScalars* ks, const cplx* h1, double zr, double zi, double tol,
-                  int arnoldi, cudaStream_t s) {
+                  int arnoldi, const Publish& pub, cudaStream_t s) {
     const int G = red_blocks_for(n);
-    orth_second_kernel<<<G, T, 0, s>>>(V, ld, nv, partial_in, w, n, G, partial_norm, ks, h1, zr, zi, tol, arnoldi);
+    orth_second_kernel<<<G, T, 0, s>>>(V, ld, nv, partial_in, w, n, G, partial_norm, ks, h1, zr, zi, tol, arnoldi,
+                                       pub);
     return 1;
 }
 
@@ -995,9 +1028,24 @@ int k_combine(const cplx* V, long long ld, int nv, const KrylovScalars* ks, cplx
     return 1;
 }
 
-int k_krylov_start_ex(KrylovScalars* ks, const double* nrm2_partial, long long n, cudaStream_t s) {
-    krylov_start_kernel<<<1, 32, 0, s>>>(ks, nrm2_partial, red_blocks_for(n));
+int k_krylov_start(KrylovScalars* ks, const cplx* x, long long n, double* partial, cudaStream_t s) {
+    const int G = red_blocks_for(n);
+    krylov_start_kernel<<<G, T, 0, s>>>(ks, x, n, G, partial, &ks->arrived);
     return 1;
+}
+
+bool wait_status(const HostStatus* hs, unsigned seq, cudaStream_t s) {
+    const volatile unsigned* p = &hs->seq;
+    auto there = [&] { return (int)(*p - seq) >= 0; };
+    for (unsigned i = 1;; ++i) {
+        if (there()) break;
+        if ((i & 0xFFF) == 0 && cudaStreamQuery(s) != cudaErrorNotReady) {   // done or failed
+            if (there()) break;
+            return false;
+        }
+    }
+    std::atomic_thread_fence(std::memory_order_acquire);
+    return true;
 }
 
 int k_permute3(const cplx* x, cplx* y, int d0, int d1, int d2, int p0, int p1, int p2, int inverse,
@@ -1067,7 +1115,7 @@ int k_weighted_sum(const cplx* N, int nb, long long n, const double* W, int r, c
 }
 
 int k_small_krylov(const int* d, const cplx* hb0, const cplx* hb1, const cplx* hb2, const SmallPairs& pp, cplx* x,
-                   double zr, double zi, double tol, int mmax, int arnoldi, KrylovScalars* ks, cudaStream_t s) {
+                   double zr, double zi, double tol, int mmax, int arnoldi, const Publish& pub, cudaStream_t s) {
     const int n = d[0] * d[1] * d[2], R = (n + SK_CL - 1) / SK_CL;
     const size_t smem = sizeof(cplx) * ((size_t)R * n + (size_t)(mmax + 1) * n);
     // the shared-memory limit is a per-device attribute of the kernel: set it
@@ -1087,6 +1135,6 @@ int k_small_krylov(const int* d, const cplx* hb0, const cplx* hb1, const cplx* h
         }
     }
     small_krylov_kernel<<<SK_CL, SK_THREADS, smem, s>>>(d[0], d[1], d[2], hb0, hb1, hb2, pp, x, zr, zi, tol, mmax,
-                                                        arnoldi, ks);
+                                                        arnoldi, pub);
     return 1;
 }

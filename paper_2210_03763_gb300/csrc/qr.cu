@@ -34,6 +34,7 @@
 #include "common.cuh"
 
 #include <algorithm>
+#include <cstring>
 #include <mutex>
 
 namespace {
@@ -632,7 +633,7 @@ __device__ void la_dots(int P, PairF pair, cplx* out, const cplx* A, long long M
 template <int RB>
 __global__ void __launch_bounds__(QB) qr_coop_kernel(cplx* A, long long M, int D, cplx* R, int* flags, cplx* part,
                                                      cplx* red_out, unsigned* bar, int* err, int nc_max, double tol,
-                                                     int la_max, int rpb) {
+                                                     int la_max, int rpb, Publish pub) {
     // dynamic shared memory: nc_max cached columns of RB + 1 rows, then the
     // look-ahead window of at most la_max (<= LA_WMAX) columns (this block's
     // rows of v1_j)
@@ -898,6 +899,13 @@ __global__ void __launch_bounds__(QB) qr_coop_kernel(cplx* A, long long M, int D
         }
         if (k0 >= D) break;     // every column decided and finalised
         k = k0 - 1;             // the loop's increment brings it to k0
+    }
+    if (b0 && pub.hs) {         // block 0 decided the flags: report them
+        __syncthreads();
+        for (int k = t; k < D; k += QB) pub.hs->qr_dep[k] = flags[k];
+        __threadfence_system();
+        __syncthreads();
+        if (t == 0) *(volatile unsigned*)&pub.hs->seq = pub.seq;
     }
 }
 
@@ -1347,6 +1355,7 @@ struct CoopArgs {
     double tol;
     int la;
     int rpb;
+    Publish pub;
 };
 
 std::mutex g_coop_mu;
@@ -1405,7 +1414,7 @@ bool launch_coop(CoopArgs& a, cudaStream_t s, int& nl) {
     if (G > (long long)nsm * per_sm) return false;
     // the barrier leaves its arrival count at zero after every completed
     // wait, so it needs a reset only after an error
-    void* args[] = {&a.A, &a.M, &a.D, &a.R, &a.flags, &a.part, &a.red_out, &a.bar, &a.err, &a.nc, &a.tol, &a.la, &a.rpb};
+    void* args[] = {&a.A, &a.M, &a.D, &a.R, &a.flags, &a.part, &a.red_out, &a.bar, &a.err, &a.nc, &a.tol, &a.la, &a.rpb, &a.pub};
     nl = 1;
     if (cudaLaunchCooperativeKernel((const void*)qr_coop_kernel<RB>, dim3((unsigned)G), dim3(QB), args, smem, s) ==
         cudaSuccess)
@@ -1440,6 +1449,7 @@ int qr_cgs2(cplx* A, int M, int D, cplx* R, const int* cand, int ncand, QrScratc
     // per call: 81 x 81 2.49 -> 1.11, 128 x 128 7.2 -> 1.95, 6561 x 128 8.5 ->
     // 4.2 (blocks of 128 rows before)
     bool coop_done = false;
+    const Publish pub = ws.hs ? Publish{ws.hs, ++*ws.seq, nullptr} : Publish{};
     if (D <= MAXD) {
         const int nsm = std::min(coop_sms(), QR_SMALL_BLOCKS);
         // few columns and rows: one block, no synchronisation at all
@@ -1461,7 +1471,7 @@ int qr_cgs2(cplx* A, int M, int D, cplx* R, const int* cand, int ncand, QrScratc
         }
         for (int i = 0; i < nopt && !coop_done; ++i) {
             int nc = opts[i].nc, la = opts[i].la, nl = 0;
-            CoopArgs a{A, MM, D, R, ws.flags, ws.part, ws.h, ws.bar, ws.err, nc, tol, la, rpb};
+            CoopArgs a{A, MM, D, R, ws.flags, ws.part, ws.h, ws.bar, ws.err, nc, tol, la, rpb, pub};
             switch (rb) {
                 case 8: coop_done = launch_coop<8>(a, s, nl); break;
                 case 16: coop_done = launch_coop<16>(a, s, nl); break;
@@ -1488,10 +1498,14 @@ int qr_cgs2(cplx* A, int M, int D, cplx* R, const int* cand, int ncand, QrScratc
 
     // dependent columns -> completion
     static thread_local int hflags[MAXD], herr;
-    cudaMemcpyAsync(hflags, ws.flags, sizeof(int) * D, cudaMemcpyDeviceToHost, s);
     herr = 0;
-    if (coop_done) cudaMemcpyAsync(&herr, ws.err, sizeof(int), cudaMemcpyDeviceToHost, s);
-    cudaStreamSynchronize(s);
+    if (coop_done && ws.hs && wait_status(ws.hs, pub.seq, s)) {
+        std::memcpy(hflags, ws.hs->qr_dep, sizeof(int) * D);
+    } else {
+        cudaMemcpyAsync(hflags, ws.flags, sizeof(int) * D, cudaMemcpyDeviceToHost, s);
+        if (coop_done) cudaMemcpyAsync(&herr, ws.err, sizeof(int), cudaMemcpyDeviceToHost, s);
+        cudaStreamSynchronize(s);
+    }
     if (herr) {   // a grid-barrier wait gave up: clear the flag, report
         cudaMemsetAsync(ws.err, 0, sizeof(int), s);
         cudaMemsetAsync(ws.bar, 0, 2 * sizeof(unsigned), s);

@@ -121,8 +121,14 @@ __global__ void __launch_bounds__(CT) panel_chol_kernel(const cplx* Sw, long lon
 // R's panel (columns n.., leading dimension D): rows < n: S1 + S2 R1, rows
 // n .. n + bp: R2 R1.  (S1, S2: leading dimension ld; R1, R2: PB.)
 __global__ void panel_r_kernel(const cplx* S1, const cplx* S2, long long ld, const cplx* R1, const cplx* R2, int n,
-                               int bp, cplx* R, int D, int* dep) {
+                               int bp, cplx* R, int D, int* dep, const int* flag, Publish pub) {
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
+    if (e == 0 && pub.hs) {
+        pub.hs->qr_flag = *flag;
+        if (pub.tc_flag && *(volatile const int*)pub.tc_flag) pub.hs->tc_flag = 1;
+        __threadfence_system();
+        *(volatile unsigned*)&pub.hs->seq = pub.seq;
+    }
     if (e < bp) dep[n + e] = 0;
     if (e >= (n + bp) * bp) return;
     const int i = e % (n + bp), j = e / (n + bp);
@@ -178,7 +184,7 @@ size_t qr_panel_workspace(int M, int D) {
 }
 
 int qr_panel(cplx* A, int M, int D, cplx* R, QrScratch& ws, cudaStream_t s, void* workspace, size_t workspace_bytes,
-             int first, int last) {
+             int first, int last, const Publish& pub) {
     cplx* S1 = ws.panel;
     cplx* S2 = S1 + (long long)(D + PB) * PB;
     cplx* C = S2 + (long long)(D + PB) * PB;
@@ -218,7 +224,8 @@ int qr_panel(cplx* A, int M, int D, cplx* R, QrScratch& ws, cudaStream_t s, void
             if (l < 0) return -1;
             launches += l;
         }
-        panel_r_kernel<<<((n + bp) * bp + 127) / 128, 128, 0, s>>>(S1, S2, ld, R1, R2, n, bp, R, D, ws.flags);
+        panel_r_kernel<<<((n + bp) * bp + 127) / 128, 128, 0, s>>>(S1, S2, ld, R1, R2, n, bp, R, D, ws.flags,
+                                                                    flag, n + PB >= std::min(D, last) ? pub : Publish{});
         ++launches;
     }
     return launches;

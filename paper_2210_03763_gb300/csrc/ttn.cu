@@ -94,6 +94,7 @@ struct Env {
     cplx* dops = nullptr;          // 3 * |driven| * D*D
     int* d_sites = nullptr;        // device copies of the id lists
     int* d_driven = nullptr;
+    std::vector<int> sites_up, driven_up;   // what the device copies hold
     size_t cap_n = 0, cap_d = 0;   // capacity in matrices
 };
 
@@ -145,12 +146,9 @@ struct ttn_ctx {
     double* kpn = nullptr;    // RED_BLOCKS
     double* apx = nullptr;    // RED_BLOCKS: norm^2 partials of an absorbed node
     double* apr = nullptr;    // RED_BLOCKS: norm^2 partials of the absorbed link matrix
-    struct HostStatus {
-        KrylovStatus krylov;
-        int tc_flag;
-        int qr_flag;
-    };
-    HostStatus* hstat = nullptr;   // pinned host: status read back from the device
+    HostStatus* hstat = nullptr;   // pinned host memory that kernels report into
+    unsigned seq = 0;              // last sequence number used with it
+    std::map<std::pair<const Env*, const Env*>, int> kry_hint;   // Krylov steps of a node or link last time
     QrScratch qr{};
     std::map<std::pair<int, int>, int*> cand;   // (node, leg) -> candidate rows
     std::map<std::pair<int, int>, int> ncand;
@@ -943,8 +941,27 @@ bool env_has_block(const Env& e) { return e.has_H || !e.sites.empty(); }
 // x <- exp(z H) x with H given by `apply`; z = (zr, zi).  Lanczos: the
 // three-term recurrence, then a pass against the whole basis; with decay
 // (non-Hermitian H) Arnoldi, two passes against the whole basis.
+// Where the next reporting launch reports.
+Publish next_publish(ttn_ctx* c) { return {c->hstat, ++c->seq, reinterpret_cast<const int*>(c->split_ws)}; }
+
+void wait_published(ttn_ctx* c) {
+    if (!wait_status(c->hstat, c->seq, c->stream)) {
+        CUDA_OK(cudaStreamSynchronize(c->stream));
+        throw TtnError(TTN_ERR_CUDA, "a kernel ended without its status");
+    }
+    if (c->hstat->tc_flag) {   // a tensor-core wait that gave up leaves garbage: report it first
+        CUDA_OK(cudaStreamSynchronize(c->stream));
+        c->hstat->tc_flag = 0;
+        check_split_flag(c);
+    }
+}
+
+// `hint`: the steps that this node or link took last time (0: unknown).  That
+// many are launched before the host looks at the first status; every step's
+// status and coefficients are kept, so that the run ends at the first converged
+// step whatever was launched beyond it.
 template <class F>
-void krylov(ttn_ctx* c, cplx* x, long long n, double zr, double zi, F apply) {
+void krylov(ttn_ctx* c, cplx* x, long long n, double zr, double zi, int& hint, F apply) {
     cudaStream_t s = c->stream;
     const double tol = (c->prec == TTN_FP64) ? 1e-13 : 1e-9;
     const int mmax = test_krylov_mmax();
@@ -952,21 +969,18 @@ void krylov(ttn_ctx* c, cplx* x, long long n, double zr, double zi, F apply) {
     const long long ld = n;
     {
         ProfScope ps(c, PK_KRY, 0.0, 48.0 * n);
-        c->stats[3] += k_norm2_partial(x, n, c->kpn, s);
-        c->stats[3] += k_krylov_start_ex(c->ks, c->kpn, n, s);
+        c->stats[3] += k_krylov_start(c->ks, x, n, c->kpn, s);
         c->stats[3] += k_scale_copy_dev(x, n, &c->ks->inv_scale, V, s);
     }
-    const KrylovStatus& st = c->hstat->krylov;
-    int j = 0;
-    for (;; ++j) {
+    int m = -1, seen = 0;   // the converged step, steps whose status has been read
+    for (int j = 0; m < 0 && j < mmax; ++j) {
         cplx* vj = V + (long long)j * ld;
         cplx* w = V + (long long)(j + 1) * ld;
         apply(vj, w);
-        c->stats[1] += 1;
         {
             // bytes: the basis is read twice (Arnoldi: three times), w read and written twice
             const bool arnoldi = c->gamma != 0.0;   // non-Hermitian generator (decay)
-            ProfScope ps(c, PK_KRY, 0.0, 16.0 * n * ((arnoldi ? 3.0 : 2.0) * (j + 1) + 7.0));
+            ProfScope ps(c, PK_KRY, 0.0, 16.0 * n * ((arnoldi ? 3.0 : 2.0) * (j + 1) + 9.0));
             cplx* part2 = c->kpart + (size_t)RED_BLOCKS * (KRYLOV_MMAX + 1);
             if (arnoldi) {
                 c->stats[3] += k_dots(V, ld, j + 1, w, n, c->kpart, s);
@@ -975,26 +989,29 @@ void krylov(ttn_ctx* c, cplx* x, long long n, double zr, double zi, F apply) {
                 c->stats[3] += k_dots(vj, ld, 1, w, n, c->kpart, s);
                 c->stats[3] += k_lanczos_first(V, ld, j, c->kpart, c->ks, w, n, part2, c->kh1, s);
             }
-            c->stats[3] += k_orth_second(V, ld, j + 1, part2, w, n, c->kpn, c->ks, c->kh1, zr, zi, tol, arnoldi, s);
+            c->stats[3] += k_orth_second(V, ld, j + 1, part2, w, n, c->kpn, c->ks, c->kh1, zr, zi, tol, arnoldi,
+                                         next_publish(c), s);
+            if (j + 1 < mmax) c->stats[3] += k_scale_copy_dev(w, n, &c->ks->inv_scale, w, s);
         }
-        CUDA_OK(cudaMemcpyAsync(&c->hstat->krylov, &c->ks->st, sizeof(st), cudaMemcpyDeviceToHost, s));
-        c->hstat->tc_flag = 0;
-        if (c->split_ws)   // a tensor-core wait that gave up leaves garbage: report it first
-            CUDA_OK(cudaMemcpyAsync(&c->hstat->tc_flag, c->split_ws, sizeof(int), cudaMemcpyDeviceToHost, s));
-        CUDA_OK(cudaStreamSynchronize(s));
-        if (c->hstat->tc_flag) check_split_flag(c);
-        if (st.nonfinite) throw TtnError(TTN_ERR_NUMERIC, "non-finite value in Lanczos");
-        if (st.converged || j == mmax - 1) break;
-        ProfScope ps(c, PK_KRY, 0.0, 32.0 * n);
-        c->stats[3] += k_scale_copy_dev(w, n, &c->ks->inv_scale, w, s);
+        if (j + 1 < std::min(hint, mmax)) continue;
+        wait_published(c);
+        for (; seen <= j && m < 0; ++seen) {
+            const KrylovStatus& st = c->hstat->krylov[seen];
+            if (st.nonfinite) throw TtnError(TTN_ERR_NUMERIC, "non-finite value in Lanczos");
+            if (st.converged) m = seen;
+        }
     }
-    if (!st.converged) {
-        c->max_err = std::max(c->max_err, st.err);
-        if (st.err > 1e-6) throw TtnError(TTN_ERR_KRYLOV, "Lanczos did not converge in m_max steps");
+    if (m < 0) {
+        m = mmax - 1;
+        const double err = c->hstat->krylov[m].err;
+        c->max_err = std::max(c->max_err, err);
+        if (err > 1e-6) throw TtnError(TTN_ERR_KRYLOV, "Lanczos did not converge in m_max steps");
     }
+    hint = m + 1;
     c->stats[0] += 1;
-    ProfScope ps(c, PK_KRY, 0.0, 16.0 * n * (j + 2));
-    c->stats[3] += k_combine(V, ld, j + 1, c->ks, x, n, s);
+    c->stats[1] += m + 1;
+    ProfScope ps(c, PK_KRY, 0.0, 16.0 * n * (m + 2));
+    c->stats[3] += k_combine(V, ld, m + 1, c->ks, x, n, s);
 }
 
 // Small nodes and links (s <= SMALL_S): the whole Krylov exponential in one
@@ -1019,11 +1036,10 @@ bool small_evolve(ttn_ctx* c, const int* d, cplx* const* hb, const Pair* pairs, 
     {
         ProfScope ps(c, PK_KRY, 0.0, 0.0);
         c->stats[3] += k_small_krylov(d, hb[0], hb[1], hb[2], pp, x, zr, zi, tol, test_krylov_mmax(),
-                                      c->gamma != 0.0 ? 1 : 0, c->ks, c->stream);
+                                      c->gamma != 0.0 ? 1 : 0, next_publish(c), c->stream);
     }
-    KrylovStatus& st = c->hstat->krylov;
-    CUDA_OK(cudaMemcpyAsync(&st, &c->ks->st, sizeof(st), cudaMemcpyDeviceToHost, c->stream));
-    CUDA_OK(cudaStreamSynchronize(c->stream));
+    wait_published(c);
+    const KrylovStatus& st = c->hstat->krylov[0];
     if (st.nonfinite) throw TtnError(TTN_ERR_NUMERIC, "non-finite value in Lanczos");
     c->stats[0] += 1;
     c->stats[1] += st.iters;
@@ -1041,13 +1057,24 @@ void ensure_env_capacity(ttn_ctx* c, Env& E, size_t nn, size_t nd) {
     if (nn > E.cap_n) {
         E.nops = (cplx*)dalloc(c, sizeof(cplx) * DD * nn);
         E.d_sites = (int*)dalloc(c, sizeof(int) * nn);
+        E.sites_up.clear();
         E.cap_n = nn;
     }
     if (nd > E.cap_d) {
         E.dops = (cplx*)dalloc(c, sizeof(cplx) * DD * 3 * nd);
         E.d_driven = (int*)dalloc(c, sizeof(int) * nd);
+        E.driven_up.clear();
         E.cap_d = nd;
     }
+}
+
+// Device copy of an id list, sent when it differs from what was sent before
+// (two blocking copies per environment otherwise; the lists only change with
+// the schedule).
+void upload_ids(const std::vector<int>& ids, std::vector<int>& sent, int* d, cudaStream_t s) {
+    if (ids.empty() || ids == sent) return;
+    CUDA_OK(cudaMemcpyAsync(d, ids.data(), sizeof(int) * ids.size(), cudaMemcpyHostToDevice, s));
+    sent = ids;
 }
 
 // Split-precision renormalisation of an operator stack (a2): for every op_i
@@ -1182,10 +1209,8 @@ void renormalize(ttn_ctx* c, const cplx* X, const int* d, int o, const Env& eu, 
     ensure_env_capacity(c, E, E.sites.size(), E.driven.size());
     long long DDo = (long long)E.D * E.D;
     cudaStream_t s = c->stream;
-    if (!E.sites.empty())
-        CUDA_OK(cudaMemcpyAsync(E.d_sites, E.sites.data(), sizeof(int) * E.sites.size(), cudaMemcpyHostToDevice, s));
-    if (!E.driven.empty())
-        CUDA_OK(cudaMemcpyAsync(E.d_driven, E.driven.data(), sizeof(int) * E.driven.size(), cudaMemcpyHostToDevice, s));
+    upload_ids(E.sites, E.sites_up, E.d_sites, s);
+    upload_ids(E.driven, E.driven_up, E.d_driven, s);
     // static block: X^H (Hs_u + Hs_v + sum V n n) X
     const Env* e3[3];
     e3[u] = &eu;
@@ -1269,15 +1294,15 @@ int gauge_qr(ttn_ctx* c, cplx*& A, cplx*& spare, int M, int D, cplx* R, const in
             int gave_up = 0;
             for (int first = 0; first < D && !gave_up;) {
                 const int last = hint == 1 || first > 0 ? D : QR_PANEL;
-                const int n = qr_panel(spare, M, D, R, q, c->stream, c->split_ws, c->split_cap, first, last);
+                const int n = qr_panel(spare, M, D, R, q, c->stream, c->split_ws, c->split_cap, first, last,
+                                       next_publish(c));
                 if (n < 0) {
-                    gave_up = 2;
+                    gave_up = 1;
                     break;
                 }
                 c->stats[3] += n;
                 c->digits_run = true;
-                CUDA_OK(cudaMemcpyAsync(&c->hstat->qr_flag, q.err + 1, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-                CUDA_OK(cudaStreamSynchronize(c->stream));
+                wait_published(c);
                 gave_up = c->hstat->qr_flag;
                 first = last;
             }
@@ -1372,7 +1397,7 @@ void node_evolve(ttn_ctx* c, int k, double tau) {
     if (small_evolve(c, nd.d, hbs, pairs, np, c->T[k], 0.0, -tau)) return;
     SplitHeff S;
     const bool sp = split_heff_prepare(c, S, nd.d, hbs, pairs, np);
-    krylov(c, c->T[k], nd.s, 0.0, -tau, [&](const cplx* x, cplx* y) {
+    krylov(c, c->T[k], nd.s, 0.0, -tau, c->kry_hint[{e[0], e[1]}], [&](const cplx* x, cplx* y) {
         if (sp) split_heff_apply(c, S, x, y);
         else heff_apply(c, nd.d, hbs, Dl, pairs, np, x, y);
     });
@@ -1394,7 +1419,7 @@ void link_evolve(ttn_ctx* c, const Env& er, const Env& ec, double tau) {
     if (small_evolve(c, d, hbs, pairs, np, c->Rbuf, 0.0, tau)) return;
     SplitHeff S;
     const bool sp = split_heff_prepare(c, S, d, hbs, pairs, np);
-    krylov(c, c->Rbuf, (long long)d[0] * d[1], 0.0, tau, [&](const cplx* x, cplx* y) {
+    krylov(c, c->Rbuf, (long long)d[0] * d[1], 0.0, tau, c->kry_hint[{e[0], e[1]}], [&](const cplx* x, cplx* y) {
         if (sp) split_heff_apply(c, S, x, y);
         else heff_apply(c, d, hbs, Dl, pairs, np, x, y);
     });
@@ -1631,6 +1656,8 @@ void alloc_qr_scratch(ttn_ctx* c, long long maxM, int maxD, QrScratch& q) {
     q.row_rank = (int*)dalloc(c, sizeof(int) * std::max<long long>(maxM, 1));
     q.cand_used = (int*)dalloc(c, sizeof(int) * std::max<long long>(maxM, 1));
     q.panel = (cplx*)dalloc(c, sizeof(cplx) * (3 * (size_t)(maxD + QR_PANEL) * QR_PANEL + 3 * QR_PANEL * QR_PANEL));
+    q.hs = c->hstat;
+    q.seq = &c->seq;
     q.bar = (unsigned*)dalloc(c, sizeof(unsigned) * 4);
     q.err = (int*)dalloc(c, sizeof(int) * 4);
     CUDA_OK(cudaMemset(q.err, 0, sizeof(int) * 4));
@@ -1664,6 +1691,7 @@ void allocate(ttn_ctx* c) {
     c->Rbuf = (cplx*)dalloc(c, sizeof(cplx) * MAX_CHI * MAX_CHI);
     c->Kbasis = (cplx*)dalloc(c, sizeof(cplx) * (KRYLOV_MMAX + 1) * c->smax);
     c->ks = (KrylovScalars*)dalloc(c, sizeof(KrylovScalars));
+    CUDA_OK(cudaMemset(c->ks, 0, sizeof(KrylovScalars)));   // block counters start at zero
     c->kh1 = (cplx*)dalloc(c, sizeof(cplx) * (KRYLOV_MMAX + 1));
     c->kpart = (cplx*)dalloc(c, sizeof(cplx) * 2 * RED_BLOCKS * (MAX_CHI + 2));
     c->kpn = (double*)dalloc(c, sizeof(double) * RED_BLOCKS);
@@ -1675,7 +1703,9 @@ void allocate(ttn_ctx* c) {
     alloc_qr_scratch(c, mq, MAX_CHI, c->qr);
     c->d_coef = (double*)dalloc(c, sizeof(double) * 5 * c->N);
     c->h_coef.assign(5 * c->N, 0.0);
-    CUDA_OK(cudaMallocHost(&c->hstat, sizeof(ttn_ctx::HostStatus)));
+    CUDA_OK(cudaMallocHost(&c->hstat, sizeof(HostStatus)));
+    std::memset(c->hstat, 0, sizeof(HostStatus));
+    c->qr.hs = c->hstat;
     c->up.assign(nn, Env());
     c->down.assign(nn, Env());
     c->phys.assign(c->n_leaves, Env());
@@ -2492,7 +2522,8 @@ ttn_status ttn_selftest_qr(const double* A, int M, int D, const int* cand, int n
                 t->hstat = nullptr;
             }
         } fr{&tmp};
-        CUDA_OK(cudaMallocHost(&tmp.hstat, sizeof(ttn_ctx::HostStatus)));
+        CUDA_OK(cudaMallocHost(&tmp.hstat, sizeof(HostStatus)));
+        std::memset(tmp.hstat, 0, sizeof(HostStatus));
         QrScratch q;
         alloc_qr_scratch(&tmp, M, D, q);
         cplx* dA = (cplx*)dalloc(&tmp, sizeof(cplx) * (size_t)M * D);
