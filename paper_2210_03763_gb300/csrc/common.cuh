@@ -271,6 +271,16 @@ int qr_cgs2(cplx* A, int M, int D, cplx* R, const int* cand, int ncand,
 // (R_in V = R_out).  One cooperative launch; bar: 2 unsigned, err: set when a
 // grid-barrier wait gave up; info[0]: sweeps run.  Returns launches, -1 if
 // the cooperative launch failed.
+struct JacobiTask {
+    cplx* R;
+    cplx* V;
+    int N;
+    unsigned* bar;
+    int* info;
+};
+constexpr int SVD_BATCH = 48;   // matrices per launch at most
+// The same for n independent matrices, as many per launch as are co-resident.
+int svd_jacobi_batch(const JacobiTask* tasks, int n, int max_sweeps, double tol, int* err, cudaStream_t s);
 int svd_jacobi_square(cplx* R, cplx* V, int N, int max_sweeps, double tol, unsigned* bar, int* err, int* info,
                       cudaStream_t s);
 // sigma_i = |r_i|, descending order, kept k = min(chi, #{sigma >= eps sigma_max})

@@ -74,13 +74,29 @@ __device__ void pair_of(int k, int r, int Np, int& i, int& j) {
     j = at(Np - 1 - k);
 }
 
+// Several matrices in one launch: a sweep over one matrix is a chain of
+// barriers between its N / 2 blocks (4 ms at N = 64, nearly all of it waiting),
+// so the bonds of a tree run side by side, each with its own barrier.
+struct JacobiBatch {
+    JacobiTask t[SVD_BATCH];
+    int first[SVD_BATCH + 1];   // first block of each matrix
+    int n;
+};
+
 // info: [0] sweeps run, [1] unused, [2], [3] rotation counters (alternating sweeps)
-__global__ void __launch_bounds__(SVD_THREADS) jacobi_kernel(cplx* R, cplx* V, int N, int Np, int max_sweeps,
-                                                            double tol, unsigned* bar, int* err, int* info) {
+__global__ void __launch_bounds__(SVD_THREADS) jacobi_kernel(const __grid_constant__ JacobiBatch jb, int max_sweeps,
+                                                            double tol, int* err) {
     __shared__ double red[3][SVD_THREADS / 32];
     __shared__ double rot[4];   // c, s, cos phi, sin phi; rot[0] < 0: skip
-    const unsigned nb = gridDim.x;
-    const int k = blockIdx.x;
+    int m = 0;
+    while ((int)blockIdx.x >= jb.first[m + 1]) ++m;
+    cplx* R = jb.t[m].R;
+    cplx* V = jb.t[m].V;
+    const int N = jb.t[m].N, Np = N + (N & 1);
+    unsigned* bar = jb.t[m].bar;
+    int* info = jb.t[m].info;
+    const unsigned nb = jb.first[m + 1] - jb.first[m];
+    const int k = (int)blockIdx.x - jb.first[m];
     // |R|_F^2, the same in every block (same summation order): pairs whose
     // inner product is below 1e-30 |R|_F^2 are left alone -- columns that
     // rank deficiency has already reduced to rounding noise would otherwise
@@ -169,8 +185,8 @@ __global__ void __launch_bounds__(SVD_THREADS) jacobi_kernel(cplx* R, cplx* V, i
                 __syncthreads();
                 if (rot[0] >= 0.0) {
                     const double c = rot[0], s = rot[1], pc = rot[2], ps = rot[3];   // e^{-i phi} = pc - i ps
-                    for (int m = 0; m < 2; ++m) {
-                        cplx* X = m == 0 ? R : V;
+                    for (int w = 0; w < 2; ++w) {
+                        cplx* X = w == 0 ? R : V;
                         cplx* xi = X + (long long)i * N;
                         cplx* xj = X + (long long)j * N;
                         for (int e = threadIdx.x; e < N; e += SVD_THREADS) {
@@ -258,20 +274,43 @@ __global__ void identity_kernel(cplx* V, int N) {
 
 }  // namespace
 
+int svd_jacobi_batch(const JacobiTask* tasks, int n, int max_sweeps, double tol, int* err, cudaStream_t s) {
+    int dev = 0, nsm = 0, per_sm = 0, launches = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, jacobi_kernel, SVD_THREADS, 0);
+    const int room = nsm * per_sm;
+    for (int i = 0; i < n;) {
+        JacobiBatch jb;
+        jb.n = 0;
+        jb.first[0] = 0;
+        for (; i < n && jb.n < SVD_BATCH; ++i) {   // as many matrices as are co-resident
+            const JacobiTask& t = tasks[i];
+            const int blocks = (t.N + 1) / 2;
+            if (jb.n > 0 && jb.first[jb.n] + blocks > room) break;
+            identity_kernel<<<(t.N * t.N + 255) / 256, 256, 0, s>>>(t.V, t.N);
+            cudaMemsetAsync(t.bar, 0, 2 * sizeof(unsigned), s);
+            cudaMemsetAsync(t.info, 0, 4 * sizeof(int), s);
+            ++launches;
+            if (t.N < 2) continue;   // nothing to rotate
+            jb.t[jb.n] = t;
+            jb.first[jb.n + 1] = jb.first[jb.n] + blocks;
+            ++jb.n;
+        }
+        if (jb.n == 0) continue;
+        void* args[] = {(void*)&jb, (void*)&max_sweeps, (void*)&tol, (void*)&err};
+        if (cudaLaunchCooperativeKernel((const void*)jacobi_kernel, dim3(jb.first[jb.n]), dim3(SVD_THREADS), args, 0,
+                                        s) != cudaSuccess)
+            return -1;
+        ++launches;
+    }
+    return launches;
+}
+
 int svd_jacobi_square(cplx* R, cplx* V, int N, int max_sweeps, double tol, unsigned* bar, int* err, int* info,
                       cudaStream_t s) {
-    const int Np = N + (N & 1);
-    identity_kernel<<<(N * N + 255) / 256, 256, 0, s>>>(V, N);
-    cudaMemsetAsync(bar, 0, 2 * sizeof(unsigned), s);
-    cudaMemsetAsync(info, 0, 4 * sizeof(int), s);
-    if (Np < 2) return 1;
-    int blocks = Np / 2;
-    void* args[] = {(void*)&R, (void*)&V, (void*)&N, (void*)&Np, (void*)&max_sweeps, (void*)&tol,
-                    (void*)&bar, (void*)&err, (void*)&info};
-    if (cudaLaunchCooperativeKernel((const void*)jacobi_kernel, dim3(blocks), dim3(SVD_THREADS), args, 0, s) !=
-        cudaSuccess)
-        return -1;
-    return 2;
+    const JacobiTask t{R, V, N, bar, info};
+    return svd_jacobi_batch(&t, 1, max_sweeps, tol, err, s);
 }
 
 int svd_finish(const cplx* R, const cplx* V, int N, int chi, double eps, cplx* Ur, cplx* Vh, double* S, int* k,

@@ -2726,80 +2726,107 @@ ttn_status ttn_compress(ttn_ctx* src, ttn_ctx* dst, double* discarded) {
         centre_to_root(c);
         CUDA_OK(cudaStreamSynchronize(c->stream));
         const int nn = (int)c->nodes.size();
-        std::vector<void*> temp;
-        struct Free {
-            std::vector<void*>& t;
-            ~Free() {
-                for (void* p : t) cudaFree(p);
-            }
-        } fr{temp};
-        auto tmalloc = [&](size_t bytes) {
-            void* p = nullptr;
-            if (test_take_alloc_fail() || cudaMalloc(&p, std::max<size_t>(bytes, 16)) != cudaSuccess)
-                throw TtnError(TTN_ERR_ALLOC, "compress buffers");
-            temp.push_back(p);
-            return p;
+        // one allocation: per bond the Gram (overwritten by the rotations), its V
+        // and eigenvectors, the kept ones transposed, the eigenvalues
+        struct Bond {
+            cplx *G, *V, *U, *UT;
+            double* S;
+            unsigned* bar;
+            int* info;
         };
+        std::vector<Bond> bd(nn);
+        uint8_t* arena = nullptr;
+        size_t used = 0;
+        auto take = [&](size_t bytes) {
+            uint8_t* p = arena + used;
+            used += (std::max<size_t>(bytes, 16) + 255) / 256 * 256;
+            return (void*)p;
+        };
+        int *err = nullptr, *order = nullptr, *dk = nullptr;
+        double *ddisc = nullptr, *dS = nullptr;
+        cplx* Vh = nullptr;   // of the bond at hand, not used
+        auto lay_out = [&] {
+            used = 0;
+            err = (int*)take(sizeof(int) * 4);
+            order = (int*)take(sizeof(int) * MAX_CHI);
+            dk = (int*)take(sizeof(int) * 4);
+            ddisc = (double*)take(sizeof(double));
+            dS = (double*)take(sizeof(double) * MAX_CHI * (size_t)nn);
+            Vh = (cplx*)take(sizeof(cplx) * MAX_CHI * MAX_CHI);
+            for (int k = 0; k < nn; ++k) {
+                const size_t D = c->nodes[k].d[2], Dn = dst->nodes[k].d[2];
+                bd[k].G = (cplx*)take(sizeof(cplx) * D * D);
+                if (k == c->root) continue;
+                bd[k].V = (cplx*)take(sizeof(cplx) * D * D);
+                bd[k].U = (cplx*)take(sizeof(cplx) * D * D);
+                bd[k].UT = (cplx*)take(sizeof(cplx) * D * Dn);
+                bd[k].S = dS + (size_t)MAX_CHI * k;
+                bd[k].bar = (unsigned*)take(sizeof(unsigned) * 2);
+                bd[k].info = (int*)take(sizeof(int) * 4);
+            }
+        };
+        lay_out();
+        struct Free {
+            uint8_t*& p;
+            ~Free() { cudaFree(p); }
+        } fr{arena};
+        if (test_take_alloc_fail() || cudaMalloc(&arena, used) != cudaSuccess) {
+            arena = nullptr;
+            cudaGetLastError();
+            throw TtnError(TTN_ERR_ALLOC, "compress buffers");
+        }
+        lay_out();
         // bond Grams top-down: G_k(a, a') = <R_a|R_a'>, G_root = [[1]]
-        std::vector<cplx*> G(nn, nullptr);
-        G[c->root] = (cplx*)tmalloc(sizeof(cplx));
-        const cplx one = C(1.0);
-        CUDA_OK(cudaMemcpyAsync(G[c->root], &one, sizeof(cplx), cudaMemcpyHostToDevice, c->stream));
+        c->stats[3] += k_fill(bd[c->root].G, 1, C(1.0), c->stream);
         for (int li = (int)c->level_nodes.size() - 1; li >= 0; --li)
             for (int p : c->level_nodes[li]) {
                 const Node& np_ = c->nodes[p];
-                leg_apply(c, G[p], np_.d[2], c->T[p], np_.d, 2, c->tmp[0], 0.0);
+                leg_apply(c, bd[p].G, np_.d[2], c->T[p], np_.d, 2, c->tmp[0], 0.0);
                 for (int u = 0; u < 2; ++u) {
                     const int k = np_.child[u];
-                    if (k < 0) continue;
-                    const long long D = np_.d[u];
-                    G[k] = (cplx*)tmalloc(sizeof(cplx) * D * D);
-                    project(c, c->T[p], np_.d, c->tmp[0], np_.d, u, G[k], 1, 0, 0);
+                    if (k >= 0) project(c, c->T[p], np_.d, c->tmp[0], np_.d, u, bd[k].G, 1, 0, 0);
                 }
             }
         // Schmidt bases: one-sided Jacobi on each Gram (Hermitian PSD: its left
         // singular vectors are its eigenvectors), all D columns in descending
         // order; the kept ones are the first D' (their conjugates in the
         // subtree basis)
-        unsigned* bar = (unsigned*)tmalloc(sizeof(unsigned) * 4);
-        int* err = (int*)tmalloc(sizeof(int) * 4);
-        int* info = (int*)tmalloc(sizeof(int) * 4);
-        int* order = (int*)tmalloc(sizeof(int) * MAX_CHI);
-        int* dk = (int*)tmalloc(sizeof(int) * 4);
-        double* ddisc = (double*)tmalloc(sizeof(double));
-        double* dS = (double*)tmalloc(sizeof(double) * MAX_CHI);
-        cplx* Rw = (cplx*)tmalloc(sizeof(cplx) * MAX_CHI * MAX_CHI);
-        cplx* Vw = (cplx*)tmalloc(sizeof(cplx) * MAX_CHI * MAX_CHI);
-        cplx* Vh = (cplx*)tmalloc(sizeof(cplx) * MAX_CHI * MAX_CHI);
-        std::vector<cplx*> UT(nn, nullptr), UHc(nn, nullptr);   // U^T (no conj) and conj(U)^T per bond
         CUDA_OK(cudaMemsetAsync(err, 0, sizeof(int) * 4, c->stream));
-        double dsum = 0.0, dmax = 0.0;
-        std::vector<double> hS(MAX_CHI);
+        std::vector<JacobiTask> tasks;
+        for (int k = 0; k < nn; ++k)
+            if (k != c->root) tasks.push_back({bd[k].G, bd[k].V, c->nodes[k].d[2], bd[k].bar, bd[k].info});
+        const int nj = svd_jacobi_batch(tasks.data(), (int)tasks.size(), 60, 1e-15, err, c->stream);
+        if (nj < 0) throw TtnError(TTN_ERR_CUDA, "Jacobi launch failed");
+        c->stats[3] += nj;
+        std::vector<cplx*> UT(nn, nullptr);   // U^T (no conj) per bond
         for (int k = 0; k < nn; ++k) {
             if (k == c->root) continue;
             const int D = c->nodes[k].d[2], Dn = dst->nodes[k].d[2];
-            CUDA_OK(cudaMemcpyAsync(Rw, G[k], sizeof(cplx) * D * D, cudaMemcpyDeviceToDevice, c->stream));
-            if (svd_jacobi_square(Rw, Vw, D, 60, 1e-15, bar, err, info, c->stream) < 0)
-                throw TtnError(TTN_ERR_CUDA, "Jacobi launch failed");
-            cplx* Ur = (cplx*)tmalloc(sizeof(cplx) * D * D);
-            svd_finish(Rw, Vw, D, D, -1.0, Ur, Vh, dS, dk, ddisc, order, c->stream);
-            int herr = 0;
-            CUDA_OK(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
-            CUDA_OK(cudaMemcpyAsync(hS.data(), dS, sizeof(double) * D, cudaMemcpyDeviceToHost, c->stream));
-            CUDA_OK(cudaStreamSynchronize(c->stream));
-            if (herr) throw TtnError(TTN_ERR_TIMEOUT, "Jacobi grid barrier wait timed out");
+            c->stats[3] += svd_finish(bd[k].G, bd[k].V, D, D, -1.0, bd[k].U, Vh, bd[k].S, dk, ddisc, order,
+                                      c->stream);
+            // U: D x D, its first Dn columns are the kept eigenvectors of G_k;
+            // transposed to Dn x D (the leg matrices below)
+            UT[k] = bd[k].UT;
+            c->stats[3] += k_permute3(bd[k].U, UT[k], D, Dn, 1, 1, 0, 2, 0, c->stream);
+        }
+        std::vector<double> hS((size_t)MAX_CHI * nn);
+        int herr = 0;
+        CUDA_OK(cudaMemcpyAsync(hS.data(), dS, sizeof(double) * hS.size(), cudaMemcpyDeviceToHost, c->stream));
+        CUDA_OK(cudaMemcpyAsync(&herr, err, sizeof(int), cudaMemcpyDeviceToHost, c->stream));
+        CUDA_OK(cudaStreamSynchronize(c->stream));
+        if (herr) throw TtnError(TTN_ERR_TIMEOUT, "Jacobi grid barrier wait timed out");
+        check_digits(c);
+        double dsum = 0.0, dmax = 0.0;
+        for (int k = 0; k < nn; ++k) {
+            if (k == c->root) continue;
             double tot = 0.0, drop = 0.0;   // eigenvalues of the Gram are its singular values
-            for (int t = 0; t < D; ++t) {
-                tot += hS[t];
-                if (t >= Dn) drop += hS[t];
+            for (int t = 0; t < c->nodes[k].d[2]; ++t) {
+                tot += hS[(size_t)MAX_CHI * k + t];
+                if (t >= dst->nodes[k].d[2]) drop += hS[(size_t)MAX_CHI * k + t];
             }
             const double e = tot > 0.0 ? drop / tot : 0.0;
             dsum += e;
             dmax = std::max(dmax, e);
-            // Ur: D x D, its first Dn columns are the kept eigenvectors of G_k;
-            // transpose them to Dn x D (the leg matrices below)
-            UT[k] = (cplx*)tmalloc(sizeof(cplx) * Dn * D);
-            c->stats[3] += k_permute3(Ur, UT[k], D, Dn, 1, 1, 0, 2, 0, c->stream);
         }
         // projected tensors: children legs by U_c^H = Ur_c^T, parent leg by
         // U_k^T = conj(Ur_k)^T, then into dst
