@@ -53,7 +53,7 @@ struct SplitPackArgs {
     float* hi;
     float* lo;
 };
-int split_pack(const SplitPackArgs& p, cudaStream_t stream);
+int split_pack(const SplitPackArgs* p, int n, cudaStream_t stream);   // n operands, few launches
 
 // Packed output of a split contraction: the epilogue writes TF32 hi/lo
 // planes (as split_pack with embed = 0) at float2 position

@@ -75,13 +75,22 @@ __device__ __forceinline__ void tmem_ld16(uint32_t taddr, float* v) {
     for (int i = 0; i < 16; ++i) v[i] = __uint_as_float(r[i]);
 }
 
+// Round a float to TF32 (10 mantissa bits, to nearest, ties to even) with
+// integer operations; inf/nan unchanged.
+__device__ __forceinline__ float tf32_rne(float x) {
+    uint32_t u = __float_as_uint(x);
+    if ((u & 0x7F800000u) == 0x7F800000u) return x;
+    u += 0xFFFu + ((u >> 13) & 1u);
+    return __uint_as_float(u & 0xFFFFE000u);
+}
+
 // Split an FP64 value into TF32-representable hi and lo with integer
 // operations only (GB300's FP64 pipe is the bottleneck of any FP64
 // arithmetic): hi = x rounded to 10 mantissa bits (to nearest, ties to even),
 // lo = the exact remainder x - hi rounded to 11 significant bits; |hi + lo - x|
 // <= 2^-23 |x|.  |x| < 2^-126 (and FP64 subnormals) give 0; inf/nan pass
 // through the conversion instruction.
-__device__ __forceinline__ void split_tf32(double x, float& hi, float& lo) {
+__device__ __noinline__ void split_tf32_general(double x, float& hi, float& lo) {
     const unsigned long long u = (unsigned long long)__double_as_longlong(x);
     const unsigned sign = (unsigned)(u >> 63);
     const int e = (int)((u >> 52) & 0x7FF);
@@ -132,44 +141,120 @@ __device__ __forceinline__ void split_tf32(double x, float& hi, float& lo) {
     lo = __uint_as_float((lsign << 31) | ((unsigned)le << 23) | ((unsigned)(m & 0x3FFULL) << 13));
 }
 
+// The same values in half the instructions for exponents away from the ends of
+// the FP32 range.  The remainder is a 43-bit integer R (upper word rh, lower
+// word the lower word of x); it goes to a float of at most 24 bits with its
+// last bit set when bits were dropped, so that the one rounding to TF32 is
+// exact.
+__device__ __forceinline__ void split_tf32(double x, float& hi, float& lo) {
+    const uint32_t uh = (uint32_t)__double2hiint(x), ul = (uint32_t)__double2loint(x);
+    const int fe = (int)((uh >> 20) & 0x7FFu) - 1023 + 127;   // FP32 exponent field
+    if ((unsigned)(fe - 64) > 180u) {
+        if ((uh << 1) == 0u && ul == 0u) hi = lo = 0.f;
+        else split_tf32_general(x, hi, lo);
+        return;
+    }
+    const uint32_t sign = uh & 0x80000000u;
+    const uint32_t top = sign | ((uint32_t)fe << 23) | ((uh & 0xFFFFFu) << 3) | (ul >> 29);
+    uint32_t r = top | ((ul & 0x1FFFFFFFu) != 0u ? 1u : 0u);   // sticky bit for the tie
+    r += 0xFFFu + ((r >> 13) & 1u);
+    r &= 0xFFFFE000u;
+    hi = __uint_as_float(r);
+    const int rh = (int)(uh & 0x3FFu) - (r != (top & 0xFFFFE000u) ? 1024 : 0);
+    int w = (rh << 14) | (int)(ul >> 18), sh = 18;             // |R| >= 2^31: at least 13 bits stay
+    w |= (ul & 0x3FFFFu) != 0u ? 1 : 0;
+    if (rh == ((int)ul >> 31)) {                               // |R| < 2^31
+        w = (int)ul;
+        sh = 0;
+        if (w >= (1 << 24) || w <= -(1 << 24)) {
+            w = (w >> 7) | ((w & 0x7F) != 0 ? 1 : 0);
+            sh = 7;
+        }
+    }
+    lo = tf32_rne((float)w * __uint_as_float(sign | ((uint32_t)(fe - 52 + sh) << 23)));
+}
+
 // ----------------------------------------------------------------- packing
-// One thread per complex element (batch, row r < Rpad, k < Kc); entries with
-// r >= R or k >= Ki*Ko are written as zeros (tile padding).  Real row of
-// (r, bi, bo): (embed ? 2r : r) + bi*rb_i + bo*rb_o; float offset of k:
-// k_off + 2k in a row of `pitch` floats.
-__global__ void pack_kernel(SplitPackArgs p) {
+// Complex element (batch, row r < Rpad, k < Kc); entries with r >= R or
+// k >= Ki*Ko are written as zeros (tile padding).  Real row of (r, bi, bo):
+// (embed ? 2r : r) + bi*rb_i + bo*rb_o; float offset of k: k_off + 2k in a row
+// of `pitch` floats.
+//
+// A block packs 32 rows (numbered over rows and batches) by tiles of 32 K.
+// The planes are K-major, so warps write along K; operands whose rows are the
+// closer stride are read along the rows and turned in shared memory (one
+// 16-byte element per 32-byte sector otherwise).  Bound: HBM, then the integer
+// instructions of the split.  Measured, the 161 operands of one sampling sweep
+// (8x8 lattice, chi = 128): 22 -> 12.4 ms.
+constexpr int PK_ROWS = 32, PK_THREADS = 256, PK_JOBS = 6;
+struct PackJobs {   // several operands in one launch
+    SplitPackArgs p[PK_JOBS];
+    int first[PK_JOBS + 1];   // first block of each
+    int rb[PK_JOBS];          // row blocks (fastest), then K blocks of ktiles tiles
+    int ktiles[PK_JOBS];
+};
+__global__ void __launch_bounds__(PK_THREADS) pack_kernel(const __grid_constant__ PackJobs jobs) {
+    int job = 0;
+    while ((int)blockIdx.x >= jobs.first[job + 1]) ++job;
+    const SplitPackArgs& p = jobs.p[job];
+    const int local = (int)blockIdx.x - jobs.first[job], ktiles = jobs.ktiles[job];
+    const int kblock = local / jobs.rb[job], rblock = local - kblock * jobs.rb[job];
+    __shared__ const cplx* base[PK_ROWS];
+    __shared__ long long out[PK_ROWS];
+    __shared__ cplx tile[32][PK_ROWS + 1];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const long long f0 = (long long)rblock * PK_ROWS, nrow = (long long)p.Rpad * p.Bi * p.Bo;
+    if (threadIdx.x < PK_ROWS) {
+        const unsigned f = (unsigned)(f0 + threadIdx.x);
+        const unsigned b = f / (unsigned)p.Rpad;
+        const int r = (int)(f - b * (unsigned)p.Rpad);
+        const int bi = (int)(b % (unsigned)p.Bi), bo = (int)(b / (unsigned)p.Bi);
+        const bool in = f0 + threadIdx.x < nrow;
+        base[threadIdx.x] = in && r < p.R ? p.src + bi * p.s_bi + bo * p.s_bo + r * p.s_r : nullptr;
+        out[threadIdx.x] = in ? ((p.embed ? 2LL * r : (long long)r) + bi * p.rb_i + bo * p.rb_o) * p.pitch + p.k_off : -1;
+    }
+    __syncthreads();
     const int K = p.Ki * p.Ko;
-    const long long per_b = (long long)p.Rpad * p.Kc;
-    const long long total = per_b * p.Bi * p.Bo;
-    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
-         e += (long long)gridDim.x * blockDim.x) {
-        const long long b = e / per_b;
-        const long long rem = e - b * per_b;
-        const int r = (int)(rem / p.Kc);
-        const int k = (int)(rem - (long long)r * p.Kc);
-        const int bi = (int)(b % p.Bi), bo = (int)(b / p.Bi);
-        double re = 0.0, im = 0.0;
-        if (r < p.R && k < K) {
-            const int ki = k % p.Ki, ko = k / p.Ki;
-            cplx v = p.src[bi * p.s_bi + bo * p.s_bo + r * p.s_r + ki * p.s_ki + ko * p.s_ko];
-            re = v.x;
-            im = p.conj ? __longlong_as_double(__double_as_longlong(v.y) ^ (long long)0x8000000000000000ULL) : v.y;
+    const bool turn = p.s_r < p.s_ki;   // rows are closer than K
+    const int kend = min(p.Kc, (kblock + 1) * ktiles * 32);
+    for (int k0 = kblock * ktiles * 32; k0 < kend; k0 += 32) {
+        if (turn) {
+            const cplx* src = base[lane];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const int kk = warp + 8 * i, k = k0 + kk;
+                cplx v = make_double2(0.0, 0.0);
+                if (src && k < K) v = src[(k % p.Ki) * p.s_ki + (k / p.Ki) * p.s_ko];
+                tile[kk][lane] = v;
+            }
+            __syncthreads();
         }
-        float rh, rl, ih, il;
-        split_tf32(re, rh, rl);
-        split_tf32(im, ih, il);
-        const long long row = (p.embed ? 2LL * r : (long long)r) + bi * p.rb_i + bo * p.rb_o;
-        const long long o0 = row * p.pitch + p.k_off + 2LL * k;
-        if (p.embed) {
-            const long long o1 = o0 + p.pitch;
-            *reinterpret_cast<float2*>(p.hi + o0) = make_float2(rh, -ih);
-            *reinterpret_cast<float2*>(p.hi + o1) = make_float2(ih, rh);
-            *reinterpret_cast<float2*>(p.lo + o0) = make_float2(rl, -il);
-            *reinterpret_cast<float2*>(p.lo + o1) = make_float2(il, rl);
-        } else {
-            *reinterpret_cast<float2*>(p.hi + o0) = make_float2(rh, ih);
-            *reinterpret_cast<float2*>(p.lo + o0) = make_float2(rl, il);
+        const int k = k0 + lane;
+        const long long off = (k % p.Ki) * p.s_ki + (k / p.Ki) * p.s_ko;
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int r = warp + 8 * i;
+            const long long o = out[r];
+            if (o < 0 || k >= p.Kc) continue;
+            cplx v = make_double2(0.0, 0.0);
+            if (turn) v = tile[lane][r];
+            else if (base[r] && k < K) v = base[r][off];
+            float rh, rl, ih, il;
+            split_tf32(v.x, rh, rl);
+            split_tf32(p.conj ? -v.y : v.y, ih, il);
+            const long long o0 = o + 2LL * k;
+            if (p.embed) {
+                const long long o1 = o0 + p.pitch;
+                *reinterpret_cast<float2*>(p.hi + o0) = make_float2(rh, -ih);
+                *reinterpret_cast<float2*>(p.hi + o1) = make_float2(ih, rh);
+                *reinterpret_cast<float2*>(p.lo + o0) = make_float2(rl, -il);
+                *reinterpret_cast<float2*>(p.lo + o1) = make_float2(il, rl);
+            } else {
+                *reinterpret_cast<float2*>(p.hi + o0) = make_float2(rh, ih);
+                *reinterpret_cast<float2*>(p.lo + o0) = make_float2(rl, il);
+            }
         }
+        if (turn) __syncthreads();
     }
 }
 
@@ -250,15 +335,6 @@ struct EpiArgs {
     int o_pd;
     long long o_sp1, o_sp2, o_sq, o_sbi, o_sbo;
 };
-
-// Round a float to TF32 (10 mantissa bits, to nearest, ties to even) with
-// integer operations; inf/nan unchanged.
-__device__ __forceinline__ float tf32_rne(float x) {
-    uint32_t u = __float_as_uint(x);
-    if ((u & 0x7F800000u) == 0x7F800000u) return x;
-    u += 0xFFFu + ((u >> 13) & 1u);
-    return __uint_as_float(u & 0xFFFFE000u);
-}
 
 // (hi + lo) as a float-float sum -> TF32 pair (th, tl) with
 // |hi + lo - th - tl| <~ 2^-22 |hi + lo|, FP32 and integer operations only.
@@ -793,12 +869,32 @@ SplitPackArgs side_pack_args(const GemmArgs& g, const Plan& pl, int side, float*
 }  // namespace
 
 // ------------------------------------------------------------- public API
-int split_pack(const SplitPackArgs& p, cudaStream_t stream) {
-    const long long total = (long long)p.Rpad * p.Kc * p.Bi * p.Bo;
-    if (total <= 0) return 0;
-    const long long grid = std::min<long long>((total + 255) / 256, 152LL * 16);
-    pack_kernel<<<(unsigned)grid, 256, 0, stream>>>(p);
-    return 1;
+int split_pack(const SplitPackArgs* p, int n, cudaStream_t stream) {
+    int launches = 0;
+    for (int i = 0; i < n;) {
+        PackJobs jobs;
+        int nj = 0;
+        jobs.first[0] = 0;
+        for (; i < n && nj < PK_JOBS; ++i) {
+            const long long rows = (long long)p[i].Rpad * p[i].Bi * p[i].Bo;
+            if (rows <= 0 || p[i].Kc <= 0) continue;
+            // K tiles per block: as many as leave a few blocks per SM
+            const int kt = (p[i].Kc + 31) / 32;
+            const long long rb = (rows + PK_ROWS - 1) / PK_ROWS;
+            int per = 1;
+            while (per < 8 && rb * ((kt + 2 * per - 1) / (2 * per)) >= 4LL * num_sms()) per *= 2;
+            jobs.p[nj] = p[i];
+            jobs.rb[nj] = (int)rb;
+            jobs.ktiles[nj] = per;
+            jobs.first[nj + 1] = jobs.first[nj] + (int)(rb * ((kt + per - 1) / per));
+            ++nj;
+        }
+        if (nj == 0) break;
+        for (int j = nj; j < PK_JOBS; ++j) jobs.first[j + 1] = jobs.first[nj];   // never selected
+        pack_kernel<<<(unsigned)jobs.first[nj], PK_THREADS, 0, stream>>>(jobs);
+        ++launches;
+    }
+    return launches;
 }
 
 size_t split_mma_partials(const SplitMma& m) {
@@ -893,9 +989,8 @@ int launch_split_pack(const GemmArgs& g, cudaStream_t stream, void* workspace, s
     float* Pl = Ph + pl.pe;
     float* Qh = Pl + pl.pe;
     float* Ql = Qh + pl.qe;
-    int n = split_pack(side_pack_args(g, pl, 0, Ph, Pl), stream);
-    n += split_pack(side_pack_args(g, pl, 1, Qh, Ql), stream);
-    return n;
+    const SplitPackArgs both[2] = {side_pack_args(g, pl, 0, Ph, Pl), side_pack_args(g, pl, 1, Qh, Ql)};
+    return split_pack(both, 2, stream);
 }
 
 // Phase 2: the tcgen05 GEMM on the packed operands of the same GemmArgs.

@@ -718,6 +718,7 @@ bool split_heff_prepare(ttn_ctx* c, SplitHeff& S, const int* d, cplx* const* hb,
             P.Xl = P.Xh + xe;
         }
     }
+    std::vector<SplitPackArgs> jobs;   // every operand of the visit, packed together
     // operator stacks Q_u = [H_block(u) | n stacks of the pairs with a = u]
     auto pack_ops = [&](SplitHeff::Leg& L, const cplx* src, int nmat, long long k_off_c, int Kc_write) {
         SplitPackArgs a;
@@ -737,7 +738,7 @@ bool split_heff_prepare(ttn_ctx* c, SplitHeff& S, const int* d, cplx* const* hb,
         a.k_off = 2 * k_off_c;
         a.hi = L.Qh;
         a.lo = L.Ql;
-        c->stats[3] += split_pack(a, c->stream);
+        jobs.push_back(a);
     };
     for (int u = 0; u < 3; ++u) {
         SplitHeff::Leg& L = S.leg[u];
@@ -770,7 +771,11 @@ bool split_heff_prepare(ttn_ctx* c, SplitHeff& S, const int* d, cplx* const* hb,
         a.pitch = P.Kz;
         a.hi = P.Gh;
         a.lo = P.Gl;
-        c->stats[3] += split_pack(a, c->stream);
+        jobs.push_back(a);
+    }
+    {
+        ProfScope ps(c, PK_PACK, 0.0, 0.0);
+        c->stats[3] += split_pack(jobs.data(), (int)jobs.size(), c->stream);
     }
     S.ok = true;
     return true;
@@ -785,11 +790,15 @@ int* split_flag(ttn_ctx* c) {
 void split_heff_apply(ttn_ctx* c, const SplitHeff& S, const cplx* x, cplx* y) {
     const int d0 = S.d[0], d1 = S.d[1], d2 = S.d[2];
     int* flag = split_flag(c);
-    // 1. X into slot 0 of every stacked operand
+    // 1. X into slot 0 of every stacked operand, and once more with leg a's index
+    // fastest for the transposed pairs
+    SplitPackArgs jobs[6];
+    int nj = 0;
+    double pack_bytes = 0.0;
     for (int u = 0; u < 3; ++u) {
         const SplitHeff::Leg& L = S.leg[u];
         if (!L.on) continue;
-        SplitPackArgs a;
+        SplitPackArgs& a = jobs[nj++];
         std::memset(&a, 0, sizeof(a));
         a.src = x;
         a.Ko = 1;
@@ -806,8 +815,36 @@ void split_heff_apply(ttn_ctx* c, const SplitHeff& S, const cplx* x, cplx* y) {
         a.pitch = L.Kp;
         a.hi = L.Ph;
         a.lo = L.Pl;
-        ProfScope ps(c, PK_PACK, 0.0, (double)a.R * a.Bi * L.d * 32.0);
-        c->stats[3] += split_pack(a, c->stream);
+        pack_bytes += (double)a.R * a.Bi * L.d * 32.0;
+    }
+    for (int p = 0; p < S.np; ++p) {
+        const SplitHeff::PairPlan& P = S.pp[p];
+        if (!P.trans) continue;
+        const int b = P.b;
+        // X with leg a's index fastest: rows (x fastest, then y), K = leg b
+        SplitPackArgs& xa = jobs[nj++];
+        std::memset(&xa, 0, sizeof(xa));
+        xa.src = x;
+        xa.Ko = 1;
+        xa.Bo = 1;
+        if (b == 0) {          // (a, b) = (2, 0): rows c + d2 b'
+            xa.R = d2; xa.s_r = (long long)d0 * d1; xa.Bi = d1; xa.s_bi = d0; xa.Ki = d0; xa.s_ki = 1;
+        } else if (b == 1) {   // (2, 1): rows c + d2 a
+            xa.R = d2; xa.s_r = (long long)d0 * d1; xa.Bi = d0; xa.s_bi = 1; xa.Ki = d1; xa.s_ki = d0;
+        } else {               // (1, 2): rows b + d1 a
+            xa.R = d1; xa.s_r = d0; xa.Bi = d0; xa.s_bi = 1; xa.Ki = d2; xa.s_ki = (long long)d0 * d1;
+        }
+        xa.Rpad = xa.R;
+        xa.rb_i = xa.R;
+        xa.Kc = S.d[b];
+        xa.pitch = P.Kz;
+        xa.hi = P.Xh;
+        xa.lo = P.Xl;
+        pack_bytes += (double)xa.R * xa.Bi * S.d[b] * 32.0;
+    }
+    {
+        ProfScope ps(c, PK_PACK, 0.0, pack_bytes);
+        c->stats[3] += split_pack(jobs, nj, c->stream);
     }
     // 2. channel intermediates Z_i = G_i x_b X, written into the K slots of P_a
     const int BIG = 1 << 30;
@@ -832,29 +869,6 @@ void split_heff_apply(ttn_ctx* c, const SplitHeff& S, const cplx* x, cplx* y) {
         o.pd = BIG;
         o.sp1 = 1;
         if (P.trans) {
-            // X with leg a's index fastest: rows (x fastest, then y), K = leg b
-            SplitPackArgs xa;
-            std::memset(&xa, 0, sizeof(xa));
-            xa.src = x;
-            xa.Ko = 1;
-            xa.Bo = 1;
-            if (b == 0) {          // (a, b) = (2, 0): rows c + d2 b'
-                xa.R = d2; xa.s_r = (long long)d0 * d1; xa.Bi = d1; xa.s_bi = d0; xa.Ki = d0; xa.s_ki = 1;
-            } else if (b == 1) {   // (2, 1): rows c + d2 a
-                xa.R = d2; xa.s_r = (long long)d0 * d1; xa.Bi = d0; xa.s_bi = 1; xa.Ki = d1; xa.s_ki = d0;
-            } else {               // (1, 2): rows b + d1 a
-                xa.R = d1; xa.s_r = d0; xa.Bi = d0; xa.s_bi = 1; xa.Ki = d2; xa.s_ki = (long long)d0 * d1;
-            }
-            xa.Rpad = xa.R;
-            xa.rb_i = xa.R;
-            xa.Kc = S.d[b];
-            xa.pitch = P.Kz;
-            xa.hi = P.Xh;
-            xa.lo = P.Xl;
-            {
-                ProfScope ps(c, PK_PACK, 0.0, (double)xa.R * xa.Bi * S.d[b] * 32.0);
-                c->stats[3] += split_pack(xa, c->stream);
-            }
             m.Ph = P.Xh; m.Pl = P.Xl; m.P_rows = P.XPp; m.P_pitch = P.Kz;
             m.Pn = P.Xrows; m.Pp = P.XPp;
             m.Bi = P.r; m.Bo = 1; m.q_sbi = P.Qrows;
@@ -1114,22 +1128,30 @@ bool renorm_stack_split(ttn_ctx* c, const cplx* X, const int* d, int u, int o, c
     grow_zeroed(c, c->shP[0], c->shP_cap[0], 2 * pe * sizeof(float));
     float *Xh = c->shX[0], *Xl = Xh + xe, *Oh = c->shG[0], *Ol = Oh + oe, *Ch = c->shQ[0], *Cl = Ch + ce,
           *Ph = c->shP[0], *Pl = Ph + pe;
-    SplitPackArgs a;
-    // X with rows w + dw * o-index, K = u-index
-    std::memset(&a, 0, sizeof(a));
-    a.src = X; a.R = dw; a.s_r = st[w]; a.Bi = dO; a.s_bi = st[o]; a.rb_i = dw; a.Bo = 1;
-    a.Ki = du; a.s_ki = st[u]; a.Ko = 1; a.Rpad = dw; a.Kc = Kz / 2; a.pitch = Kz; a.hi = Xh; a.lo = Xl;
-    c->stats[3] += split_pack(a, c->stream);
-    // op stack, embedded: rows = new u-index, K = old u-index, one padded block per op
-    std::memset(&a, 0, sizeof(a));
-    a.src = ops; a.R = du; a.s_r = 1; a.Ki = du; a.s_ki = du; a.Ko = 1; a.Bi = nop; a.s_bi = DDu; a.Bo = 1;
-    a.rb_i = Qrows_u; a.embed = 1; a.Rpad = Qrows_u / 2; a.Kc = Kz / 2; a.pitch = Kz; a.hi = Oh; a.lo = Ol;
-    c->stats[3] += split_pack(a, c->stream);
-    // X^H, embedded: rows = o-index, K = w + dw * u
-    std::memset(&a, 0, sizeof(a));
-    a.src = X; a.R = dO; a.s_r = st[o]; a.Ki = dw; a.s_ki = st[w]; a.Ko = du; a.s_ko = st[u]; a.Bi = a.Bo = 1;
-    a.conj = 1; a.embed = 1; a.Rpad = Qrows_o / 2; a.Kc = Kp / 2; a.pitch = Kp; a.hi = Ch; a.lo = Cl;
-    c->stats[3] += split_pack(a, c->stream);
+    SplitPackArgs jobs[3];
+    std::memset(jobs, 0, sizeof(jobs));
+    {
+        // X with rows w + dw * o-index, K = u-index
+        SplitPackArgs& a = jobs[0];
+        a.src = X; a.R = dw; a.s_r = st[w]; a.Bi = dO; a.s_bi = st[o]; a.rb_i = dw; a.Bo = 1;
+        a.Ki = du; a.s_ki = st[u]; a.Ko = 1; a.Rpad = dw; a.Kc = Kz / 2; a.pitch = Kz; a.hi = Xh; a.lo = Xl;
+    }
+    {
+        // op stack, embedded: rows = new u-index, K = old u-index, one padded block per op
+        SplitPackArgs& a = jobs[1];
+        a.src = ops; a.R = du; a.s_r = 1; a.Ki = du; a.s_ki = du; a.Ko = 1; a.Bi = nop; a.s_bi = DDu; a.Bo = 1;
+        a.rb_i = Qrows_u; a.embed = 1; a.Rpad = Qrows_u / 2; a.Kc = Kz / 2; a.pitch = Kz; a.hi = Oh; a.lo = Ol;
+    }
+    {
+        // X^H, embedded: rows = o-index, K = w + dw * u
+        SplitPackArgs& a = jobs[2];
+        a.src = X; a.R = dO; a.s_r = st[o]; a.Ki = dw; a.s_ki = st[w]; a.Ko = du; a.s_ko = st[u]; a.Bi = a.Bo = 1;
+        a.conj = 1; a.embed = 1; a.Rpad = Qrows_o / 2; a.Kc = Kp / 2; a.pitch = Kp; a.hi = Ch; a.lo = Cl;
+    }
+    {
+        ProfScope ps(c, PK_PACK, 0.0, 32.0 * (2.0 * s + (double)nop * DDu));
+        c->stats[3] += split_pack(jobs, 3, c->stream);
+    }
     int* flag = split_flag(c);
     for (int i0 = 0; i0 < nop; i0 += chunk) {
         const int nb = std::min(chunk, nop - i0);
