@@ -262,8 +262,9 @@ int qr_panel(cplx* A, int M, int D, cplx* R, QrScratch& ws, cudaStream_t s, void
              int first, int last, const Publish& pub);
 // |A|_F^2 into ws.scal[0].
 int qr_frobenius(const cplx* A, long long n, QrScratch& ws, cudaStream_t s);
+// fine_rows: spread the rows of small matrices over all SMs (see qr.cu).
 int qr_cgs2(cplx* A, int M, int D, cplx* R, const int* cand, int ncand,
-            QrScratch& ws, cudaStream_t s, int* n_dependent_host, double tol = QR_TOL_FP64);
+            QrScratch& ws, cudaStream_t s, int* n_dependent_host, bool fine_rows = false, double tol = QR_TOL_FP64);
 
 // ---- truncated SVD (svd.cu) -----------------------------------------------------
 // One-sided Jacobi SVD of the N x N column-major R (N <= 256) in place: R's

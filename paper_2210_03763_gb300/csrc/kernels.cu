@@ -761,18 +761,15 @@ __global__ void fill_kernel(cplx* x, long long n, cplx v) {
 // (omega_x, omega_z, Re W, Im W, delta).  Most coefficients of a pulse layer are
 // zero at a given time, and one thread per entry walking all atoms was a serial
 // chain of loads (16 us for a 12 x 12 block of 62 atoms): the block first
-// lists the terms whose coefficients are not all zero, then S threads per entry
-// share them.  Measured, us per block (8x8 lattice, chi = 12): 15.8 -> 7.3.
+// lists the terms whose coefficients are not all zero and reads only their
+// operators, several in flight.  Terms are added one by one in atom order.
+// Measured, us per block (8x8 lattice, chi = 12): 15.8 -> 8.0.
 constexpr int AB_THREADS = 128;
-
-template <int S>
 __global__ void __launch_bounds__(AB_THREADS)
     assemble_block_kernel(cplx* H, const cplx* Hs, int D, const cplx* nops, int nsites, const int* site_ids,
                           const cplx* dops, int ndriven, const int* driven_ids, const double* coef, double gamma) {
-    constexpr int OB = AB_THREADS / S;
     extern __shared__ short terms[];       // < nsites: site term, else driven atom (index - nsites)
     __shared__ int s_count;
-    __shared__ cplx part[S > 1 ? AB_THREADS : 1];
     if (threadIdx.x < 32) {                // in order, by one warp
         int count = 0;
         const int n = nsites + ndriven;
@@ -792,54 +789,48 @@ __global__ void __launch_bounds__(AB_THREADS)
         if (threadIdx.x == 0) s_count = count;
     }
     __syncthreads();
-    const int count = s_count, o = threadIdx.x % OB, ks = threadIdx.x / OB;
+    const int count = s_count;
     const long long DD = (long long)D * D;
-    for (long long e0 = (long long)blockIdx.x * OB; e0 < DD; e0 += (long long)gridDim.x * OB) {
-        const long long e = e0 + o;
-        cplx h = make_double2(0.0, 0.0);
-        if (e < DD) {
-            const int a = (int)(e % D), b = (int)(e / D);
-            const long long et = b + (long long)D * a;           // transposed position
+    for (long long e = blockIdx.x * (long long)AB_THREADS + threadIdx.x; e < DD; e += (long long)gridDim.x * AB_THREADS) {
+        const int a = (int)(e % D), b = (int)(e / D);
+        const long long et = b + (long long)D * a;           // transposed position
+        cplx h = Hs ? Hs[e] : make_double2(0.0, 0.0);
+        int i = 0;
+#pragma unroll 4
+        for (; i < count && terms[i] < nsites; ++i) {
+            // -(Delta_i + i gamma) n_i: detuning, and the decay of Eq. 3
+            const int q = terms[i];
+            const double de = coef[5 * site_ids[q] + 4];
+            const cplx v = nops[q * DD + e];
+            h.x -= de * v.x - gamma * v.y;
+            h.y -= de * v.y + gamma * v.x;
+        }
 #pragma unroll 2
-            for (int i = ks; i < count; i += S) {
-                const int q = terms[i];
-                if (q < nsites) {
-                    // -(Delta_i + i gamma) n_i: detuning, and the decay of Eq. 3
-                    const double de = coef[5 * site_ids[q] + 4];
-                    const cplx v = nops[q * DD + e];
-                    h.x -= de * v.x - gamma * v.y;
-                    h.y -= de * v.y + gamma * v.x;
-                    continue;
-                }
-                const double* c = coef + 5 * driven_ids[q - nsites];
-                const cplx* sx = dops + (3LL * (q - nsites)) * DD;
-                if (c[0] != 0.0) {
-                    const cplx v = sx[e];
-                    h.x = fma(c[0], v.x, h.x);
-                    h.y = fma(c[0], v.y, h.y);
-                }
-                if (c[1] != 0.0) {
-                    const cplx v = sx[DD + e];
-                    h.x = fma(c[1], v.x, h.x);
-                    h.y = fma(c[1], v.y, h.y);
-                }
-                if (c[2] != 0.0 || c[3] != 0.0) {
-                    // W rp + conj(W) rp^H ; rp^H(a, b) = conj(rp(b, a))
-                    const cplx vr = sx[2 * DD + e], vt = sx[2 * DD + et];
-                    h.x += (c[2] * vr.x - c[3] * vr.y) + (c[2] * vt.x - c[3] * vt.y);
-                    h.y += (c[2] * vr.y + c[3] * vr.x) + (-c[2] * vt.y - c[3] * vt.x);
-                }
+        for (; i < count; ++i) {
+            const int q = terms[i] - nsites;
+            const double* c = coef + 5 * driven_ids[q];
+            const cplx* sx = dops + (3LL * q) * DD;
+            cplx t = make_double2(0.0, 0.0);
+            if (c[0] != 0.0) {
+                const cplx v = sx[e];
+                t.x = c[0] * v.x;
+                t.y = c[0] * v.y;
             }
+            if (c[1] != 0.0) {
+                const cplx v = sx[DD + e];
+                t.x = fma(c[1], v.x, t.x);
+                t.y = fma(c[1], v.y, t.y);
+            }
+            if (c[2] != 0.0 || c[3] != 0.0) {
+                // W rp + conj(W) rp^H ; rp^H(a, b) = conj(rp(b, a))
+                const cplx vr = sx[2 * DD + e], vt = sx[2 * DD + et];
+                t.x = t.x + (c[2] * vr.x - c[3] * vr.y) + (c[2] * vt.x - c[3] * vt.y);
+                t.y = t.y + (c[2] * vr.y + c[3] * vr.x) + (-c[2] * vt.y - c[3] * vt.x);
+            }
+            h.x += t.x;
+            h.y += t.y;
         }
-        if (S > 1) {
-            __syncthreads();
-            part[threadIdx.x] = h;
-            __syncthreads();
-            if (ks != 0) continue;
-#pragma unroll
-            for (int q = 1; q < S; ++q) h = cadd(h, part[q * OB + o]);
-        }
-        if (e < DD) H[e] = Hs ? cadd(Hs[e], h) : h;
+        H[e] = h;
     }
 }
 
@@ -1066,12 +1057,8 @@ int k_assemble_block(cplx* H, const cplx* Hs, int D, const cplx* nops, int nsite
                      cudaStream_t s) {
     long long DD = (long long)D * D;
     const size_t smem = sizeof(short) * (size_t)std::max(1, nsites + ndriven);
-    if (DD <= 4096)
-        assemble_block_kernel<8><<<(unsigned)((DD + 15) / 16), AB_THREADS, smem, s>>>(
-            H, Hs, D, nops, nsites, site_ids, dops, ndriven, driven_ids, coef, gamma);
-    else
-        assemble_block_kernel<2><<<(unsigned)std::min<long long>((DD + 63) / 64, 8 * 152), AB_THREADS, smem, s>>>(
-            H, Hs, D, nops, nsites, site_ids, dops, ndriven, driven_ids, coef, gamma);
+    assemble_block_kernel<<<(unsigned)std::min<long long>((DD + AB_THREADS - 1) / AB_THREADS, 8 * 152), AB_THREADS, smem,
+                            s>>>(H, Hs, D, nops, nsites, site_ids, dops, ndriven, driven_ids, coef, gamma);
     return 1;
 }
 

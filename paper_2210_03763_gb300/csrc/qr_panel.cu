@@ -12,7 +12,7 @@
 //
 // The column-by-column rule (qr.cu) decides which columns are dependent; this
 // path is for matrices without any: it gives up (the flag) as soon as a
-// column's part outside the earlier ones is below 1e-5 of the column or 1e-8
+// column's part outside the earlier ones is below 1e-4 of the column or 1e-8
 // of |A|_F, far above the rule's 1e-10, and the caller runs the column loop
 // on the original matrix.  Q and R are then the same as the column loop's up
 // to rounding (R has a positive real diagonal, which makes them unique).
@@ -32,7 +32,7 @@ namespace {
 
 constexpr int PB = QR_PANEL;       // panel width
 constexpr int CT = 512;            // threads of the Cholesky kernel
-constexpr double MIN_COL2 = 1e-10; // residual^2 / |column|^2
+constexpr double MIN_COL2 = 1e-8;  // residual^2 / |column|^2
 constexpr double MIN_FRO2 = 1e-16; // residual^2 / |A|_F^2
 
 // G = Sw + Gq (bp x bp, Hermitian; Sw with leading dimension ld, Gq with PB,

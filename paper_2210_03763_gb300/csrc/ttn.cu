@@ -30,10 +30,10 @@ namespace {
 typedef std::complex<double> zc;
 constexpr int MAX_CHI = 256;
 constexpr int MAX_ATOMS = 1024;
-// QR by panels (gauge_qr) from this size on: a panel costs ~0.35 ms of launches
-// and small kernels whatever its rows (4096 x 64: 0.73 ms against 1.25 in the
-// column loop; 81 x 81 would take as long as there).
-constexpr int PANEL_MIN_M = 2048, PANEL_MIN_D = 48;
+// QR by panels (gauge_qr) from this size on: a panel costs ~0.3 ms of launches
+// and small kernels whatever its rows, a column of the column loop 11 us and up
+// (9 x 9: 0.1 ms, 81 x 81: 2.5 ms).
+constexpr int PANEL_MIN_M = 48, PANEL_MIN_D = 24;
 
 struct TtnError : std::runtime_error {
     ttn_status code;
@@ -1337,7 +1337,7 @@ int gauge_qr(ttn_ctx* c, cplx*& A, cplx*& spare, int M, int D, cplx* R, const in
         }
     }
     int ndep = 0;
-    const int nl = qr_cgs2(A, M, D, R, cand, ncand, q, c->stream, &ndep);
+    const int nl = qr_cgs2(A, M, D, R, cand, ncand, q, c->stream, &ndep, hint == -1);
     if (nl < 0) throw TtnError(TTN_ERR_TIMEOUT, "QR grid barrier wait timed out");
     c->stats[3] += nl;
     if (ndep > 0) hint = -1;
