@@ -269,25 +269,19 @@ struct DigitGemm {
     int* err;
 };
 
-// 64-byte swizzle, K-major, 8-row groups 512 bytes apart.
-__device__ __forceinline__ uint64_t sdesc64(uint32_t addr) {
-    uint64_t d = 0;
-    d |= (uint64_t)((addr & 0x3FFFF) >> 4);
-    d |= (uint64_t)1 << 16;
-    d |= (uint64_t)(512 >> 4) << 32;
-    d |= (uint64_t)1 << 46;
-    d |= (uint64_t)4 << 61;
-    return d;
-}
+// 64-byte swizzle, K-major, 8-row groups 512 bytes apart; the address (lower
+// word) varies.
+constexpr uint32_t DESC_HI = (512u >> 4) | (1u << 14) | (4u << 29);
+__device__ __forceinline__ uint32_t desc_lo(uint32_t addr) { return ((addr & 0x3FFFF) >> 4) | (1u << 16); }
 
 // D = F32, A = B = BF16, K-major, M = 128, N = 64.
 constexpr uint32_t IDESC = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(BN >> 3) << 17) | ((uint32_t)(BM >> 4) << 24);
 
-__device__ __forceinline__ void mma_bf16(uint32_t dt, uint64_t a, uint64_t b, uint32_t acc) {
+__device__ __forceinline__ void mma_bf16(uint32_t dt, uint32_t a, uint32_t b, uint32_t acc) {
     asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(
-            dt),
-        "l"(a), "l"(b), "r"(IDESC), "r"(acc));
+        "{\n .reg .pred p;\n .reg .b64 da, db;\n setp.ne.b32 p, %4, 0;\n mov.b64 da, {%1, %5};\n mov.b64 db, {%2, %5};\n"
+        " tcgen05.mma.cta_group::1.kind::f16 [%0], da, db, %3, p;\n}\n" ::"r"(dt),
+        "r"(a), "r"(b), "r"(IDESC), "r"(acc), "r"(DESC_HI));
 }
 
 __device__ __forceinline__ void tma_load_3d(void* dst, const CUtensorMap* map, uint64_t* bar, int x, int y, int z) {
@@ -451,52 +445,57 @@ __global__ void __launch_bounds__(THREADS, 1)
         }
         __syncwarp();
     } else if (warp == MMA_WARP) {
-        if (lane == 0) {
-            unsigned it = 0, cg = 0;
-            bool ok = true;
-            for (long long t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-                const int ks = (int)(t / (grid_tiles * ea.batches));
-                const int st1 = min(ea.nst, (ks + 1) * ea.cps * CHUNK_ST);
-                for (int c0 = ks * ea.cps * CHUNK_ST; c0 < st1 && ok; c0 += CHUNK_ST, ++cg) {
-                    const int c1 = min(st1, c0 + CHUNK_ST);
-                    for (int st = c0; st < c1 && ok; ++st, ++it) {
-                        const unsigned s = it % STAGES, round = it / STAGES;
-                        if (!mbar_wait(&full[s], round & 1, ea.err)) {
-                            ok = false;
-                            break;
-                        }
-                        asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-                        const uint32_t base = smem_u32(smem + s * STAGE_BYTES);
-                        const uint64_t dp = sdesc64(base), dq = sdesc64(base + P_BYTES);
-                        // unrolled: the descriptors are then immediate offsets (a loop over the digits
-                        // took 110 clk per MMA to issue, the MMA 32 to 48)
+        // the whole warp walks the loop, one elected lane issues: unrolled, the
+        // descriptors are immediate offsets from uniform registers (a loop over the
+        // digits took 110 clk per MMA to issue, unrolled in one lane's branch 70; the
+        // MMA takes 32 to 48).  Uniform: 128 x 128 x 16384 204 -> 187 us, 4096 x 64 x 64
+        // in batches of 4 61 -> 55 us.
+        const uint32_t lo0 = desc_lo(smem_u32(smem));
+        unsigned it = 0, cg = 0;
+        bool ok = true;
+        for (long long t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
+            const int ks = (int)(t / (grid_tiles * ea.batches));
+            const int st1 = min(ea.nst, (ks + 1) * ea.cps * CHUNK_ST);
+            for (int c0 = ks * ea.cps * CHUNK_ST; c0 < st1 && ok; c0 += CHUNK_ST, ++cg) {
+                const int c1 = min(st1, c0 + CHUNK_ST);
+                for (int st = c0; st < c1 && ok; ++st, ++it) {
+                    const unsigned s = it % STAGES, round = it / STAGES;
+                    if (!__all_sync(0xffffffffu, mbar_wait(&full[s], round & 1, ea.err))) {
+                        ok = false;
+                        break;
+                    }
+                    asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    const uint32_t dp = lo0 + s * (STAGE_BYTES >> 4), dq = dp + (P_BYTES >> 4);
 #pragma unroll
-                        for (int l = 0; l < NLEV; ++l) {
-                            if (!ok) break;
-                            if (st == c0 && cg > 0) {
-                                if (!mbar_wait(&lempty[l], (cg - 1) & 1, ea.err)) {
-                                    ok = false;
-                                    break;
-                                }
-                                asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                    for (int l = 0; l < NLEV; ++l) {
+                        if (!ok) break;
+                        if (st == c0 && cg > 0) {
+                            if (!__all_sync(0xffffffffu, mbar_wait(&lempty[l], (cg - 1) & 1, ea.err))) {
+                                ok = false;
+                                break;
                             }
-                            const int i0 = l > ND - 1 ? l - (ND - 1) : 0, i1 = l < ND - 1 ? l : ND - 1;
+                            asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
+                        }
+                        const int i0 = l > ND - 1 ? l - (ND - 1) : 0, i1 = l < ND - 1 ? l : ND - 1;
+                        if (elect_one()) {
 #pragma unroll
                             for (int i = i0; i <= i1; ++i) {
-                                const uint64_t a = dp + (uint64_t)(i * P_PLANE >> 4);
-                                const uint64_t q = dq + (uint64_t)((l - i) * Q_PLANE >> 4);
+                                const uint32_t a = dp + (i * P_PLANE >> 4), q = dq + ((l - i) * Q_PLANE >> 4);
                                 mma_bf16(tmem + l * BN, a, q, (st > c0 || i > i0) ? 1u : 0u);
                                 mma_bf16(tmem + l * BN, a + 2, q + 2, 1u);   // 16 bf16 = 32 bytes along K
                             }
                             if (st == c1 - 1) mma_commit(&lfull[l]);
                         }
-                        mma_commit(&empty[s]);
+                        __syncwarp();
                     }
+                    if (elect_one()) mma_commit(&empty[s]);
+                    __syncwarp();
                 }
             }
-            mma_commit(mdone);
-            mbar_drain(mdone, 0);
         }
+        if (elect_one()) mma_commit(mdone);
+        __syncwarp();
+        mbar_drain(mdone, 0);
         __syncwarp();
     } else {
         const int quad = warp & 3, col0 = (warp >> 2) * DCOLS;
