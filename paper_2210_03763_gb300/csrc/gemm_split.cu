@@ -351,6 +351,28 @@ __device__ __forceinline__ double f32_to_f64(float f) {
     return __longlong_as_double((long long)bits);
 }
 
+// hi + lo in double, rounded once, the same bits as
+// f32_to_f64(hi) + f32_to_f64(lo) without the FP64 pipe, which the epilogue of
+// a short K was bound by (a 128 x 128 tile of FP64 adds takes 9700 clocks per SM,
+// its products at K' = 256 6700).  s + e = hi + lo exactly (TwoSum); e counted in
+// units of s's last double bit is an integer of at most 2^28 after one rounding,
+// which ties to even as the sum does (s itself is even), and is added to s's bits.
+// Measured, 128 x 128 x 16384 outputs of K = 128 in batches of 50: 1140 -> 887 us.
+__device__ __forceinline__ double ff_to_f64(float hi, float lo) {
+    const float s = __fadd_rn(hi, lo), b = __fsub_rn(s, hi);
+    const float e = __fadd_rn(__fsub_rn(hi, __fsub_rn(s, b)), __fsub_rn(lo, b));
+    const uint32_t u = __float_as_uint(s), ex = (u >> 23) & 0xFFu;
+    if (ex - 64u > 180u || (u & 0x7FFFFFu) == 0u) {   // far exponents; powers of two (finer bits below s)
+        if ((u << 1) == 0u) return __hiloint2double((int)u, 0);
+        return f32_to_f64(hi) + f32_to_f64(lo);
+    }
+    int d = __float2int_rn(e * __uint_as_float((127u + 52u + 127u - ex) << 23));
+    if ((int)u < 0) d = -d;
+    const uint32_t top = (u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + ((1023u - 127u) << 20));
+    const unsigned long long w = ((unsigned long long)top << 32 | (u << 29)) + (unsigned long long)(long long)d;
+    return __longlong_as_double((long long)w);
+}
+
 // Knuth's TwoSum, hi + lo += x, on two lanes at once with packed f32x2
 // arithmetic (round to nearest per lane, the same results as scalar FADDs in
 // half the instructions: the drain warps are issue-bound, and this cut the
@@ -595,35 +617,42 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
                     }
                     continue;
                 }
-                cplx* C = ea.C + bi * ea.c_bi + bo * ea.c_bo + (long long)(p % ea.c_pd) * ea.c_p +
-                          (long long)(p / ea.c_pd) * ea.c_p2;
+                cplx* C = Wt ? Wt + p
+                             : ea.C + bi * ea.c_bi + bo * ea.c_bo + (long long)(p % ea.c_pd) * ea.c_p +
+                                   (long long)(p / ea.c_pd) * ea.c_p2;
+                const long long c_q = Wt ? ea.Pn : ea.c_q;
+                int q = q0;
+                // groups of 4 outputs, the next ones moved down: the code stays short
+                // (a launch with a tile per block runs it cold, 16 bytes an instruction)
+#pragma unroll 1
+                for (int g = 0; g < DCOLS; g += 8) {
 #pragma unroll
-                for (int j = 0; j < DCOLS; j += 2) {
-                    const int q = (qt * BN + col0 + j) >> 1;       // complex row of Q
-                    if (q >= ea.Qn) continue;
-                    const double re = f32_to_f64(hi[j]) + f32_to_f64(lo[j]);
-                    const double im = f32_to_f64(hi[j + 1]) + f32_to_f64(lo[j + 1]);
-                    if (Wt) {
-                        Wt[p + (long long)q * ea.Pn] = make_double2(re, im);
-                        continue;
-                    }
-                    cplx* cp = C + q * ea.c_q;
-                    cplx r;
-                    if (ea.mode == 0) {                 // alpha = 1, beta = 0
-                        r = make_double2(re, im);
-                    } else if (ea.mode == 1) {          // alpha = 1, beta = 1
-                        cplx o = *cp;
-                        r = make_double2(o.x + re, o.y + im);
-                    } else {
-                        r.x = ea.alpha.x * re - ea.alpha.y * im;
-                        r.y = ea.alpha.x * im + ea.alpha.y * re;
-                        if (!beta0) {
-                            cplx o = *cp;
-                            r.x += ea.beta.x * o.x - ea.beta.y * o.y;
-                            r.y += ea.beta.x * o.y + ea.beta.y * o.x;
+                    for (int j = 0; j < 8; j += 2, ++q) {
+                        if (q >= ea.Qn) continue;
+                        const double re = ff_to_f64(hi[j], lo[j]), im = ff_to_f64(hi[j + 1], lo[j + 1]);
+                        cplx* cp = C + q * c_q;
+                        cplx r = make_double2(re, im);
+                        if (!Wt && ea.mode != 0) {
+                            if (ea.mode == 1) {                 // alpha = 1, beta = 1
+                                cplx o = *cp;
+                                r = make_double2(o.x + re, o.y + im);
+                            } else {
+                                r.x = ea.alpha.x * re - ea.alpha.y * im;
+                                r.y = ea.alpha.x * im + ea.alpha.y * re;
+                                if (!beta0) {
+                                    cplx o = *cp;
+                                    r.x += ea.beta.x * o.x - ea.beta.y * o.y;
+                                    r.y += ea.beta.x * o.y + ea.beta.y * o.x;
+                                }
+                            }
                         }
+                        *cp = r;
                     }
-                    *cp = r;
+#pragma unroll
+                    for (int j = 0; j + 8 < DCOLS; ++j) {
+                        hi[j] = hi[j + 8];
+                        lo[j] = lo[j + 8];
+                    }
                 }
             }
         }
