@@ -155,6 +155,7 @@ __device__ __forceinline__ uint32_t bf16_pair(float lo, float hi) {
 
 // Row exponents over blocks of K (long K only): exps zeroed before.
 __global__ void __launch_bounds__(PK_THREADS) digit_max_kernel(DigitSide sp, DigitSide sq, int nbp, int kb) {
+    pdl_begin();
     const DigitSide& s = (int)blockIdx.x < nbp ? sp : sq;
     const long long f0 = (long long)((int)blockIdx.x < nbp ? blockIdx.x : blockIdx.x - nbp) * PK_ROWS;
     __shared__ const cplx* base[PK_ROWS];
@@ -174,6 +175,7 @@ __global__ void __launch_bounds__(PK_THREADS) digit_max_kernel(DigitSide sp, Dig
 // and finds the exponents itself.
 __global__ void __launch_bounds__(PK_THREADS) digit_pack_kernel(DigitSide sp, DigitSide sq, int nbp, int kb,
                                                                int one_pass) {
+    pdl_begin();
     const bool isp = (int)blockIdx.x < nbp;
     const DigitSide& s = isp ? sp : sq;
     const long long f0 = (long long)(isp ? blockIdx.x : blockIdx.x - nbp) * PK_ROWS;
@@ -357,6 +359,7 @@ __device__ __noinline__ cplx plain_output(const GemmArgs& g, int m, int n, int b
 
 __global__ void __launch_bounds__(THREADS, 1)
     digit_gemm_kernel(const __grid_constant__ CUtensorMap mP, const __grid_constant__ CUtensorMap mQ, DigitGemm ea) {
+    pdl_wait();
     extern __shared__ __align__(1024) uint8_t smem_raw[];
     uint8_t* smem = (uint8_t*)(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     uint64_t* full = reinterpret_cast<uint64_t*>(smem + STAGES * STAGE_BYTES);
@@ -771,10 +774,10 @@ int launch_zgemm_digits(const GemmArgs& g, cudaStream_t stream, void* workspace,
     const dim3 grid(nbp + nbq, (Kc + kb - 1) / kb);
     if (!one) {
         if (cudaMemsetAsync(ws + pl.ep_off, 0, pl.p_off - pl.ep_off, stream) != cudaSuccess) return -1;
-        digit_max_kernel<<<grid, PK_THREADS, 0, stream>>>(sp, sq, nbp, kb);
+        launch(digit_max_kernel, grid, PK_THREADS, 0, stream, sp, sq, nbp, kb);
         ++launches;
     }
-    digit_pack_kernel<<<grid, PK_THREADS, 0, stream>>>(sp, sq, nbp, kb, one);
+    launch(digit_pack_kernel, grid, PK_THREADS, 0, stream, sp, sq, nbp, kb, one);
     ++launches;
     CUtensorMap mP, mQ;
     if (!make_map3(&mP, sp.planes, sp.rows, pl.Kp, BM) || !make_map3(&mQ, sq.planes, sq.rows, pl.Kp, BN)) return -1;
@@ -797,7 +800,7 @@ int launch_zgemm_digits(const GemmArgs& g, cudaStream_t stream, void* workspace,
     d.W = d.nsplit > 1 ? reinterpret_cast<cplx*>(ws + pl.w_off) : nullptr;
     d.err = reinterpret_cast<int*>(ws);
     const long long nt = (long long)d.n_ptiles * d.n_qtiles * d.batches * d.nsplit;
-    digit_gemm_kernel<<<(unsigned)std::min<long long>(nt, N_SM), THREADS, SMEM_BYTES, stream>>>(mP, mQ, d);
+    launch(digit_gemm_kernel, (unsigned)std::min<long long>(nt, N_SM), THREADS, SMEM_BYTES, stream, mP, mQ, d);
     ++launches;
     if (d.nsplit > 1) launches += launch_splitk_f64(g, d.nsplit, d.W, stream);
     return launches;

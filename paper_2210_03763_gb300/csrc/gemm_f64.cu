@@ -34,6 +34,7 @@ __device__ __forceinline__ cplx cmul_acc(cplx acc, cplx a, cplx b) {
 // batch-major, m fastest); a second kernel adds the ranges in fixed order.
 template <int BM, int BN>
 __global__ void __launch_bounds__(THREADS) zgemm_f64_kernel(GemmArgs g, int ks_len, cplx* W) {
+    pdl_begin();
     constexpr int TM = BM / 16, TN = BN / 16;
     // K slice per shared-memory stage: 8, or 32 for 16 x 16 tiles, whose small
     // outputs (9 x 9 blocks) otherwise spend a global-memory round trip on
@@ -152,6 +153,7 @@ __global__ void __launch_bounds__(THREADS) zgemm_f64_kernel(GemmArgs g, int ks_l
 
 // C = alpha sum_ks W[ks] + beta C in fixed order.
 __global__ void splitk_f64_kernel(GemmArgs g, int nsplit, const cplx* W) {
+    pdl_begin();
     const long long MN = (long long)g.M * g.N, nbatch = (long long)g.Bi * g.Bo, total = MN * nbatch;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
          e += (long long)gridDim.x * blockDim.x) {
@@ -191,6 +193,7 @@ constexpr int DIRECT_THREADS = 128;
 
 template <int S>
 __global__ void __launch_bounds__(DIRECT_THREADS) zgemm_f64_direct_kernel(GemmArgs g, int kc) {
+    pdl_begin();
     constexpr int OB = DIRECT_THREADS / S;   // outputs per block
     __shared__ cplx part[S > 1 ? DIRECT_THREADS : 1];
     const int o = threadIdx.x % OB, ks = threadIdx.x / OB;
@@ -256,7 +259,7 @@ template <int BM, int BN>
 void launch_tile(const GemmArgs& g, cudaStream_t stream, int nsplit, int ks_len, cplx* W) {
     long long batches = (long long)g.Bi * g.Bo;
     dim3 grid((g.N + BN - 1) / BN, (g.M + BM - 1) / BM, (unsigned)(batches * nsplit));
-    zgemm_f64_kernel<BM, BN><<<grid, THREADS, 0, stream>>>(g, nsplit > 1 ? ks_len : 0, W);
+    launch(zgemm_f64_kernel<BM, BN>, grid, THREADS, 0, stream, g, nsplit > 1 ? ks_len : 0, W);
 }
 
 // Tile width for one dimension: the widest of 16, 32, 64 whose padded size is
@@ -316,12 +319,12 @@ void launch_direct(const GemmArgs& g, cudaStream_t stream, int S, int kc) {
     const long long outs = (long long)g.M * g.N * g.Bi * (long long)g.Bo;
     const unsigned grid = (unsigned)((outs * S + DIRECT_THREADS - 1) / DIRECT_THREADS);
     switch (S) {
-        case 1: zgemm_f64_direct_kernel<1><<<grid, DIRECT_THREADS, 0, stream>>>(g, kc); break;
-        case 2: zgemm_f64_direct_kernel<2><<<grid, DIRECT_THREADS, 0, stream>>>(g, kc); break;
-        case 4: zgemm_f64_direct_kernel<4><<<grid, DIRECT_THREADS, 0, stream>>>(g, kc); break;
-        case 8: zgemm_f64_direct_kernel<8><<<grid, DIRECT_THREADS, 0, stream>>>(g, kc); break;
-        case 16: zgemm_f64_direct_kernel<16><<<grid, DIRECT_THREADS, 0, stream>>>(g, kc); break;
-        default: zgemm_f64_direct_kernel<32><<<grid, DIRECT_THREADS, 0, stream>>>(g, kc); break;
+        case 1: launch(zgemm_f64_direct_kernel<1>, grid, DIRECT_THREADS, 0, stream, g, kc); break;
+        case 2: launch(zgemm_f64_direct_kernel<2>, grid, DIRECT_THREADS, 0, stream, g, kc); break;
+        case 4: launch(zgemm_f64_direct_kernel<4>, grid, DIRECT_THREADS, 0, stream, g, kc); break;
+        case 8: launch(zgemm_f64_direct_kernel<8>, grid, DIRECT_THREADS, 0, stream, g, kc); break;
+        case 16: launch(zgemm_f64_direct_kernel<16>, grid, DIRECT_THREADS, 0, stream, g, kc); break;
+        default: launch(zgemm_f64_direct_kernel<32>, grid, DIRECT_THREADS, 0, stream, g, kc); break;
     }
 }
 
@@ -355,6 +358,6 @@ int launch_zgemm_f64(const GemmArgs& g, cudaStream_t stream, void* workspace, si
 int launch_splitk_f64(const GemmArgs& g, int nsplit, const cplx* W, cudaStream_t stream) {
     const long long total = (long long)g.M * g.N * g.Bi * g.Bo;
     const unsigned grid = (unsigned)std::min<long long>((total + 63) / 64, 152 * 16);   // small outputs: more SMs
-    splitk_f64_kernel<<<grid, 64, 0, stream>>>(g, nsplit, W);
+    launch(splitk_f64_kernel, grid, 64, 0, stream, g, nsplit, W);
     return 1;
 }

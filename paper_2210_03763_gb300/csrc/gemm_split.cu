@@ -188,6 +188,7 @@ struct PackJobs {   // several operands in one launch
     int ktiles[PK_JOBS];
 };
 __global__ void __launch_bounds__(PK_THREADS) pack_kernel(const __grid_constant__ PackJobs jobs) {
+    pdl_begin();
     int job = 0;
     while ((int)blockIdx.x >= jobs.first[job + 1]) ++job;
     const SplitPackArgs& p = jobs.p[job];
@@ -396,6 +397,7 @@ template <int BN_>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap mPh, const __grid_constant__ CUtensorMap mPl,
                    const __grid_constant__ CUtensorMap mQh, const __grid_constant__ CUtensorMap mQl, EpiArgs ea) {
+    pdl_wait();
     using T = TileCfg<BN_>;
     constexpr int BN = T::BN, STAGES = T::STAGES, B_TILE = T::B_TILE, STAGE_BYTES = T::STAGE_BYTES,
                   DCOLS = T::DCOLS;
@@ -667,6 +669,7 @@ __global__ void __launch_bounds__(GEMM_THREADS, 1)
 
 // C = alpha sum_ks W[ks] + beta C, summing the K ranges in increasing order.
 __global__ void splitk_reduce_kernel(EpiArgs ea) {
+    pdl_begin();
     const long long PQ = (long long)ea.Pn * ea.Qn, total = PQ * ea.batches;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
          e += (long long)gridDim.x * blockDim.x) {
@@ -923,7 +926,7 @@ int split_pack(const SplitPackArgs* p, int n, cudaStream_t stream) {
         }
         if (nj == 0) break;
         for (int j = nj; j < PK_JOBS; ++j) jobs.first[j + 1] = jobs.first[nj];   // never selected
-        pack_kernel<<<(unsigned)jobs.first[nj], PK_THREADS, 0, stream>>>(jobs);
+        launch(pack_kernel, (unsigned)jobs.first[nj], PK_THREADS, 0, stream, jobs);
         ++launches;
     }
     return launches;
@@ -994,13 +997,13 @@ int split_mma(const SplitMma& m, int* err_flag, void* partials, size_t partial_b
     const long long ntiles = (long long)ea.n_ptiles * ea.n_qtiles * ea.batches * sk.nsplit;
     const unsigned grid = (unsigned)std::min<long long>(ntiles, num_sms());
     if (bn == 128)
-        tc_gemm_kernel<128><<<grid, GEMM_THREADS, smem_bytes, stream>>>(mPh, mPl, mQh, mQl, ea);
+        launch(tc_gemm_kernel<128>, grid, GEMM_THREADS, smem_bytes, stream, mPh, mPl, mQh, mQl, ea);
     else
-        tc_gemm_kernel<64><<<grid, GEMM_THREADS, smem_bytes, stream>>>(mPh, mPl, mQh, mQl, ea);
+        launch(tc_gemm_kernel<64>, grid, GEMM_THREADS, smem_bytes, stream, mPh, mPl, mQh, mQl, ea);
     if (sk.nsplit == 1) return 1;
     const long long total = (long long)m.Pn * m.Qn * ea.batches;
     const unsigned rg = (unsigned)std::min<long long>((total + 255) / 256, (long long)num_sms() * 8);
-    splitk_reduce_kernel<<<rg, 256, 0, stream>>>(ea);
+    launch(splitk_reduce_kernel, rg, 256, 0, stream, ea);
     return 2;
 }
 

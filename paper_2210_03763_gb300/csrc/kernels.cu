@@ -165,6 +165,7 @@ __device__ void block_dots(const cplx* V, long long ld, int nv, const cplx* w, l
 
 __global__ void __launch_bounds__(T) dots_kernel(const cplx* V, long long ld, int nv, const cplx* w, long long n, int G,
                                                  cplx* partial) {
+    pdl_begin();
     __shared__ DotSmem sm;
     long long lo, hi;
     chunk_of(n, G, lo, hi);
@@ -175,6 +176,7 @@ __global__ void __launch_bounds__(T) dots_kernel(const cplx* V, long long ld, in
 // (stored to h_out), w -= sum_i V_i h_i, partial dots of the new w.
 __global__ void __launch_bounds__(T) orth_first_kernel(const cplx* V, long long ld, int nv, const cplx* partial_in,
                                                        cplx* w, long long n, int G, cplx* partial_dots, cplx* h_out) {
+    pdl_begin();
     __shared__ cplx sh_h[KRYLOV_MMAX + 1];
     __shared__ DotSmem sm;
     reduce_partials_to_shared(partial_in, nv, G, sh_h);
@@ -199,6 +201,7 @@ __global__ void __launch_bounds__(T) orth_first_kernel(const cplx* V, long long 
 __global__ void __launch_bounds__(T) lanczos_first_kernel(const cplx* V, long long ld, int j, const cplx* partial_in,
                                                           const KrylovScalars* ks, cplx* w, long long n, int G,
                                                           cplx* partial_dots, cplx* h_out) {
+    pdl_begin();
     __shared__ cplx sh_h[1];
     __shared__ DotSmem sm;
     reduce_partials_to_shared(partial_in, 1, G, sh_h);
@@ -239,6 +242,7 @@ __global__ void __launch_bounds__(T) orth_second_kernel(const cplx* V, long long
                                                         cplx* w, long long n, int G, double* partial_norm,
                                                         KrylovScalars* ks, const cplx* h1, double zr, double zi,
                                                         double tol, int arnoldi, Publish pub) {
+    pdl_begin();
     __shared__ cplx sh_h[KRYLOV_MMAX + 1];
     __shared__ double shd[T / 32];
     __shared__ int last;
@@ -265,6 +269,7 @@ __global__ void __launch_bounds__(T) orth_second_kernel(const cplx* V, long long
 }
 
 __global__ void norm2_partial_kernel(const cplx* x, long long n, int G, double* partial) {
+    pdl_begin();
     __shared__ double shd[T / 32];
     long long lo, hi;
     chunk_of(n, G, lo, hi);
@@ -275,6 +280,7 @@ __global__ void norm2_partial_kernel(const cplx* x, long long n, int G, double* 
 }
 
 __global__ void scale_copy_kernel(const cplx* x, long long n, const double* scale, cplx* y) {
+    pdl_begin();
     double f = scale[0];
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
          e += (long long)gridDim.x * blockDim.x) {
@@ -286,6 +292,7 @@ __global__ void scale_copy_kernel(const cplx* x, long long n, const double* scal
 // x <- x * sqrt(sum(pr) / sum(px)): rescale x to the norm given by the
 // partial sums pr (each block sums both partial lists in the same order).
 __global__ void rescale_to_norm_kernel(cplx* x, long long n, const double* px, int Gx, const double* pr, int Gr) {
+    pdl_begin();
     __shared__ double f;
     if (threadIdx.x < 32) {
         const double a = reduce_norm_partials(px, Gx), b = reduce_norm_partials(pr, Gr);
@@ -302,6 +309,7 @@ __global__ void rescale_to_norm_kernel(cplx* x, long long n, const double* px, i
 
 __global__ void combine_kernel(const cplx* V, long long ld, int nv, const KrylovScalars* ks, cplx* y,
                                long long n) {
+    pdl_begin();
     __shared__ cplx c[KRYLOV_MMAX];
     if (threadIdx.x < nv) {
         cplx ci = ks->c[nv - 1][threadIdx.x];
@@ -390,6 +398,7 @@ __device__ void tridiag_expm_warp(const double* a, const double* b, int m, doubl
 // |x|^2; the last block to finish sets the start scalars.
 __global__ void __launch_bounds__(T) krylov_start_kernel(KrylovScalars* ks, const cplx* x, long long n, int G,
                                                          double* partial, unsigned* arrived) {
+    pdl_begin();
     __shared__ double shd[T / 32];
     __shared__ int last;
     long long lo, hi;
@@ -574,6 +583,7 @@ __device__ cplx small_heff(int xr, int yc, int d0, int d1, int d2, const cplx* h
 __global__ void __cluster_dims__(SK_CL, 1, 1) __launch_bounds__(SK_THREADS)
     small_krylov_kernel(int d0, int d1, int d2, const cplx* hb0, const cplx* hb1, const cplx* hb2, SmallPairs pp,
                         cplx* x, double zr, double zi, double tol, int mmax, int arnoldi, Publish pub) {
+    pdl_begin();
     namespace cg = cooperative_groups;
     cg::cluster_group cl = cg::this_cluster();
     extern __shared__ cplx smem_c[];
@@ -732,6 +742,7 @@ __global__ void __cluster_dims__(SK_CL, 1, 1) __launch_bounds__(SK_THREADS)
 
 __global__ void permute3_kernel(const cplx* x, cplx* y, int d0, int d1, int d2, int p0, int p1, int p2,
                                 int inverse) {
+    pdl_begin();
     // y has axes (x-axis p0, x-axis p1, x-axis p2), first fastest
     long long n = (long long)d0 * d1 * d2;
     int dims[3] = {d0, d1, d2};
@@ -752,6 +763,7 @@ __global__ void permute3_kernel(const cplx* x, cplx* y, int d0, int d1, int d2, 
 }
 
 __global__ void fill_kernel(cplx* x, long long n, cplx v) {
+    pdl_begin();
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
          e += (long long)gridDim.x * blockDim.x)
         x[e] = v;
@@ -768,6 +780,7 @@ constexpr int AB_THREADS = 128;
 __global__ void __launch_bounds__(AB_THREADS)
     assemble_block_kernel(cplx* H, const cplx* Hs, int D, const cplx* nops, int nsites, const int* site_ids,
                           const cplx* dops, int ndriven, const int* driven_ids, const double* coef, double gamma) {
+    pdl_begin();
     extern __shared__ short terms[];       // < nsites: site term, else driven atom (index - nsites)
     __shared__ int s_count;
     if (threadIdx.x < 32) {                // in order, by one warp
@@ -850,6 +863,7 @@ __global__ void check_finite_kernel(const cplx* x, long long n, int* flag) {
 template <int WSUM_GROUP>
 __global__ void weighted_sum_kernel(const cplx* __restrict__ N, int nb, long long n, const double* __restrict__ W,
                                     int r, cplx* __restrict__ G, int staged) {
+    pdl_begin();
     extern __shared__ double sw_smem[];
     const double* sw = W;   // weights from global memory unless they fit in shared memory
     if (staged) {
@@ -888,6 +902,7 @@ template <int S>
 __global__ void __launch_bounds__(128) weighted_sum_small_kernel(const cplx* __restrict__ N, int nb, int n,
                                                                  const double* __restrict__ W, int r,
                                                                  cplx* __restrict__ G) {
+    pdl_begin();
     constexpr int OB = 128 / S;
     __shared__ cplx part[128];
     const int o = threadIdx.x % OB, ks = threadIdx.x / OB;
@@ -970,27 +985,27 @@ int red_blocks_for(long long n) {
 
 int k_norm2_partial(const cplx* x, long long n, double* partial, cudaStream_t s) {
     int G = red_blocks_for(n);
-    norm2_partial_kernel<<<G, T, 0, s>>>(x, n, G, partial);
+    launch(norm2_partial_kernel, G, T, 0, s, x, n, G, partial);
     return 1;
 }
 
 int k_dots(const cplx* V, long long ld, int nv, const cplx* w, long long n, cplx* partial, cudaStream_t s) {
     const int G = red_blocks_for(n);
-    dots_kernel<<<G, T, 0, s>>>(V, ld, nv, w, n, G, partial);
+    launch(dots_kernel, G, T, 0, s, V, ld, nv, w, n, G, partial);
     return 1;
 }
 
 int k_orth_first(const cplx* V, long long ld, int nv, const cplx* partial_in, cplx* w, long long n, cplx* partial_dots,
                  cplx* h_out, cudaStream_t s) {
     const int G = red_blocks_for(n);
-    orth_first_kernel<<<G, T, 0, s>>>(V, ld, nv, partial_in, w, n, G, partial_dots, h_out);
+    launch(orth_first_kernel, G, T, 0, s, V, ld, nv, partial_in, w, n, G, partial_dots, h_out);
     return 1;
 }
 
 int k_lanczos_first(const cplx* V, long long ld, int j, const cplx* partial_in, const KrylovScalars* ks, cplx* w,
                     long long n, cplx* partial_dots, cplx* h_out, cudaStream_t s) {
     const int G = red_blocks_for(n);
-    lanczos_first_kernel<<<G, T, 0, s>>>(V, ld, j, partial_in, ks, w, n, G, partial_dots, h_out);
+    launch(lanczos_first_kernel, G, T, 0, s, V, ld, j, partial_in, ks, w, n, G, partial_dots, h_out);
     return 1;
 }
 
@@ -998,30 +1013,30 @@ int k_orth_second(const cplx* V, long long ld, int nv, const cplx* partial_in, c
                   double* partial_norm, KrylovScalars* ks, const cplx* h1, double zr, double zi, double tol,
                   int arnoldi, const Publish& pub, cudaStream_t s) {
     const int G = red_blocks_for(n);
-    orth_second_kernel<<<G, T, 0, s>>>(V, ld, nv, partial_in, w, n, G, partial_norm, ks, h1, zr, zi, tol, arnoldi,
-                                       pub);
+    launch(orth_second_kernel, G, T, 0, s, V, ld, nv, partial_in, w, n, G, partial_norm, ks, h1, zr, zi, tol, arnoldi,
+           pub);
     return 1;
 }
 
 int k_scale_copy_dev(const cplx* x, long long n, const double* scale, cplx* y, cudaStream_t s) {
-    scale_copy_kernel<<<grid_for(n), 256, 0, s>>>(x, n, scale, y);
+    launch(scale_copy_kernel, grid_for(n), 256, 0, s, x, n, scale, y);
     return 1;
 }
 
 int k_rescale_to_norm(cplx* x, long long n, const double* px, int Gx, const double* pr, int Gr, cudaStream_t s) {
-    rescale_to_norm_kernel<<<grid_for(n), 256, 0, s>>>(x, n, px, Gx, pr, Gr);
+    launch(rescale_to_norm_kernel, grid_for(n), 256, 0, s, x, n, px, Gx, pr, Gr);
     return 1;
 }
 
 int k_combine(const cplx* V, long long ld, int nv, const KrylovScalars* ks, cplx* y, long long n,
               cudaStream_t s) {
-    combine_kernel<<<grid_for(n), 256, 0, s>>>(V, ld, nv, ks, y, n);
+    launch(combine_kernel, grid_for(n), 256, 0, s, V, ld, nv, ks, y, n);
     return 1;
 }
 
 int k_krylov_start(KrylovScalars* ks, const cplx* x, long long n, double* partial, cudaStream_t s) {
     const int G = red_blocks_for(n);
-    krylov_start_kernel<<<G, T, 0, s>>>(ks, x, n, G, partial, &ks->arrived);
+    launch(krylov_start_kernel, G, T, 0, s, ks, x, n, G, partial, &ks->arrived);
     return 1;
 }
 
@@ -1042,13 +1057,13 @@ bool wait_status(const HostStatus* hs, unsigned seq, cudaStream_t s) {
 int k_permute3(const cplx* x, cplx* y, int d0, int d1, int d2, int p0, int p1, int p2, int inverse,
                cudaStream_t s) {
     long long n = (long long)d0 * d1 * d2;
-    permute3_kernel<<<grid_for(n), 256, 0, s>>>(x, y, d0, d1, d2, p0, p1, p2, inverse);
+    launch(permute3_kernel, grid_for(n), 256, 0, s, x, y, d0, d1, d2, p0, p1, p2, inverse);
     return 1;
 }
 
 int k_fill(cplx* x, long long n, cplx v, cudaStream_t s) {
     if (n <= 0) return 0;
-    fill_kernel<<<grid_for(n), 256, 0, s>>>(x, n, v);
+    launch(fill_kernel, grid_for(n), 256, 0, s, x, n, v);
     return 1;
 }
 
@@ -1057,8 +1072,8 @@ int k_assemble_block(cplx* H, const cplx* Hs, int D, const cplx* nops, int nsite
                      cudaStream_t s) {
     long long DD = (long long)D * D;
     const size_t smem = sizeof(short) * (size_t)std::max(1, nsites + ndriven);
-    assemble_block_kernel<<<(unsigned)std::min<long long>((DD + AB_THREADS - 1) / AB_THREADS, 8 * 152), AB_THREADS, smem,
-                            s>>>(H, Hs, D, nops, nsites, site_ids, dops, ndriven, driven_ids, coef, gamma);
+    launch(assemble_block_kernel, (unsigned)std::min<long long>((DD + AB_THREADS - 1) / AB_THREADS, 8 * 152),
+           AB_THREADS, smem, s, H, Hs, D, nops, nsites, site_ids, dops, ndriven, driven_ids, coef, gamma);
     return 1;
 }
 
@@ -1084,9 +1099,10 @@ int k_weighted_sum(const cplx* N, int nb, long long n, const double* W, int r, c
     if (n <= 0 || r <= 0) return 0;
     if (n * r <= 64 * 1024) {   // below that the chip is not full with one thread per entry
         const int outs = (int)(n * r);
-        if (nb >= 32 && outs <= 16 * 1024) weighted_sum_small_kernel<16><<<(outs + 7) / 8, 128, 0, s>>>(N, nb, (int)n, W, r, G);
-        else if (nb >= 4) weighted_sum_small_kernel<4><<<(outs + 31) / 32, 128, 0, s>>>(N, nb, (int)n, W, r, G);
-        else weighted_sum_small_kernel<1><<<(outs + 127) / 128, 128, 0, s>>>(N, nb, (int)n, W, r, G);
+        if (nb >= 32 && outs <= 16 * 1024) launch(weighted_sum_small_kernel<16>, (outs + 7) / 8, 128, 0, s, N, nb,
+                                                  (int)n, W, r, G);
+        else if (nb >= 4) launch(weighted_sum_small_kernel<4>, (outs + 31) / 32, 128, 0, s, N, nb, (int)n, W, r, G);
+        else launch(weighted_sum_small_kernel<1>, (outs + 127) / 128, 128, 0, s, N, nb, (int)n, W, r, G);
         return 1;
     }
     const size_t need = sizeof(double) * (size_t)nb * r;
@@ -1095,9 +1111,9 @@ int k_weighted_sum(const cplx* N, int nb, long long n, const double* W, int r, c
     // entries over every SM
     const long long blocks = std::min<long long>((n + 63) / 64, 16 * 152);
     if (r <= 4)   // few outputs: small register groups, more loads in flight
-        weighted_sum_kernel<4><<<(unsigned)blocks, 64, staged ? need : 0, s>>>(N, nb, n, W, r, G, staged);
+        launch(weighted_sum_kernel<4>, (unsigned)blocks, 64, staged ? need : 0, s, N, nb, n, W, r, G, staged);
     else
-        weighted_sum_kernel<16><<<(unsigned)blocks, 64, staged ? need : 0, s>>>(N, nb, n, W, r, G, staged);
+        launch(weighted_sum_kernel<16>, (unsigned)blocks, 64, staged ? need : 0, s, N, nb, n, W, r, G, staged);
     return 1;
 }
 
@@ -1121,7 +1137,7 @@ int k_small_krylov(const int* d, const cplx* hb0, const cplx* hb1, const cplx* h
             attr[dev] = true;
         }
     }
-    small_krylov_kernel<<<SK_CL, SK_THREADS, smem, s>>>(d[0], d[1], d[2], hb0, hb1, hb2, pp, x, zr, zi, tol, mmax,
-                                                        arnoldi, pub);
+    launch(small_krylov_kernel, SK_CL, SK_THREADS, smem, s, d[0], d[1], d[2], hb0, hb1, hb2, pp, x, zr, zi, tol, mmax,
+           arnoldi, pub);
     return 1;
 }

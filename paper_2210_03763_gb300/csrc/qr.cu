@@ -102,6 +102,7 @@ __device__ double block_sum_d(double s, double* sh) {
 
 // Frobenius norm partials of the whole matrix.
 __global__ void frob_partial_kernel(const cplx* A, long long n, double* partial) {
+    pdl_begin();
     __shared__ double sh[32];
     double s = 0.0;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n; e += (long long)gridDim.x * blockDim.x)
@@ -111,6 +112,7 @@ __global__ void frob_partial_kernel(const cplx* A, long long n, double* partial)
 }
 
 __global__ void frob_finish_kernel(const double* partial, int G, double* scal) {
+    pdl_begin();
     double s = 0.0;
     for (int g = threadIdx.x; g < G; g += 32) s += partial[g];
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
@@ -1427,8 +1429,8 @@ bool launch_coop(CoopArgs& a, cudaStream_t s, int& nl) {
 
 int qr_frobenius(const cplx* A, long long n, QrScratch& ws, cudaStream_t s) {
     const int Gf = (int)std::min<long long>((n + 255) / 256, QR_FROB_BLOCKS);
-    frob_partial_kernel<<<Gf, 256, 0, s>>>(A, n, ws.pnorm);
-    frob_finish_kernel<<<1, 32, 0, s>>>(ws.pnorm, Gf, ws.scal);
+    launch(frob_partial_kernel, Gf, 256, 0, s, A, n, ws.pnorm);
+    launch(frob_finish_kernel, 1, 32, 0, s, ws.pnorm, Gf, ws.scal);
     return 2;
 }
 

@@ -42,6 +42,7 @@ constexpr double MIN_FRO2 = 1e-16; // residual^2 / |A|_F^2
 // matrix near the identity.  Sets *flag when a pivot is too small.
 __global__ void __launch_bounds__(CT) panel_chol_kernel(const cplx* Sw, long long ld, const cplx* Gq, int bp, cplx* C,
                                                         cplx* Rm, const double* fro2, int pass, int* flag) {
+    pdl_begin();
     __shared__ cplx G[PB][PB + 1], X[PB][PB + 1];
     __shared__ double norm2[PB], s_inv, s_r;
     __shared__ int bad;
@@ -122,6 +123,7 @@ __global__ void __launch_bounds__(CT) panel_chol_kernel(const cplx* Sw, long lon
 // n .. n + bp: R2 R1.  (S1, S2: leading dimension ld; R1, R2: PB.)
 __global__ void panel_r_kernel(const cplx* S1, const cplx* S2, long long ld, const cplx* R1, const cplx* R2, int n,
                                int bp, cplx* R, int D, int* dep, const int* flag, Publish pub) {
+    pdl_begin();
     const int e = blockIdx.x * blockDim.x + threadIdx.x;
     if (e == 0 && pub.hs) {
         pub.hs->qr_flag = *flag;
@@ -208,8 +210,8 @@ int qr_panel(cplx* A, int M, int D, cplx* R, QrScratch& ws, cudaStream_t s, void
                 g.alpha = make_double2(-1.0, 0.0);
                 launches += launch_zgemm_f64(g, s);
             }
-            panel_chol_kernel<<<1, CT, 0, s>>>(S + n, ld, n > 0 ? Gq : nullptr, bp, C + n, pass == 1 ? R1 : R2, ws.scal,
-                                               pass, flag);
+            launch(panel_chol_kernel, 1, CT, 0, s, S + n, ld, n > 0 ? Gq : nullptr, bp, C + n, pass == 1 ? R1 : R2,
+                   ws.scal, pass, flag);
             ++launches;
             if (n > 0) {   // -S_q T
                 GemmArgs g = args(n, bp, bp);
@@ -224,8 +226,8 @@ int qr_panel(cplx* A, int M, int D, cplx* R, QrScratch& ws, cudaStream_t s, void
             if (l < 0) return -1;
             launches += l;
         }
-        panel_r_kernel<<<((n + bp) * bp + 127) / 128, 128, 0, s>>>(S1, S2, ld, R1, R2, n, bp, R, D, ws.flags,
-                                                                    flag, n + PB >= std::min(D, last) ? pub : Publish{});
+        launch(panel_r_kernel, ((n + bp) * bp + 127) / 128, 128, 0, s, S1, S2, ld, R1, R2, n, bp, R, D, ws.flags,
+               flag, n + PB >= std::min(D, last) ? pub : Publish{});
         ++launches;
     }
     return launches;

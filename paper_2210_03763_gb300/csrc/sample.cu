@@ -29,6 +29,7 @@ __device__ double block_sum(double v, double* sh) {
 // G_b <- G_b / max(Re tr G_b, 1e-300) for the D x D matrices of S shots
 // (stride ld complex); one block per shot.
 __global__ void __launch_bounds__(NT) trace_normalize_kernel(cplx* G, int D, long long ld) {
+    pdl_begin();
     __shared__ double sh[NT / 32];
     __shared__ double sfac;
     cplx* g = G + blockIdx.x * ld;
@@ -46,6 +47,7 @@ __global__ void __launch_bounds__(NT) trace_normalize_kernel(cplx* G, int D, lon
 
 // w_b <- w_b / |w_b| (unchanged when zero) for S vectors of length D.
 __global__ void __launch_bounds__(NT) vec_normalize_kernel(cplx* w, int D, long long ld) {
+    pdl_begin();
     __shared__ double sh[NT / 32];
     __shared__ double sfac;
     cplx* x = w + blockIdx.x * ld;
@@ -63,6 +65,7 @@ __global__ void __launch_bounds__(NT) vec_normalize_kernel(cplx* w, int D, long 
 // outcome into out[b * N + atom]; w_b = e_s.
 __global__ void leaf_draw_kernel(const cplx* G, const double* U, long long ldu, int j, int atom, int* out, int N,
                                  cplx* w, int S) {
+    pdl_begin();
     const int b = blockIdx.x * blockDim.x + threadIdx.x;
     if (b >= S) return;
     int s = 0;
@@ -88,19 +91,19 @@ __global__ void leaf_draw_kernel(const cplx* G, const double* U, long long ldu, 
 
 int k_trace_normalize(cplx* G, int D, long long ld, int S, cudaStream_t s) {
     if (S <= 0) return 0;
-    trace_normalize_kernel<<<S, NT, 0, s>>>(G, D, ld);
+    launch(trace_normalize_kernel, S, NT, 0, s, G, D, ld);
     return 1;
 }
 
 int k_vec_normalize(cplx* w, int D, long long ld, int S, cudaStream_t s) {
     if (S <= 0) return 0;
-    vec_normalize_kernel<<<S, NT, 0, s>>>(w, D, ld);
+    launch(vec_normalize_kernel, S, NT, 0, s, w, D, ld);
     return 1;
 }
 
 int k_leaf_draw(const cplx* G, const double* U, long long ldu, int j, int atom, int* out, int N, cplx* w, int S,
                 cudaStream_t s) {
     if (S <= 0) return 0;
-    leaf_draw_kernel<<<(S + 127) / 128, 128, 0, s>>>(G, U, ldu, j, atom, out, N, w, S);
+    launch(leaf_draw_kernel, (S + 127) / 128, 128, 0, s, G, U, ldu, j, atom, out, N, w, S);
     return 1;
 }
