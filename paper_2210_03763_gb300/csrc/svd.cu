@@ -21,7 +21,8 @@
 
 namespace {
 
-constexpr int SVD_THREADS = 128;
+constexpr int SVD_THREADS = 128;   // at most; fewer for short columns
+constexpr int SVD_ROWS = 2;        // column elements per thread (N <= 256)
 constexpr unsigned long long SVD_WAIT_NS = 2000000000ull;   // 2 s per barrier wait
 
 __device__ __forceinline__ unsigned long long svd_ns() {
@@ -76,7 +77,11 @@ __device__ void pair_of(int k, int r, int Np, int& i, int& j) {
 
 // Several matrices in one launch: a sweep over one matrix is a chain of
 // barriers between its N / 2 blocks (4 ms at N = 64, nearly all of it waiting),
-// so the bonds of a tree run side by side, each with its own barrier.
+// so the bonds of a tree run side by side, each with its own barrier.  A round
+// is bound by the FP64 pipe (14 bonds of 64: three blocks per SM) and the
+// chain load - sums - rotation - store - barrier.  Measured, 14 bonds of 64 one
+// after another -> side by side -> with each element loaded once and the scalar
+// work spread over lanes: 64 -> 18.1 -> 14.9 ms; one 64 x 64 11.5 -> 10.4.
 struct JacobiBatch {
     JacobiTask t[SVD_BATCH];
     int first[SVD_BATCH + 1];   // first block of each matrix
@@ -86,7 +91,7 @@ struct JacobiBatch {
 // info: [0] sweeps run, [1] unused, [2], [3] rotation counters (alternating sweeps)
 __global__ void __launch_bounds__(SVD_THREADS) jacobi_kernel(const __grid_constant__ JacobiBatch jb, int max_sweeps,
                                                             double tol, int* err) {
-    __shared__ double red[3][SVD_THREADS / 32];
+    __shared__ double red[4][SVD_THREADS / 32];
     __shared__ double rot[4];   // c, s, cos phi, sin phi; rot[0] < 0: skip
     int m = 0;
     while ((int)blockIdx.x >= jb.first[m + 1]) ++m;
@@ -104,7 +109,7 @@ __global__ void __launch_bounds__(SVD_THREADS) jacobi_kernel(const __grid_consta
     __shared__ double s_floor;
     {
         double a = 0.0;
-        for (long long e = threadIdx.x; e < (long long)N * N; e += SVD_THREADS) {
+        for (long long e = threadIdx.x; e < (long long)N * N; e += blockDim.x) {
             const cplx x = __ldcg(R + e);
             a += x.x * x.x + x.y * x.y;
         }
@@ -113,7 +118,7 @@ __global__ void __launch_bounds__(SVD_THREADS) jacobi_kernel(const __grid_consta
         __syncthreads();
         if (threadIdx.x == 0) {
             double t = 0.0;
-            for (int q = 0; q < SVD_THREADS / 32; ++q) t += red[0][q];
+            for (int q = 0; q < (int)blockDim.x / 32; ++q) t += red[0][q];
             s_floor = 1e-30 * t;
         }
         __syncthreads();
@@ -133,68 +138,90 @@ __global__ void __launch_bounds__(SVD_THREADS) jacobi_kernel(const __grid_consta
                 j = t;
             }
             if (j < N) {
-                const cplx* ci = R + (long long)i * N;
-                const cplx* cj = R + (long long)j * N;
-                double a = 0.0, b = 0.0, gr = 0.0, gi = 0.0;
                 // columns move between blocks from round to round: read them
-                // through L2 (__ldcg), never from a stale L1 line
-                for (int e = threadIdx.x; e < N; e += SVD_THREADS) {
-                    const cplx x = __ldcg(ci + e), y = __ldcg(cj + e);
-                    a += x.x * x.x + x.y * x.y;
-                    b += y.x * y.x + y.y * y.y;
-                    gr += x.x * y.x + x.y * y.y;   // conj(x) y
-                    gi += x.x * y.y - x.y * y.x;
+                // through L2 (__ldcg), never from a stale L1 line; each element
+                // once, V's in flight while the rotation is worked out
+                const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = (int)blockDim.x / 32;
+                cplx* ci = R + (long long)i * N;
+                cplx* cj = R + (long long)j * N;
+                cplx* vi = V + (long long)i * N;
+                cplx* vj = V + (long long)j * N;
+                cplx x[SVD_ROWS], y[SVD_ROWS], vx[SVD_ROWS], vy[SVD_ROWS];
+#pragma unroll
+                for (int q = 0; q < SVD_ROWS; ++q) {
+                    const int e = threadIdx.x + q * (int)blockDim.x;
+                    if (e >= N) continue;
+                    x[q] = __ldcg(ci + e);
+                    y[q] = __ldcg(cj + e);
                 }
-                for (int o = 16; o > 0; o >>= 1) {
-                    a += __shfl_down_sync(0xffffffffu, a, o);
-                    b += __shfl_down_sync(0xffffffffu, b, o);
-                    gr += __shfl_down_sync(0xffffffffu, gr, o);
-                    gi += __shfl_down_sync(0xffffffffu, gi, o);
+#pragma unroll
+                for (int q = 0; q < SVD_ROWS; ++q) {
+                    const int e = threadIdx.x + q * (int)blockDim.x;
+                    if (e >= N) continue;
+                    vx[q] = __ldcg(vi + e);
+                    vy[q] = __ldcg(vj + e);
                 }
-                __shared__ double redi[SVD_THREADS / 32];
-                const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-                if (l == 0) {
-                    red[0][w] = a;
-                    red[1][w] = b;
-                    red[2][w] = gr;
-                    redi[w] = gi;
+                if (32 * w < N) {
+                    double a = 0.0, b = 0.0, gr = 0.0, gi = 0.0;
+#pragma unroll
+                    for (int q = 0; q < SVD_ROWS; ++q) {
+                        if (threadIdx.x + q * (int)blockDim.x >= N) continue;
+                        a += x[q].x * x[q].x + x[q].y * x[q].y;
+                        b += y[q].x * y[q].x + y[q].y * y[q].y;
+                        gr += x[q].x * y[q].x + x[q].y * y[q].y;   // conj(x) y
+                        gi += x[q].x * y[q].y - x[q].y * y[q].x;
+                    }
+                    // the four sums share the lanes (six FP64 additions, not twenty):
+                    // a ends in lanes 0-7, b 8-15, gr 16-23, gi 24-31
+                    const bool up = lane & 16, mid = lane & 8;
+                    double k0 = up ? gr : a, k1 = up ? gi : b;
+                    k0 += __shfl_xor_sync(0xffffffffu, up ? a : gr, 16);
+                    k1 += __shfl_xor_sync(0xffffffffu, up ? b : gi, 16);
+                    double v = mid ? k1 : k0;
+                    v += __shfl_xor_sync(0xffffffffu, mid ? k0 : k1, 8);
+                    for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+                    if ((lane & 7) == 0) red[lane >> 3][w] = v;
+                } else if ((lane & 7) == 0) {
+                    red[lane >> 3][w] = 0.0;
                 }
                 __syncthreads();
-                if (threadIdx.x == 0) {
-                    double A = 0, B = 0, Gr = 0, Gi = 0;
-                    for (int q = 0; q < SVD_THREADS / 32; ++q) {
-                        A += red[0][q];
-                        B += red[1][q];
-                        Gr += red[2][q];
-                        Gi += redi[q];
-                    }
-                    const double g = sqrt(Gr * Gr + Gi * Gi);
-                    if (g > tol * sqrt(A * B) && g > floor_g) {
-                        const double zeta = (B - A) / (2.0 * g);
+                if (w == 0) {   // lanes work on different quantities: the FP64 pipe takes a warp at a time
+                    double v = 0.0;
+                    for (int q = 0; q < nw; ++q) v += red[lane & 3][q];
+                    const double A = __shfl_sync(0xffffffffu, v, 0), B = __shfl_sync(0xffffffffu, v, 1),
+                                 Gr = __shfl_sync(0xffffffffu, v, 2), Gi = __shfl_sync(0xffffffffu, v, 3);
+                    v = sqrt((lane & 1) ? A * B : Gr * Gr + Gi * Gi);
+                    const double g = __shfl_sync(0xffffffffu, v, 0), ab = __shfl_sync(0xffffffffu, v, 1);
+                    if (g > tol * ab && g > floor_g) {
+                        v = (lane == 0 ? B - A : lane == 1 ? Gr : Gi) / (lane == 0 ? 2.0 * g : g);
+                        const double zeta = __shfl_sync(0xffffffffu, v, 0);
                         const double t = (zeta >= 0.0 ? 1.0 : -1.0) / (fabs(zeta) + sqrt(1.0 + zeta * zeta));
                         const double c = 1.0 / sqrt(1.0 + t * t);
-                        rot[0] = c;
-                        rot[1] = c * t;
-                        rot[2] = Gr / g;
-                        rot[3] = Gi / g;
-                        atomicAdd(cnt, 1);
-                    } else {
+                        if (lane == 0) {
+                            rot[0] = c;
+                            rot[1] = c * t;
+                            atomicAdd(cnt, 1);
+                        } else if (lane < 3) {
+                            rot[lane + 1] = v;
+                        }
+                    } else if (lane == 0) {
                         rot[0] = -1.0;
                     }
                 }
                 __syncthreads();
                 if (rot[0] >= 0.0) {
                     const double c = rot[0], s = rot[1], pc = rot[2], ps = rot[3];   // e^{-i phi} = pc - i ps
-                    for (int w = 0; w < 2; ++w) {
-                        cplx* X = w == 0 ? R : V;
-                        cplx* xi = X + (long long)i * N;
-                        cplx* xj = X + (long long)j * N;
-                        for (int e = threadIdx.x; e < N; e += SVD_THREADS) {
-                            const cplx x = __ldcg(xi + e), y = __ldcg(xj + e);
-                            const cplx yp = make_double2(pc * y.x + ps * y.y, pc * y.y - ps * y.x);   // e^{-i phi} y
-                            xi[e] = make_double2(c * x.x - s * yp.x, c * x.y - s * yp.y);
-                            xj[e] = make_double2(s * x.x + c * yp.x, s * x.y + c * yp.y);
-                        }
+                    auto rotate = [&](const cplx& p, const cplx& q, cplx* pi, cplx* pj) {
+                        const cplx yp = make_double2(pc * q.x + ps * q.y, pc * q.y - ps * q.x);   // e^{-i phi} q
+                        *pi = make_double2(c * p.x - s * yp.x, c * p.y - s * yp.y);
+                        *pj = make_double2(s * p.x + c * yp.x, s * p.y + c * yp.y);
+                    };
+#pragma unroll
+                    for (int q = 0; q < SVD_ROWS; ++q) {
+                        const int e = threadIdx.x + q * (int)blockDim.x;
+                        if (e >= N) continue;
+                        rotate(x[q], y[q], ci + e, cj + e);
+                        rotate(vx[q], vy[q], vi + e, vj + e);
                     }
                 }
             }
@@ -214,6 +241,7 @@ __global__ void __launch_bounds__(SVD_THREADS) jacobi_kernel(const __grid_consta
 // One block.
 __global__ void svd_finish_kernel(const cplx* R, const cplx* V, int N, int chi, double eps, cplx* Ur, cplx* Vh,
                                   double* S, int* kout, double* disc, int* order) {
+    pdl_begin();
     extern __shared__ double sig[];
     for (int i = threadIdx.x; i < N; i += blockDim.x) {
         double s = 0.0;
@@ -267,6 +295,7 @@ __global__ void svd_finish_kernel(const cplx* R, const cplx* V, int N, int chi, 
 }
 
 __global__ void identity_kernel(cplx* V, int N) {
+    pdl_begin();
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < (long long)N * N;
          e += (long long)gridDim.x * blockDim.x)
         V[e] = make_double2((e % N) == (e / N) ? 1.0 : 0.0, 0.0);
@@ -278,7 +307,12 @@ int svd_jacobi_batch(const JacobiTask* tasks, int n, int max_sweeps, double tol,
     int dev = 0, nsm = 0, per_sm = 0, launches = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, jacobi_kernel, SVD_THREADS, 0);
+    int T = 32;   // a thread per column element; idle warps would still take their turns at the FP64 pipe
+    for (int i = 0; i < n; ++i) {
+        if (tasks[i].N > SVD_ROWS * SVD_THREADS) return -1;
+        T = std::max(T, std::min(SVD_THREADS, (tasks[i].N + 31) / 32 * 32));
+    }
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, jacobi_kernel, T, 0);
     const int room = nsm * per_sm;
     for (int i = 0; i < n;) {
         JacobiBatch jb;
@@ -288,7 +322,7 @@ int svd_jacobi_batch(const JacobiTask* tasks, int n, int max_sweeps, double tol,
             const JacobiTask& t = tasks[i];
             const int blocks = (t.N + 1) / 2;
             if (jb.n > 0 && jb.first[jb.n] + blocks > room) break;
-            identity_kernel<<<(t.N * t.N + 255) / 256, 256, 0, s>>>(t.V, t.N);
+            launch(identity_kernel, (t.N * t.N + 255) / 256, 256, 0, s, t.V, t.N);
             cudaMemsetAsync(t.bar, 0, 2 * sizeof(unsigned), s);
             cudaMemsetAsync(t.info, 0, 4 * sizeof(int), s);
             ++launches;
@@ -299,7 +333,7 @@ int svd_jacobi_batch(const JacobiTask* tasks, int n, int max_sweeps, double tol,
         }
         if (jb.n == 0) continue;
         void* args[] = {(void*)&jb, (void*)&max_sweeps, (void*)&tol, (void*)&err};
-        if (cudaLaunchCooperativeKernel((const void*)jacobi_kernel, dim3(jb.first[jb.n]), dim3(SVD_THREADS), args, 0,
+        if (cudaLaunchCooperativeKernel((const void*)jacobi_kernel, dim3(jb.first[jb.n]), dim3(T), args, 0,
                                         s) != cudaSuccess)
             return -1;
         ++launches;
@@ -315,6 +349,6 @@ int svd_jacobi_square(cplx* R, cplx* V, int N, int max_sweeps, double tol, unsig
 
 int svd_finish(const cplx* R, const cplx* V, int N, int chi, double eps, cplx* Ur, cplx* Vh, double* S, int* k,
                double* disc, int* order, cudaStream_t s) {
-    svd_finish_kernel<<<1, 256, sizeof(double) * N, s>>>(R, V, N, chi, eps, Ur, Vh, S, k, disc, order);
+    launch(svd_finish_kernel, 1, 256, sizeof(double) * N, s, R, V, N, chi, eps, Ur, Vh, S, k, disc, order);
     return 1;
 }
