@@ -36,13 +36,6 @@ bool digits_wanted(const GemmArgs& g);
 size_t digits_workspace_bytes(const GemmArgs& g);
 int launch_zgemm_digits(const GemmArgs& g, cudaStream_t stream, void* workspace, size_t workspace_bytes);
 
-// ---- split-precision building blocks (gemm_split.cu) -------------------------
-// Packing of one side of a split contraction into TF32 hi/lo planes: complex
-// element (row r, k, batch bi, bo) of src (strides s_r, s_ki (k % Ki),
-// s_ko (k / Ki), s_bi, s_bo) goes to real row (embed ? 2r : r) + bi*rb_i +
-// bo*rb_o, floats k_off + 2k of a row `pitch` floats long; embed = 1 is the
-// real embedding of the Q side (rows (Re, -Im) and (Im, Re)).  Rows
-// r in [R, Rpad) and k in [Ki*Ko, Kc) are written as zeros.
 // Programmatic dependent launch for small kernels: the next kernel of the
 // stream is brought up while this one runs, and waits in pdl_begin() until all
 // before it is complete and visible.  Every kernel started with launch() calls
@@ -75,6 +68,13 @@ inline void launch(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cud
 }
 #endif
 
+// ---- split-precision building blocks (gemm_split.cu) -------------------------
+// Packing of one side of a split contraction into TF32 hi/lo planes: complex
+// element (row r, k, batch bi, bo) of src (strides s_r, s_ki (k % Ki),
+// s_ko (k / Ki), s_bi, s_bo) goes to real row (embed ? 2r : r) + bi*rb_i +
+// bo*rb_o, floats k_off + 2k of a row `pitch` floats long; embed = 1 is the
+// real embedding of the Q side (rows (Re, -Im) and (Im, Re)).  Rows
+// r in [R, Rpad) and k in [Ki*Ko, Kc) are written as zeros.
 struct SplitPackArgs {
     const cplx* src;
     long long s_r, s_ki, s_ko, s_bi, s_bo;

@@ -848,6 +848,7 @@ __global__ void __launch_bounds__(AB_THREADS)
 }
 
 __global__ void check_finite_kernel(const cplx* x, long long n, int* flag) {
+    pdl_begin();
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < n;
          e += (long long)gridDim.x * blockDim.x) {
         cplx v = x[e];
@@ -1079,7 +1080,7 @@ int k_assemble_block(cplx* H, const cplx* Hs, int D, const cplx* nops, int nsite
 
 int k_check_finite(const cplx* x, long long n, int* flag, cudaStream_t s) {
     if (n <= 0) return 0;
-    check_finite_kernel<<<grid_for(n), 256, 0, s>>>(x, n, flag);
+    launch(check_finite_kernel, grid_for(n), 256, 0, s, x, n, flag);
     return 1;
 }
 

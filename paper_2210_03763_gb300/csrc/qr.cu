@@ -1083,6 +1083,7 @@ __global__ void __launch_bounds__(QB) normalize_col_kernel(cplx* A, long long M,
 // M += y_t y_t^H / nu_t^2 (Sherman-Morrison).  The selection touches only
 // candidate rows (O(L r^2)); the vectors are one M x r x m product.
 __global__ void sc_init_kernel(int* row_rank, long long M, int* cand_used, int ncand) {
+    pdl_begin();
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < M; i += (long long)gridDim.x * blockDim.x)
         row_rank[i] = 0x7FFFFFFF;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < ncand;
@@ -1120,6 +1121,7 @@ __device__ double sc_residual(const cplx* A, long long M, const int* kept, int r
 __global__ void __launch_bounds__(SC_THREADS) sc_select_kernel(const cplx* A, long long M, const int* kept, int r,
                                                                int m, const int* cand, int ncand, int* acc_rows,
                                                                cplx* Y, double* nu, int* row_rank, int* cand_used) {
+    pdl_begin();
     extern __shared__ cplx sm[];
     cplx* Mi = sm;
     cplx* y = Mi + r * r;
@@ -1204,6 +1206,7 @@ __global__ void __launch_bounds__(SC_THREADS) sc_select_kernel(const cplx* A, lo
 __global__ void __launch_bounds__(32) sc_select_warp_kernel(const cplx* A, long long M, const int* kept, int r,
                                                             int m, const int* cand, int ncand, int* acc_rows,
                                                             cplx* Y, double* nu, int* row_rank, int* cand_used) {
+    pdl_begin();
     extern __shared__ cplx sm[];
     cplx* Mi = sm;               // r x r
     cplx* ys = Mi + r * r;       // r
@@ -1314,6 +1317,7 @@ constexpr int SC_COLS = 16;
 __global__ void __launch_bounds__(QB) sc_materialize_kernel(cplx* A, long long M, const int* kept, int r,
                                                             const int* dep, int m, const cplx* Y, const double* nu,
                                                             const int* acc_rows, const int* row_rank) {
+    pdl_begin();
     extern __shared__ cplx sY[];
     __shared__ int sacc[SC_COLS], sdep[SC_COLS];
     __shared__ double sinv[SC_COLS];   // 1 / nu_t: one division per column, not one per entry
@@ -1535,7 +1539,7 @@ int qr_cgs2(cplx* A, int M, int D, cplx* R, const int* cand, int ncand, QrScratc
         cudaMemcpyAsync(ws.kept, hk, sizeof(int) * std::max(nk, 1), cudaMemcpyHostToDevice, s);
         cudaMemcpyAsync(ws.dep, hd, sizeof(int) * nd, cudaMemcpyHostToDevice, s);
         int gi = (int)std::min<long long>((std::max<long long>(MM, ncand) + 255) / 256, 1024);
-        sc_init_kernel<<<gi, 256, 0, s>>>(ws.row_rank, MM, ws.cand_used, ncand);
+        launch(sc_init_kernel, gi, 256, 0, s, ws.row_rank, MM, ws.cand_used, ncand);
         static bool attr[64] = {};   // shared memory above 48 KB (kept rank up to 64), per device
         {
             std::lock_guard<std::mutex> lock(g_coop_mu);
@@ -1548,16 +1552,16 @@ int qr_cgs2(cplx* A, int M, int D, cplx* R, const int* cand, int ncand, QrScratc
             }
         }
         if (r <= 32) {
-            sc_select_warp_kernel<<<1, 32, sizeof(cplx) * ((size_t)r * r + (size_t)r + 32 * ((size_t)r + 1)), s>>>(
-                A, MM, ws.kept, r, nd, cand, ncand, ws.acc_rows, ws.Y, ws.nu, ws.row_rank, ws.cand_used);
+            launch(sc_select_warp_kernel, 1, 32, sizeof(cplx) * ((size_t)r * r + (size_t)r + 32 * ((size_t)r + 1)), s,
+                   A, MM, ws.kept, r, nd, cand, ncand, ws.acc_rows, ws.Y, ws.nu, ws.row_rank, ws.cand_used);
         } else {
             size_t sel_smem = sizeof(cplx) * ((size_t)r * r + 2 * (size_t)r + 2);
-            sc_select_kernel<<<1, SC_THREADS, sel_smem, s>>>(A, MM, ws.kept, r, nd, cand, ncand, ws.acc_rows, ws.Y,
-                                                             ws.nu, ws.row_rank, ws.cand_used);
+            launch(sc_select_kernel, 1, SC_THREADS, sel_smem, s, A, MM, ws.kept, r, nd, cand, ncand, ws.acc_rows, ws.Y,
+                   ws.nu, ws.row_rank, ws.cand_used);
         }
         const size_t mat_smem = sizeof(cplx) * (size_t)r * SC_COLS;
-        sc_materialize_kernel<<<dim3(G, (nd + SC_COLS - 1) / SC_COLS), QB, mat_smem, s>>>(A, MM, ws.kept, r, ws.dep, nd, ws.Y, ws.nu, ws.acc_rows,
-                                                      ws.row_rank);
+        launch(sc_materialize_kernel, dim3(G, (nd + SC_COLS - 1) / SC_COLS), QB, mat_smem, s, A, MM, ws.kept, r, ws.dep,
+               nd, ws.Y, ws.nu, ws.acc_rows, ws.row_rank);
         launches += 3;
         return launches;
     }
