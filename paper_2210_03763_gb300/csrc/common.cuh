@@ -41,10 +41,10 @@ int launch_zgemm_digits(const GemmArgs& g, cudaStream_t stream, void* workspace,
 // before it is complete and visible.  Every kernel started with launch() calls
 // pdl_begin() before anything else (GEMMs that fill the SMs pdl_wait()).
 // Only between grids of at most a block per SM: blocks brought up early take
-// the free places of the SMs as they come, and large grids spread unevenly (all
-// launches: 4x4 chi = 64 FP64 127 -> 143 ms).  Measured, ms per step: 8x8
-// chi = 12 FP64 99 -> 82, 4x4 chi = 64 FP64 127 -> 120, 8x8 chi = 128 split 374
-// -> 356.
+// the free places of the SMs as they come, and large grids spread unevenly.  ms
+// per step with a limit of 76, 152, 304, 608 blocks: 8x8 chi = 128 split 364,
+// 357, 363, 364, its entangled start 700, 692, 717, 725, 4x4 chi = 64 FP64 123,
+// 120, 124, 131.  Without it: 374, 721, 127; 8x8 chi = 12 FP64 99 -> 82.
 #ifdef __CUDACC__
 constexpr unsigned PDL_MAX_BLOCKS = 152;
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
