@@ -21,8 +21,8 @@
 // 16384 x 128 matrix, and its 128 columns as many grid synchronisations
 // (8.5 ms measured); here the rows are read by ~10 launches per panel and
 // pass.  Measured, ms per call, column loop (with its rows spread over all SMs)
-// and panels: 16384 x 128 7.5 and 2.1, 10368 x 81 2.9 and 1.25, 6561 x 128 4.2
-// and 1.6, 4096 x 64 1.25 and 0.73.
+// and panels: 16384 x 128 7.5 and 1.95, 10368 x 81 2.9 and 1.14, 6561 x 128 4.2
+// and 1.5, 4096 x 64 1.25 and 0.67, 81 x 81 1.1 and 0.46.
 #include "common.cuh"
 
 #include <algorithm>
