@@ -60,8 +60,8 @@ extern "C" ttn_status ttn_contract_split_noalloc(const double* A, const double* 
         ttn_status st = scratch_for_current_device(&scratch);
         if (st != TTN_OK) return st;
         // the error flag at the start of the scratch is zero: it starts so and
-        // is cleared whenever a call has found it set (a memset here took 2 to 3 us
-        // of a call of 30)
+        // is cleared whenever a call has found it set (clearing it here was a launch
+        // of its own in a call of 30 us)
         packed = launch_split_pack(g, s, scratch, NOALLOC_SCRATCH_BYTES, 1);
         if (packed == -2) return TTN_ERR_ARG;
     }
