@@ -271,7 +271,7 @@ struct QrScratch {
     int* cand_used;     // M: candidate accepted flags
     unsigned* bar;      // 2: grid barrier of the cooperative column loop
     int* err;           // [0] set when a bounded device wait gave up, [1] when the panel path gave up
-    cplx* panel;        // panel path: 3 (D + QR_PANEL) QR_PANEL + 3 QR_PANEL^2
+    cplx* panel;        // panel path: qr_panel_scratch(D)
     HostStatus* hs;     // status in host memory (null: read back by copies)
     unsigned* seq;      // last sequence number used with it
 };
@@ -285,16 +285,16 @@ constexpr int QR_SC_MAXR = 64;   // structured completion when the kept rank r <
 // library).
 constexpr double QR_TOL_FP64 = 1e-10;
 constexpr int QR_PANEL = 32;
-// QR of a well-conditioned matrix by panels (qr_panel.cu): columns [first,
-// last) of A in place and of R (zeroed before), ws.scal[0] = |A|_F^2 and
-// ws.err[1] = 0 before the first call.  Reports qr_flag with the last launch;
-// not 0: not well-conditioned, A and R undefined.  Workspace as launch_zgemm_digits (of
-// qr_panel_workspace bytes).  Returns launches, -1 when not available.
+// QR of a well-conditioned matrix by panels (qr_panel.cu): A = Q R, A kept, Q
+// in a buffer of its own.  Columns [first, last) of Q, in calls one after
+// another; the one that ends at D writes R.  Reports qr_flag with the last
+// launch; not 0: not well-conditioned, Q and R undefined.  Workspace as
+// launch_zgemm_digits (of qr_panel_workspace bytes); ws.panel of
+// qr_panel_scratch(D) complex.  Returns launches, -1 when not available.
+size_t qr_panel_scratch(int D);
 size_t qr_panel_workspace(int M, int D);
-int qr_panel(cplx* A, int M, int D, cplx* R, QrScratch& ws, cudaStream_t s, void* workspace, size_t workspace_bytes,
-             int first, int last, const Publish& pub);
-// |A|_F^2 into ws.scal[0].
-int qr_frobenius(const cplx* A, long long n, QrScratch& ws, cudaStream_t s);
+int qr_panel(const cplx* A, cplx* Q, int M, int D, cplx* R, QrScratch& ws, cudaStream_t s, void* workspace,
+             size_t workspace_bytes, int first, int last, const Publish& pub);
 // fine_rows: spread the rows of small matrices over all SMs (see qr.cu).
 int qr_cgs2(cplx* A, int M, int D, cplx* R, const int* cand, int ncand,
             QrScratch& ws, cudaStream_t s, int* n_dependent_host, bool fine_rows = false, double tol = QR_TOL_FP64);

@@ -1429,14 +1429,15 @@ bool launch_coop(CoopArgs& a, cudaStream_t s, int& nl) {
     return false;
 }
 
-}  // namespace
-
+// |A|_F^2 into ws.scal[0].
 int qr_frobenius(const cplx* A, long long n, QrScratch& ws, cudaStream_t s) {
     const int Gf = (int)std::min<long long>((n + 255) / 256, QR_FROB_BLOCKS);
     launch(frob_partial_kernel, Gf, 256, 0, s, A, n, ws.pnorm);
     launch(frob_finish_kernel, 1, 32, 0, s, ws.pnorm, Gf, ws.scal);
     return 2;
 }
+
+}  // namespace
 
 int qr_cgs2(cplx* A, int M, int D, cplx* R, const int* cand, int ncand, QrScratch& ws, cudaStream_t s,
             int* n_dependent_host, bool fine_rows, double tol) {

@@ -1297,8 +1297,8 @@ bool panel_applies(int M, int D) { return D >= PANEL_MIN_D && M >= PANEL_MIN_M; 
 
 // A (M x D) = Q R, Q in A's place: by panels on the tensor cores when the
 // matrix is large and well-conditioned, else by the column
-// loop, which decides and completes dependent columns.  The panel path works
-// on a copy in `spare` (swapped with A when it succeeds) and gives up on
+// loop, which decides and completes dependent columns.  The panel path puts Q
+// in `spare` (swapped with A when it succeeds) and gives up on
 // matrices that are not well-conditioned, so it is tried where it is likely
 // to succeed.  hint: 1 it succeeded here last time; 0 unknown (its first panel
 // is checked before the rest is launched); -1 dependent columns last time; < -1
@@ -1309,14 +1309,10 @@ int gauge_qr(ttn_ctx* c, cplx*& A, cplx*& spare, int M, int D, cplx* R, const in
     if (hint >= 0 && panel_applies(M, D)) {
         const size_t need = qr_panel_workspace(M, D);
         if (try_grow_split_ws(c, need)) {
-            CUDA_OK(cudaMemsetAsync(R, 0, sizeof(cplx) * (size_t)D * D, c->stream));
-            CUDA_OK(cudaMemsetAsync(q.err + 1, 0, sizeof(int), c->stream));
-            CUDA_OK(cudaMemcpyAsync(spare, A, sizeof(cplx) * (size_t)M * D, cudaMemcpyDeviceToDevice, c->stream));
-            c->stats[3] += qr_frobenius(A, (long long)M * D, q, c->stream);
             int gave_up = 0;
             for (int first = 0; first < D && !gave_up;) {
                 const int last = hint == 1 || first > 0 ? D : QR_PANEL;
-                const int n = qr_panel(spare, M, D, R, q, c->stream, c->split_ws, c->split_cap, first, last,
+                const int n = qr_panel(A, spare, M, D, R, q, c->stream, c->split_ws, c->split_cap, first, last,
                                        next_publish(c));
                 if (n < 0) {
                     gave_up = 1;
@@ -1677,7 +1673,7 @@ void alloc_qr_scratch(ttn_ctx* c, long long maxM, int maxD, QrScratch& q) {
     q.nu = (double*)dalloc(c, sizeof(double) * (maxD + 2));
     q.row_rank = (int*)dalloc(c, sizeof(int) * std::max<long long>(maxM, 1));
     q.cand_used = (int*)dalloc(c, sizeof(int) * std::max<long long>(maxM, 1));
-    q.panel = (cplx*)dalloc(c, sizeof(cplx) * (3 * (size_t)(maxD + QR_PANEL) * QR_PANEL + 3 * QR_PANEL * QR_PANEL));
+    q.panel = (cplx*)dalloc(c, sizeof(cplx) * qr_panel_scratch(maxD));
     q.hs = c->hstat;
     q.seq = &c->seq;
     q.bar = (unsigned*)dalloc(c, sizeof(unsigned) * 4);
