@@ -28,13 +28,17 @@ int launch_zgemm_f64(const GemmArgs& g, cudaStream_t stream, void* workspace = n
 size_t f64_workspace_bytes(const GemmArgs& g);
 // C = alpha sum_ks W[ks] + beta C, W[((ks * Bo + bo) * Bi + bi) * M * N + m + n M].
 int launch_splitk_f64(const GemmArgs& g, int nsplit, const cplx* W, cudaStream_t stream);
-// The same contraction by exact digit products on the tensor cores
-// (gemm_digits.cu): whether it pays for this shape, its workspace (first int:
-// the error flag a timed-out wait sets), and the launch (kernels launched; -1
-// when it is not handled there, -2 when the workspace is too small).
+// The same contraction by digit products on the tensor cores (gemm_digits.cu):
+// whether it pays for this shape, its workspace (first int: the error flag a
+// timed-out wait sets; second: outputs that the last launch left to FMA
+// chains), and the launch (kernels launched; -1 when it is not handled there,
+// -2 when the workspace is too small).  elementwise: every output has the error
+// bound of an FMA chain; else its error is relative to |row||column|, C may
+// overlap A and B when it is one batch, and rows with an infinity or a NaN give NaNs.
 bool digits_wanted(const GemmArgs& g);
-size_t digits_workspace_bytes(const GemmArgs& g);
-int launch_zgemm_digits(const GemmArgs& g, cudaStream_t stream, void* workspace, size_t workspace_bytes);
+size_t digits_workspace_bytes(const GemmArgs& g, bool elementwise);
+int launch_zgemm_digits(const GemmArgs& g, bool elementwise, cudaStream_t stream, void* workspace,
+                        size_t workspace_bytes);
 
 // Programmatic dependent launch for small kernels: the next kernel of the
 // stream is brought up while this one runs, and waits in pdl_begin() until all

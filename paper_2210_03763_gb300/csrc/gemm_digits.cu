@@ -15,9 +15,24 @@
 // |v_l| <= 7 * 128 * 2^14 < 2^24 for 128 values of k, so the FP32
 // accumulation of a K chunk of 128 reals has no rounding at all; chunks are
 // added in 64-bit integers, and the one rounding of the result is the final
-// conversion to FP64.  Against the 53-bit products and sums of an FMA chain
-// the error is smaller (measured, uniform operands, rms relative to |row|
-// |column|: 7e-18 at K = 64, below the 3.3e-17 of an FMA chain).
+// conversion to FP64.
+//
+// Accuracy.  What is lost is the part of an entry below its row's grid:
+//   |error| <= 2^-56 (2^Ep sum_k |q_k| + 2^Eq sum_k |p_k|) + K 2^-60 2^(Ep + Eq).
+// For operands of one size along K that is less than the roundings of an FMA
+// chain (uniform operands, rms relative to |row||column|: 7e-18 at K = 64, the
+// chain 3.3e-17).  Not so where small entries of one row meet large ones of
+// the other: graded against each other over 2^32, digits alone are off by
+// 2e-8 of sum |p_k||q_k|.  So digit_check_kernel computes a lower bound of
+// sum_k |p_k||q_k| for every output (a bf16 product of the magnitudes, a
+// hundredth of the work) and marks the outputs whose error bound above exceeds
+// that of an FMA chain, 2 K 2^-53 sum |p_k||q_k|; digit_fix_kernel computes
+// those by FMA chains.  Every output so has an FMA chain's bound, whatever the
+// operands hold.  Callers whose analysis needs no more than |row||column|
+// (the panel QR, whose operands are columns of norm about 1) leave the check
+// out (elementwise = false).  The check costs 7 us of a small contraction and 6
+// to 11 % of a large one (4096 x 64 x 64 48 -> 55 us, 16384 x 128 x 128 180 -> 200);
+// in steps and observables of this library 0 to 0.02 % of the outputs are marked.
 //
 // Why: GB300's FP64 pipe gives 1.06 TFLOP/s; 34 bf16 products give one FP64
 // product at up to 1908 / 34 = 56 TFLOP/s.  Measured, packing included, against
@@ -42,6 +57,7 @@
 
 #include <algorithm>
 #include <cstring>
+#include <math_constants.h>
 
 namespace {
 
@@ -71,6 +87,8 @@ struct DigitSide {
     long long rows;                          // real rows in a plane
     uint16_t* planes;                        // ND planes of rows x 2 Kc bf16
     int* exps;                               // per complex row: biased exponent field of its largest entry
+    uint16_t* mag;                           // rows x Kc bf16: max(|re|, |im|) 2^-E, rounded down; null: no check
+    unsigned long long* l1;                  // per complex row: sum of (|re| + |im|) 2^-E in units of 2^-16
 };
 
 constexpr int PK_ROWS = 32, PK_THREADS = 256, PK_KT = 32;
@@ -154,7 +172,22 @@ __device__ __forceinline__ uint32_t bf16_pair(float lo, float hi) {
     return __byte_perm(__float_as_uint(lo), __float_as_uint(hi), 0x7632);
 }
 
-// Row exponents over blocks of K (long K only): exps zeroed before.
+// max(|re|, |im|) 2^-E of an entry as bf16, rounded down; at least 2^-60 unless
+// the entry is zero (a product of two is zero only if one of them is).
+__device__ __forceinline__ uint16_t magnitude(cplx v, int emax) {
+    const uint32_t hx = (uint32_t)__double2hiint(v.x) & 0x7FFFFFFFu, hy = (uint32_t)__double2hiint(v.y) & 0x7FFFFFFFu;
+    const uint32_t h = hx > hy ? hx : hy;
+    const int e = (int)(h >> 20), d = emax - e;
+    if (e > 0 && d < 60) return (uint16_t)(((126 - d) << 7) | ((h >> 13) & 0x7Fu));
+    return (h | (uint32_t)__double2loint(v.x) | (uint32_t)__double2loint(v.y)) ? (uint16_t)((126 - 59) << 7) : (uint16_t)0;
+}
+// |t| of biased digits in units of 2^39 (2^-16 of the row's largest), rounded up.
+__device__ __forceinline__ unsigned l1_units(unsigned long long biased) {
+    const long long t = (long long)(biased - 0x808080808080ULL);
+    return (unsigned)(((t < 0 ? -t : t) + ((1LL << 39) - 1)) >> 39);
+}
+
+// Row exponents over blocks of K (long K only): exps and l1 zeroed before.
 __global__ void __launch_bounds__(PK_THREADS) digit_max_kernel(DigitSide sp, DigitSide sq, int nbp, int kb) {
     pdl_begin();
     const DigitSide& s = (int)blockIdx.x < nbp ? sp : sq;
@@ -175,19 +208,22 @@ __global__ void __launch_bounds__(PK_THREADS) digit_max_kernel(DigitSide sp, Dig
 // Digits of 32 rows over a block of K.  one_pass: this block sees the whole K
 // and finds the exponents itself.
 __global__ void __launch_bounds__(PK_THREADS) digit_pack_kernel(DigitSide sp, DigitSide sq, int nbp, int kb,
-                                                               int one_pass) {
+                                                               int one_pass, int* marked) {
     pdl_begin();
+    if (marked && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *marked = 0;
     const bool isp = (int)blockIdx.x < nbp;
     const DigitSide& s = isp ? sp : sq;
     const long long f0 = (long long)(isp ? blockIdx.x : blockIdx.x - nbp) * PK_ROWS;
     __shared__ const cplx* base[PK_ROWS];
     __shared__ int mx[PK_ROWS];
     __shared__ cplx tile[PK_KT][PK_ROWS + 1];
+    __shared__ unsigned long long l1[PK_ROWS];   // row r: added to by its own warp's lane 0 only
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const long long nrow = (long long)s.Rpad * s.Bi * s.Bo;
     if (threadIdx.x < PK_ROWS) {
         base[threadIdx.x] = row_base(s, f0 + threadIdx.x);
         mx[threadIdx.x] = 0;
+        l1[threadIdx.x] = 0;
     }
     __syncthreads();
     const int K = s.Ki * s.Ko;
@@ -228,30 +264,47 @@ __global__ void __launch_bounds__(PK_THREADS) digit_pack_kernel(DigitSide sp, Di
         for (int i = 0; i < PK_ROWS / 8; ++i) {
             const int r = warp + 8 * i;
             const long long f = f0 + r;
-            if (f >= nrow || k >= s.Kc) continue;
-            uint16_t* o = s.planes + (s.embed ? 2 * f : f) * 2LL * s.Kc + 2LL * k;
-            if (!base[r] || mx[r] == 0x7FF) {   // padding; rows that the epilogue recomputes
+            if (f >= nrow) continue;
+            unsigned l = 0;
+            if (k < s.Kc) {
+                uint16_t* o = s.planes + (s.embed ? 2 * f : f) * 2LL * s.Kc + 2LL * k;
+                if (!base[r] || mx[r] == 0x7FF) {   // padding; rows with infinities or NaNs
 #pragma unroll
-                for (int q = 0; q < ND; ++q) {
-                    *reinterpret_cast<uint32_t*>(o + q * plane) = 0u;
-                    if (s.embed) *reinterpret_cast<uint32_t*>(o + q * plane + 2LL * s.Kc) = 0u;
-                }
-                continue;
-            }
-            const cplx v = tile[lane][r];
-            const unsigned long long tr = biased_digits(v.x, mx[r]), ti = biased_digits(s.conj ? -v.y : v.y, mx[r]);
-#pragma unroll
-            for (int q = 0; q < ND; ++q) {
-                const uint32_t w = bf16_pair(digit_float(tr, q), digit_float(ti, q));   // (re, im)
-                if (s.embed) {   // (re, -im) and (im, re)
-                    *reinterpret_cast<uint32_t*>(o + q * plane) = w ^ 0x80000000u;
-                    *reinterpret_cast<uint32_t*>(o + q * plane + 2LL * s.Kc) = __byte_perm(w, 0u, 0x1032);
+                    for (int q = 0; q < ND; ++q) {
+                        *reinterpret_cast<uint32_t*>(o + q * plane) = 0u;
+                        if (s.embed) *reinterpret_cast<uint32_t*>(o + q * plane + 2LL * s.Kc) = 0u;
+                    }
+                    if (s.mag) s.mag[f * s.Kc + k] = 0;
                 } else {
-                    *reinterpret_cast<uint32_t*>(o + q * plane) = w;
+                    const cplx v = tile[lane][r];
+                    const unsigned long long tr = biased_digits(v.x, mx[r]),
+                                             ti = biased_digits(s.conj ? -v.y : v.y, mx[r]);
+#pragma unroll
+                    for (int q = 0; q < ND; ++q) {
+                        const uint32_t w = bf16_pair(digit_float(tr, q), digit_float(ti, q));   // (re, im)
+                        if (s.embed) {   // (re, -im) and (im, re)
+                            *reinterpret_cast<uint32_t*>(o + q * plane) = w ^ 0x80000000u;
+                            *reinterpret_cast<uint32_t*>(o + q * plane + 2LL * s.Kc) = __byte_perm(w, 0u, 0x1032);
+                        } else {
+                            *reinterpret_cast<uint32_t*>(o + q * plane) = w;
+                        }
+                    }
+                    if (s.mag) {
+                        s.mag[f * s.Kc + k] = magnitude(v, mx[r]);
+                        l = l1_units(tr) + l1_units(ti);
+                    }
                 }
+            }
+            if (s.mag) {
+                l = __reduce_add_sync(0xffffffffu, l);
+                if (lane == 0) l1[r] += l;
             }
         }
         __syncthreads();
+    }
+    if (s.mag && threadIdx.x < PK_ROWS && f0 + threadIdx.x < nrow) {
+        if (gridDim.y == 1) s.l1[f0 + threadIdx.x] = l1[threadIdx.x];
+        else atomicAdd(&s.l1[f0 + threadIdx.x], l1[threadIdx.x]);
     }
 }
 
@@ -268,6 +321,13 @@ struct DigitGemm {
     int nsplit, cps;             // K ranges per tile, chunks per range
     const int* expP;             // 0x7FF: the row holds an infinity or a NaN
     const int* expQ;
+    // outputs left to digit_fix_kernel, null: none; bit i of word ((b n_qtiles +
+    // qt) Pp + p): complex Q row 32 qt + i
+    uint32_t* mask;
+    int* marked;                 // how many
+    const uint16_t *magP, *magQ;
+    const unsigned long long *l1P, *l1Q;
+    int Kc;
     cplx* W;                     // partial sums of split K (layout of splitk_f64_kernel)
     int* err;
 };
@@ -340,22 +400,214 @@ __device__ __forceinline__ double to_double(long long h, long long lo, int sc) {
     return scalbn(d, sc);
 }
 
-// One output in plain FP64 (rows with infinities or NaNs), over this work
-// item's K range.
-__device__ __noinline__ cplx plain_output(const GemmArgs& g, int m, int n, int bi, int bo, int k0, int k1) {
-    const cplx* A = g.A + bi * g.a_bi + bo * g.a_bo + m * g.a_m;
-    const cplx* B = g.B + bi * g.b_bi + bo * g.b_bo + n * g.b_n;
-    cplx s = make_double2(0.0, 0.0);
-    for (int k = k0; k < k1; ++k) {
-        cplx a = A[(k % g.Ki) * g.a_ki + (k / g.Ki) * g.a_ko], b = B[(k % g.Ki) * g.b_ki + (k / g.Ki) * g.b_ko];
-        if (g.conjA) a.y = -a.y;
-        if (g.conjB) b.y = -b.y;
-        s.x = fma(a.x, b.x, s.x);
-        s.x = fma(-a.y, b.y, s.x);
-        s.y = fma(a.x, b.y, s.y);
-        s.y = fma(a.y, b.x, s.y);
+// Plane row (complex P rows, real Q rows) where batch b starts.
+__device__ __forceinline__ int first_row(const DigitGemm& ea, int b, int vbi, int vbo, int pad) {
+    const int bi = b % ea.g.Bi, bo = b / ea.g.Bi;
+    return ((vbi ? bi : 0) + (vbo ? bo * (vbi ? ea.g.Bi : 1) : 0)) * pad;
+}
+
+__device__ __forceinline__ void store_output(const DigitGemm& ea, int m, int n, int bi, int bo, cplx r) {
+    const GemmArgs& g = ea.g;
+    cplx* cp = g.C + bi * g.c_bi + bo * g.c_bo + m * g.c_m + n * g.c_n;
+    if (!(g.alpha.x == 1.0 && g.alpha.y == 0.0)) {
+        const cplx v = r;
+        r.x = g.alpha.x * v.x - g.alpha.y * v.y;
+        r.y = g.alpha.x * v.y + g.alpha.y * v.x;
     }
-    return s;
+    if (!(g.beta.x == 0.0 && g.beta.y == 0.0)) {
+        const cplx o = *cp;
+        if (g.beta.x == 1.0 && g.beta.y == 0.0) {
+            r.x += o.x;
+            r.y += o.y;
+        } else {
+            r.x += g.beta.x * o.x - g.beta.y * o.y;
+            r.y += g.beta.x * o.y + g.beta.y * o.x;
+        }
+    }
+    *cp = r;
+}
+
+// --------------------------------------------------------------- the check
+// S = sum_k max(|re|, |im|)_p max(|re|, |im|)_q 2^-(Ep + Eq), at most
+// sum |p_k||q_k| in those units, for 32 x 32 outputs per warp.  With l the l1
+// sums, the digits' error is below 2^-56 (l_p + l_q) + K 2^-60 and an FMA chain's
+// bound is 2 K 2^-53 S: marked is what has S < (l_p + l_q) / (16 K) + 2^-8, except
+// S = 0 (every product zero, and so is the digits' result), and rows with
+// infinities or NaNs.  Operands of one size reach the threshold within the
+// first few dozen K, and the warp stops there: only graded and sparse rows
+// are summed to the end.  The order of K is free, so a lane loads 16 bytes of
+// a row and feeds them to two k16 steps.
+constexpr int CK_THREADS = 128;
+__global__ void __launch_bounds__(CK_THREADS) digit_check_kernel(DigitGemm ea) {
+    pdl_begin();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nqc = ea.n_qtiles, npc = ea.Pp / 64, nq2 = (nqc + 1) / 2;   // 32-wide Q groups, 64 x 64 blocks
+    const int blk = (int)(blockIdx.x % (unsigned)(npc * nq2)), b = (int)(blockIdx.x / (unsigned)(npc * nq2));
+    const int p0 = (blk % npc) * 64 + (warp & 1) * 32, qt = (blk / npc) * 2 + (warp >> 1), q0 = qt * 32;
+    if (qt >= nqc) return;
+    const long long prow = first_row(ea, b, ea.p_vbi, ea.p_vbo, ea.Pp) + p0;
+    const long long qrow = first_row(ea, b, ea.q_vbi, ea.q_vbo, ea.Qp) / 2 + q0;
+    const int g8 = lane >> 2, j4 = lane & 3;
+    const float c1 = 1.01f / (16.0f * 65536.0f * (float)(ea.g.Ki * ea.g.Ko));
+    float lp[4], lq[8];                        // thresholds' parts: rows g8 + 8 i, columns 8 i + 2 j4 and + 1
+    bool pbad[4], qbad[8];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        lp[i] = 0.00391f + c1 * (float)ea.l1P[prow + g8 + 8 * i];
+        pbad[i] = ea.expP[prow + g8 + 8 * i] == 0x7FF;
+    }
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+        const int c = 8 * (i >> 1) + 2 * j4 + (i & 1);
+        lq[i] = c1 * (float)ea.l1Q[qrow + c];
+        qbad[i] = ea.expQ[qrow + c] == 0x7FF;
+    }
+    float acc[2][4][4];
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) acc[i][j][e] = 0.f;
+    // marks of this lane: row i (g8 + 8 i), column c (8 (c >> 1) + 2 j4 + (c & 1))
+    auto marks = [&](bool final) {
+        unsigned out[4] = {0u, 0u, 0u, 0u}, any = 0;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const float S = acc[i >> 1][c >> 1][(i & 1) * 2 + (c & 1)];
+                const bool valid = p0 + g8 + 8 * i < ea.Pn && q0 + 8 * (c >> 1) + 2 * j4 + (c & 1) < ea.Qn;
+                const bool low = S < lp[i] + lq[c] && !(final && S == 0.f);
+                if (valid && (low || (final && (pbad[i] || qbad[c])))) out[i] |= 1u << (8 * (c >> 1) + 2 * j4 + (c & 1));
+            }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) any |= out[i];
+        if (final) {
+            unsigned n = 0;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                unsigned w = out[i];
+                w |= __shfl_xor_sync(0xffffffffu, w, 1);
+                w |= __shfl_xor_sync(0xffffffffu, w, 2);
+                if (j4 == 0) {
+                    ea.mask[((long long)b * nqc + qt) * ea.Pp + p0 + g8 + 8 * i] = w;
+                    n += __popc(w);
+                }
+            }
+            n = __reduce_add_sync(0xffffffffu, n);
+            if (lane == 0 && n) atomicAdd(ea.marked, (int)n);
+        }
+        return any != 0;
+    };
+    const uint16_t* mp = ea.magP + (prow + g8) * ea.Kc;
+    const uint16_t* mq = ea.magQ + (qrow + g8) * ea.Kc;
+    for (int k0 = 0, it = 1; k0 < ea.Kc; k0 += 32, ++it) {
+        const int k = k0 + 8 * j4;
+        const bool in = k < ea.Kc;             // Kc is a multiple of 16
+        uint4 a[4], bq[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            a[i] = in ? *reinterpret_cast<const uint4*>(mp + 8LL * i * ea.Kc + k) : make_uint4(0, 0, 0, 0);
+            bq[i] = in ? *reinterpret_cast<const uint4*>(mq + 8LL * i * ea.Kc + k) : make_uint4(0, 0, 0, 0);
+        }
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                float* d = acc[i][j];
+                asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                             : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                             : "r"(a[2 * i].x), "r"(a[2 * i + 1].x), "r"(a[2 * i].y), "r"(a[2 * i + 1].y), "r"(bq[j].x), "r"(bq[j].y));
+                asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
+                             : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+                             : "r"(a[2 * i].z), "r"(a[2 * i + 1].z), "r"(a[2 * i].w), "r"(a[2 * i + 1].w), "r"(bq[j].z), "r"(bq[j].w));
+            }
+        if ((it & 3) == 0 && !__any_sync(0xffffffffu, marks(false))) break;
+    }
+    marks(true);
+}
+
+// The marked outputs in plain FP64.  A block takes 256 words of the mask (8192
+// outputs) at a time, lists its marked outputs and gives each 1 to 32 lanes,
+// as many as keep its 256 threads busy; the lanes' sums are added in a fixed
+// order.
+constexpr int FX_THREADS = 256;
+__global__ void __launch_bounds__(FX_THREADS) digit_fix_kernel(DigitGemm ea) {
+    pdl_begin();
+    if (*(volatile int*)ea.marked == 0) return;
+    __shared__ uint16_t list[FX_THREADS * 32];
+    __shared__ int wsum[FX_THREADS / 32];
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const GemmArgs& g = ea.g;
+    const int K = g.Ki * g.Ko;
+    const long long words = (long long)ea.batches * ea.n_qtiles * ea.Pp;   // a multiple of 128
+    for (long long w0 = (long long)blockIdx.x * FX_THREADS; w0 < words; w0 += (long long)gridDim.x * FX_THREADS) {
+        unsigned w = w0 + t < words ? ea.mask[w0 + t] : 0u;
+        int pos = __popc(w);
+        for (int o = 1; o < 32; o *= 2) {
+            const int v = __shfl_up_sync(0xffffffffu, pos, o);
+            if (lane >= o) pos += v;
+        }
+        __syncthreads();   // the list of the last round has been read
+        if (lane == 31) wsum[warp] = pos;
+        __syncthreads();
+        int n = 0;
+        pos -= __popc(w);
+        for (int q = 0; q < FX_THREADS / 32; ++q) {
+            if (q < warp) pos += wsum[q];
+            n += wsum[q];
+        }
+        while (w) {
+            const int i = __ffs((int)w) - 1;
+            w &= w - 1;
+            list[pos++] = (uint16_t)(t * 32 + i);
+        }
+        __syncthreads();
+        int L = 1;
+        while (L < 32 && n * L * 2 <= FX_THREADS) L *= 2;
+        for (int e0 = 0; e0 < n; e0 += FX_THREADS / L) {
+            const int e = e0 + t / L;
+            cplx s = make_double2(0.0, 0.0);
+            int m = 0, nn = 0, bi = 0, bo = 0, b = 0;
+            if (e < n) {
+                const long long word = w0 + (list[e] >> 5);
+                const int p = (int)(word % ea.Pp);
+                const long long rest = word / ea.Pp;
+                const int q = (int)(rest % ea.n_qtiles) * 32 + (list[e] & 31);
+                b = (int)(rest / ea.n_qtiles);
+                bi = b % g.Bi;
+                bo = b / g.Bi;
+                m = ea.swapped ? q : p;
+                nn = ea.swapped ? p : q;
+                const cplx* A = g.A + bi * g.a_bi + bo * g.a_bo + m * g.a_m;
+                const cplx* B = g.B + bi * g.b_bi + bo * g.b_bo + nn * g.b_n;
+#pragma unroll 4
+                for (int k = t % L; k < K; k += L) {
+                    const int ki = k % g.Ki, ko = k / g.Ki;
+                    cplx a = A[ki * g.a_ki + ko * g.a_ko], v = B[ki * g.b_ki + ko * g.b_ko];
+                    if (g.conjA) a.y = -a.y;
+                    if (g.conjB) v.y = -v.y;
+                    s.x = fma(a.x, v.x, s.x);
+                    s.x = fma(-a.y, v.y, s.x);
+                    s.y = fma(a.x, v.y, s.y);
+                    s.y = fma(a.y, v.x, s.y);
+                }
+            }
+            for (int o = L / 2; o > 0; o /= 2) {
+                s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
+                s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
+            }
+            if (e < n && t % L == 0) {
+                if (ea.nsplit > 1) {   // the whole sum in the first range's place
+                    for (int ks = 0; ks < ea.nsplit; ++ks)
+                        ea.W[(((long long)ks * ea.batches + b) * g.N + nn) * g.M + m] = ks ? make_double2(0.0, 0.0) : s;
+                } else {
+                    store_output(ea, m, nn, bi, bo, s);
+                }
+            }
+        }
+    }
 }
 
 __global__ void __launch_bounds__(THREADS, 1)
@@ -372,13 +624,15 @@ __global__ void __launch_bounds__(THREADS, 1)
 
     // an earlier launch on this workspace gave up: do nothing (the host
     // reports the error at its next check)
-    __shared__ int s_skip;
-    if (threadIdx.x == 0) s_skip = *(volatile int*)ea.err;
+    __shared__ int s_skip, s_marked;
+    if (threadIdx.x == 0) {
+        s_skip = *(volatile int*)ea.err;
+        s_marked = ea.mask && *(volatile int*)ea.marked;
+    }
     __syncthreads();
     if (s_skip) return;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int nchunk = (ea.nst + CHUNK_ST - 1) / CHUNK_ST;
     const long long grid_tiles = (long long)ea.n_ptiles * ea.n_qtiles;
     const long long ntiles = grid_tiles * ea.batches * ea.nsplit;
     auto tile_of = [&](long long t, int& pt, int& qt, int& b, int& ks) {
@@ -393,12 +647,6 @@ __global__ void __launch_bounds__(THREADS, 1)
         b = (int)(rest % ea.batches);
         ks = (int)(rest / ea.batches);
     };
-    // plane rows (complex P rows, real Q rows) where batch b starts
-    auto row0 = [&](int b, int vbi, int vbo, int pad) {
-        const int bi = b % ea.g.Bi, bo = b / ea.g.Bi;
-        return ((vbi ? bi : 0) + (vbo ? bo * (vbi ? ea.g.Bi : 1) : 0)) * pad;
-    };
-
     if (threadIdx.x == 0) {
         for (int s = 0; s < STAGES; ++s) {
             mbar_init(&full[s], 1);
@@ -428,8 +676,8 @@ __global__ void __launch_bounds__(THREADS, 1)
             for (long long t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
                 int pt, qt, b, ks;
                 tile_of(t, pt, qt, b, ks);
-                const int prow = row0(b, ea.p_vbi, ea.p_vbo, ea.Pp) + pt * BM;
-                const int qrow = row0(b, ea.q_vbi, ea.q_vbo, ea.Qp) + qt * BN;
+                const int prow = first_row(ea, b, ea.p_vbi, ea.p_vbo, ea.Pp) + pt * BM;
+                const int qrow = first_row(ea, b, ea.q_vbi, ea.q_vbo, ea.Qp) + qt * BN;
                 const int st0 = ks * ea.cps * CHUNK_ST, st1 = min(ea.nst, (ks + 1) * ea.cps * CHUNK_ST);
                 for (int st = st0; st < st1; ++st, ++it) {
                     const unsigned s = it % STAGES, round = it / STAGES;
@@ -503,9 +751,6 @@ __global__ void __launch_bounds__(THREADS, 1)
         __syncwarp();
     } else {
         const int quad = warp & 3, col0 = (warp >> 2) * DCOLS;
-        const bool a1 = ea.g.alpha.x == 1.0 && ea.g.alpha.y == 0.0;
-        const bool b0 = ea.g.beta.x == 0.0 && ea.g.beta.y == 0.0;
-        const bool b1 = ea.g.beta.x == 1.0 && ea.g.beta.y == 0.0;
         unsigned cg = 0;
         bool ok = true;
         for (long long t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
@@ -541,45 +786,29 @@ __global__ void __launch_bounds__(THREADS, 1)
             }
             if (!ok) break;
             const int p = pt * BM + quad * 32 + lane;
-            if (p >= ea.Pn) continue;
-            const int bi = b % ea.g.Bi, bo = b / ea.g.Bi;
-            const int ep = ea.expP[row0(b, ea.p_vbi, ea.p_vbo, ea.Pp) + p];
-            const int* eq = ea.expQ + row0(b, ea.q_vbi, ea.q_vbo, ea.Qp) / 2;
+            if (p < ea.Pn) {
+                const int bi = b % ea.g.Bi, bo = b / ea.g.Bi;
+                const int ep = ea.expP[first_row(ea, b, ea.p_vbi, ea.p_vbo, ea.Pp) + p];
+                const int* eq = ea.expQ + first_row(ea, b, ea.q_vbi, ea.q_vbo, ea.Qp) / 2;
+                const uint32_t left = s_marked ? ea.mask[((long long)b * ea.n_qtiles + qt) * ea.Pp + p] >> (col0 >> 1) : 0u;
 #pragma unroll
-            for (int j = 0; j < DCOLS; j += 2) {
-                const int q = (qt * BN + col0 + j) >> 1;
-                if (q >= ea.Qn) continue;
-                const int e = eq[q];
-                const int m = ea.swapped ? q : p, n = ea.swapped ? p : q;
-                cplx r;
-                if (ep == 0x7FF || e == 0x7FF) {
-                    r = plain_output(ea.g, m, n, bi, bo, st0 * BK / 2, min(ea.g.Ki * ea.g.Ko, st1 * BK / 2));
-                } else {
-                    const int sc = max(ep, 1) + max(e, 1) - 2 * 1022 - 70;   // E_p + E_q - 110 + 40
-                    r = make_double2(to_double(sh[j], sl[j], sc), to_double(sh[j + 1], sl[j + 1], sc));
-                }
-                if (ea.nsplit > 1) {
-                    ea.W[(((long long)ks * ea.batches + b) * ea.g.N + n) * ea.g.M + m] = r;
-                    continue;
-                }
-                cplx* cp = ea.g.C + bi * ea.g.c_bi + bo * ea.g.c_bo + m * ea.g.c_m + n * ea.g.c_n;
-                if (!a1) {
-                    const cplx v = r;
-                    r.x = ea.g.alpha.x * v.x - ea.g.alpha.y * v.y;
-                    r.y = ea.g.alpha.x * v.y + ea.g.alpha.y * v.x;
-                }
-                if (!b0) {
-                    const cplx o = *cp;
-                    if (b1) {
-                        r.x += o.x;
-                        r.y += o.y;
+                for (int j = 0; j < DCOLS; j += 2) {
+                    const int q = (qt * BN + col0 + j) >> 1;
+                    if (q >= ea.Qn || ((left >> (j >> 1)) & 1u)) continue;
+                    const int e = eq[q];
+                    const int m = ea.swapped ? q : p, n = ea.swapped ? p : q;
+                    cplx r;
+                    if (ep == 0x7FF || e == 0x7FF) {   // only without the check
+                        r = make_double2(CUDART_NAN, CUDART_NAN);
                     } else {
-                        r.x += ea.g.beta.x * o.x - ea.g.beta.y * o.y;
-                        r.y += ea.g.beta.x * o.y + ea.g.beta.y * o.x;
+                        const int sc = max(ep, 1) + max(e, 1) - 2 * 1022 - 70;   // E_p + E_q - 110 + 40
+                        r = make_double2(to_double(sh[j], sl[j], sc), to_double(sh[j + 1], sl[j + 1], sc));
                     }
+                    if (ea.nsplit > 1) ea.W[(((long long)ks * ea.batches + b) * ea.g.N + n) * ea.g.M + m] = r;
+                    else store_output(ea, m, n, bi, bo, r);
                 }
-                *cp = r;
             }
+            __syncwarp();
         }
     }
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -601,10 +830,10 @@ struct DPlan {
     DigitGemm d{};
     long long np = 0, nq = 0;             // packed batches of P and Q
     int Kp = 0;
-    size_t p_off = 0, q_off = 0, ep_off = 0, eq_off = 0, w_off = 0, bytes = 0;
+    size_t p_off = 0, q_off = 0, ep_off = 0, eq_off = 0, lp_off = 0, lq_off = 0, mp_off = 0, mq_off = 0, mask_off = 0, w_off = 0, bytes = 0;
 };
 
-DPlan plan(const GemmArgs& g) {
+DPlan plan(const GemmArgs& g, bool elementwise) {
     DPlan pl;
     const long long K = (long long)g.Ki * g.Ko;
     if (g.M <= 0 || g.N <= 0 || K <= 0 || g.Bi <= 0 || g.Bo <= 0) return pl;
@@ -657,8 +886,18 @@ DPlan plan(const GemmArgs& g) {
     };
     pl.ep_off = take(sizeof(int) * pl.np * d.Pp);
     pl.eq_off = take(sizeof(int) * pl.nq * (d.Qp / 2));
+    if (elementwise) {
+        pl.lp_off = take(sizeof(unsigned long long) * pl.np * d.Pp);
+        pl.lq_off = take(sizeof(unsigned long long) * pl.nq * (d.Qp / 2));
+    }
     pl.p_off = take((size_t)ND * pl.np * d.Pp * pl.Kp * 2);
     pl.q_off = take((size_t)ND * pl.nq * d.Qp * pl.Kp * 2);
+    d.Kc = pl.Kp / 2;
+    if (elementwise) {
+        pl.mp_off = take((size_t)pl.np * d.Pp * d.Kc * 2);
+        pl.mq_off = take((size_t)pl.nq * (d.Qp / 2) * d.Kc * 2);
+        pl.mask_off = take(sizeof(uint32_t) * (size_t)d.batches * d.n_qtiles * d.Pp);
+    }
     if (d.nsplit > 1) pl.w_off = take((size_t)d.nsplit * d.batches * g.M * (size_t)g.N * sizeof(cplx));
     pl.bytes = off;
     pl.ok = pl.np * d.Pp < (1LL << 31) && pl.nq * d.Qp < (1LL << 31);
@@ -703,38 +942,39 @@ bool halve(const GemmArgs& g, GemmArgs& lo, GemmArgs& hi) {
 }  // namespace
 
 // Rule: digits pay once the FP64 pipe would take longer than the fixed cost
-// of packing both sides plus the tile work (measured at the border: 4096 x 64 x
-// 64 280 us on the FP64 pipe, 48 in digits; 64 x 64 x 64 9 us and 13).
+// of packing and checking both sides plus the tile work (measured at the border:
+// 4096 x 64 x 64 280 us on the FP64 pipe, 55 in digits; 64 x 64 x 64 9 us and 20).
 bool digits_wanted(const GemmArgs& g) {
     const double K = (double)g.Ki * g.Ko, macs = (double)g.M * g.N * K * g.Bi * (double)g.Bo;
     if (std::min(g.M, g.N) < 16 || std::max(g.M, g.N) < 32 || K < 16) return false;
-    DPlan pl = plan(g);
+    DPlan pl = plan(g, true);
     if (!pl.ok || !encode_fn()) return false;
     const double f64_us = 4.0 + 8.0 * macs / 1.0e6;
     const double chunks = (double)pl.d.n_ptiles * pl.d.n_qtiles * pl.d.batches * ((pl.d.nst + CHUNK_ST - 1) / CHUNK_ST);
-    const double us = 16.0 + 6.5 * std::max(1.0, chunks / N_SM) + (double)pl.bytes / 2.0e6;
+    const double us = 23.0 + 6.5 * std::max(1.0, chunks / N_SM) + (double)pl.bytes / 2.0e6;
     return us < f64_us;
 }
 
-size_t digits_workspace_bytes(const GemmArgs& g) {
-    DPlan pl = plan(g);
+size_t digits_workspace_bytes(const GemmArgs& g, bool elementwise) {
+    DPlan pl = plan(g, elementwise);
     if (!pl.ok) return 0;
     if ((long long)pl.bytes > MAX_PLANE_BYTES) {
         GemmArgs lo, hi;
-        if (halve(g, lo, hi)) return std::max(digits_workspace_bytes(lo), digits_workspace_bytes(hi));
+        if (halve(g, lo, hi)) return std::max(digits_workspace_bytes(lo, elementwise), digits_workspace_bytes(hi, elementwise));
     }
     return pl.bytes;
 }
 
-int launch_zgemm_digits(const GemmArgs& g, cudaStream_t stream, void* workspace, size_t workspace_bytes) {
-    DPlan pl = plan(g);
+int launch_zgemm_digits(const GemmArgs& g, bool elementwise, cudaStream_t stream, void* workspace,
+                        size_t workspace_bytes) {
+    DPlan pl = plan(g, elementwise);
     if (!pl.ok || !encode_fn()) return -1;
     if ((long long)pl.bytes > MAX_PLANE_BYTES) {
         GemmArgs lo, hi;
         if (halve(g, lo, hi)) {
-            const int a = launch_zgemm_digits(lo, stream, workspace, workspace_bytes);
+            const int a = launch_zgemm_digits(lo, elementwise, stream, workspace, workspace_bytes);
             if (a < 0) return a;
-            const int b = launch_zgemm_digits(hi, stream, workspace, workspace_bytes);
+            const int b = launch_zgemm_digits(hi, elementwise, stream, workspace, workspace_bytes);
             return b < 0 ? b : a + b;
         }
     }
@@ -762,6 +1002,10 @@ int launch_zgemm_digits(const GemmArgs& g, cudaStream_t stream, void* workspace,
         s.rows = p ? pl.np * d.Pp : pl.nq * d.Qp;
         s.planes = reinterpret_cast<uint16_t*>(ws + (p ? pl.p_off : pl.q_off));
         s.exps = reinterpret_cast<int*>(ws + (p ? pl.ep_off : pl.eq_off));
+        if (elementwise) {
+            s.mag = reinterpret_cast<uint16_t*>(ws + (p ? pl.mp_off : pl.mq_off));
+            s.l1 = reinterpret_cast<unsigned long long*>(ws + (p ? pl.lp_off : pl.lq_off));
+        }
         return s;
     };
     const DigitSide sp = side(true), sq = side(false);
@@ -778,7 +1022,8 @@ int launch_zgemm_digits(const GemmArgs& g, cudaStream_t stream, void* workspace,
         launch(digit_max_kernel, grid, PK_THREADS, 0, stream, sp, sq, nbp, kb);
         ++launches;
     }
-    launch(digit_pack_kernel, grid, PK_THREADS, 0, stream, sp, sq, nbp, kb, one);
+    d.marked = elementwise ? reinterpret_cast<int*>(ws) + 1 : nullptr;
+    launch(digit_pack_kernel, grid, PK_THREADS, 0, stream, sp, sq, nbp, kb, one, d.marked);
     ++launches;
     CUtensorMap mP, mQ;
     if (!make_map3(&mP, sp.planes, sp.rows, pl.Kp, BM) || !make_map3(&mQ, sq.planes, sq.rows, pl.Kp, BN)) return -1;
@@ -800,9 +1045,24 @@ int launch_zgemm_digits(const GemmArgs& g, cudaStream_t stream, void* workspace,
     d.expQ = sq.exps;
     d.W = d.nsplit > 1 ? reinterpret_cast<cplx*>(ws + pl.w_off) : nullptr;
     d.err = reinterpret_cast<int*>(ws);
+    if (elementwise) {
+        d.mask = reinterpret_cast<uint32_t*>(ws + pl.mask_off);
+        d.magP = sp.mag;
+        d.magQ = sq.mag;
+        d.l1P = sp.l1;
+        d.l1Q = sq.l1;
+        launch(digit_check_kernel, (unsigned)((d.Pp / 64) * ((d.n_qtiles + 1) / 2) * d.batches), CK_THREADS, 0, stream, d);
+        ++launches;
+    }
     const long long nt = (long long)d.n_ptiles * d.n_qtiles * d.batches * d.nsplit;
     launch(digit_gemm_kernel, (unsigned)std::min<long long>(nt, N_SM), THREADS, SMEM_BYTES, stream, mP, mQ, d);
     ++launches;
+    if (elementwise) {
+        const long long words = (long long)d.batches * d.n_qtiles * d.Pp;
+        launch(digit_fix_kernel, (unsigned)std::min<long long>((words + FX_THREADS - 1) / FX_THREADS, N_SM), FX_THREADS, 0,
+               stream, d);
+        ++launches;
+    }
     if (d.nsplit > 1) launches += launch_splitk_f64(g, d.nsplit, d.W, stream);
     return launches;
 }

@@ -286,11 +286,11 @@ size_t qr_panel_scratch(int D) {   // complex: S and C, Gq, column norms and exp
 }
 
 size_t qr_panel_workspace(int M, int D) {
-    size_t need = digits_workspace_bytes(r_args(nullptr, nullptr, M, D, nullptr));
+    size_t need = digits_workspace_bytes(r_args(nullptr, nullptr, M, D, nullptr), false);
     for (int n = 0; n < D; n += PB) {
         const int bp = std::min(PB, D - n);
-        need = std::max(need, std::max(digits_workspace_bytes(gram_args(nullptr, M, n, bp, nullptr)),
-                                       digits_workspace_bytes(update_args(nullptr, M, n, bp, nullptr))));
+        need = std::max(need, std::max(digits_workspace_bytes(gram_args(nullptr, M, n, bp, nullptr), false),
+                                       digits_workspace_bytes(update_args(nullptr, M, n, bp, nullptr), false)));
     }
     return need;
 }
@@ -313,7 +313,7 @@ int qr_panel(const cplx* A, cplx* Q, int M, int D, cplx* R, QrScratch& ws, cudaS
     for (int n = first; n < last; n += PB) {
         const int bp = std::min(PB, D - n), ld = n + bp;
         for (int pass = 1; pass <= 2; ++pass) {
-            int l = launch_zgemm_digits(gram_args(Q, M, n, bp, S), s, workspace, workspace_bytes);
+            int l = launch_zgemm_digits(gram_args(Q, M, n, bp, S), false, s, workspace, workspace_bytes);
             if (l < 0) return -1;
             launches += l;
             if (n > 0) {   // -S_q^H S_q
@@ -336,7 +336,7 @@ int qr_panel(const cplx* A, cplx* Q, int M, int D, cplx* R, QrScratch& ws, cudaS
                 launches += launch_zgemm_f64(g, s);
             }
             // in place: the operands are packed before the first output is written
-            l = launch_zgemm_digits(update_args(Q, M, n, bp, C), s, workspace, workspace_bytes);
+            l = launch_zgemm_digits(update_args(Q, M, n, bp, C), false, s, workspace, workspace_bytes);
             if (l < 0) return -1;
             launches += l;
         }
@@ -345,7 +345,7 @@ int qr_panel(const cplx* A, cplx* Q, int M, int D, cplx* R, QrScratch& ws, cudaS
         launch(panel_report_kernel, 1, 1, 0, s, flag, pub);
         return launches + 1;
     }
-    const int l = launch_zgemm_digits(r_args(Q, A, M, D, R), s, workspace, workspace_bytes);
+    const int l = launch_zgemm_digits(r_args(Q, A, M, D, R), false, s, workspace, workspace_bytes);
     if (l < 0) return -1;
     launch(panel_finish_kernel, 1, FT, 0, s, R, D, flag, pub);
     return launches + l + 1;

@@ -345,10 +345,10 @@ void gemm(ttn_ctx* c, const GemmArgs& g) {
         }
     }
     if (n < 0 && digits_wanted(g)) {   // large FP64 contractions: exact digit products on the tensor cores
-        const size_t need = digits_workspace_bytes(g);
+        const size_t need = digits_workspace_bytes(g, true);
         if (try_grow_split_ws(c, need)) {   // no room: the FP64 kernels below need none
             ProfScope ps(c, PK_F64, fl, 0.0, &g);
-            n = launch_zgemm_digits(g, c->stream, c->split_ws, c->split_cap);
+            n = launch_zgemm_digits(g, true, c->stream, c->split_ws, c->split_cap);
             if (n >= 0) c->digits_run = true;
         }
     }
