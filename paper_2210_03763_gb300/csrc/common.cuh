@@ -299,7 +299,12 @@ size_t qr_panel_scratch(int D);
 size_t qr_panel_workspace(int M, int D);
 int qr_panel(const cplx* A, cplx* Q, int M, int D, cplx* R, QrScratch& ws, cudaStream_t s, void* workspace,
              size_t workspace_bytes, int first, int last, const Publish& pub);
-// fine_rows: spread the rows of small matrices over all SMs (see qr.cu).
+// Reports qr_flag != 0 if R, from another QR of the matrix, has a diagonal
+// that qr_panel is sure to refuse.  Returns launches.
+int qr_panel_verdict(const cplx* R, int D, cudaStream_t s, const Publish& pub);
+// fine_rows: spread the rows of small matrices over all SMs (see qr.cu);
+// qr_one_block: no difference, a single block either way.
+constexpr bool qr_one_block(int M, int D) { return M <= QR_ROWS && D <= 16; }
 int qr_cgs2(cplx* A, int M, int D, cplx* R, const int* cand, int ncand,
             QrScratch& ws, cudaStream_t s, int* n_dependent_host, bool fine_rows = false, double tol = QR_TOL_FP64);
 

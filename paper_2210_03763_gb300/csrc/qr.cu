@@ -1453,19 +1453,18 @@ int qr_cgs2(cplx* A, int M, int D, cplx* R, const int* cand, int ncand, QrScratc
     // (with no cached columns and a window of 4, the 512 blocks of 65536-row
     // matrices are co-resident); with fine_rows at least 8, as many as spread
     // the matrix over every SM (at most 64 rows: most of the kept columns then
-    // stay in shared memory; up to 128: 64 of them).  The caller asks for that
-    // where it expects dependent columns: full-rank matrices go to the panel
-    // path, and the ill-conditioned ones that it leaves keep 128 rows and with
-    // them the order of the sums, to whose rounding their nearly dependent
-    // columns are sensitive.  Measured, full rank, ms per call, blocks of 128
-    // rows -> fine_rows: 81 x 81 2.49 -> 1.11, 128 x 128 7.2 -> 1.95, 6561 x 128
-    // 8.5 -> 4.2
+    // stay in shared memory; up to 128: 64 of them).  The caller takes that for
+    // matrices with dependent columns: full-rank ones go to the panel path, and
+    // the ill-conditioned ones that it leaves keep 128 rows and with them the
+    // order of the sums, to whose rounding their nearly dependent columns are
+    // sensitive.  Measured, full rank, ms per call, blocks of 128 rows ->
+    // fine_rows: 81 x 81 2.49 -> 1.11, 128 x 128 7.2 -> 1.95, 6561 x 128 8.5 -> 4.2
     bool coop_done = false;
     const Publish pub = ws.hs ? Publish{ws.hs, ++*ws.seq, nullptr} : Publish{};
     if (D <= MAXD) {
         const int nsm = std::min(coop_sms(), QR_SMALL_BLOCKS);
         // few columns and rows: one block, no synchronisation at all
-        const bool coarse = !fine_rows || nsm == 0 || (M <= QB && D <= 16);
+        const bool coarse = !fine_rows || nsm == 0 || qr_one_block(M, D);
         int rpb = coarse ? QB : std::min(QB, std::max(8, (M + nsm - 1) / nsm)), rb = 8;
         while (rb < rpb) rb *= 2;
         struct Opt {

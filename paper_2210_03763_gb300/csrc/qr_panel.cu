@@ -14,7 +14,7 @@
 // Accuracy.  A digit contraction holds a row of its operand on one grid, 2^-55 of
 // the row's largest entry, so the rows of [Q W] are only held well if Q and W
 // are of one size: unscaled, W lost 1e-15 / |A| of itself (1e-9 of a matrix of
-// norm 1e-6).  Scaled, |Q R - A| is below 5e-16 of every column on its own scale
+// norm 1e-6).  Scaled, |Q R - A| is below 1e-15 of every column on its own scale
 // (the column loop: 2e-16).  R multiplied up from the passes' factors instead of
 // Q^H A lost up to the panel's condition number times 2^-55 (1e-13 of a column
 // 2e-4 away from the span of the others); the product costs 0.16 ms of 16384 x 128
@@ -23,9 +23,8 @@
 // The column-by-column rule (qr.cu) decides which columns are dependent; this
 // path is for matrices without any: it gives up (the flag) as soon as a
 // column's part outside the earlier ones is below 1e-4 of the column or 1e-8
-// of |A|_F, far above the rule's 1e-10, and when |A| is within 2^+-480 of the
-// ends of the FP64 range, and the caller runs the column loop on the original
-// matrix.  Q and R are then the same as the column loop's up to rounding (R has
+// of |A|_F, far above the rule's 1e-10, and when |A| lies outside 2^+-480, and the
+// caller runs the column loop on the original matrix.  Q and R are then the same as the column loop's up to rounding (R has
 // a positive real diagonal, which makes them unique).
 //
 // Why: 16 M D^2 flops of the column loop take 4.1 ms on the FP64 pipe for a
@@ -201,47 +200,71 @@ __global__ void panel_report_kernel(const int* flag, Publish pub) {
     panel_publish(pub, *flag);
 }
 
+// By a whole block, col2 and diag (of D) in shared memory: squared column
+// norms and the diagonal of the upper triangular R.  A warp per column; tidy:
+// clear what is below the diagonal and the diagonal's imaginary part first.
+__device__ void r_columns(cplx* R, int D, bool tidy, double* col2, double* diag) {
+    const int lane = threadIdx.x & 31;
+    for (int k = threadIdx.x >> 5; k < D; k += FT / 32) {
+        cplx* r = R + (long long)k * D;
+        double s = 0.0;
+        for (int i = lane; i < (tidy ? D : k + 1); i += 32) {
+            cplx x = r[i];
+            if (i > k) x = make_double2(0.0, 0.0);
+            if (i == k) {
+                x.y = 0.0;
+                diag[k] = x.x;
+            }
+            if (tidy && i >= k) r[i] = x;
+            s = fma(x.x, x.x, fma(x.y, x.y, s));
+        }
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (lane == 0) col2[k] = s;
+    }
+    __syncthreads();
+}
+
+// By one warp: does a diagonal entry lie below `margin` times the limits?
+__device__ bool r_refused(const double* col2, const double* diag, int D, double margin) {
+    const int lane = threadIdx.x & 31;
+    double f = 0.0;
+    for (int k = lane; k < D; k += 32) f += col2[k];
+    for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
+    bool bad = false;
+    for (int k = lane; k < D; k += 32) {
+        const double d = diag[k], d2 = d * d;
+        if (!(d > 0.0 && d2 >= margin * MIN_COL2 * col2[k] && d2 > margin * MIN_FRO2 * f)) bad = true;
+    }
+    return __any_sync(0xffffffffu, bad);
+}
+
 // R = Q^H A made upper triangular with a real diagonal, and the residuals
-// checked once more on the final R: sets *flag as panel_chol_kernel.  One
-// block, a warp per column.
+// checked once more on the final R (the Gram matrices know them less well):
+// sets *flag as panel_chol_kernel.  One block.
 __global__ void __launch_bounds__(FT) panel_finish_kernel(cplx* R, int D, int* flag, Publish pub) {
     pdl_begin();
     __shared__ double col2[256], diag[256];
-    const int lane = threadIdx.x & 31;
     const bool gave_up = *(volatile int*)flag != 0;   // R has not been written
     __syncthreads();
-    if (!gave_up)
-        for (int k = threadIdx.x >> 5; k < D; k += FT / 32) {
-            cplx* r = R + (long long)k * D;
-            double s = 0.0;
-            for (int i = lane; i < D; i += 32) {
-                cplx x = r[i];
-                if (i > k) x = make_double2(0.0, 0.0);
-                if (i == k) {
-                    x.y = 0.0;
-                    diag[k] = x.x;
-                }
-                if (i >= k) r[i] = x;
-                s = fma(x.x, x.x, fma(x.y, x.y, s));
-            }
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if (lane == 0) col2[k] = s;
-        }
-    __syncthreads();
+    if (!gave_up) r_columns(R, D, true, col2, diag);
     if (threadIdx.x >= 32) return;
-    int bad = gave_up;
-    if (!gave_up) {
-        double f = 0.0;
-        for (int k = lane; k < D; k += 32) f += col2[k];
-        for (int o = 16; o > 0; o >>= 1) f += __shfl_xor_sync(0xffffffffu, f, o);
-        for (int k = lane; k < D; k += 32) {
-            const double d = diag[k], d2 = d * d;
-            if (!(d > 0.0 && d2 >= MIN_COL2 * col2[k] && d2 > MIN_FRO2 * f)) bad = 1;
-        }
-        bad = __any_sync(0xffffffffu, bad);
-        if (bad && lane == 0) *flag = 1;
+    const bool bad = gave_up || r_refused(col2, diag, D, 1.0);
+    if (threadIdx.x == 0) {
+        if (bad) *flag = 1;
+        panel_publish(pub, bad);
     }
-    if (lane == 0) panel_publish(pub, bad);
+}
+
+// The final check on another QR's R: its diagonal agrees with the panels' to
+// 1e-11 at the limits (2^-53 |a| against 1e-4 |a|), so what is below 0.9 of them is
+// refused for certain.  One block.
+__global__ void __launch_bounds__(FT) panel_verdict_kernel(cplx* R, int D, Publish pub) {
+    pdl_begin();
+    __shared__ double col2[256], diag[256];
+    r_columns(R, D, false, col2, diag);
+    if (threadIdx.x >= 32) return;
+    const bool bad = r_refused(col2, diag, D, 0.9);
+    if (threadIdx.x == 0) panel_publish(pub, bad);
 }
 
 GemmArgs args(int M, int N, int K) {
@@ -349,4 +372,9 @@ int qr_panel(const cplx* A, cplx* Q, int M, int D, cplx* R, QrScratch& ws, cudaS
     if (l < 0) return -1;
     launch(panel_finish_kernel, 1, FT, 0, s, R, D, flag, pub);
     return launches + l + 1;
+}
+
+int qr_panel_verdict(const cplx* R, int D, cudaStream_t s, const Publish& pub) {
+    launch(panel_verdict_kernel, 1, FT, 0, s, const_cast<cplx*>(R), D, pub);
+    return 1;
 }

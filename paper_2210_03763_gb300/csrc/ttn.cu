@@ -152,7 +152,7 @@ struct ttn_ctx {
     QrScratch qr{};
     std::map<std::pair<int, int>, int*> cand;   // (node, leg) -> candidate rows
     std::map<std::pair<int, int>, int> ncand;
-    std::map<std::pair<int, int>, int> qr_hint;   // (node, leg): how its last QR went (see gauge_qr)
+    std::map<std::pair<int, int>, int> qr_hint;   // (node, leg): how its last QR went (QrHint)
 
     std::vector<Env> up, down, phys;
     Env dummy;
@@ -1295,50 +1295,73 @@ void rebuild_up_envs(ttn_ctx* c) {
 // ----------------------------------------------------------- QR & moves
 bool panel_applies(int M, int D) { return D >= PANEL_MIN_D && M >= PANEL_MIN_M; }
 
-// A (M x D) = Q R, Q in A's place: by panels on the tensor cores when the
-// matrix is large and well-conditioned, else by the column
-// loop, which decides and completes dependent columns.  The panel path puts Q
-// in `spare` (swapped with A when it succeeds) and gives up on
-// matrices that are not well-conditioned, so it is tried where it is likely
-// to succeed.  hint: 1 it succeeded here last time; 0 unknown (its first panel
-// is checked before the rest is launched); -1 dependent columns last time; < -1
-// that many more QRs without a try (full rank, badly conditioned).  Returns
-// the dependent columns.
+// How the last QR of a node's leg went.  It decides what is tried first, never
+// the result.
+enum QrHint { QR_UNKNOWN = 0, QR_PANELS, QR_DEPENDENT, QR_ILL_CONDITIONED };
+
+// A (M x D) = Q R, Q in A's place.  The result is a function of A alone:
+//   panels on the tensor cores (qr_panel.cu) if they take A, else
+//   the column loop with its rows spread over the SMs if it finds dependent
+//   columns, which it completes, else
+//   the column loop with 128 rows per block.
+// A matrix with dependent columns (residual at most 1e-10 |A|_F) or with R's
+// diagonal below the panels' limits is refused by the panels whatever order is
+// tried, so after a bond that had dependent columns or was ill-conditioned last
+// time the column loop goes first and the panels are left out if it confirms
+// that.  Every attempt works in `spare`, swapped with A in the end (small
+// matrices, and without a spare: the column loop in place).  Returns the
+// dependent columns.
 int gauge_qr(ttn_ctx* c, cplx*& A, cplx*& spare, int M, int D, cplx* R, const int* cand, int ncand, QrScratch& q,
              int& hint) {
-    if (hint >= 0 && panel_applies(M, D)) {
-        const size_t need = qr_panel_workspace(M, D);
-        if (try_grow_split_ws(c, need)) {
-            int gave_up = 0;
-            for (int first = 0; first < D && !gave_up;) {
-                const int last = hint == 1 || first > 0 ? D : QR_PANEL;
-                const int n = qr_panel(A, spare, M, D, R, q, c->stream, c->split_ws, c->split_cap, first, last,
-                                       next_publish(c));
-                if (n < 0) {
-                    gave_up = 1;
-                    break;
-                }
-                c->stats[3] += n;
-                c->digits_run = true;
-                wait_published(c);
-                gave_up = c->hstat->qr_flag;
-                first = last;
-            }
-            if (!gave_up) {
-                std::swap(A, spare);
-                hint = 1;
-                return 0;
-            }
-            hint = -9;
+    auto columns = [&](cplx* X, bool fine) {
+        if (X != A)
+            CUDA_OK(cudaMemcpyAsync(X, A, sizeof(cplx) * (size_t)M * D, cudaMemcpyDeviceToDevice, c->stream));
+        int ndep = 0;
+        const int nl = qr_cgs2(X, M, D, R, cand, ncand, q, c->stream, &ndep, fine);
+        if (nl < 0) throw TtnError(TTN_ERR_TIMEOUT, "QR grid barrier wait timed out");
+        c->stats[3] += nl;
+        return ndep;
+    };
+    if (!spare || qr_one_block(M, D)) return columns(A, false);   // one block: one way to split its rows
+    auto done = [&](int how, int ndep) {
+        std::swap(A, spare);
+        hint = how;
+        return ndep;
+    };
+    const bool panels = panel_applies(M, D) && try_grow_split_ws(c, qr_panel_workspace(M, D));
+    bool full_rank = false;   // known from the column loop
+    if (hint == QR_DEPENDENT) {
+        if (const int ndep = columns(spare, true)) return done(QR_DEPENDENT, ndep);
+        full_rank = true;
+    } else if (hint == QR_ILL_CONDITIONED) {
+        if (columns(spare, false) == 0) {
+            if (!panels) return done(QR_ILL_CONDITIONED, 0);
+            c->stats[3] += qr_panel_verdict(R, D, c->stream, next_publish(c));
+            wait_published(c);
+            if (c->hstat->qr_flag) return done(QR_ILL_CONDITIONED, 0);
         }
     }
-    int ndep = 0;
-    const int nl = qr_cgs2(A, M, D, R, cand, ncand, q, c->stream, &ndep, hint == -1);
-    if (nl < 0) throw TtnError(TTN_ERR_TIMEOUT, "QR grid barrier wait timed out");
-    c->stats[3] += nl;
-    if (ndep > 0) hint = -1;
-    else if (hint < 0) ++hint;
-    return ndep;
+    if (panels) {
+        int gave_up = 0;
+        for (int first = 0; first < D && !gave_up;) {   // all at once where it is likely to succeed
+            const int last = hint == QR_PANELS || first > 0 ? D : QR_PANEL;
+            const int n = qr_panel(A, spare, M, D, R, q, c->stream, c->split_ws, c->split_cap, first, last,
+                                   next_publish(c));
+            if (n < 0) {
+                gave_up = 1;
+                break;
+            }
+            c->stats[3] += n;
+            c->digits_run = true;
+            wait_published(c);
+            gave_up = c->hstat->qr_flag;
+            first = last;
+        }
+        if (!gave_up) return done(QR_PANELS, 0);
+    }
+    if (!full_rank)
+        if (const int ndep = columns(spare, true)) return done(QR_DEPENDENT, ndep);
+    return done(QR_ILL_CONDITIONED, columns(spare, false));
 }
 
 // X (node k) = Q x_o R; Q replaces the node tensor, R (D x D) into Rbuf.
@@ -2546,11 +2569,13 @@ ttn_status ttn_selftest_qr(const double* A, int M, int D, const int* cand, int n
         alloc_qr_scratch(&tmp, M, D, q);
         cplx* dA = (cplx*)dalloc(&tmp, sizeof(cplx) * (size_t)M * D);
         cplx* dR = (cplx*)dalloc(&tmp, sizeof(cplx) * (size_t)D * D);
-        cplx* spare = nullptr;   // the panel path's copy, where it applies and fits
-        int hint = -1;
-        if (panel_applies(M, D) && cudaMalloc(&spare, sizeof(cplx) * (size_t)M * D) == cudaSuccess) {
+        cplx* spare = nullptr;   // where it fits
+        int hint = QR_UNKNOWN;
+        if (cudaMalloc(&spare, sizeof(cplx) * (size_t)M * D) == cudaSuccess) {
             tmp.allocs.push_back(spare);
-            if (try_grow_split_ws(&tmp, qr_panel_workspace(M, D))) hint = 0;   // outside the timed region
+            if (panel_applies(M, D)) try_grow_split_ws(&tmp, qr_panel_workspace(M, D));   // outside the timed region
+        } else {
+            spare = nullptr;
         }
         cudaGetLastError();
         const int nc = cand ? ncand : M;
