@@ -339,9 +339,14 @@ ttn_status ttn_selftest_fp64_peak(int method, double* tflops);
  *                          TTN_ERR_KRYLOV;
  *   TTN_INJECT_ALLOC_FAIL  the next `value` device allocations fail
  *                          (TTN_ERR_ALLOC);
+ *   TTN_INJECT_QR_GIVE_UP  in the next `value` cooperative QR column loops one
+ *                          block ends before its last rows are written, as
+ *                          after a grid-barrier wait that ran out
+ *                          (TTN_ERR_TIMEOUT);
  *   TTN_INJECT_NONE        clears every hook.
  * Hooks are process-wide.  Bad kind or value -> TTN_ERR_ARG. */
-enum { TTN_INJECT_NONE = 0, TTN_INJECT_TC_STALL = 1, TTN_INJECT_KRYLOV_MMAX = 2, TTN_INJECT_ALLOC_FAIL = 3 };
+enum { TTN_INJECT_NONE = 0, TTN_INJECT_TC_STALL = 1, TTN_INJECT_KRYLOV_MMAX = 2, TTN_INJECT_ALLOC_FAIL = 3,
+       TTN_INJECT_QR_GIVE_UP = 4 };
 ttn_status ttn_test_inject(int kind, long long value);
 
 /* ---- allocation-free contraction ----------------------------------------

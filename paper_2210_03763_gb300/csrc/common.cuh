@@ -171,7 +171,7 @@ struct HostStatus {
     KrylovStatus krylov[KRYLOV_MMAX];   // per Krylov step (one-launch runs: [0])
     int tc_flag;                        // a tensor-core wait gave up
     int qr_flag;                        // panel QR: not well-conditioned
-    int qr_dep[256];                    // column loop: dependent columns
+    int qr_dep[256];                    // column loop: dependent columns (no report when a block gave up)
     unsigned seq;
 };
 struct Publish {                        // where and as which launch a kernel reports; hs null: not at all
@@ -273,7 +273,7 @@ struct QrScratch {
     double* nu;         // D: squared residual norms
     int* row_rank;      // M: step at which a row was accepted (INT_MAX: never)
     int* cand_used;     // M: candidate accepted flags
-    unsigned* bar;      // 2: grid barrier of the cooperative column loop
+    unsigned* bar;      // 3: grid barrier of the cooperative column loop, blocks that have finished it
     int* err;           // [0] set when a bounded device wait gave up, [1] when the panel path gave up
     cplx* panel;        // panel path: qr_panel_scratch(D)
     HostStatus* hs;     // status in host memory (null: read back by copies)
@@ -351,5 +351,6 @@ int k_leaf_draw(const cplx* G, const double* U, long long ldu, int j, int atom, 
 unsigned long long test_take_tc_stall();
 int test_krylov_mmax();
 bool test_take_alloc_fail();
+bool test_take_qr_give_up();
 
 #define TTN_LAUNCH_CHECK() (cudaGetLastError())

@@ -635,7 +635,7 @@ __device__ void la_dots(int P, PairF pair, cplx* out, const cplx* A, long long M
 template <int RB>
 __global__ void __launch_bounds__(QB) qr_coop_kernel(cplx* A, long long M, int D, cplx* R, int* flags, cplx* part,
                                                      cplx* red_out, unsigned* bar, int* err, int nc_max, double tol,
-                                                     int la_max, int rpb, Publish pub) {
+                                                     int la_max, int rpb, Publish pub, int give_up) {
     // dynamic shared memory: nc_max cached columns of RB + 1 rows, then the
     // look-ahead window of at most la_max (<= LA_WMAX) columns (this block's
     // rows of v1_j)
@@ -902,9 +902,23 @@ __global__ void __launch_bounds__(QB) qr_coop_kernel(cplx* A, long long M, int D
         if (k0 >= D) break;     // every column decided and finalised
         k = k0 - 1;             // the loop's increment brings it to k0
     }
-    if (b0 && pub.hs) {         // block 0 decided the flags: report them
+    if (give_up && blockIdx.x == G - 1) {   // test hook: as if its last barrier wait had given up
+        if (t == 0) atomicExch(err, 1);
+        return;
+    }
+    // the last block to finish reports: a block that gave up never gets here, no
+    // report is made then, and the host reads *err
+    if (pub.hs) {
         __syncthreads();
-        for (int k = t; k < D; k += QB) pub.hs->qr_dep[k] = flags[k];
+        if (t == 0) {
+            __threadfence();
+            sm.ok = atomicAdd(bar + 2, 1u) == (unsigned)G - 1;
+            if (sm.ok) bar[2] = 0u;
+            __threadfence();
+        }
+        __syncthreads();
+        if (!sm.ok) return;
+        for (int k = t; k < D; k += QB) pub.hs->qr_dep[k] = ((volatile int*)flags)[k];   // decided by block 0
         __threadfence_system();
         __syncthreads();
         if (t == 0) *(volatile unsigned*)&pub.hs->seq = pub.seq;
@@ -1362,6 +1376,7 @@ struct CoopArgs {
     int la;
     int rpb;
     Publish pub;
+    int give_up;
 };
 
 std::mutex g_coop_mu;
@@ -1418,9 +1433,9 @@ bool launch_coop(CoopArgs& a, cudaStream_t s, int& nl) {
         }
     }
     if (G > (long long)nsm * per_sm) return false;
-    // the barrier leaves its arrival count at zero after every completed
-    // wait, so it needs a reset only after an error
-    void* args[] = {&a.A, &a.M, &a.D, &a.R, &a.flags, &a.part, &a.red_out, &a.bar, &a.err, &a.nc, &a.tol, &a.la, &a.rpb, &a.pub};
+    // the barrier and the count of finished blocks are at zero after every
+    // completed loop, so they need a reset only after an error
+    void* args[] = {&a.A, &a.M, &a.D, &a.R, &a.flags, &a.part, &a.red_out, &a.bar, &a.err, &a.nc, &a.tol, &a.la, &a.rpb, &a.pub, &a.give_up};
     nl = 1;
     if (cudaLaunchCooperativeKernel((const void*)qr_coop_kernel<RB>, dim3((unsigned)G), dim3(QB), args, smem, s) ==
         cudaSuccess)
@@ -1462,6 +1477,7 @@ int qr_cgs2(cplx* A, int M, int D, cplx* R, const int* cand, int ncand, QrScratc
     bool coop_done = false;
     const Publish pub = ws.hs ? Publish{ws.hs, ++*ws.seq, nullptr} : Publish{};
     if (D <= MAXD) {
+        const int give_up = test_take_qr_give_up();
         const int nsm = std::min(coop_sms(), QR_SMALL_BLOCKS);
         // few columns and rows: one block, no synchronisation at all
         const bool coarse = !fine_rows || nsm == 0 || qr_one_block(M, D);
@@ -1483,7 +1499,7 @@ int qr_cgs2(cplx* A, int M, int D, cplx* R, const int* cand, int ncand, QrScratc
         }
         for (int i = 0; i < nopt && !coop_done; ++i) {
             int nc = opts[i].nc, la = opts[i].la, nl = 0;
-            CoopArgs a{A, MM, D, R, ws.flags, ws.part, ws.h, ws.bar, ws.err, nc, tol, la, rpb, pub};
+            CoopArgs a{A, MM, D, R, ws.flags, ws.part, ws.h, ws.bar, ws.err, nc, tol, la, rpb, pub, give_up};
             switch (rb) {
                 case 8: coop_done = launch_coop<8>(a, s, nl); break;
                 case 16: coop_done = launch_coop<16>(a, s, nl); break;
@@ -1520,7 +1536,7 @@ int qr_cgs2(cplx* A, int M, int D, cplx* R, const int* cand, int ncand, QrScratc
     }
     if (herr) {   // a grid-barrier wait gave up: clear the flag, report
         cudaMemsetAsync(ws.err, 0, sizeof(int), s);
-        cudaMemsetAsync(ws.bar, 0, 2 * sizeof(unsigned), s);
+        cudaMemsetAsync(ws.bar, 0, 3 * sizeof(unsigned), s);
         cudaStreamSynchronize(s);
         return -1;
     }

@@ -193,6 +193,7 @@ struct ttn_ctx {
 static std::atomic<long long> g_inj_tc_stall{0};     // tensor-core launches still to stall
 static std::atomic<int> g_inj_mmax{0};               // Krylov dimension cap, 0: KRYLOV_MMAX
 static std::atomic<long long> g_inj_alloc_fail{0};   // device allocations still to fail
+static std::atomic<long long> g_inj_qr_give_up{0};   // cooperative QR loops in which a block is still to give up
 constexpr unsigned long long INJ_STALL_NS = 1000000ull;   // 1 ms wait that runs out
 
 namespace {
@@ -212,6 +213,7 @@ int test_krylov_mmax() {
     const int m = g_inj_mmax.load();
     return (m >= 1 && m < KRYLOV_MMAX) ? m : KRYLOV_MMAX;
 }
+bool test_take_qr_give_up() { return take_one(g_inj_qr_give_up); }
 bool test_take_alloc_fail() { return take_one(g_inj_alloc_fail); }
 
 namespace {
@@ -3353,6 +3355,7 @@ ttn_status ttn_test_inject(int kind, long long value) {
             g_inj_tc_stall = 0;
             g_inj_mmax = 0;
             g_inj_alloc_fail = 0;
+            g_inj_qr_give_up = 0;
             return TTN_OK;
         case TTN_INJECT_TC_STALL: g_inj_tc_stall = value; return TTN_OK;
         case TTN_INJECT_KRYLOV_MMAX:
@@ -3360,6 +3363,7 @@ ttn_status ttn_test_inject(int kind, long long value) {
             g_inj_mmax = (int)value;
             return TTN_OK;
         case TTN_INJECT_ALLOC_FAIL: g_inj_alloc_fail = value; return TTN_OK;
+        case TTN_INJECT_QR_GIVE_UP: g_inj_qr_give_up = value; return TTN_OK;
         default: return TTN_ERR_ARG;
     }
 }

@@ -74,7 +74,7 @@ SIGNATURES = [
 ]
 
 # fault-injection hooks of ttn_test_inject
-INJECT_NONE, INJECT_TC_STALL, INJECT_KRYLOV_MMAX, INJECT_ALLOC_FAIL = 0, 1, 2, 3
+INJECT_NONE, INJECT_TC_STALL, INJECT_KRYLOV_MMAX, INJECT_ALLOC_FAIL, INJECT_QR_GIVE_UP = 0, 1, 2, 3, 4
 
 _lib = None
 
