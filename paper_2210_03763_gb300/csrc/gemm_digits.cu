@@ -328,6 +328,7 @@ struct DigitGemm {
     const uint16_t *magP, *magQ;
     const unsigned long long *l1P, *l1Q;
     int Kc;
+    unsigned long long stall_ns; // test hook: > 0 makes the drain warps wait this long on a barrier that nothing arrives at
     cplx* W;                     // partial sums of split K (layout of splitk_f64_kernel)
     int* err;
 };
@@ -620,7 +621,8 @@ __global__ void __launch_bounds__(THREADS, 1)
     uint64_t* lfull = empty + STAGES;      // [NLEV] level accumulated
     uint64_t* lempty = lfull + NLEV;       // [NLEV] level drained
     uint64_t* mdone = lempty + NLEV;
-    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(mdone + 1);
+    uint64_t* stallbar = mdone + 1;        // test hook: never arrived at
+    uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(stallbar + 1);
 
     // an earlier launch on this workspace gave up: do nothing (the host
     // reports the error at its next check)
@@ -657,6 +659,7 @@ __global__ void __launch_bounds__(THREADS, 1)
             mbar_init(&lempty[i], DRAIN_THREADS);
         }
         mbar_init(mdone, 1);
+        mbar_init(stallbar, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     }
     if (warp == 0) {
@@ -753,6 +756,8 @@ __global__ void __launch_bounds__(THREADS, 1)
         const int quad = warp & 3, col0 = (warp >> 2) * DCOLS;
         unsigned cg = 0;
         bool ok = true;
+        // test hook: the other roles see the error flag and abort as after a real timeout
+        if (ea.stall_ns > 0 && !__all_sync(0xffffffffu, mbar_wait(stallbar, 0, ea.err, ea.stall_ns))) ok = false;
         for (long long t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
             int pt, qt, b, ks;
             tile_of(t, pt, qt, b, ks);
@@ -1045,6 +1050,7 @@ int launch_zgemm_digits(const GemmArgs& g, bool elementwise, cudaStream_t stream
     d.expQ = sq.exps;
     d.W = d.nsplit > 1 ? reinterpret_cast<cplx*>(ws + pl.w_off) : nullptr;
     d.err = reinterpret_cast<int*>(ws);
+    d.stall_ns = test_take_tc_stall();
     if (elementwise) {
         d.mask = reinterpret_cast<uint32_t*>(ws + pl.mask_off);
         d.magP = sp.mag;

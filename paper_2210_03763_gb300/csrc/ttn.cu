@@ -2900,6 +2900,7 @@ ttn_status ttn_compress(ttn_ctx* src, ttn_ctx* dst, double* discarded) {
             CUDA_OK(cudaMemcpyAsync(dst->T[k], cur, sizeof(cplx) * sz, cudaMemcpyDeviceToDevice, c->stream));
         }
         CUDA_OK(cudaStreamSynchronize(c->stream));
+        check_digits(c);
         // canonical form of dst: QR of every non-root node towards its parent, bottom-up
         for (auto& lev : dst->level_nodes)
             for (int k : lev) {
