@@ -90,7 +90,8 @@ struct SplitPackArgs {
     float* hi;
     float* lo;
 };
-int split_pack(const SplitPackArgs* p, int n, cudaStream_t stream);   // n operands, few launches
+// n operands, few launches; clear (may be null): an int that the first sets to zero.
+int split_pack(const SplitPackArgs* p, int n, cudaStream_t stream, int* clear = nullptr);
 
 // Packed output of a split contraction: the epilogue writes TF32 hi/lo
 // planes (as split_pack with embed = 0) at float2 position
@@ -146,7 +147,7 @@ int launch_zgemm_split(const GemmArgs& g, cudaStream_t stream, void* workspace,
 constexpr int SPLIT_K_MAX = 1 << 20;
 size_t split_workspace_bytes(const GemmArgs& g, int max_split = SPLIT_K_MAX);
 int launch_split_pack(const GemmArgs& g, cudaStream_t stream, void* workspace, size_t workspace_bytes,
-                      int max_split = SPLIT_K_MAX);
+                      int max_split = SPLIT_K_MAX, bool clear_flag = false);
 int launch_split_mma(const GemmArgs& g, cudaStream_t stream, void* workspace, size_t workspace_bytes,
                      int max_split = SPLIT_K_MAX);
 

@@ -186,9 +186,11 @@ struct PackJobs {   // several operands in one launch
     int first[PK_JOBS + 1];   // first block of each
     int rb[PK_JOBS];          // row blocks (fastest), then K blocks of ktiles tiles
     int ktiles[PK_JOBS];
+    int* clear;               // error word to set to zero, or null
 };
 __global__ void __launch_bounds__(PK_THREADS) pack_kernel(const __grid_constant__ PackJobs jobs) {
     pdl_begin();
+    if (jobs.clear && blockIdx.x == 0 && threadIdx.x == 0) *jobs.clear = 0;
     int job = 0;
     while ((int)blockIdx.x >= jobs.first[job + 1]) ++job;
     const SplitPackArgs& p = jobs.p[job];
@@ -904,10 +906,11 @@ SplitPackArgs side_pack_args(const GemmArgs& g, const Plan& pl, int side, float*
 }  // namespace
 
 // ------------------------------------------------------------- public API
-int split_pack(const SplitPackArgs* p, int n, cudaStream_t stream) {
+int split_pack(const SplitPackArgs* p, int n, cudaStream_t stream, int* clear) {
     int launches = 0;
     for (int i = 0; i < n;) {
         PackJobs jobs;
+        jobs.clear = clear;
         int nj = 0;
         jobs.first[0] = 0;
         for (; i < n && nj < PK_JOBS; ++i) {
@@ -1014,9 +1017,9 @@ size_t split_workspace_bytes(const GemmArgs& g, int max_split) {
 
 // Phase 1 of a split contraction: pack both operands.  Returns kernels
 // launched, -1 if the shape is not handled here (caller uses FP64), -2 if the
-// workspace is too small.
+// workspace is too small.  clear_flag: the workspace's error flag starts at zero.
 int launch_split_pack(const GemmArgs& g, cudaStream_t stream, void* workspace, size_t workspace_bytes,
-                      int max_split) {
+                      int max_split, bool clear_flag) {
     Plan pl = plan_for(g, max_split);
     if (!pl.ok || !encode_fn()) return -1;
     if (!workspace || workspace_bytes < pl.bytes) return -2;
@@ -1025,7 +1028,7 @@ int launch_split_pack(const GemmArgs& g, cudaStream_t stream, void* workspace, s
     float* Qh = Pl + pl.pe;
     float* Ql = Qh + pl.qe;
     const SplitPackArgs both[2] = {side_pack_args(g, pl, 0, Ph, Pl), side_pack_args(g, pl, 1, Qh, Ql)};
-    return split_pack(both, 2, stream);
+    return split_pack(both, 2, stream, clear_flag ? reinterpret_cast<int*>(workspace) : nullptr);
 }
 
 // Phase 2: the tcgen05 GEMM on the packed operands of the same GemmArgs.

@@ -59,10 +59,9 @@ extern "C" ttn_status ttn_contract_split_noalloc(const double* A, const double* 
     if (need > 0) {
         ttn_status st = scratch_for_current_device(&scratch);
         if (st != TTN_OK) return st;
-        // the error flag at the start of the scratch is zero: it starts so and
-        // is cleared whenever a call has found it set (clearing it here was a launch
-        // of its own in a call of 30 us)
-        packed = launch_split_pack(g, s, scratch, NOALLOC_SCRATCH_BYTES, 1);
+        // the packing also clears the error flag at the start of the scratch: a call
+        // that ended early (a launch error) may have left it set
+        packed = launch_split_pack(g, s, scratch, NOALLOC_SCRATCH_BYTES, 1, true);
         if (packed == -2) return TTN_ERR_ARG;
     }
     if (packed < 0) {
