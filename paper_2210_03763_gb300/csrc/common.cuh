@@ -34,11 +34,13 @@ int launch_splitk_f64(const GemmArgs& g, int nsplit, const cplx* W, cudaStream_t
 // chains), and the launch (kernels launched; -1 when it is not handled there,
 // -2 when the workspace is too small).  elementwise: every output has the error
 // bound of an FMA chain; else its error is relative to |row||column|, C may
-// overlap A and B when it is one batch, and rows with an infinity or a NaN give NaNs.
+// overlap A and B when it is one batch, and rows with an infinity or a NaN give
+// NaNs.  skip (device memory, may be null): when it is set the operands are not
+// even read, and C is undefined.
 bool digits_wanted(const GemmArgs& g);
 size_t digits_workspace_bytes(const GemmArgs& g, bool elementwise);
 int launch_zgemm_digits(const GemmArgs& g, bool elementwise, cudaStream_t stream, void* workspace,
-                        size_t workspace_bytes);
+                        size_t workspace_bytes, const int* skip = nullptr);
 
 // Programmatic dependent launch for small kernels: the next kernel of the
 // stream is brought up while this one runs, and waits in pdl_begin() until all

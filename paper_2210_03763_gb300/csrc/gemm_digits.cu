@@ -188,8 +188,10 @@ __device__ __forceinline__ unsigned l1_units(unsigned long long biased) {
 }
 
 // Row exponents over blocks of K (long K only): exps and l1 zeroed before.
-__global__ void __launch_bounds__(PK_THREADS) digit_max_kernel(DigitSide sp, DigitSide sq, int nbp, int kb) {
+__global__ void __launch_bounds__(PK_THREADS) digit_max_kernel(DigitSide sp, DigitSide sq, int nbp, int kb,
+                                                              const int* skip) {
     pdl_begin();
+    if (skip && *(volatile const int*)skip) return;
     const DigitSide& s = (int)blockIdx.x < nbp ? sp : sq;
     const long long f0 = (long long)((int)blockIdx.x < nbp ? blockIdx.x : blockIdx.x - nbp) * PK_ROWS;
     __shared__ const cplx* base[PK_ROWS];
@@ -208,8 +210,9 @@ __global__ void __launch_bounds__(PK_THREADS) digit_max_kernel(DigitSide sp, Dig
 // Digits of 32 rows over a block of K.  one_pass: this block sees the whole K
 // and finds the exponents itself.
 __global__ void __launch_bounds__(PK_THREADS) digit_pack_kernel(DigitSide sp, DigitSide sq, int nbp, int kb,
-                                                               int one_pass, int* marked) {
+                                                               int one_pass, int* marked, const int* skip) {
     pdl_begin();
+    if (skip && *(volatile const int*)skip) return;
     if (marked && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *marked = 0;
     const bool isp = (int)blockIdx.x < nbp;
     const DigitSide& s = isp ? sp : sq;
@@ -331,6 +334,7 @@ struct DigitGemm {
     unsigned long long stall_ns; // test hook: > 0 makes the drain warps wait this long on a barrier that nothing arrives at
     cplx* W;                     // partial sums of split K (layout of splitk_f64_kernel)
     int* err;
+    const int* skip;             // not null and set: nothing to do
 };
 
 // 64-byte swizzle, K-major, 8-row groups 512 bytes apart; the address (lower
@@ -624,11 +628,11 @@ __global__ void __launch_bounds__(THREADS, 1)
     uint64_t* stallbar = mdone + 1;        // test hook: never arrived at
     uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(stallbar + 1);
 
-    // an earlier launch on this workspace gave up: do nothing (the host
-    // reports the error at its next check)
+    // an earlier launch on this workspace gave up (the host reports the error at
+    // its next check), or the caller's flag is set: do nothing
     __shared__ int s_skip, s_marked;
     if (threadIdx.x == 0) {
-        s_skip = *(volatile int*)ea.err;
+        s_skip = *(volatile int*)ea.err || (ea.skip && *(volatile const int*)ea.skip);
         s_marked = ea.mask && *(volatile int*)ea.marked;
     }
     __syncthreads();
@@ -971,15 +975,15 @@ size_t digits_workspace_bytes(const GemmArgs& g, bool elementwise) {
 }
 
 int launch_zgemm_digits(const GemmArgs& g, bool elementwise, cudaStream_t stream, void* workspace,
-                        size_t workspace_bytes) {
+                        size_t workspace_bytes, const int* skip) {
     DPlan pl = plan(g, elementwise);
     if (!pl.ok || !encode_fn()) return -1;
     if ((long long)pl.bytes > MAX_PLANE_BYTES) {
         GemmArgs lo, hi;
         if (halve(g, lo, hi)) {
-            const int a = launch_zgemm_digits(lo, elementwise, stream, workspace, workspace_bytes);
+            const int a = launch_zgemm_digits(lo, elementwise, stream, workspace, workspace_bytes, skip);
             if (a < 0) return a;
-            const int b = launch_zgemm_digits(hi, elementwise, stream, workspace, workspace_bytes);
+            const int b = launch_zgemm_digits(hi, elementwise, stream, workspace, workspace_bytes, skip);
             return b < 0 ? b : a + b;
         }
     }
@@ -1024,11 +1028,11 @@ int launch_zgemm_digits(const GemmArgs& g, bool elementwise, cudaStream_t stream
     const dim3 grid(nbp + nbq, (Kc + kb - 1) / kb);
     if (!one) {
         if (cudaMemsetAsync(ws + pl.ep_off, 0, pl.p_off - pl.ep_off, stream) != cudaSuccess) return -1;
-        launch(digit_max_kernel, grid, PK_THREADS, 0, stream, sp, sq, nbp, kb);
+        launch(digit_max_kernel, grid, PK_THREADS, 0, stream, sp, sq, nbp, kb, skip);
         ++launches;
     }
     d.marked = elementwise ? reinterpret_cast<int*>(ws) + 1 : nullptr;
-    launch(digit_pack_kernel, grid, PK_THREADS, 0, stream, sp, sq, nbp, kb, one, d.marked);
+    launch(digit_pack_kernel, grid, PK_THREADS, 0, stream, sp, sq, nbp, kb, one, d.marked, skip);
     ++launches;
     CUtensorMap mP, mQ;
     if (!make_map3(&mP, sp.planes, sp.rows, pl.Kp, BM) || !make_map3(&mQ, sq.planes, sq.rows, pl.Kp, BN)) return -1;
@@ -1050,6 +1054,7 @@ int launch_zgemm_digits(const GemmArgs& g, bool elementwise, cudaStream_t stream
     d.expQ = sq.exps;
     d.W = d.nsplit > 1 ? reinterpret_cast<cplx*>(ws + pl.w_off) : nullptr;
     d.err = reinterpret_cast<int*>(ws);
+    d.skip = skip;
     d.stall_ns = test_take_tc_stall();
     if (elementwise) {
         d.mask = reinterpret_cast<uint32_t*>(ws + pl.mask_off);

@@ -24,7 +24,8 @@
 // path is for matrices without any: it gives up (the flag) as soon as a
 // column's part outside the earlier ones is below 1e-4 of the column or 1e-8
 // of |A|_F, far above the rule's 1e-10, and when |A| lies outside 2^+-480, and the
-// caller runs the column loop on the original matrix.  Q and R are then the same as the column loop's up to rounding (R has
+// caller runs the column loop on the original matrix; what has been launched
+// beyond that point does nothing.  Q and R are then the same as the column loop's up to rounding (R has
 // a positive real diagonal, which makes them unique).
 //
 // Why: 16 M D^2 flops of the column loop take 4.1 ms on the FP64 pipe for a
@@ -336,7 +337,7 @@ int qr_panel(const cplx* A, cplx* Q, int M, int D, cplx* R, QrScratch& ws, cudaS
     for (int n = first; n < last; n += PB) {
         const int bp = std::min(PB, D - n), ld = n + bp;
         for (int pass = 1; pass <= 2; ++pass) {
-            int l = launch_zgemm_digits(gram_args(Q, M, n, bp, S), false, s, workspace, workspace_bytes);
+            int l = launch_zgemm_digits(gram_args(Q, M, n, bp, S), false, s, workspace, workspace_bytes, flag);
             if (l < 0) return -1;
             launches += l;
             if (n > 0) {   // -S_q^H S_q
@@ -359,7 +360,7 @@ int qr_panel(const cplx* A, cplx* Q, int M, int D, cplx* R, QrScratch& ws, cudaS
                 launches += launch_zgemm_f64(g, s);
             }
             // in place: the operands are packed before the first output is written
-            l = launch_zgemm_digits(update_args(Q, M, n, bp, C), false, s, workspace, workspace_bytes);
+            l = launch_zgemm_digits(update_args(Q, M, n, bp, C), false, s, workspace, workspace_bytes, flag);
             if (l < 0) return -1;
             launches += l;
         }
@@ -368,7 +369,7 @@ int qr_panel(const cplx* A, cplx* Q, int M, int D, cplx* R, QrScratch& ws, cudaS
         launch(panel_report_kernel, 1, 1, 0, s, flag, pub);
         return launches + 1;
     }
-    const int l = launch_zgemm_digits(r_args(Q, A, M, D, R), false, s, workspace, workspace_bytes);
+    const int l = launch_zgemm_digits(r_args(Q, A, M, D, R), false, s, workspace, workspace_bytes, flag);
     if (l < 0) return -1;
     launch(panel_finish_kernel, 1, FT, 0, s, R, D, flag, pub);
     return launches + l + 1;
