@@ -244,7 +244,8 @@ ttn_status ttn_refresh_envs(ttn_ctx* ctx);
 ttn_status ttn_apply_heff(ttn_ctx* ctx, int node, const double* x, double* y);
 
 /* Counters since the last ttn_reset_stats: [0] Krylov runs, [1] Krylov
- * matvecs, [2] max Krylov error estimate (as double bits), [3] kernel launches
+ * matvecs run (a run first launches as many as its node or link took last
+ * time, so some may lie beyond the step it ends at), [2] max Krylov error estimate (as double bits), [3] kernel launches
  * issued by the library, [4] QR calls, [5] dependent columns completed. */
 ttn_status ttn_get_stats(const ttn_ctx* ctx, int64_t* out6);
 

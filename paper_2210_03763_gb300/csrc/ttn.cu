@@ -993,6 +993,7 @@ void krylov(ttn_ctx* c, cplx* x, long long n, double zr, double zi, int& hint, F
         cplx* vj = V + (long long)j * ld;
         cplx* w = V + (long long)(j + 1) * ld;
         apply(vj, w);
+        c->stats[1] += 1;
         {
             // bytes: the basis is read twice (Arnoldi: three times), w read and written twice
             const bool arnoldi = c->gamma != 0.0;   // non-Hermitian generator (decay)
@@ -1025,7 +1026,6 @@ void krylov(ttn_ctx* c, cplx* x, long long n, double zr, double zi, int& hint, F
     }
     hint = m + 1;
     c->stats[0] += 1;
-    c->stats[1] += m + 1;
     ProfScope ps(c, PK_KRY, 0.0, 16.0 * n * (m + 2));
     c->stats[3] += k_combine(V, ld, m + 1, c->ks, x, n, s);
 }
