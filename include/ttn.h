@@ -20,6 +20,9 @@
  *  - The context owns all device memory; nothing is shared between contexts.
  *  - Work is issued on the context's stream (ttn_set_stream); calls that
  *    return host scalars synchronise that stream.
+ *    While a call waits for the device its host thread polls, one core per
+ *    context; on a device set to cudaDeviceScheduleYield it yields between
+ *    polls, on one set to cudaDeviceScheduleBlockingSync it sleeps.
  *  - No call throws.  Each returns a ttn_status; on error the context keeps a
  *    message (ttn_last_error).  Invalid arguments return TTN_ERR_ARG and leave
  *    the context unchanged.  Device-side numerical failures (NaN/Inf) are

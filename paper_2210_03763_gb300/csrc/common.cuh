@@ -183,7 +183,8 @@ struct Publish {                        // where and as which launch a kernel re
     const int* tc_flag;                 // may be null
 };
 // Wait until launch `seq` on stream s has reported.  False: the stream ran dry
-// (or failed) without it.
+// (or failed) without it.  The host thread polls, yields between polls or
+// sleeps as the device's scheduling flag says (cudaSetDeviceFlags).
 bool wait_status(const HostStatus* hs, unsigned seq, cudaStream_t s);
 
 struct KrylovScalars {

@@ -10,6 +10,7 @@
 #include <atomic>
 #include <cmath>
 #include <mutex>
+#include <sched.h>
 
 namespace {
 
@@ -1044,9 +1045,19 @@ int k_krylov_start(KrylovScalars* ks, const cplx* x, long long n, double* partia
 bool wait_status(const HostStatus* hs, unsigned seq, cudaStream_t s) {
     const volatile unsigned* p = &hs->seq;
     auto there = [&] { return (int)(*p - seq) >= 0; };
+    unsigned schedule = cudaDeviceScheduleAuto;
     for (unsigned i = 1;; ++i) {
         if (there()) break;
-        if ((i & 0xFFF) == 0 && cudaStreamQuery(s) != cudaErrorNotReady) {   // done or failed
+        if ((i & 0xFFF) != 0) continue;
+        // a long wait (some 10 us): as the device's scheduling flag has it, and
+        // look whether the stream is done or has failed
+        if (i == 0x1000) {
+            if (cudaGetDeviceFlags(&schedule) != cudaSuccess) cudaGetLastError();
+            schedule &= cudaDeviceScheduleMask;
+        }
+        if (schedule == cudaDeviceScheduleYield) sched_yield();
+        if (schedule == cudaDeviceScheduleBlockingSync ? cudaStreamSynchronize(s) != cudaErrorNotReady
+                                                       : cudaStreamQuery(s) != cudaErrorNotReady) {
             if (there()) break;
             return false;
         }
