@@ -1,9 +1,9 @@
 // Vector, reduction and small-matrix kernels of the TDVP update.
 //
-// Reductions never use atomics: each of G blocks writes a partial sum for a
-// contiguous chunk of the vector, and every consumer sums the G partials in
-// the same fixed order, so repeated runs are bitwise identical and every
-// block of a kernel sees the same reduced value.
+// Each of G blocks of a reduction writes a partial sum for a contiguous chunk
+// of the vector, and every consumer sums the G partials in the same fixed order,
+// so repeated runs are bitwise identical and every block of a kernel sees the
+// same reduced value.  Atomics only count the blocks that have finished.
 #include "common.cuh"
 #include <cooperative_groups.h>
 #include <algorithm>
@@ -17,13 +17,6 @@ namespace {
 constexpr int T = RED_THREADS;
 
 __device__ __forceinline__ cplx cadd(cplx a, cplx b) { return make_double2(a.x + b.x, a.y + b.y); }
-__device__ __forceinline__ cplx cmul(cplx a, cplx b) {
-    return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
-}
-// conj(a) * b
-__device__ __forceinline__ cplx cdotc(cplx a, cplx b) {
-    return make_double2(a.x * b.x + a.y * b.y, a.x * b.y - a.y * b.x);
-}
 // The vector kernels below are bound by GB300's FP64 pipe (about 1/64 of its
 // FP32 rate), not by HBM, so the complex multiply-accumulates are written as
 // four fused multiply-adds (s += conj(a) b, x -= a h) instead of two
@@ -51,22 +44,6 @@ __device__ __forceinline__ void chunk_of(long long n, int G, long long& lo, long
     long long c = (n + G - 1) / G;
     lo = (long long)blockIdx.x * c;
     hi = lo + c < n ? lo + c : n;
-}
-
-// Block-wide sum of one complex value per thread (result valid in thread 0).
-__device__ cplx block_sum_c(cplx v, cplx* sh) {
-    for (int o = 16; o > 0; o >>= 1) {
-        v.x += __shfl_down_sync(0xffffffffu, v.x, o);
-        v.y += __shfl_down_sync(0xffffffffu, v.y, o);
-    }
-    const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-    __syncthreads();
-    if (l == 0) sh[w] = v;
-    __syncthreads();
-    cplx r = make_double2(0.0, 0.0);
-    if (threadIdx.x == 0)
-        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) r = cadd(r, sh[i]);
-    return r;
 }
 
 __device__ double block_sum_d(double v, double* sh) {
