@@ -307,6 +307,20 @@ ttn_status ttn_reset_stats(ttn_ctx* ctx);
 ttn_status ttn_selftest_contract_host(const double* A, const double* B, double* C, int M, int N, int K,
                                       int precision, int* path, float* ms);
 
+/* Which kernels ran in this host thread's last ttn_selftest_contract_host or
+ * ttn_selftest_qr, and (recomputed, may be NULL) how many outputs of a digit
+ * contraction its error check left to FP64 FMA chains. */
+enum {
+    TTN_PATH_F64_DIRECT = 0,      /* FP64, one thread per output and K slice     */
+    TTN_PATH_F64_TILES = 1,       /* FP64, shared-memory tiles                   */
+    TTN_PATH_F64_DIGITS = 2,      /* FP64 by digit products, tensor cores        */
+    TTN_PATH_SPLIT = 3,           /* split TF32, tensor cores                    */
+    TTN_PATH_QR_COLUMNS = 4,      /* QR column loop, 128 rows per block          */
+    TTN_PATH_QR_COLUMNS_FINE = 5, /* QR column loop, rows spread over the SMs    */
+    TTN_PATH_QR_PANELS = 6        /* QR by panels, tensor cores                  */
+};
+ttn_status ttn_selftest_last_path(int* path, int* recomputed);
+
 /* Truncated singular value decomposition of a bond matrix, no context needed
  * (Sec. "Tensor network simulations": the bond dimension chi caps the kept
  * singular values; discarding sigma_i < eps * sigma_max as well).

@@ -26,6 +26,7 @@ struct GemmArgs {
 // tiles cannot fill the GPU split K into ranges summed in fixed order.
 int launch_zgemm_f64(const GemmArgs& g, cudaStream_t stream, void* workspace = nullptr, size_t workspace_bytes = 0);
 size_t f64_workspace_bytes(const GemmArgs& g);
+bool f64_direct(const GemmArgs& g);   // taken by the direct kernel, not the tiled one
 // C = alpha sum_ks W[ks] + beta C, W[((ks * Bo + bo) * Bi + bi) * M * N + m + n M].
 int launch_splitk_f64(const GemmArgs& g, int nsplit, const cplx* W, cudaStream_t stream);
 // The same contraction by digit products on the tensor cores (gemm_digits.cu):

@@ -330,6 +330,11 @@ void launch_direct(const GemmArgs& g, cudaStream_t stream, int S, int kc) {
 
 }  // namespace
 
+bool f64_direct(const GemmArgs& g) {
+    int kc = 0;
+    return direct_slices(g, tile_for(g.M), tile_for(g.N), kc) > 0;
+}
+
 size_t f64_workspace_bytes(const GemmArgs& g) {
     if (g.M <= 0 || g.N <= 0 || g.Bi <= 0 || g.Bo <= 0) return 0;
     int ks_len = 0, kc = 0;

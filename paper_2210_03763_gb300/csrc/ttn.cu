@@ -167,6 +167,7 @@ struct ttn_ctx {
     size_t ev_next = 0;
     void* split_ws = nullptr;   // packed operands of the tensor-core GEMMs (+ error flag)
     size_t split_cap = 0;
+    int last_path = 0;          // TTN_PATH_* of the last contraction or QR
     bool digits_run = false;    // an FP64 contraction ran on the tensor cores since the flag was last read
     cplx* obs_ws = nullptr;     // densities of ttn_measure, overlap environments
     size_t obs_cap = 0;
@@ -213,6 +214,7 @@ int test_krylov_mmax() {
     const int m = g_inj_mmax.load();
     return (m >= 1 && m < KRYLOV_MMAX) ? m : KRYLOV_MMAX;
 }
+thread_local int g_selftest_path = 0, g_selftest_recomputed = 0;   // of this thread's last self-test
 bool test_take_qr_give_up() { return take_one(g_inj_qr_give_up); }
 bool test_take_alloc_fail() { return take_one(g_inj_alloc_fail); }
 
@@ -339,6 +341,7 @@ void gemm(ttn_ctx* c, const GemmArgs& g) {
                 n = launch_split_pack(g, c->stream, c->split_ws, c->split_cap);
             }
             if (n >= 0) {
+                c->last_path = TTN_PATH_SPLIT;
                 ProfScope ps(c, PK_TC, fl, 0.5 * need + nb * (double)g.M * g.N * 16.0, &g);
                 int m = launch_split_mma(g, c->stream, c->split_ws, c->split_cap);
                 if (m < 0) throw TtnError(TTN_ERR_CUDA, "split GEMM launch failed after packing");
@@ -351,10 +354,14 @@ void gemm(ttn_ctx* c, const GemmArgs& g) {
         if (try_grow_split_ws(c, need)) {   // no room: the FP64 kernels below need none
             ProfScope ps(c, PK_F64, fl, 0.0, &g);
             n = launch_zgemm_digits(g, true, c->stream, c->split_ws, c->split_cap);
-            if (n >= 0) c->digits_run = true;
+            if (n >= 0) {
+                c->digits_run = true;
+                c->last_path = TTN_PATH_F64_DIGITS;
+            }
         }
     }
     if (n < 0) {
+        c->last_path = f64_direct(g) ? TTN_PATH_F64_DIRECT : TTN_PATH_F64_TILES;
         const size_t wb = f64_workspace_bytes(g);
         if (wb > c->f64_cap) {   // split-K partials of small-output FP64 contractions
             CUDA_OK(cudaStreamSynchronize(c->stream));
@@ -1324,10 +1331,12 @@ int gauge_qr(ttn_ctx* c, cplx*& A, cplx*& spare, int M, int D, cplx* R, const in
         c->stats[3] += nl;
         return ndep;
     };
+    c->last_path = TTN_PATH_QR_COLUMNS;
     if (!spare || qr_one_block(M, D)) return columns(A, false);   // one block: one way to split its rows
     auto done = [&](int how, int ndep) {
         std::swap(A, spare);
         hint = how;
+        if (how != QR_ILL_CONDITIONED) c->last_path = how == QR_PANELS ? TTN_PATH_QR_PANELS : TTN_PATH_QR_COLUMNS_FINE;
         return ndep;
     };
     const bool panels = panel_applies(M, D) && try_grow_split_ws(c, qr_panel_workspace(M, D));
@@ -2599,6 +2608,8 @@ ttn_status ttn_selftest_qr(const double* A, int M, int D, const int* cand, int n
         cudaEventDestroy(e1);
         CUDA_OK(cudaGetLastError());
         check_digits(&tmp);
+        g_selftest_path = tmp.last_path;
+        g_selftest_recomputed = 0;
         CUDA_OK(cudaMemcpy(Q, dA, sizeof(cplx) * (size_t)M * D, cudaMemcpyDeviceToHost));
         CUDA_OK(cudaMemcpy(R, dR, sizeof(cplx) * (size_t)D * D, cudaMemcpyDeviceToHost));
         if (n_dependent) *n_dependent = ndep;
@@ -2652,9 +2663,20 @@ ttn_status ttn_selftest_contract_host(const double* A, const double* B, double* 
         CUDA_OK(cudaGetLastError());
         check_split_flag(&tmp);
         CUDA_OK(cudaMemcpy(Cout, dC, sizeof(cplx) * (size_t)M * N, cudaMemcpyDeviceToHost));
+        g_selftest_path = tmp.last_path;
+        g_selftest_recomputed = 0;
+        if (tmp.last_path == TTN_PATH_F64_DIGITS)
+            CUDA_OK(cudaMemcpy(&g_selftest_recomputed, (int*)tmp.split_ws + 1, sizeof(int), cudaMemcpyDeviceToHost));
         if (path) *path = tc ? 1 : 0;
         if (ms) *ms = t;
     });
+}
+
+ttn_status ttn_selftest_last_path(int* path, int* recomputed) {
+    if (!path) return TTN_ERR_ARG;
+    *path = g_selftest_path;
+    if (recomputed) *recomputed = g_selftest_recomputed;
+    return TTN_OK;
 }
 
 ttn_status ttn_selftest_fp64_peak(int method, double* tflops) {

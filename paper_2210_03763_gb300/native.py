@@ -67,6 +67,7 @@ SIGNATURES = [
     ("ttn_contract_split_noalloc", ctypes.c_int, [_P, _P, _P, ctypes.c_int, ctypes.c_int, ctypes.c_int, _P]),
     ("ttn_selftest_contract_host", ctypes.c_int, [_D, _D, _D, ctypes.c_int, ctypes.c_int, ctypes.c_int,
                                                   ctypes.c_int, _I, ctypes.POINTER(ctypes.c_float)]),
+    ("ttn_selftest_last_path", ctypes.c_int, [_I, _I]),
     ("ttn_selftest_fp64_peak", ctypes.c_int, [ctypes.c_int, _D]),
     ("ttn_test_inject", ctypes.c_int, [ctypes.c_int, ctypes.c_longlong]),
     ("ttn_svd_truncate", ctypes.c_int, [_D, ctypes.c_int, ctypes.c_int, ctypes.c_int, ctypes.c_double, _D, _D, _D,
@@ -146,6 +147,19 @@ def contract_host(A, B, precision):
     if st != 0:
         raise TTNError(st, "selftest_contract_host(%d, %d, %d)" % (M, N, K))
     return C, bool(path.value), ms.value
+
+
+PATHS = ("f64_direct", "f64_tiles", "f64_digits", "split", "qr_columns", "qr_columns_fine", "qr_panels")
+
+
+def selftest_last_path():
+    """(name of the kernels that this thread's last contract_host or
+    selftest_qr ran, outputs of a digit contraction left to FMA chains)."""
+    path, n = ctypes.c_int(0), ctypes.c_int(0)
+    st = load().ttn_selftest_last_path(ctypes.byref(path), ctypes.byref(n))
+    if st != 0:
+        raise TTNError(st, "selftest_last_path")
+    return PATHS[path.value], n.value
 
 
 def fp64_peak(method=0):
