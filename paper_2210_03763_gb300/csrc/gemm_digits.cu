@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(PK_THREADS) digit_pack_kernel(DigitSide sp, Di
                                                                int one_pass, int* marked, const int* skip) {
     pdl_begin();
     if (skip && *(volatile const int*)skip) return;
-    if (marked && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) *marked = 0;
+    if (marked && blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) marked[0] = marked[1] = 0;
     const bool isp = (int)blockIdx.x < nbp;
     const DigitSide& s = isp ? sp : sq;
     const long long f0 = (long long)(isp ? blockIdx.x : blockIdx.x - nbp) * PK_ROWS;
@@ -327,7 +327,8 @@ struct DigitGemm {
     // outputs left to digit_fix_kernel, null: none; bit i of word ((b n_qtiles +
     // qt) Pp + p): complex Q row 32 qt + i
     uint32_t* mask;
-    int* marked;                 // how many
+    int* marked;                 // [0] how many, [1] in how many words
+    uint32_t* list;              // those words, in any order
     const uint16_t *magP, *magQ;
     const unsigned long long *l1P, *l1Q;
     int Kc;
@@ -439,17 +440,25 @@ __device__ __forceinline__ void store_output(const DigitGemm& ea, int m, int n, 
 // bound is 2 K 2^-53 S: marked is what has S < (l_p + l_q) / (16 K) + 2^-8, except
 // S = 0 (every product zero, and so is the digits' result), and rows with
 // infinities or NaNs.  Operands of one size reach the threshold within the
-// first few dozen K, and the warp stops there: only graded and sparse rows
-// are summed to the end.  The order of K is free, so a lane loads 16 bytes of
-// a row and feeds them to two k16 steps.
-constexpr int CK_THREADS = 128;
+// first few dozen K and stop there: only graded and sparse rows are summed to
+// the end.  For a long K and few outputs that is a chain of loads (128 x 128 x
+// 16384: 390 us with a warp per 32 x 32 tile), so there (LONG) one of a block's 4
+// warps looks at the first 128 K, and if that is not enough all of them share
+// the tile's K, load ahead, and add their sums in a fixed order (109 us; the
+// step below 1.83 -> 1.74 s).  The order of K is free, so a lane loads 16 bytes of a
+// row and feeds them to two k16 steps.
+constexpr int CK_WARPS = 4, CK_THREADS = 32 * CK_WARPS;
+template <bool LONG>
 __global__ void __launch_bounds__(CK_THREADS) digit_check_kernel(DigitGemm ea) {
     pdl_begin();
+    __shared__ float sums[LONG ? CK_WARPS : 1][32][32];   // [warp][accumulator][lane]
+    __shared__ int s_more;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int nqc = ea.n_qtiles, npc = ea.Pp / 64, nq2 = (nqc + 1) / 2;   // 32-wide Q groups, 64 x 64 blocks
-    const int blk = (int)(blockIdx.x % (unsigned)(npc * nq2)), b = (int)(blockIdx.x / (unsigned)(npc * nq2));
-    const int p0 = (blk % npc) * 64 + (warp & 1) * 32, qt = (blk / npc) * 2 + (warp >> 1), q0 = qt * 32;
-    if (qt >= nqc) return;
+    const int nqc = ea.n_qtiles, npc = ea.Pp / 32;   // 32 x 32 outputs per warp (LONG: per block)
+    const long long tile = LONG ? blockIdx.x : (long long)blockIdx.x * CK_WARPS + warp;
+    if (tile >= (long long)npc * nqc * ea.batches) return;
+    const int b = (int)(tile / (npc * nqc)), rest = (int)(tile % (npc * nqc));
+    const int p0 = rest % npc * 32, qt = rest / npc, q0 = qt * 32;
     const long long prow = first_row(ea, b, ea.p_vbi, ea.p_vbo, ea.Pp) + p0;
     const long long qrow = first_row(ea, b, ea.q_vbi, ea.q_vbo, ea.Qp) / 2 + q0;
     const int g8 = lane >> 2, j4 = lane & 3;
@@ -496,7 +505,9 @@ __global__ void __launch_bounds__(CK_THREADS) digit_check_kernel(DigitGemm ea) {
                 w |= __shfl_xor_sync(0xffffffffu, w, 1);
                 w |= __shfl_xor_sync(0xffffffffu, w, 2);
                 if (j4 == 0) {
-                    ea.mask[((long long)b * nqc + qt) * ea.Pp + p0 + g8 + 8 * i] = w;
+                    const long long word = ((long long)b * nqc + qt) * ea.Pp + p0 + g8 + 8 * i;
+                    ea.mask[word] = w;
+                    if (w) ea.list[atomicAdd(ea.marked + 1, 1)] = (uint32_t)word;
                     n += __popc(w);
                 }
             }
@@ -507,15 +518,17 @@ __global__ void __launch_bounds__(CK_THREADS) digit_check_kernel(DigitGemm ea) {
     };
     const uint16_t* mp = ea.magP + (prow + g8) * ea.Kc;
     const uint16_t* mq = ea.magQ + (qrow + g8) * ea.Kc;
-    for (int k0 = 0, it = 1; k0 < ea.Kc; k0 += 32, ++it) {
-        const int k = k0 + 8 * j4;
+    uint4 a[4], bq[4];
+    auto load = [&](int slice, uint4* x, uint4* y) {   // 32 K of every row
+        const int k = 32 * slice + 8 * j4;
         const bool in = k < ea.Kc;             // Kc is a multiple of 16
-        uint4 a[4], bq[4];
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-            a[i] = in ? *reinterpret_cast<const uint4*>(mp + 8LL * i * ea.Kc + k) : make_uint4(0, 0, 0, 0);
-            bq[i] = in ? *reinterpret_cast<const uint4*>(mq + 8LL * i * ea.Kc + k) : make_uint4(0, 0, 0, 0);
+            x[i] = in ? *reinterpret_cast<const uint4*>(mp + 8LL * i * ea.Kc + k) : make_uint4(0, 0, 0, 0);
+            y[i] = in ? *reinterpret_cast<const uint4*>(mq + 8LL * i * ea.Kc + k) : make_uint4(0, 0, 0, 0);
         }
+    };
+    auto multiply = [&] {
 #pragma unroll
         for (int i = 0; i < 2; ++i)
 #pragma unroll
@@ -528,88 +541,124 @@ __global__ void __launch_bounds__(CK_THREADS) digit_check_kernel(DigitGemm ea) {
                              : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
                              : "r"(a[2 * i].z), "r"(a[2 * i + 1].z), "r"(a[2 * i].w), "r"(a[2 * i + 1].w), "r"(bq[j].z), "r"(bq[j].w));
             }
-        if ((it & 3) == 0 && !__any_sync(0xffffffffu, marks(false))) break;
+    };
+    const int slices = (ea.Kc + 31) / 32;
+    auto sum_slices = [&](int first, int step, bool stop) {   // the next one in flight
+        uint4 an[4], bn[4];
+        load(first, a, bq);
+        for (int it = first; it < slices; it += step) {
+            load(it + step, an, bn);
+            multiply();
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                a[i] = an[i];
+                bq[i] = bn[i];
+            }
+            if (stop && (it & 3) == 3 && !__any_sync(0xffffffffu, marks(false))) break;
+        }
+    };
+    if (!LONG) {
+        sum_slices(0, 1, true);
+        marks(true);
+        return;
     }
-    marks(true);
+    if (warp == 0) {   // are the first four slices enough?
+        for (int it = 0; it < 4; ++it) {
+            load(it, a, bq);
+            multiply();
+        }
+        const bool more = __any_sync(0xffffffffu, marks(false));
+        if (lane == 0) s_more = more;
+    }
+    __syncthreads();
+    if (s_more) {
+        float* d = &acc[0][0][0];
+#pragma unroll
+        for (int i = 0; i < 32; ++i) d[i] = 0.f;
+        sum_slices(warp, CK_WARPS, false);
+#pragma unroll
+        for (int i = 0; i < 32; ++i) sums[warp][i][lane] = d[i];
+        __syncthreads();
+        if (warp == 0)
+#pragma unroll
+            for (int i = 0; i < 32; ++i)
+                for (int w = 1; w < CK_WARPS; ++w) d[i] += sums[w][i][lane];
+    }
+    if (warp == 0) marks(true);
 }
 
-// The marked outputs in plain FP64.  A block takes 256 words of the mask (8192
-// outputs) at a time, lists its marked outputs and gives each 1 to 32 lanes,
-// as many as keep its 256 threads busy; the lanes' sums are added in a fixed
-// order.
-constexpr int FX_THREADS = 256;
+// The marked outputs in plain FP64.  Few are marked, often of a long K, so the
+// words that hold any are spread over the SMs, each to W warps, as many as there
+// are warps for (1 to all 8 of a block), and a word's outputs share its 32 W
+// lanes, each summing every L-th K; the lanes' sums are added in a fixed
+// order.  Measured, a step of 8x8, chi = 128 from a product state, 0.01 to 2 % of
+// the outputs of its K = 10368 and 16384 contractions marked: 2.90 s with
+// 256 words to a block wherever their marked outputs lie, 1.83 s so.
+constexpr int FX_THREADS = 256, FX_WARPS = FX_THREADS / 32;
 __global__ void __launch_bounds__(FX_THREADS) digit_fix_kernel(DigitGemm ea) {
     pdl_begin();
-    if (*(volatile int*)ea.marked == 0) return;
-    __shared__ uint16_t list[FX_THREADS * 32];
-    __shared__ int wsum[FX_THREADS / 32];
-    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int nwords = *(volatile int*)(ea.marked + 1);
+    if (nwords == 0) return;
+    __shared__ cplx part[FX_WARPS];
     const GemmArgs& g = ea.g;
     const int K = g.Ki * g.Ko;
-    const long long words = (long long)ea.batches * ea.n_qtiles * ea.Pp;   // a multiple of 128
-    for (long long w0 = (long long)blockIdx.x * FX_THREADS; w0 < words; w0 += (long long)gridDim.x * FX_THREADS) {
-        unsigned w = w0 + t < words ? ea.mask[w0 + t] : 0u;
-        int pos = __popc(w);
-        for (int o = 1; o < 32; o *= 2) {
-            const int v = __shfl_up_sync(0xffffffffu, pos, o);
-            if (lane >= o) pos += v;
-        }
-        __syncthreads();   // the list of the last round has been read
-        if (lane == 31) wsum[warp] = pos;
-        __syncthreads();
-        int n = 0;
-        pos -= __popc(w);
-        for (int q = 0; q < FX_THREADS / 32; ++q) {
-            if (q < warp) pos += wsum[q];
-            n += wsum[q];
-        }
-        while (w) {
-            const int i = __ffs((int)w) - 1;
-            w &= w - 1;
-            list[pos++] = (uint16_t)(t * 32 + i);
-        }
-        __syncthreads();
-        int L = 1;
-        while (L < 32 && n * L * 2 <= FX_THREADS) L *= 2;
-        for (int e0 = 0; e0 < n; e0 += FX_THREADS / L) {
-            const int e = e0 + t / L;
-            cplx s = make_double2(0.0, 0.0);
-            int m = 0, nn = 0, bi = 0, bo = 0, b = 0;
-            if (e < n) {
-                const long long word = w0 + (list[e] >> 5);
-                const int p = (int)(word % ea.Pp);
-                const long long rest = word / ea.Pp;
-                const int q = (int)(rest % ea.n_qtiles) * 32 + (list[e] & 31);
-                b = (int)(rest / ea.n_qtiles);
-                bi = b % g.Bi;
-                bo = b / g.Bi;
-                m = ea.swapped ? q : p;
-                nn = ea.swapped ? p : q;
-                const cplx* A = g.A + bi * g.a_bi + bo * g.a_bo + m * g.a_m;
-                const cplx* B = g.B + bi * g.b_bi + bo * g.b_bo + nn * g.b_n;
+    int W = 1;
+    while (W < FX_WARPS && (long long)nwords * W * 2 <= (long long)gridDim.x * FX_WARPS) W *= 2;
+    const int per = FX_WARPS / W, grp = (int)threadIdx.x / (32 * W), t = (int)threadIdx.x % (32 * W);
+    for (long long i0 = (long long)blockIdx.x * per; i0 < nwords; i0 += (long long)gridDim.x * per) {
+        const bool on = i0 + grp < nwords;
+        const uint32_t word = on ? ea.list[i0 + grp] : 0u;
+        uint32_t w = on ? ea.mask[word] : 0u;
+        const int n = max(1, __popc(w));
+        int L = W;                              // n <= 32: lanes per output
+        while (n * L * 2 <= 32 * W) L *= 2;
+        const int o = t / L;                    // output of the word
+        const bool mine = o < __popc(w);
+        cplx s = make_double2(0.0, 0.0);
+        int m = 0, nn = 0, bi = 0, bo = 0, b = 0;
+        if (mine) {
+            for (int i = 0; i < o; ++i) w &= w - 1;
+            const int p = (int)(word % (uint32_t)ea.Pp), rest = (int)(word / (uint32_t)ea.Pp);
+            const int q = rest % ea.n_qtiles * 32 + __ffs((int)w) - 1;
+            b = rest / ea.n_qtiles;
+            bi = b % g.Bi;
+            bo = b / g.Bi;
+            m = ea.swapped ? q : p;
+            nn = ea.swapped ? p : q;
+            const cplx* A = g.A + bi * g.a_bi + bo * g.a_bo + m * g.a_m;
+            const cplx* B = g.B + bi * g.b_bi + bo * g.b_bo + nn * g.b_n;
 #pragma unroll 4
-                for (int k = t % L; k < K; k += L) {
-                    const int ki = k % g.Ki, ko = k / g.Ki;
-                    cplx a = A[ki * g.a_ki + ko * g.a_ko], v = B[ki * g.b_ki + ko * g.b_ko];
-                    if (g.conjA) a.y = -a.y;
-                    if (g.conjB) v.y = -v.y;
-                    s.x = fma(a.x, v.x, s.x);
-                    s.x = fma(-a.y, v.y, s.x);
-                    s.y = fma(a.x, v.y, s.y);
-                    s.y = fma(a.y, v.x, s.y);
-                }
+            for (int k = t % L; k < K; k += L) {
+                const int ki = k % g.Ki, ko = k / g.Ki;
+                cplx a = A[ki * g.a_ki + ko * g.a_ko], v = B[ki * g.b_ki + ko * g.b_ko];
+                if (g.conjA) a.y = -a.y;
+                if (g.conjB) v.y = -v.y;
+                s.x = fma(a.x, v.x, s.x);
+                s.x = fma(-a.y, v.y, s.x);
+                s.y = fma(a.x, v.y, s.y);
+                s.y = fma(a.y, v.x, s.y);
             }
-            for (int o = L / 2; o > 0; o /= 2) {
-                s.x += __shfl_xor_sync(0xffffffffu, s.x, o);
-                s.y += __shfl_xor_sync(0xffffffffu, s.y, o);
-            }
-            if (e < n && t % L == 0) {
-                if (ea.nsplit > 1) {   // the whole sum in the first range's place
-                    for (int ks = 0; ks < ea.nsplit; ++ks)
-                        ea.W[(((long long)ks * ea.batches + b) * g.N + nn) * g.M + m] = ks ? make_double2(0.0, 0.0) : s;
-                } else {
-                    store_output(ea, m, nn, bi, bo, s);
+        }
+        for (int d = min(L, 32) / 2; d > 0; d /= 2) {   // a warp has one L
+            s.x += __shfl_xor_sync(0xffffffffu, s.x, d);
+            s.y += __shfl_xor_sync(0xffffffffu, s.y, d);
+        }
+        if (W > 1) {   // L > 32: the warps of an output
+            __syncthreads();
+            if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+            __syncthreads();
+            if (mine && t % L == 0)
+                for (int i = 1; i < L / 32; ++i) {
+                    s.x += part[(threadIdx.x >> 5) + i].x;
+                    s.y += part[(threadIdx.x >> 5) + i].y;
                 }
+        }
+        if (mine && t % L == 0) {
+            if (ea.nsplit > 1) {   // the whole sum in the first range's place
+                for (int ks = 0; ks < ea.nsplit; ++ks)
+                    ea.W[(((long long)ks * ea.batches + b) * g.N + nn) * g.M + m] = ks ? make_double2(0.0, 0.0) : s;
+            } else {
+                store_output(ea, m, nn, bi, bo, s);
             }
         }
     }
@@ -839,7 +888,7 @@ struct DPlan {
     DigitGemm d{};
     long long np = 0, nq = 0;             // packed batches of P and Q
     int Kp = 0;
-    size_t p_off = 0, q_off = 0, ep_off = 0, eq_off = 0, lp_off = 0, lq_off = 0, mp_off = 0, mq_off = 0, mask_off = 0, w_off = 0, bytes = 0;
+    size_t p_off = 0, q_off = 0, ep_off = 0, eq_off = 0, lp_off = 0, lq_off = 0, mp_off = 0, mq_off = 0, mask_off = 0, list_off = 0, w_off = 0, bytes = 0;
 };
 
 DPlan plan(const GemmArgs& g, bool elementwise) {
@@ -906,10 +955,12 @@ DPlan plan(const GemmArgs& g, bool elementwise) {
         pl.mp_off = take((size_t)pl.np * d.Pp * d.Kc * 2);
         pl.mq_off = take((size_t)pl.nq * (d.Qp / 2) * d.Kc * 2);
         pl.mask_off = take(sizeof(uint32_t) * (size_t)d.batches * d.n_qtiles * d.Pp);
+        pl.list_off = take(sizeof(uint32_t) * (size_t)d.batches * d.n_qtiles * d.Pp);
     }
     if (d.nsplit > 1) pl.w_off = take((size_t)d.nsplit * d.batches * g.M * (size_t)g.N * sizeof(cplx));
     pl.bytes = off;
-    pl.ok = pl.np * d.Pp < (1LL << 31) && pl.nq * d.Qp < (1LL << 31);
+    pl.ok = pl.np * d.Pp < (1LL << 31) && pl.nq * d.Qp < (1LL << 31) &&
+            (long long)d.batches * d.n_qtiles * d.Pp < (1LL << 31);   // words of the mask
     return pl;
 }
 
@@ -1058,11 +1109,14 @@ int launch_zgemm_digits(const GemmArgs& g, bool elementwise, cudaStream_t stream
     d.stall_ns = test_take_tc_stall();
     if (elementwise) {
         d.mask = reinterpret_cast<uint32_t*>(ws + pl.mask_off);
+        d.list = reinterpret_cast<uint32_t*>(ws + pl.list_off);
         d.magP = sp.mag;
         d.magQ = sq.mag;
         d.l1P = sp.l1;
         d.l1Q = sq.l1;
-        launch(digit_check_kernel, (unsigned)((d.Pp / 64) * ((d.n_qtiles + 1) / 2) * d.batches), CK_THREADS, 0, stream, d);
+        const long long tiles = (long long)(d.Pp / 32) * d.n_qtiles * d.batches;
+        if (d.Kc >= 8192 && tiles < 4 * N_SM) launch(digit_check_kernel<true>, (unsigned)tiles, CK_THREADS, 0, stream, d);
+        else launch(digit_check_kernel<false>, (unsigned)((tiles + CK_WARPS - 1) / CK_WARPS), CK_THREADS, 0, stream, d);
         ++launches;
     }
     const long long nt = (long long)d.n_ptiles * d.n_qtiles * d.batches * d.nsplit;
@@ -1070,8 +1124,9 @@ int launch_zgemm_digits(const GemmArgs& g, bool elementwise, cudaStream_t stream
     ++launches;
     if (elementwise) {
         const long long words = (long long)d.batches * d.n_qtiles * d.Pp;
-        launch(digit_fix_kernel, (unsigned)std::min<long long>((words + FX_THREADS - 1) / FX_THREADS, N_SM), FX_THREADS, 0,
-               stream, d);
+        // a block per 256 words and 1024 of K: blocks that find nothing to do still cost their start
+        const long long blocks = (words + 255) / 256 * (1 + d.Kc / 1024);
+        launch(digit_fix_kernel, (unsigned)std::min<long long>(blocks, N_SM), FX_THREADS, 0, stream, d);
         ++launches;
     }
     if (d.nsplit > 1) launches += launch_splitk_f64(g, d.nsplit, d.W, stream);

@@ -39,7 +39,7 @@ def _check(native, A, B, rows=37, cols=29):
     assert np.all(err <= bound), float(np.max(err / np.where(bound > 0, bound, 1)))
 
 
-SHAPES = [(600, 400, 64), (4097, 65, 65), (300, 300, 500), (64, 96, 4096)]
+SHAPES = [(600, 400, 64), (4097, 65, 65), (300, 300, 500), (64, 96, 4096), (97, 65, 9001)]
 
 
 @pytest.mark.parametrize("M,N,K", SHAPES)
@@ -63,8 +63,9 @@ def test_identity_with_noise_times_triangle(native):
     _check(native, np.eye(n) + 1e-10 * A, np.triu(B))
 
 
-def test_sparse_operands_with_disjoint_supports(native):
-    A, B = _rand(600, 400, 128, 5)
+@pytest.mark.parametrize("M,N,K", [(600, 400, 128), (97, 400, 9001)])
+def test_sparse_operands_with_disjoint_supports(native, M, N, K):
+    A, B = _rand(M, N, K, 5)
     A[:, ::2] = 0
     B[1::2] = 0
     B[1, 7::50] = 1e-30
