@@ -394,7 +394,7 @@ def main():
                 "peak_source": "%s bf16_tflops_sustained x 1.1/2.25 (nominal TF32:BF16), of %s" % (
                     peak_kind, peak_kind),
                 "traffic": tc_traffic(), "launches": tc["launches"] / n_prof,
-                "traffic_source": "ncu dram__bytes_read+write per launch, mean over the first 2500 tc_gemm "
+                "traffic_source": "ncu dram__bytes_read+write per launch, mean over the first 1740 tc_gemm "
                                   "launches of the timed 8x8 chi=128 step (profiles/tc_gemm_8x8_chi128_slice.md)",
                 "share_of_step": tc["ms"] / (p_secs * 1e3),
                 "flops_counted": "algorithmic 8*M*N*K per complex contraction; tensor pipe executes 3x"}

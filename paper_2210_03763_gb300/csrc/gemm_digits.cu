@@ -35,11 +35,11 @@
 // in steps and observables of this library 0 to 0.02 % of the outputs are marked.
 //
 // Why: GB300's FP64 pipe gives 1.06 TFLOP/s; 34 bf16 products give one FP64
-// product at up to 1908 / 34 = 56 TFLOP/s.  Measured, packing included, against
-// the FMA kernels: 128 x 16384 x 128 in batches of 16 28.1 -> 2.04 ms (16.8
-// TFLOP/s), 128 x 128 x 16384 in batches of 16 40 -> 2.9 ms, 4096 x 64 x 64 in
-// batches of 4 464 -> 64 us, 64 x 4096 x 256 463 -> 99 us (55 and 93 us since
-// the MMAs are issued from a uniform warp).
+// product at up to 1908 / 34 = 56 TFLOP/s.  Measured, packing and check included,
+// against the FMA kernels: 16384 x 128 x 128 in batches of 16 28.1 -> 1.19 ms (28.9
+// TFLOP/s), 128 x 128 x 16384 in batches of 16 from a product state 40 -> 2.75 ms
+// (1.65 before the outputs were checked), 4096 x 64 x 64 in batches of 4 464 -> 58
+// us, 64 x 4096 x 256 463 -> 91 us.
 //
 // Complex numbers use the real embedding of gemm_split.cu: P rows hold
 // (Re, Im) pairs, Q rows 2n and 2n + 1 hold (Re, -Im) and (Im, Re).
