@@ -174,7 +174,7 @@ struct KrylovStatus {
 struct HostStatus {
     KrylovStatus krylov[KRYLOV_MMAX];   // per Krylov step (one-launch runs: [0])
     int tc_flag;                        // a tensor-core wait gave up
-    int qr_flag;                        // panel QR: not well-conditioned
+    int qr_flag;                        // panel QR: not well-conditioned (2: as good as dependent columns)
     int qr_dep[256];                    // column loop: dependent columns (no report when a block gave up)
     unsigned seq;
 };

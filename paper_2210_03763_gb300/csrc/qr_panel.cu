@@ -45,6 +45,7 @@ constexpr int PB = QR_PANEL;       // panel width
 constexpr int CT = 512;            // threads of the Cholesky kernel
 constexpr double MIN_COL2 = 1e-8;  // residual^2 / |column|^2
 constexpr double MIN_FRO2 = 1e-16; // residual^2 / |A|_F^2
+constexpr double DEP_COL2 = 1e-14; // below: as good as a dependent column (flag 2)
 constexpr int MAX_EXP = 480;       // |A| = 2^+-480 and beyond: squares leave the FP64 range
 constexpr int ST = 512;            // threads of the scaling kernel
 constexpr int FT = 1024;           // threads of the finishing kernel
@@ -104,7 +105,7 @@ __global__ void __launch_bounds__(ST) panel_scale_kernel(const cplx* A, int M, c
 // nullptr: none) = L L^H; T = L^-H into rows [n, n + bp) of C (leading
 // dimension ld).  One block: right-looking Cholesky, the same eliminations
 // applied to the identity give L^-1.  pass 2 expects a matrix near the
-// identity.  Sets *flag when a pivot is too small: cn2, cexp are the squared
+// identity.  Sets *flag when a pivot is too small (2: down to rounding): cn2, cexp are the squared
 // norms and exponents of all D scaled columns, the panel's first is column n.
 __global__ void __launch_bounds__(CT) panel_chol_kernel(const cplx* Sw, long long ld, const cplx* Gq, int bp, cplx* C,
                                                         const double* cn2, const int* cexp, int D, int n, int pass,
@@ -147,12 +148,12 @@ __global__ void __launch_bounds__(CT) panel_chol_kernel(const cplx* Sw, long lon
         if (t == 0) {
             const double d = G[k][k].x;
             const bool ok = pass == 1 ? (d >= MIN_COL2 * norm2[k] && d > floor2[k]) : d >= 0.25;
-            if (!ok || !isfinite(d)) bad = 1;
+            if (!ok || !isfinite(d)) bad = pass == 1 && d <= DEP_COL2 * norm2[k] ? 2 : 1;
             s_inv = rsqrt(d);
         }
         __syncthreads();
         if (bad) {
-            if (t == 0) *flag = 1;
+            if (t == 0) *flag = bad;
             return;
         }
         const double inv = s_inv;
@@ -240,20 +241,17 @@ __device__ bool r_refused(const double* col2, const double* diag, int D, double 
 }
 
 // R = Q^H A made upper triangular with a real diagonal, and the residuals
-// checked once more on the final R (the Gram matrices know them less well):
-// sets *flag as panel_chol_kernel.  One block.
+// checked once more on the final R (the Gram matrices know them less well).
+// One block.
 __global__ void __launch_bounds__(FT) panel_finish_kernel(cplx* R, int D, int* flag, Publish pub) {
     pdl_begin();
     __shared__ double col2[256], diag[256];
-    const bool gave_up = *(volatile int*)flag != 0;   // R has not been written
+    const int gave_up = *(volatile int*)flag;   // R has not been written
     __syncthreads();
     if (!gave_up) r_columns(R, D, true, col2, diag);
     if (threadIdx.x >= 32) return;
-    const bool bad = gave_up || r_refused(col2, diag, D, 1.0);
-    if (threadIdx.x == 0) {
-        if (bad) *flag = 1;
-        panel_publish(pub, bad);
-    }
+    const int bad = gave_up ? gave_up : (int)r_refused(col2, diag, D, 1.0);
+    if (threadIdx.x == 0) panel_publish(pub, bad);
 }
 
 // The final check on another QR's R: its diagonal agrees with the panels' to

@@ -1370,6 +1370,8 @@ int gauge_qr(ttn_ctx* c, cplx*& A, cplx*& spare, int M, int D, cplx* R, const in
         }
         if (!gave_up) return done(QR_PANELS, 0);
     }
+    // the likelier way of the two first
+    if (!full_rank && panels && c->hstat->qr_flag == 1 && columns(spare, false) == 0) return done(QR_ILL_CONDITIONED, 0);
     if (!full_rank)
         if (const int ndep = columns(spare, true)) return done(QR_DEPENDENT, ndep);
     return done(QR_ILL_CONDITIONED, columns(spare, false));
