@@ -349,7 +349,7 @@ void gemm(ttn_ctx* c, const GemmArgs& g) {
             }
         }
     }
-    if (n < 0 && digits_wanted(g)) {   // large FP64 contractions: exact digit products on the tensor cores
+    if (n < 0 && digits_wanted(g)) {   // large FP64 contractions: digit products on the tensor cores
         const size_t need = digits_workspace_bytes(g, true);
         if (try_grow_split_ws(c, need)) {   // no room: the FP64 kernels below need none
             ProfScope ps(c, PK_F64, fl, 0.0, &g);
@@ -1317,9 +1317,10 @@ enum QrHint { QR_UNKNOWN = 0, QR_PANELS, QR_DEPENDENT, QR_ILL_CONDITIONED };
 // diagonal below the panels' limits is refused by the panels whatever order is
 // tried, so after a bond that had dependent columns or was ill-conditioned last
 // time the column loop goes first and the panels are left out if it confirms
-// that.  Every attempt works in `spare`, swapped with A in the end (small
-// matrices, and without a spare: the column loop in place).  Returns the
-// dependent columns.
+// that.  (The two row splits agree on the dependent columns unless a residual
+// lies within rounding of the threshold.)  Every attempt works in `spare`,
+// swapped with A in the end (small matrices, and without a spare: the column
+// loop in place).  Returns the dependent columns.
 int gauge_qr(ttn_ctx* c, cplx*& A, cplx*& spare, int M, int D, cplx* R, const int* cand, int ncand, QrScratch& q,
              int& hint) {
     auto columns = [&](cplx* X, bool fine) {
