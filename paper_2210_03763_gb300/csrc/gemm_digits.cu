@@ -587,11 +587,54 @@ __global__ void __launch_bounds__(CK_THREADS) digit_check_kernel(DigitGemm ea) {
     if (warp == 0) marks(true);
 }
 
-// The marked outputs in plain FP64.  Few are marked, often of a long K, so the
-// words that hold any are spread over the SMs, each to W warps, as many as there
-// are warps for (1 to all 8 of a block), and a word's outputs share its 32 W
-// lanes, each summing every L-th K; the lanes' sums are added in a fixed
-// order.  Measured, a step of 8x8, chi = 128 from a product state, 0.01 to 2 % of
+// sum over k in [k0, k1) of A_k B_k, one FMA chain.
+__device__ __forceinline__ cplx fma_chain(const GemmArgs& g, const cplx* A0, const cplx* B0, int k0, int k1) {
+    cplx s = make_double2(0.0, 0.0);
+    int ki = k0 % g.Ki, ko = k0 / g.Ki;
+    while (k0 < k1) {
+        const int run = min(g.Ki - ki, k1 - k0);
+        const cplx* A = A0 + ki * g.a_ki + ko * g.a_ko;
+        const cplx* B = B0 + ki * g.b_ki + ko * g.b_ko;
+#pragma unroll 4
+        for (int i = 0; i < run; ++i) {
+            cplx a = *A, v = *B;
+            if (g.conjA) a.y = -a.y;
+            if (g.conjB) v.y = -v.y;
+            s.x = fma(a.x, v.x, s.x);
+            s.x = fma(-a.y, v.y, s.x);
+            s.y = fma(a.x, v.y, s.y);
+            s.y = fma(a.y, v.x, s.y);
+            A += g.a_ki;
+            B += g.b_ki;
+        }
+        k0 += run;
+        ki = 0;
+        ++ko;
+    }
+    return s;
+}
+
+// A marked output's value to where the digits' would have gone.
+__device__ __forceinline__ void store_marked(const DigitGemm& ea, int m, int n, int b, cplx s) {
+    if (ea.nsplit > 1) {   // the whole sum in the first range's place
+        for (int ks = 0; ks < ea.nsplit; ++ks)
+            ea.W[(((long long)ks * ea.batches + b) * ea.g.N + n) * ea.g.M + m] = ks ? make_double2(0.0, 0.0) : s;
+    } else {
+        store_output(ea, m, n, b % ea.g.Bi, b / ea.g.Bi, s);
+    }
+}
+
+// The marked outputs in plain FP64.
+// Few are marked, often of a long K: the words that hold any are spread over the
+// SMs, each to W warps, as many as there are warps for (1 to all 8 of a block),
+// and a word's outputs share its 32 W lanes, each with a slice of K.
+// Many (an eighth and more: operands graded against each other): 32 outputs side
+// by side, one per lane, to a warp, or where there are too few of these for two
+// warps each, to a block whose 8 warps take a slice of K each, as the direct
+// kernel of gemm_f64.cu does (all marked, whole call: 16384 x 128 x 128 3.6 ms by
+// words, 3.3 so, 2.1 by the direct kernel; 128 x 128 x 16384 17.3, 4.0, 2.2).
+// Slices are added in order.
+// Measured, a step of 8x8, chi = 128 from a product state, 0.01 to 2 % of
 // the outputs of its K = 10368 and 16384 contractions marked: 2.90 s with
 // 256 words to a block wherever their marked outputs lie, 1.83 s so.
 constexpr int FX_THREADS = 256, FX_WARPS = FX_THREADS / 32;
@@ -599,12 +642,42 @@ __global__ void __launch_bounds__(FX_THREADS) digit_fix_kernel(DigitGemm ea) {
     pdl_begin();
     const int nwords = *(volatile int*)(ea.marked + 1);
     if (nwords == 0) return;
-    __shared__ cplx part[FX_WARPS];
+    __shared__ cplx part[FX_WARPS][32];
     const GemmArgs& g = ea.g;
-    const int K = g.Ki * g.Ko;
+    const int K = g.Ki * g.Ko, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (8LL * *(volatile int*)ea.marked >= (long long)g.M * g.N * ea.batches) {
+        const int mb = (g.M + 31) / 32;
+        const long long groups = (long long)mb * g.N * ea.batches;
+        const int S = groups < 2LL * gridDim.x * FX_WARPS ? FX_WARPS : 1, kc = (K + S - 1) / S;   // slices of K
+        const int slice = warp % S;
+        for (long long i = blockIdx.x * (FX_WARPS / S) + warp / S; i < groups; i += (long long)gridDim.x * (FX_WARPS / S)) {
+            const int m = (int)(i % mb) * 32 + lane;
+            const long long r = i / mb;
+            const int n = (int)(r % g.N), b = (int)(r / g.N), p = ea.swapped ? n : m, q = ea.swapped ? m : n;
+            const bool mine = m < g.M && ((ea.mask[((long long)b * ea.n_qtiles + (q >> 5)) * ea.Pp + p] >> (q & 31)) & 1u);
+            if (!__any_sync(0xffffffffu, mine)) continue;   // S > 1: the same in every warp of the block
+            cplx s = make_double2(0.0, 0.0);
+            if (mine)
+                s = fma_chain(g, g.A + (b % g.Bi) * g.a_bi + (b / g.Bi) * g.a_bo + m * g.a_m,
+                              g.B + (b % g.Bi) * g.b_bi + (b / g.Bi) * g.b_bo + n * g.b_n, min(K, slice * kc),
+                              min(K, (slice + 1) * kc));
+            if (S > 1) {
+                part[warp][lane] = s;
+                __syncthreads();
+                if (warp == 0)
+                    for (int w = 1; w < S; ++w) {
+                        s.x += part[w][lane].x;
+                        s.y += part[w][lane].y;
+                    }
+                __syncthreads();
+            }
+            if (mine && slice == 0) store_marked(ea, m, n, b, s);
+        }
+        return;
+    }
     int W = 1;
     while (W < FX_WARPS && (long long)nwords * W * 2 <= (long long)gridDim.x * FX_WARPS) W *= 2;
-    const int per = FX_WARPS / W, grp = (int)threadIdx.x / (32 * W), t = (int)threadIdx.x % (32 * W);
+    const int per = FX_WARPS / W, grp = warp / W, t = (int)threadIdx.x % (32 * W);
     for (long long i0 = (long long)blockIdx.x * per; i0 < nwords; i0 += (long long)gridDim.x * per) {
         const bool on = i0 + grp < nwords;
         const uint32_t word = on ? ea.list[i0 + grp] : 0u;
@@ -615,29 +688,18 @@ __global__ void __launch_bounds__(FX_THREADS) digit_fix_kernel(DigitGemm ea) {
         const int o = t / L;                    // output of the word
         const bool mine = o < __popc(w);
         cplx s = make_double2(0.0, 0.0);
-        int m = 0, nn = 0, bi = 0, bo = 0, b = 0;
+        int m = 0, nn = 0, b = 0;
         if (mine) {
             for (int i = 0; i < o; ++i) w &= w - 1;
             const int p = (int)(word % (uint32_t)ea.Pp), rest = (int)(word / (uint32_t)ea.Pp);
             const int q = rest % ea.n_qtiles * 32 + __ffs((int)w) - 1;
             b = rest / ea.n_qtiles;
-            bi = b % g.Bi;
-            bo = b / g.Bi;
             m = ea.swapped ? q : p;
             nn = ea.swapped ? p : q;
-            const cplx* A = g.A + bi * g.a_bi + bo * g.a_bo + m * g.a_m;
-            const cplx* B = g.B + bi * g.b_bi + bo * g.b_bo + nn * g.b_n;
-#pragma unroll 4
-            for (int k = t % L; k < K; k += L) {
-                const int ki = k % g.Ki, ko = k / g.Ki;
-                cplx a = A[ki * g.a_ki + ko * g.a_ko], v = B[ki * g.b_ki + ko * g.b_ko];
-                if (g.conjA) a.y = -a.y;
-                if (g.conjB) v.y = -v.y;
-                s.x = fma(a.x, v.x, s.x);
-                s.x = fma(-a.y, v.y, s.x);
-                s.y = fma(a.x, v.y, s.y);
-                s.y = fma(a.y, v.x, s.y);
-            }
+            const int kc = (K + L - 1) / L;
+            s = fma_chain(g, g.A + (b % g.Bi) * g.a_bi + (b / g.Bi) * g.a_bo + m * g.a_m,
+                          g.B + (b % g.Bi) * g.b_bi + (b / g.Bi) * g.b_bo + nn * g.b_n, min(K, t % L * kc),
+                          min(K, (t % L + 1) * kc));
         }
         for (int d = min(L, 32) / 2; d > 0; d /= 2) {   // a warp has one L
             s.x += __shfl_xor_sync(0xffffffffu, s.x, d);
@@ -645,22 +707,15 @@ __global__ void __launch_bounds__(FX_THREADS) digit_fix_kernel(DigitGemm ea) {
         }
         if (W > 1) {   // L > 32: the warps of an output
             __syncthreads();
-            if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = s;
+            if (lane == 0) part[warp][0] = s;
             __syncthreads();
             if (mine && t % L == 0)
                 for (int i = 1; i < L / 32; ++i) {
-                    s.x += part[(threadIdx.x >> 5) + i].x;
-                    s.y += part[(threadIdx.x >> 5) + i].y;
+                    s.x += part[warp + i][0].x;
+                    s.y += part[warp + i][0].y;
                 }
         }
-        if (mine && t % L == 0) {
-            if (ea.nsplit > 1) {   // the whole sum in the first range's place
-                for (int ks = 0; ks < ea.nsplit; ++ks)
-                    ea.W[(((long long)ks * ea.batches + b) * g.N + nn) * g.M + m] = ks ? make_double2(0.0, 0.0) : s;
-            } else {
-                store_output(ea, m, nn, bi, bo, s);
-            }
-        }
+        if (mine && t % L == 0) store_marked(ea, m, nn, b, s);
     }
 }
 
@@ -1123,10 +1178,7 @@ int launch_zgemm_digits(const GemmArgs& g, bool elementwise, cudaStream_t stream
     launch(digit_gemm_kernel, (unsigned)std::min<long long>(nt, N_SM), THREADS, SMEM_BYTES, stream, mP, mQ, d);
     ++launches;
     if (elementwise) {
-        const long long words = (long long)d.batches * d.n_qtiles * d.Pp;
-        // a block per 256 words and 1024 of K: blocks that find nothing to do still cost their start
-        const long long blocks = (words + 255) / 256 * (1 + d.Kc / 1024);
-        launch(digit_fix_kernel, (unsigned)std::min<long long>(blocks, N_SM), FX_THREADS, 0, stream, d);
+        launch(digit_fix_kernel, N_SM, FX_THREADS, 0, stream, d);
         ++launches;
     }
     if (d.nsplit > 1) launches += launch_splitk_f64(g, d.nsplit, d.W, stream);
